@@ -12,10 +12,10 @@
 // running. A row publishes itself by writing its epoch into a flag with release semantics;
 // dependants poll the flag with acquire loads (bounded: after Ilu::spin_limit polls the kernel
 // records a timeout and returns), and read data published in the same launch through L2
-// (ld.global.cg), never through L1. The triangular sweeps claim chunks of grid-line segments per
-// CTA, one segment per warp (see ilu_sweep_kernel), so that most dependencies are resolved in
-// registers and shared memory instead of L2.
+// (ld.global.cg), never through L1. The triangular sweeps read the finished factor from per-row
+// records in their own layout and claim chunks of grid-line segments per CTA (ilu_sweep_kernel).
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "precond.h"
@@ -26,11 +26,6 @@ namespace vms {
 namespace {
 
 constexpr int ILU_FWARPS = 4;    // warps per CTA of the factorisation
-// warps per CTA of the sweeps (one segment each). Measured on the 33^3-node lattice (FP32 apply):
-// 2 or 4 warps 0.244 ms, 8 warps 0.293 ms, 16 warps 0.269 ms, with one or several CTAs per SM
-// alike; FP64 rows keep the FP64 pipe of their SM partition busy for ~1000 cycles, so FP64 sweeps
-// spread over more SMs as well.
-template <typename T> constexpr int sweep_warps() { return 4; }
 constexpr unsigned FULL = 0xffffffffu;
 
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
@@ -168,419 +163,475 @@ __global__ void __launch_bounds__(ILU_FWARPS * 32)
 
 // ---------------------------------------------------------------------------------------------
 // sweeps: y = L^-1 v (rows ascending), z = U^-1 y (rows descending)
-// A warp solves the rows of one grid-line segment in order, one lane per neighbour block of the
-// row (a node has at most 32 neighbours; FP64 rows with at most 16 blocks on the sweep's side take
-// two lanes per block): every lane waits for its own neighbour at the same time.
+//
+// What bounds them: the dependency chain. A 27-point lattice of 33^3 nodes has 224 levels (128 steps
+// along a line, 64 to the next line, 32 to the next plane on the longest path), while a sweep's
+// data, 39 MB of FP32 records, would take 6 us of HBM. So everything off the chain is moved off the
+// warp that solves a row: values of earlier chunks are fetched by one warp, records by another, and
+// a row is one sum of block products without a test in its way. Measured on 33^3 nodes (jittered
+// cavity): FP32 sweep 239 -> 129 us, FP64 524 -> 260 us; 22^3 nodes of a tetrahedral mesh 57 -> 47
+// and 160 -> 67 us. What is left: a row takes about 0.2 us (FP32; FP64 11 instructions of 64 cycles
+// each on its partition's FP64 unit, about 0.5 us), and a value from another chunk about 0.9 us from
+// its publication to the slot. Four segments a chunk: eight are alike in FP32 and slower in FP64
+// (315 us: the SM's FP64 unit is shared), and a second fetching warp changes nothing.
 // ---------------------------------------------------------------------------------------------
 
-// FP32 sweeps publish every value in one 64-bit word together with the sweep's epoch (low half:
-// the float's bits, high half: the epoch). Naturally aligned 64-bit accesses are single-copy
-// atomic, so a reader that sees the current epoch in all four words of a node also holds their
-// values: one L2 round trip detects readiness and delivers the data, with no flag and no fence.
-__device__ __forceinline__ void st_packed(unsigned long long* p, float v, uint32_t ep) {
-  const unsigned long long w = ((unsigned long long)ep << 32) | __float_as_uint(v);
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
-}
+// A sweep publishes a node's four values with single stores into buffers that hold an all-ones bit
+// pattern before the sweep (a NaN that arithmetic never produces): a global one, read through L2,
+// and the chunk's slots in shared memory. Every word is written once, so a node is ready once none
+// of its words holds the pattern: no flag, no fence, and the read that finds it ready has its values.
+constexpr uint32_t UNSET32 = 0xffffffffu;
 
-__device__ __forceinline__ void ld_relaxed2(const unsigned long long* p, unsigned long long& a,
-                                            unsigned long long& b) {
+// One attempt to read a node's values from L2 (`p`) or from a slot (`s`, a shared-memory address).
+// `m` is raised to the largest of the words (FP64: of the words' halves combined), which is all
+// ones while one of them is not written.
+__device__ __forceinline__ void words_max(uint32_t a, uint32_t b, uint32_t c, uint32_t d, uint32_t& m) {
+  m = max(max(max(a, b), max(c, d)), m);
+}
+__device__ __forceinline__ void ld_relaxed4(const float* p, float x[4], uint32_t& m) {
+  unsigned long long a, b;
   asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+  const uint32_t w[4] = {(uint32_t)a, (uint32_t)(a >> 32), (uint32_t)b, (uint32_t)(b >> 32)};
+  for (int k = 0; k < 4; ++k) x[k] = __uint_as_float(w[k]);
+  words_max(w[0], w[1], w[2], w[3], m);
 }
+__device__ __forceinline__ void pairs_max(unsigned long long a, unsigned long long b, unsigned long long c,
+                                          unsigned long long d, double x[4], uint32_t& m) {
+  x[0] = __longlong_as_double((long long)a); x[1] = __longlong_as_double((long long)b);
+  x[2] = __longlong_as_double((long long)c); x[3] = __longlong_as_double((long long)d);
+  // both halves of a word are all ones only while it is not written
+  words_max((uint32_t)a & (uint32_t)(a >> 32), (uint32_t)b & (uint32_t)(b >> 32), (uint32_t)c & (uint32_t)(c >> 32),
+            (uint32_t)d & (uint32_t)(d >> 32), m);
+}
+__device__ __forceinline__ void ld_relaxed4(const double* p, double x[4], uint32_t& m) {
+  unsigned long long a, b, c, d;
+  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
+  asm volatile("ld.relaxed.gpu.global.v2.u64 {%0, %1}, [%2];" : "=l"(c), "=l"(d) : "l"(p + 2) : "memory");
+  pairs_max(a, b, c, d, x, m);
+}
+__device__ __forceinline__ void ld_slot(unsigned s, float x[4], uint32_t& m) {
+  uint32_t a, b, c, d;
+  asm volatile("ld.volatile.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(a), "=r"(b), "=r"(c), "=r"(d) : "r"(s) : "memory");
+  x[0] = __uint_as_float(a); x[1] = __uint_as_float(b);
+  x[2] = __uint_as_float(c); x[3] = __uint_as_float(d);
+  words_max(a, b, c, d, m);
+}
+__device__ __forceinline__ void ld_slot(unsigned s, double x[4], uint32_t& m) {
+  unsigned long long a, b, c, d;
+  asm volatile("ld.volatile.shared.v2.u64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "r"(s) : "memory");
+  asm volatile("ld.volatile.shared.v2.u64 {%0, %1}, [%2];" : "=l"(c), "=l"(d) : "r"(s + 16) : "memory");
+  pairs_max(a, b, c, d, x, m);
+}
+__device__ __forceinline__ void put_slot(unsigned s, const float x[4]) {
+  asm volatile("st.volatile.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(s), "f"(x[0]), "f"(x[1]), "f"(x[2]), "f"(x[3]) : "memory");
+}
+__device__ __forceinline__ void put_slot(unsigned s, const double x[4]) {
+  asm volatile("st.volatile.shared.v2.f64 [%0], {%1, %2};" ::"r"(s), "d"(x[0]), "d"(x[1]) : "memory");
+  asm volatile("st.volatile.shared.v2.f64 [%0], {%1, %2};" ::"r"(s + 16), "d"(x[2]), "d"(x[3]) : "memory");
+}
+// Publish a node's four values with one 16-byte store per lane (generic addresses; `dst` is the
+// lane's own): FP32 lane 0 writes the shared slot, lane 1 the global publication, lane 2 the plain
+// vector; FP64 two lanes each.
+__device__ __forceinline__ void publish(int lane, const float r[4], unsigned long long dst) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t.reg .b64 a, b;\n\tsetp.lt.s32 p, %0, 3;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
+      "@p st.relaxed.gpu.v2.b64 [%1], {a, b};\n\t}"
+      ::"r"(lane), "l"(dst), "f"(r[0]), "f"(r[1]), "f"(r[2]), "f"(r[3]) : "memory");
+}
+__device__ __forceinline__ void publish(int lane, const double r[4], unsigned long long dst) {
+  const double a = lane & 1 ? r[2] : r[0], b = lane & 1 ? r[3] : r[1];
+  asm volatile("{\n\t.reg .pred p;\n\tsetp.lt.s32 p, %0, 6;\n\t@p st.relaxed.gpu.v2.f64 [%1], {%2, %3};\n\t}"
+               ::"r"(lane), "l"(dst), "d"(a), "d"(b) : "memory");
+}
+// Whether one of four values is not a number (FP32: or two infinities cancel).
+__device__ __forceinline__ bool any_nan(const float r[4]) {
+  const float s = (r[0] + r[1]) + (r[2] + r[3]);
+  return s != s;
+}
+__device__ __forceinline__ bool any_nan(const double r[4]) {
+  uint32_t m = 0;
+  for (int k = 0; k < 4; ++k) m = max(m, (uint32_t)__double2hiint(r[k]) & 0x7fffffffu);
+  return m >= 0x7ff80000u;
+}
+__device__ __forceinline__ void ld_shared4(unsigned s, int, float o[4]) {
+  asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(o[0]), "=f"(o[1]), "=f"(o[2]), "=f"(o[3]) : "r"(s));
+}
+__device__ __forceinline__ void ld_shared4(unsigned s, int half, double o[4]) {
+  asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(o[0]), "=d"(o[1]) : "r"(s));
+  asm volatile("ld.shared.v2.f64 {%0, %1}, [%2];" : "=d"(o[2]), "=d"(o[3]) : "r"(s + half));
+}
+__device__ __forceinline__ void ld_shared1(unsigned s, float& o) { asm volatile("ld.shared.f32 %0, [%1];" : "=f"(o) : "r"(s)); }
+__device__ __forceinline__ void ld_shared1(unsigned s, double& o) { asm volatile("ld.shared.f64 %0, [%1];" : "=d"(o) : "r"(s)); }
+__device__ __forceinline__ void ld_shared1(unsigned s, unsigned& o) { asm volatile("ld.shared.u32 %0, [%1];" : "=r"(o) : "r"(s)); }
 
-// Wait until the four words of a node carry `ep`, then return their values.
-__device__ __forceinline__ bool wait_packed(const unsigned long long* p, uint32_t ep, float out[4],
-                                            int* err, uint32_t lim) {
-  for (uint32_t it = 0; it <= lim; ++it) {
-    unsigned long long a, b, c, d;
-    ld_relaxed2(p, a, b);
-    ld_relaxed2(p + 2, c, d);
-    if ((uint32_t)(a >> 32) == ep && (uint32_t)(b >> 32) == ep && (uint32_t)(c >> 32) == ep &&
-        (uint32_t)(d >> 32) == ep) {
-      out[0] = __uint_as_float((uint32_t)a);
-      out[1] = __uint_as_float((uint32_t)b);
-      out[2] = __uint_as_float((uint32_t)c);
-      out[3] = __uint_as_float((uint32_t)d);
-      return true;
-    }
-    if (it >= 64) __nanosleep(32);
-    if ((it & 1023u) == 1023u && *(volatile int*)err != 0) return false;
-  }
-  atomicCAS(err, 0, ILU_ERR_TIMEOUT);
+// Bulk copies global -> shared, completed on an mbarrier.
+__device__ __forceinline__ void mbar_init(unsigned bar) {
+  asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void mbar_expect(unsigned bar, unsigned bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void bulk_copy(unsigned dst, const void* src, unsigned bytes, unsigned bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(bar) : "memory");
+}
+__device__ __forceinline__ bool mbar_try(unsigned bar, unsigned parity) {
+  uint32_t ok;
+  asm volatile("{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+               : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ bool mbar_test(unsigned bar, unsigned parity) {
+  uint32_t ok;
+  asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+               : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
+  return ok != 0;
+}
+__device__ __forceinline__ void mbar_arrive(unsigned bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+// A bulk copy completes by hardware; the limit only keeps the wait finite.
+__device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
+  for (uint32_t it = 0; it < (1u << 22); ++it)
+    if (mbar_try(bar, parity)) return true;
   return false;
 }
 
-// FP64 sweeps write into buffers filled with an all-ones bit pattern before the sweep (a NaN that
-// arithmetic never produces); a node is ready once none of its four words holds that pattern.
-constexpr unsigned long long UNSET64 = ~0ull;
-
-__device__ __forceinline__ bool wait_unset(const double* p, double out[4], int* err, uint32_t lim) {
-  const unsigned long long* w = reinterpret_cast<const unsigned long long*>(p);
-  for (uint32_t it = 0; it <= lim; ++it) {
-    unsigned long long a, b, c, d;
-    ld_relaxed2(w, a, b);
-    ld_relaxed2(w + 2, c, d);
-    if (a != UNSET64 && b != UNSET64 && c != UNSET64 && d != UNSET64) {
-      out[0] = __longlong_as_double((long long)a);
-      out[1] = __longlong_as_double((long long)b);
-      out[2] = __longlong_as_double((long long)c);
-      out[3] = __longlong_as_double((long long)d);
-      return true;
-    }
-    if (it >= 64) __nanosleep(32);
-    if ((it & 1023u) == 1023u && *(volatile int*)err != 0) return false;
-  }
-  atomicCAS(err, 0, ILU_ERR_TIMEOUT);
-  return false;
+// A row of the factor as a sweep reads it (Ilu::rec): 8 NP blocks (4 x 4), then the byte offsets of
+// their values in shared memory (8 NP words). Row q of block 8 p + g belongs to lane 8 q + g in pass
+// p: a pass holds its lanes' 16-byte pieces side by side (FP64: first halves, then second halves),
+// so that a warp's loads meet no bank twice. The forward record holds -L_ik, the last
+// place kept for the row before in the segment; the backward one -U_ii^-1 U_ij, the last place the
+// same, the one before it U_ii^-1, whose value is the right-hand side. A row is then one sum of
+// block products in either sweep (the forward one adds its right-hand side). Places without a
+// block hold zeros and point to slot 0, which holds zeros.
+template <typename T, int NP> constexpr int sweep_rec_bytes() { return 8 * NP * (16 * (int)sizeof(T) + 4); }
+// rows of a bulk copy (8: 190 us instead of 213 on 49^3 nodes, but 331 instead of 237 on lines of 151
+// nodes, and fewer blocks fit an SM), and copies in flight per warp
+template <typename T, int NP> constexpr int sweep_rb() { return NP <= 2 ? 4 : 2; }
+constexpr int SWEEP_ST = 3;
+// shared memory of a sweep: value slots (zeros, the chunk's rows, their far neighbours), the rings
+// of row records and right-hand sides, the barriers
+template <typename T, int NP>
+size_t sweep_smem_bytes(int warps, int slots) {
+  return (size_t)slots * 4 * sizeof(T) +
+         (size_t)warps * SWEEP_ST * (sweep_rb<T, NP>() * (sweep_rec_bytes<T, NP>() + 4 * sizeof(T)) + 16);
 }
 
-__device__ __forceinline__ void st_relaxed_f64(double* p, double v) {
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(__double_as_longlong(v)) : "memory");
-}
-
-// Sum of the four per-lane partials over the warp, reduce-scatter style (7 shuffles): on return
-// lane L holds the full sum of component (L >> 3) & 3.
-template <typename T>
-__device__ __forceinline__ T warp_sum4_scatter(const T a[4], int lane) {
-  const bool h16 = lane & 16, h8 = lane & 8;
-  const T s0 = h16 ? a[0] : a[2], s1 = h16 ? a[1] : a[3];
-  const T b0 = (h16 ? a[2] : a[0]) + __shfl_xor_sync(FULL, s0, 16);
-  const T b1 = (h16 ? a[3] : a[1]) + __shfl_xor_sync(FULL, s1, 16);
-  T c = (h8 ? b1 : b0) + __shfl_xor_sync(FULL, h8 ? b0 : b1, 8);
-  c += __shfl_xor_sync(FULL, c, 4);
-  c += __shfl_xor_sync(FULL, c, 2);
-  c += __shfl_xor_sync(FULL, c, 1);
-  return c;
-}
-
-// Shared-memory publication inside a chunk: the CTA fills the chunk's value slots with an all-ones
-// bit pattern (a NaN that arithmetic never produces) when it takes the chunk, each writer lane then
-// stores its value directly, and a reader polls until none of the node's four words holds the
-// pattern. Every word is written once by one lane, so no flag and no fence is needed.
-template <typename T> struct Bits;
-template <> struct Bits<float> { using U = uint32_t; static constexpr U unset = 0xffffffffu; };
-template <> struct Bits<double> { using U = unsigned long long; static constexpr U unset = ~0ull; };
-
-template <typename T>
-__device__ __forceinline__ bool wait_shared(const T* p, T out[4], int* err, uint32_t lim) {
-  using U = typename Bits<T>::U;
-  const volatile U* w = reinterpret_cast<const volatile U*>(p);
-  for (uint32_t it = 0; it <= lim; ++it) {
-    const U a = w[0], b = w[1], c = w[2], d = w[3];
-    if (a != Bits<T>::unset && b != Bits<T>::unset && c != Bits<T>::unset && d != Bits<T>::unset) {
-      const U u[4] = {a, b, c, d};
-      for (int m = 0; m < 4; ++m) {
-        if constexpr (sizeof(T) == 4) out[m] = __uint_as_float(u[m]);
-        else out[m] = __longlong_as_double((long long)u[m]);
+// The records of one sweep from the factor (CSR layout, FP64): one thread per 16-byte piece.
+template <typename T, bool LOWER, int NP>
+__global__ void sweep_pack_kernel(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ dpos,
+                                  const uint8_t* __restrict__ inl, const int32_t* __restrict__ at,
+                                  const double* __restrict__ F, const double* __restrict__ Dinv, int64_t n_nodes,
+                                  unsigned char* __restrict__ rec) {
+  constexpr int PB = (int)sizeof(T);            // 16-byte pieces of a block
+  constexpr int EP = 16 / (int)sizeof(T);       // values of a piece
+  constexpr int PIECES = 8 * NP * PB + 2 * NP;  // pieces of a record
+  for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < n_nodes * PIECES;
+       w += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t i = w / PIECES;
+    const int pc = (int)(w - i * PIECES);
+    const int l = pc & 31, half = (pc >> 5) % (PB / 4), blk = 8 * ((pc >> 5) / (PB / 4)) + (l & 7);
+    const int32_t rp = rowptr[4 * i];
+    const int deg = (rowptr[4 * i + 1] - rp) >> 2, dp = dpos[i];
+    const int has = inl[i] >> (LOWER ? 0 : 1) & 1;          // the row before in the segment is a neighbour
+    const int own = (LOWER ? dp : deg - 1 - dp) - has;      // this row's other blocks
+    if (pc < 8 * NP * PB) {
+      int kk = -1;
+      if (blk < own) kk = LOWER ? blk : deg - 1 - blk;
+      else if (blk == 8 * NP - 1 && has) kk = LOWER ? dp - 1 : dp + 1;
+      const int r = l >> 3, c0 = half * EP;
+      T o[EP];
+      for (int t = 0; t < EP; ++t) {
+        const int c = c0 + t;
+        double x = 0.0;
+        if (!LOWER && blk == 8 * NP - 2) {
+          x = Dinv[16 * i + 4 * r + c];
+        } else if (kk >= 0) {
+          const double* f = F + rp + 4 * kk + c;
+          if (LOWER) x = -f[r * 4 * deg];
+          else
+            for (int m = 0; m < 4; ++m) x -= Dinv[16 * i + 4 * r + m] * f[m * 4 * deg];
+        }
+        o[t] = T(x);
       }
-      return true;
-    }
-    if (it >= 32) __nanosleep(8);
-    if ((it & 1023u) == 1023u && *(volatile int*)err != 0) return false;
-  }
-  atomicCAS(err, 0, ILU_ERR_TIMEOUT);
-  return false;
-}
-
-// Asynchronous global -> shared copies (per thread; completion tracked per thread by groups, so a
-// thread only ever reads what it copied itself and no flag or barrier is involved).
-__device__ __forceinline__ void cp_async16(void* dst, const void* src) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_async4(void* dst, const void* src) {
-  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int N>
-__device__ __forceinline__ void cp_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
-
-// Rows of a segment in flight ahead of the row being solved, and the per-warp ring they land in:
-// for each slot, every lane's 4x4 factor block, every lane's column index and the four rows of
-// U_ii^-1 (backward sweep).
-constexpr int ILU_PF = 4;
-template <typename T>
-struct SweepSlot {
-  T f[32][16];
-  int32_t col[32];
-  T dinv[4][4];
-};
-template <typename T>
-constexpr size_t sweep_ring_bytes(int warps) {
-  return (size_t)warps * ILU_PF * sizeof(SweepSlot<T>);
-}
-
-// FP64 rows with at most 16 blocks on the sweep's side take two lanes per block (two block rows
-// each): 8 DFMA instructions per row instead of 16 (the FP64 unit of an SM partition spends a
-// full warp slot on every FP64 instruction, however many lanes are active).
-template <typename T>
-__device__ __forceinline__ bool split_rows_t(int side) { return sizeof(T) == 8 && side <= 16; }
-
-// One row of the two-lanes-per-block mapping (lane 2 bl + h: rows 2h, 2h + 1 of block bl). The
-// sums end on lanes 0, 16, 1, 17 for components 0..3. Returns false if a wait gave up.
-template <typename T, bool LOWER>
-__device__ __forceinline__ bool split_row(const SweepSlot<T>& sl, int r, int64_t i, int dp, int deg,
-                                          int lane, const T (&o_rhs)[2][4], T* sx, int64_t a,
-                                          int64_t b, void* pub, T* out, int64_t n0, uint32_t ep,
-                                          int* err, uint32_t lim) {
-  const int bl = lane >> 1, h = lane & 1;
-  const int kk = LOWER ? bl : dp + 1 + bl;
-  const bool mine = LOWER ? kk < dp : kk < deg;
-  const int qw = 2 * h + ((lane >> 4) & 1);      // the component this lane's reduction ends with
-  const bool wr = (lane & 14) == 0;              // lanes 0, 1, 16, 17
-  T rhs = T(0);
-  {
-    const int src = r & 31;
-    const bool hi = r >= 32;
-    for (int m = 0; m < 4; ++m) {
-      const T t = __shfl_sync(FULL, hi ? o_rhs[1][m] : o_rhs[0][m], src);
-      if (m == qw) rhs = t;
-    }
-  }
-  T acc0 = T(0), acc1 = T(0);
-  bool ok = true;
-  if (mine) {
-    const int64_t k = sl.col[lane] >> 2;
-    T xk[4];
-    if (k >= a && k < b) {
-      const int64_t sk = LOWER ? k - a : b - 1 - k;
-      ok = wait_shared<T>(sx + 4 * sk, xk, err, lim);
-    } else if constexpr (sizeof(T) == 4) {
-      ok = wait_packed(reinterpret_cast<const unsigned long long*>(pub) + 4 * k, ep, xk, err, lim);
+      T* dst = reinterpret_cast<T*>(rec + w * 16);
+      for (int t = 0; t < EP; ++t) dst[t] = o[t];
     } else {
-      ok = wait_unset(reinterpret_cast<const double*>(pub) + 4 * k, xk, err, lim);
-    }
-    if (ok)
-      for (int m = 0; m < 4; ++m) {
-        acc0 += sl.f[lane][m] * xk[m];
-        acc1 += sl.f[lane][4 + m] * xk[m];
+      int32_t* dst = reinterpret_cast<int32_t*>(rec + w * 16);
+      const int k0 = (pc - 8 * NP * PB) * 4;
+      for (int t = 0; t < 4; ++t) {
+        const int k = k0 + t;
+        dst[t] = k < own ? 4 * (int)sizeof(T) * at[(rp >> 4) + (LOWER ? k : deg - 1 - k)] : 0;
       }
+    }
   }
-  if (!__all_sync(FULL, ok)) return false;
-  // sum over the 16 blocks (lane bits 1..4), rows 2h (lane bit 4 clear) or 2h + 1 (set)
-  const bool b4 = lane & 16;
-  T sm = (b4 ? acc1 : acc0) + __shfl_xor_sync(FULL, b4 ? acc0 : acc1, 16);
-  sm += __shfl_xor_sync(FULL, sm, 8);
-  sm += __shfl_xor_sync(FULL, sm, 4);
-  sm += __shfl_xor_sync(FULL, sm, 2);
-  const T w = wr ? rhs - sm : T(0);
-  T res = w;
-  if constexpr (!LOWER) {
-    // components 0..3 sit on lanes 0, 16, 1, 17
-    const T w0 = __shfl_sync(FULL, w, 0), w1 = __shfl_sync(FULL, w, 16);
-    const T w2 = __shfl_sync(FULL, w, 1), w3 = __shfl_sync(FULL, w, 17);
-    res = wr ? sl.dinv[qw][0] * w0 + sl.dinv[qw][1] * w1 + sl.dinv[qw][2] * w2 + sl.dinv[qw][3] * w3
-             : T(0);
-  }
-  const int64_t si = LOWER ? i - a : b - 1 - i;
-  if (wr) {
-    *reinterpret_cast<volatile T*>(sx + 4 * si + qw) = res;
-    if constexpr (sizeof(T) == 4)
-      st_packed(reinterpret_cast<unsigned long long*>(pub) + 4 * i + qw, res, ep);
-    else
-      st_relaxed_f64(reinterpret_cast<double*>(pub) + 4 * i + qw, res);
-    if (out) out[4 * (i - n0) + qw] = res;
-  }
-  return true;
 }
 
-// T: element type of the factor (float: packed publication, double: sentinel publication).
-// Rows [n0, n0 + n_rows); `v` (forward sweep) and `out` are compact (index i - n0), the
-// publication buffer `pub`, the FP64 backward-sweep input `v` and the FP32 one `vp` are indexed by
-// node over the whole mesh.
+// T: element type of the factor.
+// Rows [n0, n0 + n_rows); `v` and `out` are compact (index i - n0), the publication buffers `pub`
+// (written) and `clr` (the other sweep's, set to all ones for its next run) are indexed by node
+// over the whole mesh. NP: passes of eight blocks (a record's 8 NP places).
 //
 // The rows are cut into segments (seg[s] .. seg[s+1]): maximal runs of consecutive nodes in which
 // every node is coupled to the one before it (a grid line in a lattice numbering), at most
-// ILU_SEG_MAX long. A CTA claims the next chunk of W segments in sweep order from the
-// global counter and each of its warps takes one segment and does its rows in order, loading the
-// next row while the current one waits. A row's dependency in the same chunk is read from shared
-// memory once its value slots no longer hold the all-ones pattern (no L2 round trip; in the warp's
-// own segment it is already there); a dependency in an earlier chunk is read from the L2
-// publication. Chunks are claimed in order by running CTAs, so every wait is for work that is
-// already in progress.
-template <typename T, bool LOWER, int W = sweep_warps<T>()>
-__global__ void __launch_bounds__(W * 32)
-    ilu_sweep_kernel(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colidx,
-                     const T* __restrict__ F, const T* __restrict__ Dinv,
-                     const int32_t* __restrict__ dpos, const int32_t* __restrict__ seg, int64_t s0,
-                     int64_t n_segs, const T* __restrict__ v,
-                     const unsigned long long* __restrict__ vp, void* pub, T* __restrict__ out,
-                     int64_t n0, int64_t n_rows, uint32_t ep, unsigned long long* ticket,
-                     unsigned long long base, int* err, uint32_t lim) {
-  constexpr int SLOTS = W * ILU_SEG_MAX;
-  __shared__ __align__(16) T sx[SLOTS * 4];
+// ILU_SEG_MAX long, and the segments into chunks of at most W (Ilu::chunk). A CTA claims the next
+// chunk in sweep order and each of its first W warps does one segment's rows in order: lane
+// 8 q + g holds row q of the blocks g, g + 8, ..., and reads every neighbour's value from the
+// chunk's slots in shared memory once it no longer holds the all-ones pattern. The rows of the
+// chunk write theirs there, and the next FW warps fetch the neighbours in earlier chunks (the
+// chunk's far list) from the L2 publication as they appear, so that the L2 round trips run beside
+// the rows instead of inside them. The last warp streams the row records and right-hand sides into
+// a ring per compute warp with bulk copies. Chunks are claimed in order by running CTAs, so every
+// wait is for work that is already in progress.
+template <typename T, bool LOWER, int NP, int W, int FW>
+__global__ void __launch_bounds__((W + FW + 1) * 32)
+    ilu_sweep_kernel(const unsigned char* __restrict__ rec, const int32_t* __restrict__ seg,
+                     const int32_t* __restrict__ chunk, const int32_t* __restrict__ farptr,
+                     const int32_t* __restrict__ far, int64_t c0, int64_t n_chunks, const T* __restrict__ v,
+                     T* pub, uint4* __restrict__ clr, T* __restrict__ out, int n0, int n_rows, int slots,
+                     unsigned long long* ticket, unsigned long long base, int* err, uint32_t lim) {
+  constexpr int ST = SWEEP_ST, RB = sweep_rb<T, NP>(), VB = 4 * (int)sizeof(T);  // VB: bytes of a node's values
+  constexpr int RS = sweep_rec_bytes<T, NP>(), STAGE = RB * (RS + VB);
+  constexpr int dir = LOWER ? 1 : -1;
   __shared__ int64_t s_chunk;
-  extern __shared__ __align__(16) unsigned char sring[];
+  extern __shared__ __align__(16) unsigned char smem[];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  SweepSlot<T>* ring = reinterpret_cast<SweepSlot<T>*>(sring) + warp * ILU_PF;
-  const int q = (lane >> 3) & 3;          // the component this lane's reduction ends with
-  const bool writer = (lane & 7) == 0;    // lanes 0, 8, 16, 24 finish components 0..3
-  const int64_t n1 = n0 + n_rows;
-  const int64_t n_chunks = (n_segs + W - 1) / W;
+  const int q = lane >> 3, g = lane & 7;
+  const int n1 = n0 + n_rows;
+  const unsigned sx = (unsigned)__cvta_generic_to_shared(smem);
+  const unsigned rings = sx + slots * VB, bars = rings + W * ST * STAGE;
+  // stage n of compute warp w: barrier `full` (its copies have landed), then `empty` (it was read)
+  auto full = [&](int w, unsigned n) { return bars + (w * ST + n % ST) * 16; };
+  auto empty = [&](int w, unsigned n) { return bars + (w * ST + n % ST) * 16 + 8; };
+  if (threadIdx.x < W * ST * 2) mbar_init(bars + 8 * threadIdx.x);
+  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  unsigned copies = 0;  // compute warp: copies read; producer lane w: copies started for warp w
   for (;;) {
     if (threadIdx.x == 0) {
-      int64_t c = n_chunks;
+      int64_t c = -1;
       if (*(volatile int*)err == 0) {
         const unsigned long long t = atomicAdd(ticket, 1ull);
         if (t < base) atomicCAS(err, 0, ILU_ERR_TIMEOUT);  // the counter was disturbed
-        else if (t - base < (unsigned long long)n_chunks) c = (int64_t)(t - base);
+        else if (t - base < (unsigned long long)n_chunks)
+          c = LOWER ? c0 + (int64_t)(t - base) : c0 + n_chunks - 1 - (int64_t)(t - base);
       }
       s_chunk = c;
     }
-    for (int l = threadIdx.x; l < 4 * SLOTS; l += blockDim.x)
-      reinterpret_cast<typename Bits<T>::U*>(sx)[l] = Bits<T>::unset;
+    for (int l = threadIdx.x; l < slots * VB / 16; l += (W + FW + 1) * 32) {
+      const uint32_t z = l < VB / 16 ? 0u : UNSET32;  // slot 0: zeros
+      reinterpret_cast<uint4*>(smem)[l] = make_uint4(z, z, z, z);
+    }
     __syncthreads();
     const int64_t c = s_chunk;
-    if (c >= n_chunks) return;
-    // segments jlo .. jhi - 1 in sweep order; their nodes form the range [a, b)
-    const int64_t jlo = c * W;
-    const int64_t jhi = jlo + W < n_segs ? jlo + W : n_segs;
-    int64_t a = LOWER ? seg[s0 + jlo] : seg[s0 + n_segs - jhi];
-    int64_t b = LOWER ? seg[s0 + jhi] : seg[s0 + n_segs - jlo];
-    a = a > n0 ? a : n0;
-    b = b < n1 ? b : n1;
-    const int64_t j = jlo + warp;
-    if (j < jhi) {
-      const int64_t s = LOWER ? s0 + j : s0 + n_segs - 1 - j;
-      int64_t r_lo = seg[s], r_hi = seg[s + 1];
-      r_lo = r_lo > n0 ? r_lo : n0;
-      r_hi = r_hi < n1 ? r_hi : n1;
-      const int len = (int)(r_hi - r_lo);
-      // rows r of the segment in sweep order: node LOWER ? r_lo + r : r_hi - 1 - r. All rows'
-      // offsets and right-hand sides are loaded at once (row r on lane r % 32, register set r / 32);
-      // factor blocks, column indices and U_ii^-1 rows stream through the ring ILU_PF - 1 rows
-      // ahead of the row being solved.
-      int32_t o_rp[2][4], o_dp[2];
-      T o_rhs[2][4];
-      for (int h = 0; h < 2; ++h) {
-        const int l = lane + 32 * h;
-        o_dp[h] = 0;
-        for (int m = 0; m < 4; ++m) { o_rp[h][m] = 0; o_rhs[h][m] = T(0); }
-        if (l < len) {
-          const int64_t il = LOWER ? r_lo + l : r_hi - 1 - l;
-          for (int m = 0; m < 4; ++m) o_rp[h][m] = rowptr[4 * il + m];
-          o_dp[h] = dpos[il];
-          for (int m = 0; m < 4; ++m) {
-            if constexpr (LOWER) {
-              o_rhs[h][m] = v[4 * (il - n0) + m];
-            } else if constexpr (sizeof(T) == 4) {
-              o_rhs[h][m] = __uint_as_float((uint32_t)vp[4 * il + m]);
-            } else {
-              o_rhs[h][m] = v[4 * il + m];
-            }
-          }
+    if (c < 0) return;
+    const int slo = chunk[c], shi = chunk[c + 1];  // its segments
+    const int a = seg[slo];                        // its first node (slot 1)
+    // rows r = 0 .. len - 1 of a segment in sweep order are the nodes first + r * dir
+    auto segment = [&](int w, int& first) {
+      const int s = LOWER ? slo + w : shi - 1 - w;
+      int lo = seg[s], hi = seg[s + 1];
+      lo = lo > n0 ? lo : n0;
+      hi = hi < n1 ? hi : n1;
+      first = LOWER ? lo : hi - 1;
+      return hi > lo ? hi - lo : 0;
+    };
+    if (warp == W + FW) {
+      // producer: lane w streams the segment of compute warp w, RB rows a copy
+      int first = 0, left = lane < W && slo + lane < shi ? segment(lane, first) : 0;
+      uint32_t idle = 0;
+      bool stop = false;
+      while (!__all_sync(FULL, left == 0)) {
+        bool sent = false;
+        if (left > 0 && (copies < ST || mbar_test(empty(lane, copies), (copies / ST - 1) & 1))) {
+          const int n = left < RB ? left : RB;
+          const int64_t i0 = LOWER ? first : first - n + 1;  // its lowest node
+          const unsigned bar = full(lane, copies), dst = rings + (lane * ST + copies % ST) * STAGE;
+          mbar_expect(bar, n * (RS + VB));
+          bulk_copy(dst, rec + i0 * RS, n * RS, bar);
+          bulk_copy(dst + RB * RS, v + 4 * (i0 - n0), n * VB, bar);
+          ++copies;
+          first += dir * n;
+          left -= n;
+          sent = true;
+        }
+        idle = __any_sync(FULL, sent) ? 0 : idle + 1;
+        if (idle > 16u) __nanosleep(40);
+        // give up after lim polls without progress or once another warp has recorded an error
+        // (uniform decisions)
+        if (idle > lim || ((idle & 63u) == 63u && __any_sync(FULL, *(volatile int*)err != 0))) {
+          stop = true;
+          break;
         }
       }
-      // offsets of row r (uniform r): broadcast from the lane that loaded them
-      auto row_offsets = [&](int r, int32_t rp[4], int& dp) {
-        const int src = r & 31;
-        const bool hi = r >= 32;
-        for (int m = 0; m < 4; ++m) rp[m] = __shfl_sync(FULL, hi ? o_rp[1][m] : o_rp[0][m], src);
-        dp = __shfl_sync(FULL, hi ? o_dp[1] : o_dp[0], src);
-      };
-      auto split_rows = [&](int dp, int deg) { return split_rows_t<T>(LOWER ? dp : deg - dp - 1); };
-      auto issue = [&](int r) {  // start the copies of row r (every lane commits one group)
-        if (r < len) {
-          int32_t rp[4], dp;
-          row_offsets(r, rp, dp);
-          const int deg = (rp[1] - rp[0]) >> 2;
-          SweepSlot<T>& sl = ring[r % ILU_PF];
-          constexpr int CH = (int)(4 * sizeof(T)) / 16;  // 16-byte pieces of a 4-value block row
-          constexpr int EPC = 16 / (int)sizeof(T);        // values per piece
-          if (split_rows(dp, deg)) {
-            // two lanes per block: lane 2 bl + h copies rows 2h, 2h + 1 of block bl
-            const int bl = lane >> 1, h = lane & 1;
-            const int kk = LOWER ? bl : dp + 1 + bl;
-            if (LOWER ? kk < dp : kk < deg) {
-              const int32_t ra = h ? rp[2] : rp[0], rb = h ? rp[3] : rp[1];
-              for (int c = 0; c < CH; ++c) {
-                cp_async16(&sl.f[lane][c * EPC], F + ra + 4 * kk + c * EPC);
-                cp_async16(&sl.f[lane][4 + c * EPC], F + rb + 4 * kk + c * EPC);
-              }
-              cp_async4(&sl.col[lane], colidx + rp[0] + 4 * kk);
-            }
+      if (stop) {
+        if (lane == 0) atomicCAS(err, 0, ILU_ERR_TIMEOUT);
+        // no copy may land after the block has ended
+        if (lane < W)
+          for (unsigned n = copies < ST ? 0 : copies - ST; n < copies; ++n) mbar_wait(full(lane, n), (n / ST) & 1);
+      }
+    } else if (warp >= W) {
+      // far neighbours: lane takes entries of the list in order, each until it is published
+      const int b = seg[shi], fb = farptr[c], nf = farptr[c + 1] - fb;
+      for (int l = (a > n0 ? a : n0) * (VB / 16) + (warp - W) * 32 + lane; l < (b < n1 ? b : n1) * (VB / 16); l += FW * 32)
+        clr[l] = make_uint4(UNSET32, UNSET32, UNSET32, UNSET32);
+      int e = (warp - W) * 32 + lane;
+      int node = e < nf ? far[fb + e] : -1;
+      int rest = 0;  // this warp's entries not delivered yet
+      for (int k = (warp - W) * 32; k < nf; k += FW * 32) rest += nf - k < 32 ? nf - k : 32;
+      uint32_t idle = 0;
+      while (rest > 0) {
+        const int en = e + FW * 32;
+        const int next = en < nf ? far[fb + en] : -1;
+        bool done = false;
+        if (node >= 0) {
+          if (node < n0 || node >= n1) {
+            done = true;  // another block's node: no row here reads it
           } else {
-            const int kk = LOWER ? lane : dp + 1 + lane;
-            if (LOWER ? kk < dp : kk < deg) {
-              for (int m = 0; m < 4; ++m)
-                for (int c = 0; c < CH; ++c)
-                  cp_async16(&sl.f[lane][4 * m + c * EPC], F + rp[m] + 4 * kk + c * EPC);
-              cp_async4(&sl.col[lane], colidx + rp[0] + 4 * kk);
+            T x[4];
+            uint32_t m = 0;
+            ld_relaxed4(pub + 4 * (int64_t)node, x, m);
+            if (m != UNSET32) {
+              put_slot(sx + (1 + b - a + e) * VB, x);
+              done = true;
             }
           }
-          if (!LOWER && writer) {
-            const int64_t ir = r_hi - 1 - r;
-            for (int c = 0; c < CH; ++c)
-              cp_async16(&sl.dinv[q][c * EPC], Dinv + 16 * ir + 4 * q + c * EPC);
-          }
         }
-        cp_commit();
-      };
-      for (int r = 0; r < ILU_PF - 1; ++r) issue(r);
-      for (int r = 0; r < len; ++r) {
-        const int64_t i = LOWER ? r_lo + r : r_hi - 1 - r;
-        issue(r + ILU_PF - 1);
-        cp_wait<ILU_PF - 1>();  // this thread's copies of row r have landed
-        __syncwarp();           // ... and every lane's (U_ii^-1 rows are read across lanes)
-        const SweepSlot<T>& sl = ring[r % ILU_PF];
-        int32_t rp[4], dp;
-        row_offsets(r, rp, dp);
-        const int deg = (rp[1] - rp[0]) >> 2;
-        if (split_rows(dp, deg)) {
-          if (!split_row<T, LOWER>(sl, r, i, dp, deg, lane, o_rhs, sx, a, b, pub, out, n0, ep, err, lim))
-            break;  // an error was recorded; the CTA stops after this chunk
-          continue;
+        if (done) {
+          e = en;
+          node = next;
         }
-        const int kk = LOWER ? lane : dp + 1 + lane;
-        const bool mine = LOWER ? kk < dp : kk < deg;
-        T rhs = T(0);
-        {
-          const int src = r & 31;
-          const bool hi = r >= 32;
-          for (int m = 0; m < 4; ++m) {
-            const T t = __shfl_sync(FULL, hi ? o_rhs[1][m] : o_rhs[0][m], src);
-            if (m == q) rhs = t;
-          }
-        }
-        T acc[4] = {T(0), T(0), T(0), T(0)};
-        bool ok = true;
-        if (mine) {
-          const int64_t k = sl.col[lane] >> 2;
-          T xk[4];
-          if (k >= a && k < b) {  // a row of this chunk: shared memory
-            const int64_t sk = LOWER ? k - a : b - 1 - k;
-            ok = wait_shared<T>(sx + 4 * sk, xk, err, lim);
-          } else if constexpr (sizeof(T) == 4) {
-            ok = wait_packed(reinterpret_cast<const unsigned long long*>(pub) + 4 * k, ep, xk, err, lim);
-          } else {
-            ok = wait_unset(reinterpret_cast<const double*>(pub) + 4 * k, xk, err, lim);
-          }
-          if (ok)
-            for (int rr = 0; rr < 4; ++rr)
-              for (int m = 0; m < 4; ++m) acc[rr] += sl.f[lane][4 * rr + m] * xk[m];
-        }
-        if (!__all_sync(FULL, ok)) break;  // an error was recorded; the CTA stops after this chunk
-        const T sum = warp_sum4_scatter(acc, lane);
-        const T w = writer ? rhs - sum : T(0);
-        T res = w;
-        if constexpr (!LOWER) {
-          T wq[4];
-          for (int m = 0; m < 4; ++m) wq[m] = __shfl_sync(FULL, w, 8 * m);
-          res = writer ? sl.dinv[q][0] * wq[0] + sl.dinv[q][1] * wq[1] + sl.dinv[q][2] * wq[2] +
-                             sl.dinv[q][3] * wq[3]
-                       : T(0);
-        }
-        const int64_t si = LOWER ? i - a : b - 1 - i;
-        if (writer) {
-          *reinterpret_cast<volatile T*>(sx + 4 * si + q) = res;
-          if constexpr (sizeof(T) == 4)
-            st_packed(reinterpret_cast<unsigned long long*>(pub) + 4 * i + q, res, ep);
-          else
-            st_relaxed_f64(reinterpret_cast<double*>(pub) + 4 * i + q, res);
-          if (out) out[4 * (i - n0) + q] = res;
+        const unsigned dm = __ballot_sync(FULL, done);
+        rest -= __popc(dm);
+        idle = dm ? 0 : idle + 1;
+        // give up after lim / 8 polls (of an L2 round trip) without progress or once another warp
+        // has recorded an error (uniform decisions)
+        if (idle > lim >> 3 || ((idle & 255u) == 255u && __any_sync(FULL, *(volatile int*)err != 0))) {
+          if (lane == 0) atomicCAS(err, 0, ILU_ERR_TIMEOUT);
+          break;
         }
       }
-      cp_wait<0>();  // no copy of this segment may land in the ring after the warp has moved on
+    } else if (slo + warp < shi) {
+      int first;
+      const int len = segment(warp, first);
+      // this lane's store address (publish); the step from row to row is dir * VB for all three
+      unsigned long long dst;
+      {
+        const int role = lane / (VB / 16), half = 16 * (lane % (VB / 16));
+        if (role == 0) dst = (unsigned long long)(smem + (1 + first - a) * VB) + half;
+        else if (role == 1) dst = (unsigned long long)(pub + 4 * (int64_t)first) + half;
+        else dst = (unsigned long long)(out + 4 * (int64_t)(first - n0)) + half;
+      }
+      T res[4] = {T(0), T(0), T(0), T(0)};  // the row before (every lane holds all four values)
+      bool ok = true;
+      // Rows are taken without asking whether their neighbours' values are there: one that is not
+      // is a NaN and makes the row's result one, which all lanes see alike. Such a row is done again
+      // with an explicit wait. Inside a batch (straight-line code for a full one) the next row's
+      // record is loaded while the sums of the current row go through the shuffles, and its
+      // neighbours' values right after.
+      unsigned rc, rv;  // the batch's first record (this lane's pieces) and right-hand side
+      unsigned from[RB][NP];
+      T f[NP][4], x[NP][4], t = T(0);
+      constexpr int RD = LOWER ? RS : -RS, VD = LOWER ? VB : -VB;
+      auto record = [&](int rr) {
+#pragma unroll
+        for (int p = 0; p < NP; ++p) ld_shared4(rc + rr * RD + p * 128 * (int)sizeof(T), 512, f[p]);
+        if (LOWER) ld_shared1(rv + rr * VD + q * (int)sizeof(T), t);
+      };
+      auto values = [&](int rr, uint32_t& um) {
+#pragma unroll
+        for (int p = 0; p < NP; ++p) ld_slot(from[rr][p], x[p], um);
+      };
+      auto products = [&]() {  // place 7 of the last pass is the row before
+        T s0 = LOWER ? (g == 0 ? t : T(0)) : T(0);
+        if constexpr (sizeof(T) == 4) {
+          T s1 = T(0);  // two chains: the latency of one FMA chain would show
+#pragma unroll
+          for (int p = 0; p < NP; ++p)
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+              const T xv = p == NP - 1 && g == 7 ? res[m] : x[p][m];
+              if (m & 1) s1 += f[p][m] * xv;
+              else s0 += f[p][m] * xv;
+            }
+          s0 += s1;
+        } else {
+#pragma unroll
+          for (int p = 0; p < NP; ++p)
+#pragma unroll
+            for (int m = 0; m < 4; ++m) s0 += f[p][m] * (p == NP - 1 && g == 7 ? res[m] : x[p][m]);
+        }
+        return s0;
+      };
+      auto batch = [&](auto whole, int n) {
+#pragma unroll
+        for (int rr = 0; rr < RB; ++rr)
+          if (whole || rr < n) {
+#pragma unroll
+            for (int p = 0; p < NP; ++p) {
+              unsigned o;
+              ld_shared1(rc - 16 * lane + rr * RD + 8 * NP * 16 * (int)sizeof(T) + 32 * p + 4 * g, o);
+              from[rr][p] = !LOWER && p == NP - 1 && g == 6 ? rv + rr * VD : sx + o;  // U_ii^-1 times the right-hand side
+            }
+          }
+        uint32_t um = 0;
+        record(0);
+        values(0, um);
+#pragma unroll
+        for (int rr = 0; rr < RB; ++rr) {
+          if (!whole && rr >= n) break;
+          const bool more = rr + 1 < RB && (whole || rr + 1 < n);
+          T sum = products();
+          if (more) record(rr + 1);
+          sum += __shfl_xor_sync(FULL, sum, 4);
+          sum += __shfl_xor_sync(FULL, sum, 2);
+          sum += __shfl_xor_sync(FULL, sum, 1);
+          T w[4];
+#pragma unroll
+          for (int m = 0; m < 4; ++m) w[m] = __shfl_sync(FULL, sum, 8 * m);
+          if (more) values(rr + 1 < RB ? rr + 1 : 0, um);
+          if (__builtin_expect(any_nan(w), 0)) {  // uniform: every lane holds the same values
+            record(rr);
+            for (uint32_t it = 0;; ++it) {
+              um = 0;
+              values(rr, um);
+              if (__all_sync(FULL, um != UNSET32)) break;
+              if (it >= 256u) __nanosleep(20);
+              // give up after lim polls or once another warp has recorded an error (uniform decisions)
+              if (it >= lim || ((it & 1023u) == 1023u && __any_sync(FULL, *(volatile int*)err != 0))) return false;
+            }
+            sum = products();
+            if (more) record(rr + 1);
+            sum += __shfl_xor_sync(FULL, sum, 4);
+            sum += __shfl_xor_sync(FULL, sum, 2);
+            sum += __shfl_xor_sync(FULL, sum, 1);
+#pragma unroll
+            for (int m = 0; m < 4; ++m) w[m] = __shfl_sync(FULL, sum, 8 * m);
+            if (more) values(rr + 1 < RB ? rr + 1 : 0, um);
+          }
+#pragma unroll
+          for (int m = 0; m < 4; ++m) res[m] = w[m];
+          publish(lane, res, dst);
+          dst += dir * VB;
+        }
+        return true;
+      };
+      for (int r0 = 0; r0 < len && ok; r0 += RB) {
+        const int n = len - r0 < RB ? len - r0 : RB;
+        if (!__all_sync(FULL, mbar_wait(full(warp, copies), (copies / ST) & 1))) {
+          ok = false;
+          break;
+        }
+        const unsigned st = rings + (warp * ST + copies % ST) * STAGE;
+        rc = st + (LOWER ? 0 : (n - 1) * RS) + 16 * lane;
+        rv = st + RB * RS + (LOWER ? 0 : (n - 1) * VB);
+        ok = n == RB ? batch(std::true_type{}, RB) : batch(std::false_type{}, n);
+        // every lane has read the stage
+        __syncwarp();
+        if (lane == 0) mbar_arrive(empty(warp, copies));
+        ++copies;
+      }
+      if (!ok && lane == 0) atomicCAS(err, 0, ILU_ERR_TIMEOUT);
     }
     __syncthreads();
   }
@@ -594,8 +645,6 @@ unsigned resident_ctas(int64_t rows, int warps_per_cta, unsigned cap) {
 uint32_t next_epoch(Ilu& p, cudaStream_t st) {
   if (++p.epoch == 0) {  // wrapped: clear every flag so no stale epoch can match
     cudaMemsetAsync(p.flags, 0, sizeof(uint32_t) * p.n_nodes, st);
-    cudaMemsetAsync(p.yp, 0, sizeof(unsigned long long) * 4 * p.n_nodes, st);
-    cudaMemsetAsync(p.xp, 0, sizeof(unsigned long long) * 4 * p.n_nodes, st);
     p.epoch = 1;
   }
   return p.epoch;
@@ -662,14 +711,93 @@ int build_pattern(vms_ctx* ctx, Ilu& p, const Mesh& m) {
     }
   }
   seg.push_back((int32_t)N);
+  // the most blocks a row has on either side, the row before in its segment not counted
+  std::vector<uint8_t> inl(N, 0);  // bit 0: the node before is in the same segment, bit 1: the node after
+  p.side_lo = p.side_up = 0;
+  for (size_t s = 0; s + 1 < seg.size(); ++s)
+    for (int32_t i = seg[s]; i < seg[s + 1]; ++i) {
+      const int deg = start[i + 1] - start[i];
+      inl[i] = (uint8_t)((i > seg[s] ? 1 : 0) | (i + 1 < seg[s + 1] ? 2 : 0));
+      p.side_lo = std::max(p.side_lo, dpos[i] - (i > seg[s] ? 1 : 0));
+      p.side_up = std::max(p.side_up, deg - 1 - dpos[i] - (i + 1 < seg[s + 1] ? 1 : 0));
+    }
+  // chunks of at most ILU_CHUNK segments, fewer where a chunk's distinct neighbours in other chunks
+  // on one side would exceed ILU_FAR_MAX (one segment alone never does: 64 rows of at most 31);
+  // every neighbour's place in its row's chunk: the chunk's own rows first, then the far list of
+  // its side
+  std::vector<int32_t> chunk(1, 0), at(adj.size(), 0), farptr[2], far[2], mark(N, -1);
+  p.slots = 0;
+  {
+    const int32_t n_segs = (int32_t)seg.size() - 1;
+    // dependency levels of the two sweeps: the far lists are in the order in which their nodes appear
+    std::vector<int32_t> level[2] = {std::vector<int32_t>(N, 0), std::vector<int32_t>(N, 0)};
+    for (int64_t i = 0; i < N; ++i)
+      for (int32_t t = start[i]; t < start[i] + dpos[i]; ++t) level[0][i] = std::max(level[0][i], level[0][adj[t]] + 1);
+    for (int64_t i = N - 1; i >= 0; --i)
+      for (int32_t t = start[i] + dpos[i] + 1; t < start[i + 1]; ++t) level[1][i] = std::max(level[1][i], level[1][adj[t]] + 1);
+    farptr[0].push_back(0);
+    farptr[1].push_back(0);
+    for (int32_t lo = 0; lo < n_segs;) {
+      int32_t hi = std::min(lo + ILU_CHUNK, n_segs);
+      for (;; --hi) {
+        const int32_t a = seg[lo], b = seg[hi];
+        size_t most = 0;
+        std::vector<int32_t> lists[2];
+        for (int side = 0; side < 2; ++side) {
+          for (int32_t t = start[a]; t < start[b]; ++t) {
+            const int32_t j = adj[t];
+            if ((side ? j >= b : j < a) && mark[j] == -1) {
+              mark[j] = 0;
+              lists[side].push_back(j);
+            }
+          }
+          std::sort(lists[side].begin(), lists[side].end(), [&](int32_t x, int32_t y) {
+            return level[side][x] != level[side][y] ? level[side][x] < level[side][y] : x < y;
+          });
+          for (size_t k = 0; k < lists[side].size(); ++k) mark[lists[side][k]] = (int32_t)k;
+          for (int32_t i = a; i < b; ++i)
+            for (int32_t t = start[i]; t < start[i + 1]; ++t) {
+              const int32_t j = adj[t];
+              if (j >= a && j < b) at[t] = 1 + j - a;
+              else if (side ? j >= b : j < a) at[t] = 1 + b - a + mark[j];
+            }
+          for (int32_t j : lists[side]) mark[j] = -1;
+          most = std::max(most, lists[side].size());
+        }
+        if (most > (size_t)ILU_FAR_MAX && hi > lo + 1) continue;
+        for (int side = 0; side < 2; ++side) {
+          far[side].insert(far[side].end(), lists[side].begin(), lists[side].end());
+          farptr[side].push_back((int32_t)far[side].size());
+        }
+        p.slots = std::max(p.slots, 1 + (int)(b - a + (int32_t)most));
+        break;
+      }
+      chunk.push_back(hi);
+      lo = hi;
+    }
+  }
+  p.n_chunks = (int64_t)chunk.size() - 1;
   p.n_nodes = N;
   p.n_lower = lptr[N];
   p.n_pairs = (int64_t)pairs.size();
   p.n_segs = (int64_t)seg.size() - 1;
   e = cudaMalloc(&p.dpos, sizeof(int32_t) * N);
+  if (e == cudaSuccess) e = cudaMalloc(&p.inl, N);
+  if (e == cudaSuccess) e = cudaMemcpy(p.inl, inl.data(), N, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMalloc(&p.seg, sizeof(int32_t) * seg.size());
   if (e == cudaSuccess) e = cudaMemcpy(p.seg, seg.data(), sizeof(int32_t) * seg.size(), cudaMemcpyHostToDevice);
-  p.seg_host = std::move(seg);
+  auto up = [&](int32_t*& d, const std::vector<int32_t>& h) {
+    if (e == cudaSuccess) e = cudaMalloc(&d, sizeof(int32_t) * std::max<size_t>(1, h.size()));
+    if (e == cudaSuccess && !h.empty()) e = cudaMemcpy(d, h.data(), sizeof(int32_t) * h.size(), cudaMemcpyHostToDevice);
+  };
+  up(p.chunk, chunk);
+  up(p.at, at);
+  for (int side = 0; side < 2; ++side) {
+    up(p.farptr[side], farptr[side]);
+    up(p.far[side], far[side]);
+  }
+  p.chunk_node.resize(chunk.size());
+  for (size_t c = 0; c < chunk.size(); ++c) p.chunk_node[c] = seg[chunk[c]];
   if (e == cudaSuccess) e = cudaMalloc(&p.lptr, sizeof(int32_t) * (N + 1));
   if (e == cudaSuccess) e = cudaMalloc(&p.pptr, sizeof(int32_t) * pptr.size());
   if (e == cudaSuccess) e = cudaMalloc(&p.pairs, sizeof(uint16_t) * std::max<size_t>(1, pairs.size()));
@@ -684,26 +812,43 @@ int build_pattern(vms_ctx* ctx, Ilu& p, const Mesh& m) {
   return VMS_OK;
 }
 
+// passes of the sweeps: the places a record needs are a row's other blocks, the row before and
+// (backward sweep) the diagonal block
+int sweep_np(const Ilu& p, int side) {
+  const int places = side ? p.side_up + 2 : p.side_lo + 1;
+  return places <= 8 ? 1 : (places <= 16 ? 2 : (places <= 24 ? 3 : 5));
+}
+template <typename T>
+size_t rec_bytes(const Ilu& p, int side) {
+  const int np = sweep_np(p, side);
+  return (size_t)p.n_nodes * (np == 1 ? sweep_rec_bytes<T, 1>() : np == 2 ? sweep_rec_bytes<T, 2>()
+                                    : np == 3 ? sweep_rec_bytes<T, 3>() : sweep_rec_bytes<T, 5>());
+}
+
 int ensure_work(vms_ctx* ctx, Ilu& p, const Mesh& m, bool fp32) {
   cudaError_t e = cudaSuccess;
   if (!p.F) {
     e = cudaMalloc(&p.F, sizeof(double) * m.nnz);
     if (e == cudaSuccess) e = cudaMalloc(&p.Dinv, sizeof(double) * 16 * m.n_nodes);
-    if (e == cudaSuccess) e = cudaMalloc(&p.y, sizeof(double) * 4 * m.n_nodes);
-    if (e == cudaSuccess) e = cudaMalloc(&p.x64, sizeof(double) * 4 * m.n_nodes);
+    for (double** b : {&p.y, &p.yp64, &p.xp64})
+      if (e == cudaSuccess) e = cudaMalloc(b, sizeof(double) * 4 * m.n_nodes);
+    for (int side = 0; side < 2; ++side)
+      if (e == cudaSuccess) e = cudaMalloc(&p.rec[side], rec_bytes<double>(p, side));
+    for (double* b : {p.yp64, p.xp64})
+      if (e == cudaSuccess) e = cudaMemset(b, 0xff, sizeof(double) * 4 * m.n_nodes);
   }
-  if (e == cudaSuccess && fp32 && !p.F32) {
-    e = cudaMalloc(&p.F32, sizeof(float) * m.nnz);
-    if (e == cudaSuccess) e = cudaMalloc(&p.Dinv32, sizeof(float) * 16 * m.n_nodes);
-    if (e == cudaSuccess) e = cudaMalloc(&p.vals64, sizeof(double) * m.nnz);
+  if (e == cudaSuccess && fp32 && !p.vals64) {
+    e = cudaMalloc(&p.vals64, sizeof(double) * m.nnz);
+    for (float** b : {&p.y32, &p.yp32, &p.xp32})
+      if (e == cudaSuccess) e = cudaMalloc(b, sizeof(float) * 4 * m.n_nodes);
+    for (float* b : {p.yp32, p.xp32})
+      if (e == cudaSuccess) e = cudaMemset(b, 0xff, sizeof(float) * 4 * m.n_nodes);
+    for (int side = 0; side < 2; ++side)
+      if (e == cudaSuccess) e = cudaMalloc(&p.rec32[side], rec_bytes<float>(p, side));
   }
   if (e == cudaSuccess && !p.flags) {
     e = cudaMalloc(&p.flags, sizeof(uint32_t) * m.n_nodes);
     if (e == cudaSuccess) e = cudaMemset(p.flags, 0, sizeof(uint32_t) * m.n_nodes);
-    if (e == cudaSuccess) e = cudaMalloc(&p.yp, sizeof(unsigned long long) * 4 * m.n_nodes);
-    if (e == cudaSuccess) e = cudaMemset(p.yp, 0, sizeof(unsigned long long) * 4 * m.n_nodes);
-    if (e == cudaSuccess) e = cudaMalloc(&p.xp, sizeof(unsigned long long) * 4 * m.n_nodes);
-    if (e == cudaSuccess) e = cudaMemset(p.xp, 0, sizeof(unsigned long long) * 4 * m.n_nodes);
     if (e == cudaSuccess) e = cudaMalloc(&p.tickets, sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMemset(p.tickets, 0, sizeof(unsigned long long));
     if (e == cudaSuccess) e = cudaMalloc(&p.err, sizeof(int));
@@ -732,12 +877,32 @@ int convert(const A* x, B* y, int64_t n, cudaStream_t st) {
   return 1;
 }
 
+// The row records of both sweeps from the factor.
+template <typename T, bool LOWER>
+void pack_side(const Ilu& p, const Mesh& m, unsigned char* rec, cudaStream_t st) {
+  auto go = [&](auto kern) {
+    kern<<<16 * (unsigned)sm_count(), 256, 0, st>>>(m.rowptr, p.dpos, p.inl, p.at, p.F, p.Dinv, m.n_nodes, rec);
+  };
+  const int np = sweep_np(p, LOWER ? 0 : 1);
+  if (np == 1) go(sweep_pack_kernel<T, LOWER, 1>);
+  else if (np == 2) go(sweep_pack_kernel<T, LOWER, 2>);
+  else if (np == 3) go(sweep_pack_kernel<T, LOWER, 3>);
+  else go(sweep_pack_kernel<T, LOWER, 5>);
+}
+template <typename T>
+int pack(const Ilu& p, const Mesh& m, unsigned char* const rec[2], cudaStream_t st) {
+  pack_side<T, true>(p, m, rec[0], st);
+  pack_side<T, false>(p, m, rec[1], st);
+  return 2;
+}
+
 }  // namespace
 
 void free_ilu(Ilu& p) {
   const uint32_t lim = p.spin_limit;  // a setting of the context, kept across meshes
-  void* bufs[] = {p.dpos, p.lptr, p.pptr, p.pairs, p.F, p.Dinv, p.y, p.x64, p.F32, p.Dinv32,
-                  p.vals64, p.flags, p.yp, p.xp, p.tickets, p.err, p.seg};
+  void* bufs[] = {p.dpos, p.lptr, p.pptr, p.pairs, p.F, p.Dinv, p.y, p.yp64, p.xp64,
+                  p.vals64, p.flags, p.yp32, p.xp32, p.tickets, p.err, p.seg, p.inl, p.chunk, p.at,
+                  p.farptr[0], p.farptr[1], p.far[0], p.far[1], p.rec[0], p.rec[1], p.rec32[0], p.rec32[1], p.y32};
   for (void* b : bufs)
     if (b) cudaFree(b);
   p = Ilu();
@@ -767,79 +932,69 @@ int ilu_factor(vms_ctx* ctx, Ilu& p, const Mesh& m, bool fp32, const void* value
       p.tickets, p.base, p.err, p.spin_limit);
   p.base += (unsigned long long)m.n_nodes + (unsigned long long)ctas * ILU_FWARPS;
   *launches += 1;
-  if (fp32) {
-    *launches += convert<double, float>(p.F, p.F32, m.nnz, st);
-    *launches += convert<double, float>(p.Dinv, p.Dinv32, 16 * m.n_nodes, st);
-  }
+  if (fp32) *launches += pack<float>(p, m, p.rec32, st);
+  p.packed64 = false;  // the FP64 records are made on the first FP64 sweep
   p.factored = true;
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? VMS_OK : ctx_fail(ctx, VMS_ERR_CUDA, cudaGetErrorString(e));
 }
 
-// Segments covering nodes [n0, n1): [s0, s0 + count). Rows outside [n0, n1) are clamped away in
-// the kernel (a block solve has no couplings outside its rows, so n0 and n1 are segment starts).
-static void segment_range(const Ilu& p, int64_t n0, int64_t n1, int64_t& s0, int64_t& count) {
-  const std::vector<int32_t>& sg = p.seg_host;
-  const int64_t a = (int64_t)(std::upper_bound(sg.begin(), sg.end() - 1, (int32_t)n0) - sg.begin()) - 1;
-  const int64_t b = (int64_t)(std::lower_bound(sg.begin(), sg.end() - 1, (int32_t)n1) - sg.begin());
-  s0 = a < 0 ? 0 : a;
-  count = b - s0;
+// One sweep over rows [n0, n1): the chunks that cover it (rows outside are clamped away in the kernel;
+// a block solve has no couplings outside its rows, so n0 and n1 are segment starts).
+template <typename T>
+struct SweepArgs {
+  const unsigned char* rec;
+  int64_t n0, n1;
+  const T* v;
+  T *pub, *clr;
+  T* out;
+};
+template <typename T, bool LOWER, int NP>
+static void launch_sweep(Ilu& p, const SweepArgs<T>& s, cudaStream_t st) {
+  const std::vector<int32_t>& cn = p.chunk_node;
+  const int64_t c0 = std::max<int64_t>(0, (int64_t)(std::upper_bound(cn.begin(), cn.end() - 1, (int32_t)s.n0) - cn.begin()) - 1);
+  const int64_t nc = (int64_t)(std::lower_bound(cn.begin(), cn.end() - 1, (int32_t)s.n1) - cn.begin()) - c0;
+  constexpr int W = ILU_CHUNK, FW = 1;
+  const int side = LOWER ? 0 : 1;
+  const size_t smem = sweep_smem_bytes<T, NP>(W, p.slots);
+  const int per_sm = (int)std::min<size_t>(48 / (W + FW + 1), (size_t)(227 << 10) / (smem + 2048));
+  const unsigned ctas = resident_ctas(nc, 1, (unsigned)std::max(1, per_sm) * sm_count());
+  auto kern = ilu_sweep_kernel<T, LOWER, NP, W, FW>;
+  // more than the default 48 KB of dynamic shared memory (set for the current device)
+  cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  kern<<<ctas, (W + FW + 1) * 32, smem, st>>>(s.rec, p.seg, p.chunk, p.farptr[side], p.far[side], c0, nc, s.v,
+                                          s.pub, (uint4*)s.clr, s.out, (int)s.n0, (int)(s.n1 - s.n0),
+                                          p.slots, p.tickets, p.base, p.err, p.spin_limit);
+  p.base += (unsigned long long)nc + ctas;  // + each CTA's last claim
+}
+template <typename T, bool LOWER>
+static void sweep(Ilu& p, const SweepArgs<T>& s, cudaStream_t st) {
+  const int np = sweep_np(p, LOWER ? 0 : 1);
+  if (np == 1) launch_sweep<T, LOWER, 1>(p, s, st);
+  else if (np == 2) launch_sweep<T, LOWER, 2>(p, s, st);
+  else if (np == 3) launch_sweep<T, LOWER, 3>(p, s, st);
+  else launch_sweep<T, LOWER, 5>(p, s, st);
 }
 
 template <>
 int ilu_apply<float, float>(Ilu& p, const Mesh& m, int64_t n0, int64_t n1, const float* v, float* z,
                             cudaStream_t st) {
-  const int64_t rows = n1 - n0;
-  int64_t s0 = 0, ns = 0;
-  segment_range(p, n0, n1, s0, ns);
-  constexpr int W = sweep_warps<float>();
-  const int64_t chunks = (ns + W - 1) / W;
-  const unsigned ctas = resident_ctas(chunks, 1, 4 * sm_count());  // at most four CTAs per SM
-  const unsigned long long claims = (unsigned long long)chunks + ctas;  // + each CTA's last claim
-  uint32_t ep = next_epoch(p, st);
-  const size_t ring = sweep_ring_bytes<float>(W);
-  // the ring needs more than the default 48 KB of dynamic shared memory (set for the current device)
-  cudaFuncSetAttribute(ilu_sweep_kernel<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring);
-  cudaFuncSetAttribute(ilu_sweep_kernel<float, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring);
-  ilu_sweep_kernel<float, true><<<ctas, W * 32, ring, st>>>(
-      m.rowptr, m.colidx, p.F32, nullptr, p.dpos, p.seg, s0, ns, v, nullptr, p.yp, nullptr, n0,
-      rows, ep, p.tickets, p.base, p.err, p.spin_limit);
-  p.base += claims;
-  ep = next_epoch(p, st);
-  ilu_sweep_kernel<float, false><<<ctas, W * 32, ring, st>>>(
-      m.rowptr, m.colidx, p.F32, p.Dinv32, p.dpos, p.seg, s0, ns, nullptr, p.yp, p.xp, z, n0,
-      rows, ep, p.tickets, p.base, p.err, p.spin_limit);
-  p.base += claims;
+  sweep<float, true>(p, {p.rec32[0], n0, n1, v, p.yp32, p.xp32, p.y32}, st);
+  sweep<float, false>(p, {p.rec32[1], n0, n1, p.y32, p.xp32, p.yp32, z}, st);
   return 2;
 }
 
 template <>
 int ilu_apply<double, double>(Ilu& p, const Mesh& m, int64_t n0, int64_t n1, const double* v,
                               double* z, cudaStream_t st) {
-  const int64_t rows = n1 - n0;
-  int64_t s0 = 0, ns = 0;
-  segment_range(p, n0, n1, s0, ns);
-  constexpr int W = sweep_warps<double>();
-  const int64_t chunks = (ns + W - 1) / W;
-  const unsigned ctas = resident_ctas(chunks, 1, 4 * sm_count());  // at most four CTAs per SM
-  const unsigned long long claims = (unsigned long long)chunks + ctas;  // + each CTA's last claim
-  double* y = p.y;
-  double* x = p.x64;
-  cudaMemsetAsync(y + 4 * n0, 0xff, sizeof(double) * 4 * rows, st);
-  const size_t ring = sweep_ring_bytes<double>(W);
-  // the ring needs more than the default 48 KB of dynamic shared memory (set for the current device)
-  cudaFuncSetAttribute(ilu_sweep_kernel<double, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring);
-  cudaFuncSetAttribute(ilu_sweep_kernel<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)ring);
-  ilu_sweep_kernel<double, true><<<ctas, W * 32, ring, st>>>(
-      m.rowptr, m.colidx, p.F, nullptr, p.dpos, p.seg, s0, ns, v, nullptr, y, nullptr, n0, rows, 0,
-      p.tickets, p.base, p.err, p.spin_limit);
-  p.base += claims;
-  cudaMemsetAsync(x + 4 * n0, 0xff, sizeof(double) * 4 * rows, st);
-  ilu_sweep_kernel<double, false><<<ctas, W * 32, ring, st>>>(
-      m.rowptr, m.colidx, p.F, p.Dinv, p.dpos, p.seg, s0, ns, y, nullptr, x, z, n0, rows, 0,
-      p.tickets, p.base, p.err, p.spin_limit);
-  p.base += claims;
-  return 4;
+  int n = 2;
+  if (!p.packed64) {
+    n += pack<double>(p, m, p.rec, st);
+    p.packed64 = true;
+  }
+  sweep<double, true>(p, {p.rec[0], n0, n1, v, p.yp64, p.xp64, p.y}, st);
+  sweep<double, false>(p, {p.rec[1], n0, n1, p.y, p.xp64, p.yp64, z}, st);
+  return n;
 }
 
 int ilu_status(vms_ctx* ctx, Ilu& p, cudaStream_t st) {
@@ -853,8 +1008,10 @@ int ilu_status(vms_ctx* ctx, Ilu& p, cudaStream_t st) {
   cudaMemsetAsync(p.err, 0, sizeof(int), st);
   cudaMemsetAsync(p.tickets, 0, sizeof(unsigned long long), st);
   cudaMemsetAsync(p.flags, 0, sizeof(uint32_t) * p.n_nodes, st);
-  cudaMemsetAsync(p.yp, 0, sizeof(unsigned long long) * 4 * p.n_nodes, st);
-  cudaMemsetAsync(p.xp, 0, sizeof(unsigned long long) * 4 * p.n_nodes, st);
+  if (p.yp32) cudaMemsetAsync(p.yp32, 0xff, sizeof(float) * 4 * p.n_nodes, st);
+  if (p.xp32) cudaMemsetAsync(p.xp32, 0xff, sizeof(float) * 4 * p.n_nodes, st);
+  cudaMemsetAsync(p.yp64, 0xff, sizeof(double) * 4 * p.n_nodes, st);
+  cudaMemsetAsync(p.xp64, 0xff, sizeof(double) * 4 * p.n_nodes, st);
   cudaStreamSynchronize(st);
   p.base = 0;
   p.epoch = 0;

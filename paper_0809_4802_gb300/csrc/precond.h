@@ -12,6 +12,8 @@ constexpr uint32_t ILU_SPIN_DEFAULT = 1u << 22;  // with a 32 ns sleep per poll:
 constexpr int ILU_ERR_PIVOT = 2;
 constexpr int ILU_MAX_DEG = 32;
 constexpr int ILU_SEG_MAX = 64;
+constexpr int ILU_CHUNK = 4;         // segments of a sweep chunk
+constexpr int ILU_FAR_MAX = 1024;    // distinct far neighbours on one side of a chunk of several segments
 
 // Block ILU(0) of the node-block matrix (4x4 blocks, natural node order), factored and applied on
 // the device by warps that each own one node row and wait for the rows their row depends on.
@@ -27,17 +29,33 @@ struct Ilu {
   int32_t* seg = nullptr;           // device, n_segs + 1
   std::vector<int32_t> seg_host;    // host copy (segment ranges of node blocks)
   int64_t n_segs = 0;
+  // chunks of segments: chunk c is segments chunk[c] .. chunk[c+1] - 1, chunk_node its first nodes
+  // (host); far[0]/far[1]: its distinct neighbours in earlier / later chunks, from farptr[.][c] on
+  int32_t* chunk = nullptr;
+  std::vector<int32_t> chunk_node;
+  int64_t n_chunks = 0;
+  int32_t* farptr[2] = {nullptr, nullptr};
+  int32_t* far[2] = {nullptr, nullptr};
+  int32_t* at = nullptr;            // per block (CSR order): its column's slot in the row's chunk
+  int slots = 0;                    // most slots of a chunk (rows + far neighbours of one side)
+  uint8_t* inl = nullptr;           // n_nodes: bit 0 / 1: the node before / after is in the same segment
+  int side_lo = 0, side_up = 0;     // most blocks of a row below / above the diagonal, the row
+                                    // before it in its segment not counted
   // factor (always eliminated in FP64) and sweep work
   double* F = nullptr;         // nnz: L (unit lower, strictly lower blocks) and U, CSR layout
   double* Dinv = nullptr;      // n_nodes * 16: inverses of the diagonal blocks of U
-  float* F32 = nullptr;        // mixed precision: F rounded to FP32 (FP32 sweeps)
-  float* Dinv32 = nullptr;     // mixed precision: Dinv rounded to FP32
+  // the factor as the sweeps read it, one record per row (forward, backward)
+  unsigned char* rec[2] = {nullptr, nullptr};    // FP64 (made on the first FP64 sweep)
+  unsigned char* rec32[2] = {nullptr, nullptr};  // rounded to FP32 (mixed precision)
+  bool packed64 = false;       // rec holds the current factor
   double* vals64 = nullptr;    // mixed precision: FP64 copy of the FP32 matrix values
-  double* y = nullptr;         // 4 n_nodes: FP64 forward-sweep publication
-  double* x64 = nullptr;       // 4 n_nodes: FP64 backward-sweep publication
-  uint32_t* flags = nullptr;   // n_nodes: row-ready epochs (factorisation, FP64 sweeps)
-  unsigned long long* yp = nullptr;  // 4 n_nodes: FP32 forward sweep, (epoch << 32 | value bits)
-  unsigned long long* xp = nullptr;  // 4 n_nodes: FP32 backward sweep, same packing
+  double* y = nullptr;         // 4 n_nodes: L^-1 v (FP64 sweeps; compact over the rows solved)
+  float* y32 = nullptr;        // 4 n_nodes: L^-1 v (FP32 sweeps)
+  double* yp64 = nullptr;      // 4 n_nodes: FP64 forward-sweep publication, all ones between sweeps
+  double* xp64 = nullptr;      // 4 n_nodes: FP64 backward-sweep publication, all ones between sweeps
+  uint32_t* flags = nullptr;   // n_nodes: row-ready epochs of the factorisation
+  float* yp32 = nullptr;       // 4 n_nodes each: the FP32 sweeps' publications, all ones between sweeps
+  float* xp32 = nullptr;
   unsigned long long* tickets = nullptr;  // row-claim counters (never reset between launches)
   int* err = nullptr;          // device error word: 0, ILU_ERR_TIMEOUT or ILU_ERR_PIVOT
   uint32_t epoch = 0;
