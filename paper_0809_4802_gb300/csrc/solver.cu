@@ -14,15 +14,17 @@
 #include <type_traits>
 #include <vector>
 
+#include "ortho.cuh"
 #include "solver.h"
 
 namespace vms {
 
 void free_solver(SolverWork& s) {
   void* bufs[] = {s.x, s.r, s.V, s.Z, s.Dinv, s.h, s.rfull, s.bf, s.xf, s.cx, s.pv, s.pz, s.Zf,
-                  s.xb, s.rb, s.band};
+                  s.xb, s.rb, s.band, s.og};
   for (void* b : bufs)
     if (b) cudaFree(b);
+  if (s.hcol) cudaFreeHost(s.hcol);
   for (BandOrder& o : s.band_orders)
     if (o.perm) cudaFree(o.perm);
   const uint32_t lim = s.ilu.spin_limit;  // a setting of the context, kept across re-allocations
@@ -169,10 +171,10 @@ __global__ void block_apply_kernel(const double* __restrict__ Dinv, const VT* __
 }
 
 constexpr int DOT_THREADS = 256;
-// device scratch layout (doubles): Gram-Schmidt coefficients of the two passes, a norm, the
-// least-squares solution, then per-block partial sums
+// device scratch layout (doubles): a norm, the least-squares solution, then per-block partial sums
 constexpr int MAX_RESTART = 480;
-constexpr int H_PASS1 = 0, H_PASS2 = 512, H_NORM = 1024, H_Y = 1025, H_PART = 1536;
+constexpr int H_NORM = 0, H_Y = 1, H_PART = 512;
+static_assert(MAX_RESTART == OG_MAX, "ortho_kernel's vectors");
 
 __device__ __forceinline__ double block_reduce(double v, double* sh) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -492,6 +494,24 @@ struct Gmres {
     return e == cudaSuccess ? VMS_OK : ctx_fail(ctx, VMS_ERR_CUDA, cudaGetErrorString(e));
   }
 
+  // Queue the orthogonalisation of V_kk against V_0..V_{kk-1} (ortho_kernel): one block per SM, with
+  // at least 128 quads of rows each (fewer blocks: shorter sums over them). The Hessenberg column goes to w.hcol (page-locked).
+  template <typename VT>
+  int orthogonalise(VT* V, int kk) {
+    int64_t nn = n;
+    int blocks = (int)std::min<int64_t>({(n / 4 + 127) / 128, (int64_t)sm_count(), (int64_t)OG_BLOCKS});
+    double *X = w.og + (w.og_turn ? OG_SET : 0), *Y = w.og + (w.og_turn ? 0 : OG_SET), *out = w.hcol;
+    out[kk + 1] = 0.0;
+    void* args[] = {&V, &nn, &kk, &X, &Y, &w.og_k, &w.og_blocks, &out};
+    const cudaError_t e = cudaLaunchCooperativeKernel((const void*)ortho_kernel<VT>, dim3((unsigned)blocks),
+                                                      dim3(OG_THREADS), args, 0, st);
+    if (e != cudaSuccess) return ctx_fail(ctx, VMS_ERR_CUDA, cudaGetErrorString(e));
+    w.og_turn = !w.og_turn;
+    w.og_k = kk;
+    w.og_blocks = blocks;
+    return VMS_OK;
+  }
+
   // One restarted GMRES solve of A x = b from x = 0 in vector type VT; matrix values type T.
   // Returns VMS_OK with *iters and *relres; x receives the solution.
   // Grow the Krylov basis (and the kept preconditioned vectors) to `restart` vectors, keeping V_0.
@@ -529,7 +549,7 @@ struct Gmres {
     VT* z = reinterpret_cast<VT*>(w.Z);
     double* hd = w.h;
     std::vector<double> H((restart + 1) * restart, 0.0), cs(restart), sn(restart), g(restart + 1);
-    std::vector<double> hh(restart + 2), hcol(H_NORM + 1);
+    std::vector<double> hh(restart + 2);
     {
       KScope zs(ctx, VMS_K_FILL);
       zs.add(launch_fill_zero(x, sizeof(VT) * n, st));
@@ -568,30 +588,23 @@ struct Gmres {
         VT* zj = Zflex ? reinterpret_cast<VT*>(Zflex) + (int64_t)j * n : z;
         precond<T, VT>(vj, zj);
         { KScope k(ctx, VMS_K_SPMV); k.add(spmv<T, VT>(m, R, values, zj, vn, st)); }
-        // CGS2 against V_0..V_j: first pass coefficients into hd[H_PASS1..], second into hd[H_PASS2..]
+        // orthogonalise against V_0..V_j and normalise; the Hessenberg column lands in host memory
         const int kk = j + 1;
-        double* partial = hd + H_PART;
-        for (int pass = 0; pass < 2; ++pass) {
-          {
-            KScope k(ctx, VMS_K_REDUCE);
-            k.add(dots<VT>(V, n, kk, vn, n, partial, hd + (pass ? H_PASS2 : H_PASS1), st));
-          }
-          KScope k(ctx, VMS_K_KRYLOV);
-          k.add(vcomb<VT>(V, n, hd + (pass ? H_PASS2 : H_PASS1), kk, -1.0, vn, vn, n, st));
-        }
-        {
-          KScope k(ctx, VMS_K_REDUCE);
-          k.add(dots<VT>(vn, n, 1, vn, n, partial, hd + H_NORM, st));
-        }
         {
           KScope k(ctx, VMS_K_KRYLOV);
-          scale_kernel<VT><<<grid_for(n), 256, 0, st>>>(vn, hd + H_NORM, vn, n);
+          if (int rc2 = orthogonalise<VT>(V, kk)) return rc2;
           k.add(1);
         }
-        // bring the Hessenberg column (both passes and the norm) to the host in one copy
-        if (int rc2 = sync_host(hcol.data(), hd, sizeof(double) * (H_NORM + 1))) return rc2;
-        const double nrm2 = hcol[H_NORM];
-        for (int i = 0; i < kk; ++i) hh[i] = hcol[H_PASS1 + i] + hcol[H_PASS2 + i];
+        cudaError_t es = cudaStreamSynchronize(st);
+        if (es != cudaSuccess) return ctx_fail(ctx, VMS_ERR_CUDA, cudaGetErrorString(es));
+        const double* hcol = w.hcol;
+        if (hcol[kk + 1] != 0.0) {  // a wait gave up: start with fresh exchange words
+          cudaMemsetAsync(w.og, 0xff, sizeof(double) * 2 * OG_SET, st);
+          w.og_k = w.og_blocks = 0;
+          return ctx_fail(ctx, VMS_ERR_TIMEOUT, "orthogonalisation: a block waited longer than its limit");
+        }
+        const double nrm2 = hcol[kk];
+        for (int i = 0; i < kk; ++i) hh[i] = hcol[i];
         hh[kk] = std::sqrt(nrm2);
         // apply previous rotations, then a new one
         for (int i = 0; i < j; ++i) {
@@ -706,6 +719,9 @@ static int ensure_solver(vms_ctx* ctx, int restart) {
   if (e == cudaSuccess) e = cudaMalloc(&w.pv, sizeof(float) * n);
   if (e == cudaSuccess) e = cudaMalloc(&w.pz, sizeof(float) * n);
   if (e == cudaSuccess) e = cudaMalloc(&w.band, sizeof(int) * 4);
+  if (e == cudaSuccess) e = cudaMallocHost(&w.hcol, sizeof(double) * (MAX_RESTART + 2));
+  if (e == cudaSuccess) e = cudaMalloc(&w.og, sizeof(double) * 2 * OG_SET);
+  if (e == cudaSuccess) e = cudaMemset(w.og, 0xff, sizeof(double) * 2 * OG_SET);
   if (e != cudaSuccess) {
     free_solver(w);
     return ctx_fail(ctx, e == cudaErrorMemoryAllocation ? VMS_ERR_OUT_OF_MEMORY : VMS_ERR_CUDA,

@@ -32,6 +32,10 @@ struct SolverWork {
   double* Z = nullptr;       // n preconditioned vector (FP32 views in mixed mode)
   double* Dinv = nullptr;    // n_nodes * 16: inverted 4x4 diagonal node blocks
   double* h = nullptr;       // device scalars for dots
+  double* hcol = nullptr;    // page-locked: the Hessenberg column of the current step (ortho_kernel)
+  double* og = nullptr;      // 2 OG_SET: exchange words of ortho_kernel, two launches' taking turns
+  bool og_turn = false;
+  int og_k = 0, og_blocks = 0;  // vectors and blocks of the last launch
   double* rfull = nullptr;   // n: FP64 refinement residual (mixed)
   float* bf = nullptr;       // n: FP32 right-hand side of the inner solve (mixed)
   float* xf = nullptr;       // n: FP32 inner correction (mixed)
