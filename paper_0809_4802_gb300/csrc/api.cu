@@ -594,7 +594,7 @@ static int mesh_upload_impl(vms_ctx* ctx, int npe, int64_t n_nodes, const double
   CK(cudaMalloc(&w.resid, sizeof(double) * (4 * n_nodes + 3 * n_elems)));
   CK(cudaMalloc(&w.partial, sizeof(double) * 1024));
   CK(cudaMalloc(&w.flags, sizeof(unsigned int)));
-  CK(cudaMalloc(&w.queues, 2 * sizeof(unsigned long long)));
+  CK(cudaMalloc(&w.queues, 4 * sizeof(unsigned long long)));
   return VMS_OK;
 }
 
@@ -700,7 +700,7 @@ static int enqueue_assembly(vms_ctx* ctx, cudaStream_t st) {
     // residual and tangent in one persistent launch, then r_e and the Dirichlet rows
     {
       KScope k(ctx, VMS_K_FILL, st);
-      k.add(launch_fill_zero(w.queues, 2 * sizeof(unsigned long long), st));
+      k.add(launch_fill_zero(w.queues, 4 * sizeof(unsigned long long), st));
     }
     {
       KScope k(ctx, VMS_K_FUSED, st);
@@ -721,7 +721,7 @@ static int enqueue_assembly(vms_ctx* ctx, cudaStream_t st) {
   CK(cudaStreamWaitEvent(w.aux, w.fork, 0));
   {
     KScope k(ctx, VMS_K_RESIDUAL, st);
-    k.add(launch_residual(m, ctx->state, kp, ctx->d_qp, w.elemR, nullptr, 0, m.n_elems, 0, w.flags, st));
+    k.add(launch_residual(m, ctx->state, kp, ctx->d_qp, w.elemR, nullptr, 0, m.n_elems, 0, w.flags, st, true));
   }
   {
     KScope k(ctx, VMS_K_TANGENT, w.aux);

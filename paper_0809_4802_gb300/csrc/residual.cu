@@ -45,6 +45,53 @@ __global__ void __launch_bounds__(THREADS) residual_kernel(
   }
 }
 
+// The residual with a lane per line of the Gauss rule (residual_lines), one warp per block.
+template <bool TRANSIENT, bool FORCE, int N1>
+__global__ void __launch_bounds__(32) residual_lines_kernel(
+    const double4_32a* __restrict__ xyz, const double4_32a* __restrict__ u,
+    const double4_32a* __restrict__ uprev, const int32_t* __restrict__ conn,
+    const double* __restrict__ beta, KParams kp, const QpRow* __restrict__ qp, int64_t first,
+    int64_t count, double* __restrict__ elemR, double* __restrict__ resid,
+    const uint32_t* __restrict__ dir_mask, int64_t n_nodes, int mode, unsigned int* __restrict__ flags) {
+  constexpr int S = N1 * N1, EPW = 32 / S;
+  __shared__ double sm[EPW][rl_doubles<N1>()];
+  const int lane = threadIdx.x, el = lane / S, ln = lane - el * S;
+  const int64_t t = (int64_t)blockIdx.x * EPW + el;
+  const bool valid = el < EPW && t < count;
+  const int64_t e = first + (valid ? t : 0);
+  const uint32_t msk = mode ? dir_mask[e] : 0u;
+  const unsigned bad = residual_lines<TRANSIENT, FORCE, N1>(
+      valid, e, ln, sm[el < EPW ? el : 0], GlobalTable{qp}, kp, xyz, u, uprev, conn, beta,
+      [&](int a, int c, double v) {
+        if (mode == 0) elemR[36 * e + 4 * a + c] = v;
+        else if (!(msk >> (4 * a + c) & 1u)) atomicAdd(resid + 4 * (int64_t)conn[8 * e + a] + c, v);
+      },
+      [&](int i, double v) {
+        if (mode == 0) elemR[36 * e + 32 + i] = v;
+        else resid[4 * n_nodes + 3 * e + i] = v;
+      });
+  if (bad) atomicOr(flags, bad);
+}
+
+template <int N1>
+static void launch_lines(const Mesh& m, const State& s, const KParams& kp, const QpRow* qp,
+                         double* elemR, double* resid, int64_t first, int64_t count, int mode,
+                         unsigned int* flags, cudaStream_t st) {
+  constexpr int EPW = 32 / (N1 * N1);
+  const unsigned grid = (unsigned)((count + EPW - 1) / EPW);
+  auto launch = [&](auto kern) {
+    kern<<<grid, 32, 0, st>>>(m.xyz, s.u, s.u_prev, m.conn, s.beta, kp, qp, first, count, elemR, resid,
+                              m.dir_mask, m.n_nodes, mode, flags);
+  };
+  if (kp.transient) {
+    if (kp.has_force) launch(residual_lines_kernel<true, true, N1>);
+    else launch(residual_lines_kernel<true, false, N1>);
+  } else {
+    if (kp.has_force) launch(residual_lines_kernel<false, true, N1>);
+    else launch(residual_lines_kernel<false, false, N1>);
+  }
+}
+
 template <int THREADS>
 static void launch_r(const Mesh& m, const State& s, const KParams& kp, const QpRow* qp,
                      double* elemR, double* resid, int64_t first, int64_t count, int mode,
@@ -65,15 +112,47 @@ static void launch_r(const Mesh& m, const State& s, const KParams& kp, const QpR
   }
 }
 
+// Elements of `count` that go to the lane-per-line kernel: those past the last whole round, a round
+// being 64 elements per SM and half an SM's threads (2 U, one warp per SM partition), where the lines
+// take less time than a part of a round of threads. Measured in us (27 points; 8; 64), U = 9,728
+// elements on 152 SMs: threads U 184, 2 U 195, 3 U 288, 4 U 371 (75, 82, 115, 146; 396, 420, 636, 815)
+// in steps of U and again from there; lines 29 up to 1,728 elements (25; 34), then 14 + 12.6 per
+// thousand (10 + 3.9; 10 + 24). The bounds below are where the two meet.
+// Beside an FP64 tangent (`beside`) the lines of up to 2 U elements fill the tangent's gaps better:
+// an assembly of 512 elements takes 130 us with lines, 228 with threads, 4,096 362 and 415, 12,167
+// 893 and 1,029, 17,576 1,279 and 1,346, 19,683 1,435 and 1,436; past that the lines' extra FP64 work
+// (a third) costs more than it hides (32,768: 2,318 and 2,253; a part of them in lines: up to 4 % more).
+int64_t residual_rest(int nq, int64_t count, bool beside) {
+  const int64_t U = 64 * (int64_t)sm_count(), r = count % (2 * U);
+  if (beside) return count <= 2 * U ? count : 0;
+  const bool half = (count / (2 * U)) & 1;  // the SMs already hold two blocks each
+  const int pct = nq == 27 ? (half ? (r <= U ? 64 : 130) : 135) : (half ? (r <= U ? 75 : 150) : 160);
+  return r * 100 <= U * pct ? r : 0;
+}
+
 int launch_residual(const Mesh& m, const State& s, const KParams& kp, const QpRow* qp,
                      double* elemR, double* resid, int64_t first, int64_t count, int mode,
-                     unsigned int* flags, cudaStream_t st) {
+                     unsigned int* flags, cudaStream_t st, bool beside) {
   if (count <= 0) return 0;
-  if (kp.residual_threads == 32)
-    launch_r<32>(m, s, kp, qp, elemR, resid, first, count, mode, flags, st);
-  else
-    launch_r<RES_THREADS>(m, s, kp, qp, elemR, resid, first, count, mode, flags, st);
-  return 1;
+  // whole rounds with a thread per element, a remainder that would leave the SMs half empty (all of a
+  // small mesh) with a lane per line
+  const int64_t rest = residual_rest(kp.nq, count, beside), whole = count - rest;
+  int n = 0;
+  if (whole > 0) {
+    if (kp.residual_threads == 32)
+      launch_r<32>(m, s, kp, qp, elemR, resid, first, whole, mode, flags, st);
+    else
+      launch_r<RES_THREADS>(m, s, kp, qp, elemR, resid, first, whole, mode, flags, st);
+    ++n;
+  }
+  if (rest > 0) {
+    const int64_t f = first + whole;
+    if (kp.nq == 27) launch_lines<3>(m, s, kp, qp, elemR, resid, f, rest, mode, flags, st);
+    else if (kp.nq == 8) launch_lines<2>(m, s, kp, qp, elemR, resid, f, rest, mode, flags, st);
+    else launch_lines<4>(m, s, kp, qp, elemR, resid, f, rest, mode, flags, st);
+    ++n;
+  }
+  return n;
 }
 
 }  // namespace vms

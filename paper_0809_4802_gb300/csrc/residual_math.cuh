@@ -62,6 +62,139 @@ VMS_HD void residual_load(const Store& C, const double X[8][3], const double U[8
   }
 }
 
+// The fields along one line of the Gauss rule (eta and zeta fixed): every one is an intercept plus xi
+// times a slope. J[.][1] = j1a + xi j1b, J[.][2] = j2a + xi j2b and J[.][0] = J0; the reference velocity
+// gradient's columns vb, g1a + xi g1b, g2a + xi g2b; v = va + xi vb; p = pa + xi pb; vbar - vbar_n = dva + xi dvb.
+struct ResLine {
+  double J0[3], j1a[3], j1b[3], j2a[3], j2b[3], g1a[3], g1b[3], g2a[3], g2b[3], va[3], vb[3], dva[3], dvb[3], pa, pb;
+};
+// Its sums: src, xi src, P0, P1, xi P1, P2, xi P2 (per component), Tp, xi Tp.
+struct ResSums {
+  double s0[3], s1[3], b0[3], c0[3], c1[3], d0[3], d1[3], t0, t1;
+};
+
+// The sums of the line whose first point is q0 (and R_f, added to); false if det J <= 0 at a point.
+template <bool TRANSIENT, bool FORCE, int N1, class Table>
+VMS_HD bool residual_line(const Table& tab, int q0, const ResLine& ln, const double bet[3], double nut, double tau,
+                          const double f[3], ResSums& o_, double Rf[3]) {
+  constexpr int n1 = N1;
+  bool ok = true;
+  // One point of the line: its source term src_i, the fluxes P_al,i paired with the
+  // reference-gradient components of the test functions, and the continuity term Tp.
+  struct Pt {
+    double src[3], P0[3], P1[3], P2[3], Tp;
+  };
+  auto point = [&](int ii, Pt& o) {
+    const int q = q0 + ii;
+    const double xi = tab.xi(q);
+    const double bq = tab.b(q), db0 = tab.db(q, 0), db1 = tab.db(q, 1), db2 = tab.db(q, 2);
+    const double wq = tab.w(q);
+
+    double J[3][3];
+    VMS_UNROLL
+    for (int i = 0; i < 3; ++i) {
+      J[i][0] = ln.J0[i];
+      J[i][1] = ln.j1a[i] + xi * ln.j1b[i];
+      J[i][2] = ln.j2a[i] + xi * ln.j2b[i];
+    }
+    double cof[3][3];
+    double det = cofactor3(J, cof);
+    if (!(det >= DET_MIN)) { ok = false; det = 1.0; }
+
+    double v[3], G[3][3];
+    VMS_UNROLL
+    for (int i = 0; i < 3; ++i) {
+      v[i] = ln.va[i] + xi * ln.vb[i] + bq * bet[i];
+      G[i][0] = ln.vb[i] + bet[i] * db0;
+      G[i][1] = ln.g1a[i] + xi * ln.g1b[i] + bet[i] * db1;
+      G[i][2] = ln.g2a[i] + xi * ln.g2b[i] + bet[i] * db2;
+    }
+    const double p = ln.pa + xi * ln.pb;
+
+    // H = G cof^T: det J times the physical velocity gradient (H[i][j] = det dv_i/dx_j)
+    double H[3][3];
+    VMS_UNROLL
+    for (int i = 0; i < 3; ++i)
+      VMS_UNROLL
+      for (int j = 0; j < 3; ++j)
+        H[i][j] = G[i][0] * cof[j][0] + G[i][1] * cof[j][1] + G[i][2] * cof[j][2];
+    // src_i = w_q (H v - det f + tau det (vbar - vbar_n))_i, Tp = -w_q tr H
+    double y[3];
+    VMS_UNROLL
+    for (int i = 0; i < 3; ++i) y[i] = H[i][0] * v[0] + H[i][1] * v[1] + H[i][2] * v[2];
+    if (FORCE) {
+      VMS_UNROLL
+      for (int i = 0; i < 3; ++i) y[i] -= det * f[i];
+    }
+    if (TRANSIENT) {
+      const double td = tau * det;
+      VMS_UNROLL
+      for (int i = 0; i < 3; ++i) y[i] += td * (ln.dva[i] + xi * ln.dvb[i]);
+    }
+    VMS_UNROLL
+    for (int i = 0; i < 3; ++i) o.src[i] = wq * y[i];
+    o.Tp = -wq * (H[0][0] + H[1][1] + H[2][2]);
+    // P = (s H - w_q p I) cof with s = w_q nut / det: w_q (nut L - p I) times det J^-T
+    const double s = wq * nut * recip_normal(det);
+    const double nwp = -wq * p;
+    VMS_UNROLL
+    for (int i = 0; i < 3; ++i)
+      VMS_UNROLL
+      for (int j = 0; j < 3; ++j) H[i][j] = i == j ? s * H[i][j] + nwp : s * H[i][j];
+    VMS_UNROLL
+    for (int i = 0; i < 3; ++i) {
+      o.P0[i] = H[i][0] * cof[0][0] + H[i][1] * cof[1][0] + H[i][2] * cof[2][0];
+      o.P1[i] = H[i][0] * cof[0][1] + H[i][1] * cof[1][1] + H[i][2] * cof[2][1];
+      o.P2[i] = H[i][0] * cof[0][2] + H[i][1] * cof[1][2] + H[i][2] * cof[2][2];
+    }
+  };
+  // The points are taken in symmetric pairs (-x, x): the Gauss points are symmetric about 0 (the middle
+  // one of an odd rule is 0), b, db1, db2 are even in xi and db0 is odd, so with
+  // u = y(x) + y(-x) and w = y(x) - y(-x) a pair adds u to a sum, x w to a xi-moment, and
+  // b(x) u_src + db0(x) w_P0 + db1(x) u_P1 + db2(x) u_P2 to R_f.
+  VMS_UNROLL
+  for (int pp = 0; pp < n1 / 2; ++pp) {
+    Pt lo, hi;
+    point(pp, lo);
+    point(n1 - 1 - pp, hi);
+    const int qh = q0 + n1 - 1 - pp;
+    const double x = tab.xi(qh), bh = tab.b(qh);
+    const double e0 = tab.db(qh, 0), e1 = tab.db(qh, 1), e2 = tab.db(qh, 2);
+    VMS_UNROLL
+    for (int i = 0; i < 3; ++i) {
+      const double us = hi.src[i] + lo.src[i], ws = hi.src[i] - lo.src[i];
+      const double u0 = hi.P0[i] + lo.P0[i], w0 = hi.P0[i] - lo.P0[i];
+      const double u1 = hi.P1[i] + lo.P1[i], w1 = hi.P1[i] - lo.P1[i];
+      const double u2 = hi.P2[i] + lo.P2[i], w2 = hi.P2[i] - lo.P2[i];
+      Rf[i] = Rf[i] + bh * us + e0 * w0 + e1 * u1 + e2 * u2;
+      if (pp == 0) {
+        o_.s0[i] = us; o_.s1[i] = x * ws; o_.b0[i] = u0; o_.c0[i] = u1; o_.c1[i] = x * w1; o_.d0[i] = u2;
+        o_.d1[i] = x * w2;
+      } else {
+        o_.s0[i] += us; o_.s1[i] += x * ws; o_.b0[i] += u0; o_.c0[i] += u1; o_.c1[i] += x * w1; o_.d0[i] += u2;
+        o_.d1[i] += x * w2;
+      }
+    }
+    const double ut = hi.Tp + lo.Tp, wt = hi.Tp - lo.Tp;
+    if (pp == 0) { o_.t0 = ut; o_.t1 = x * wt; }
+    else { o_.t0 += ut; o_.t1 += x * wt; }
+  }
+  if (n1 & 1) {
+    // the middle point, xi = 0: no xi-moment, db0 = 0
+    Pt m;
+    point(n1 / 2, m);
+    const int qm = q0 + n1 / 2;
+    const double bm = tab.b(qm), e1 = tab.db(qm, 1), e2 = tab.db(qm, 2);
+    VMS_UNROLL
+    for (int i = 0; i < 3; ++i) {
+      Rf[i] = Rf[i] + bm * m.src[i] + e1 * m.P1[i] + e2 * m.P2[i];
+      o_.s0[i] += m.src[i]; o_.b0[i] += m.P0[i]; o_.c0[i] += m.P1[i]; o_.d0[i] += m.P2[i];
+    }
+    o_.t0 += m.Tp;
+  }
+  return ok;
+}
+
 // Quadrature loop. Rcp[32] (node-major 4a+c) and Rf[3] receive the element residual; returns
 // false if det J <= 0 at some point (the offending point then uses det J = 1).
 //
@@ -124,121 +257,19 @@ VMS_HD bool residual_qp_loop_n(const Store& C, const Table& tab, const double be
         }
       }
       const double pa = apa + bpa * eta, pb = apb + bpb * eta;
-      // One point of the line: its source term src_i, the fluxes P_al,i paired with the
-      // reference-gradient components of the test functions, and the continuity term Tp.
-      struct Pt {
-        double src[3], P0[3], P1[3], P2[3], Tp;
-      };
-      auto point = [&](int ii, Pt& o) {
-        const int q = q0 + ii;
-        const double xi = tab.xi(q);
-        const double bq = tab.b(q), db0 = tab.db(q, 0), db1 = tab.db(q, 1), db2 = tab.db(q, 2);
-        const double wq = tab.w(q);
-
-        double J[3][3];
-        VMS_UNROLL
-        for (int i = 0; i < 3; ++i) {
-          J[i][0] = J0[i];
-          J[i][1] = j1a[i] + xi * j1b[i];
-          J[i][2] = j2a[i] + xi * j2b[i];
-        }
-        double cof[3][3];
-        double det = cofactor3(J, cof);
-        if (!(det >= DET_MIN)) { ok = false; det = 1.0; }
-
-        double v[3], G[3][3];
-        VMS_UNROLL
-        for (int i = 0; i < 3; ++i) {
-          v[i] = va[i] + xi * vb[i] + bq * bet[i];
-          G[i][0] = vb[i] + bet[i] * db0;
-          G[i][1] = g1a[i] + xi * g1b[i] + bet[i] * db1;
-          G[i][2] = g2a[i] + xi * g2b[i] + bet[i] * db2;
-        }
-        const double p = pa + xi * pb;
-
-        // H = G cof^T: det J times the physical velocity gradient (H[i][j] = det dv_i/dx_j)
-        double H[3][3];
-        VMS_UNROLL
-        for (int i = 0; i < 3; ++i)
-          VMS_UNROLL
-          for (int j = 0; j < 3; ++j)
-            H[i][j] = G[i][0] * cof[j][0] + G[i][1] * cof[j][1] + G[i][2] * cof[j][2];
-        // src_i = w_q (H v - det f + tau det (vbar - vbar_n))_i, Tp = -w_q tr H
-        double y[3];
-        VMS_UNROLL
-        for (int i = 0; i < 3; ++i) y[i] = H[i][0] * v[0] + H[i][1] * v[1] + H[i][2] * v[2];
-        if (FORCE) {
-          VMS_UNROLL
-          for (int i = 0; i < 3; ++i) y[i] -= det * f[i];
-        }
-        if (TRANSIENT) {
-          const double td = tau * det;
-          VMS_UNROLL
-          for (int i = 0; i < 3; ++i) y[i] += td * (dva[i] + xi * dvb[i]);
-        }
-        VMS_UNROLL
-        for (int i = 0; i < 3; ++i) o.src[i] = wq * y[i];
-        o.Tp = -wq * (H[0][0] + H[1][1] + H[2][2]);
-        // P = (s H - w_q p I) cof with s = w_q nut / det: w_q (nut L - p I) times det J^-T
-        const double s = wq * nut * recip_normal(det);
-        const double nwp = -wq * p;
-        VMS_UNROLL
-        for (int i = 0; i < 3; ++i)
-          VMS_UNROLL
-          for (int j = 0; j < 3; ++j) H[i][j] = i == j ? s * H[i][j] + nwp : s * H[i][j];
-        VMS_UNROLL
-        for (int i = 0; i < 3; ++i) {
-          o.P0[i] = H[i][0] * cof[0][0] + H[i][1] * cof[1][0] + H[i][2] * cof[2][0];
-          o.P1[i] = H[i][0] * cof[0][1] + H[i][1] * cof[1][1] + H[i][2] * cof[2][1];
-          o.P2[i] = H[i][0] * cof[0][2] + H[i][1] * cof[1][2] + H[i][2] * cof[2][2];
-        }
-      };
-      // line sums: src, xi src, P0, P1, xi P1, P2, xi P2 (per component), Tp, xi Tp. The points
-      // are taken in symmetric pairs (-x, x): the Gauss points are symmetric about 0 (the middle
-      // one of an odd rule is 0), b, db1, db2 are even in xi and db0 is odd, so with
-      // u = y(x) + y(-x) and w = y(x) - y(-x) a pair adds u to a sum, x w to a xi-moment, and
-      // b(x) u_src + db0(x) w_P0 + db1(x) u_P1 + db2(x) u_P2 to R_f.
-      double s0[3], s1[3], b0[3], c0[3], c1[3], d0[3], d1[3], t0, t1;
+      ResLine ln;
       VMS_UNROLL
-      for (int pp = 0; pp < n1 / 2; ++pp) {
-        Pt lo, hi;
-        point(pp, lo);
-        point(n1 - 1 - pp, hi);
-        const int qh = q0 + n1 - 1 - pp;
-        const double x = tab.xi(qh), bh = tab.b(qh);
-        const double e0 = tab.db(qh, 0), e1 = tab.db(qh, 1), e2 = tab.db(qh, 2);
-        VMS_UNROLL
-        for (int i = 0; i < 3; ++i) {
-          const double us = hi.src[i] + lo.src[i], ws = hi.src[i] - lo.src[i];
-          const double u0 = hi.P0[i] + lo.P0[i], w0 = hi.P0[i] - lo.P0[i];
-          const double u1 = hi.P1[i] + lo.P1[i], w1 = hi.P1[i] - lo.P1[i];
-          const double u2 = hi.P2[i] + lo.P2[i], w2 = hi.P2[i] - lo.P2[i];
-          Rf[i] = Rf[i] + bh * us + e0 * w0 + e1 * u1 + e2 * u2;
-          if (pp == 0) {
-            s0[i] = us; s1[i] = x * ws; b0[i] = u0; c0[i] = u1; c1[i] = x * w1; d0[i] = u2;
-            d1[i] = x * w2;
-          } else {
-            s0[i] += us; s1[i] += x * ws; b0[i] += u0; c0[i] += u1; c1[i] += x * w1; d0[i] += u2;
-            d1[i] += x * w2;
-          }
-        }
-        const double ut = hi.Tp + lo.Tp, wt = hi.Tp - lo.Tp;
-        if (pp == 0) { t0 = ut; t1 = x * wt; }
-        else { t0 += ut; t1 += x * wt; }
+      for (int i = 0; i < 3; ++i) {
+        ln.J0[i] = J0[i]; ln.j1a[i] = j1a[i]; ln.j1b[i] = j1b[i]; ln.j2a[i] = j2a[i]; ln.j2b[i] = j2b[i];
+        ln.g1a[i] = g1a[i]; ln.g1b[i] = g1b[i]; ln.g2a[i] = g2a[i]; ln.g2b[i] = g2b[i];
+        ln.va[i] = va[i]; ln.vb[i] = vb[i];
+        if (TRANSIENT) { ln.dva[i] = dva[i]; ln.dvb[i] = dvb[i]; }
       }
-      if (n1 & 1) {
-        // the middle point, xi = 0: no xi-moment, db0 = 0
-        Pt m;
-        point(n1 / 2, m);
-        const int qm = q0 + n1 / 2;
-        const double bm = tab.b(qm), e1 = tab.db(qm, 1), e2 = tab.db(qm, 2);
-        VMS_UNROLL
-        for (int i = 0; i < 3; ++i) {
-          Rf[i] = Rf[i] + bm * m.src[i] + e1 * m.P1[i] + e2 * m.P2[i];
-          s0[i] += m.src[i]; b0[i] += m.P0[i]; c0[i] += m.P1[i]; d0[i] += m.P2[i];
-        }
-        t0 += m.Tp;
-      }
+      ln.pa = pa; ln.pb = pb;
+      ResSums sm;
+      if (!residual_line<TRANSIENT, FORCE, N1>(tab, q0, ln, bet, nut, tau, f, sm, Rf)) ok = false;
+      const double *s0 = sm.s0, *s1 = sm.s1, *b0 = sm.b0, *c0 = sm.c0, *c1 = sm.c1, *d0 = sm.d0, *d1 = sm.d1;
+      const double t0 = sm.t0, t1 = sm.t1;
       // the line's contributions to the monomial sums: xi^a eta^b zeta^c src_i and the
       // derivatives d/dxi (P0), d/deta (P1), d/dzeta (P2) of the same monomials
       VMS_UNROLL
@@ -370,6 +401,128 @@ __device__ __forceinline__ unsigned residual_element(
   VMS_UNROLL
   for (int k = 0; k < 32; ++k) finite = finite && isfinite(Rcp[k]);
   return (ok ? 0u : 1u) | (finite ? 0u : 4u);
+}
+
+// The same residual with the N1^2 lines of the Gauss rule on as many lanes, 32 / N1^2 elements per
+// warp (an FP64 instruction takes 64 cycles of a warp, however many lanes are active, so a thread
+// per element takes about 170 us alone; a line takes a ninth of the points). The element's fields are
+// mapped to their monomial coefficients one per lane; every lane walks its line and forms its shares
+// of the 32 monomial sums and of R_f; the lanes then sum one output each and map a component each
+// back to the nodes. `sm`: the element's RL_DOUBLES in shared memory; `ln`: the lane's line; lanes
+// without an element (`valid` false) only take part in the warp's barriers. `put(a, c, value)`
+// receives R_cp, putf(i, value) R_f. Returns error bits as residual_element.
+template <int N1> constexpr int rl_doubles() { return RC_RM + 35 * N1 * N1 + 35; }
+template <bool TRANSIENT, bool FORCE, int N1, class Table, class P, class Put, class PutF>
+__device__ __forceinline__ unsigned residual_lines(
+    bool valid, int64_t e, int ln, double* sm, const Table& tab, const P& kp,
+    const double4_32a* __restrict__ xyz, const double4_32a* __restrict__ u,
+    const double4_32a* __restrict__ uprev, const int32_t* __restrict__ conn,
+    const double* __restrict__ beta, const Put& put, const PutF& putf) {
+  constexpr int S = N1 * N1;
+  double* share = sm + RC_RM;          // [35][S]
+  double* total = sm + RC_RM + 35 * S;  // [35]
+  unsigned bad = 0;
+  if (valid)
+    for (int fi = ln; fi < (TRANSIENT ? 10 : 7); fi += S) {  // x (3), v and p (4), v - v_prev (3)
+      const int comp = fi < 3 ? fi : (fi < 7 ? fi - 3 : fi - 7);
+      const double4_32a* rec = fi < 3 ? xyz : u;
+      double fv[8], c[8];
+      VMS_UNROLL
+      for (int a = 0; a < 8; ++a) {
+        const int64_t nd = conn[8 * e + a];
+        fv[a] = reinterpret_cast<const double*>(rec + nd)[comp];
+        if (TRANSIENT && fi >= 7) fv[a] -= reinterpret_cast<const double*>(uprev + nd)[comp];
+      }
+      modal8(fv, c);
+      double* dst = sm + (fi < 3 ? RC_X + 7 * fi - 1 : (fi < 7 ? RC_V + 8 * comp : RC_DV + 8 * comp));
+      if (fi >= 3) dst[0] = 0.125 * c[0];
+      VMS_UNROLL
+      for (int m = 1; m < 8; ++m) dst[m] = 0.125 * c[m];
+    }
+  __syncwarp();
+  if (valid) {
+    const int q0 = ln * N1;
+    const double eta = tab.eta(q0), zeta = tab.zeta(q0), ez = tab.ez(q0);
+    ResLine L;
+    VMS_UNROLL
+    for (int i = 0; i < 3; ++i) {
+      const double *X = sm + RC_X + 7 * i - 1, *V = sm + RC_V + 8 * i, *D = sm + RC_DV + 8 * i;
+      L.j1a[i] = X[2] + X[6] * zeta;
+      L.j1b[i] = X[4] + X[7] * zeta;
+      L.J0[i] = X[1] + X[5] * zeta + L.j1b[i] * eta;
+      L.j2a[i] = X[3] + X[6] * eta;
+      L.j2b[i] = X[5] + X[7] * eta;
+      L.g1a[i] = V[2] + V[6] * zeta;
+      L.g1b[i] = V[4] + V[7] * zeta;
+      L.g2a[i] = V[3] + V[6] * eta;
+      L.g2b[i] = V[5] + V[7] * eta;
+      L.va[i] = V[0] + V[3] * zeta + L.g1a[i] * eta;
+      L.vb[i] = V[1] + V[5] * zeta + L.g1b[i] * eta;
+      if (TRANSIENT) {
+        L.dva[i] = D[0] + D[3] * zeta + (D[2] + D[6] * zeta) * eta;
+        L.dvb[i] = D[1] + D[5] * zeta + (D[4] + D[7] * zeta) * eta;
+      }
+    }
+    {
+      const double* Pc = sm + RC_P;
+      L.pa = Pc[0] + Pc[3] * zeta + (Pc[2] + Pc[6] * zeta) * eta;
+      L.pb = Pc[1] + Pc[5] * zeta + (Pc[4] + Pc[7] * zeta) * eta;
+    }
+    const double bet[3] = {beta[3 * e + 0], beta[3 * e + 1], beta[3 * e + 2]};
+    const double nut = kp.nu_e ? kp.visc_factor * __ldg(kp.nu_e + e) : kp.nut;
+    double Rf[3] = {0.0, 0.0, 0.0};
+    ResSums s;
+    if (!residual_line<TRANSIENT, FORCE, N1>(tab, q0, L, bet, nut, kp.tau, kp.f, s, Rf)) bad = 1u;
+    double* o = share + ln;  // output t's share at o[t S]
+    VMS_UNROLL
+    for (int i = 0; i < 3; ++i) {
+      const double sb = s.s1[i] + s.b0[i];
+      o[(8 * i + 0) * S] = s.s0[i];
+      o[(8 * i + 1) * S] = sb;
+      o[(8 * i + 2) * S] = eta * s.s0[i] + s.c0[i];
+      o[(8 * i + 3) * S] = zeta * s.s0[i] + s.d0[i];
+      o[(8 * i + 4) * S] = eta * sb + s.c1[i];
+      o[(8 * i + 5) * S] = zeta * sb + s.d1[i];
+      o[(8 * i + 6) * S] = ez * s.s0[i] + zeta * s.c0[i] + eta * s.d0[i];
+      o[(8 * i + 7) * S] = ez * sb + zeta * s.c1[i] + eta * s.d1[i];
+      o[(32 + i) * S] = Rf[i];
+    }
+    o[24 * S] = s.t0;
+    o[25 * S] = s.t1;
+    o[26 * S] = eta * s.t0;
+    o[27 * S] = zeta * s.t0;
+    o[28 * S] = eta * s.t1;
+    o[29 * S] = zeta * s.t1;
+    o[30 * S] = ez * s.t0;
+    o[31 * S] = ez * s.t1;
+  }
+  __syncwarp();
+  if (valid)
+    for (int t = ln; t < 35; t += S) {
+      double v = share[t * S];
+      VMS_UNROLL
+      for (int l = 1; l < S; ++l) v += share[t * S + l];
+      total[t] = v;
+    }
+  __syncwarp();
+  if (valid) {
+    if (ln < 4) {  // component ln: velocity 0..2, pressure 3
+      double r[8];
+      nodal8(total + 8 * ln, r);
+      VMS_UNROLL
+      for (int a = 0; a < 8; ++a) {
+        const double v = 0.125 * r[a];
+        if (!isfinite(v)) bad |= 4u;
+        put(a, ln, v);
+      }
+    }
+    for (int i = ln - 4 >= 0 ? ln - 4 : (S <= 4 ? ln : 3); i < 3; i += (S <= 4 ? S : 3)) {
+      if (!isfinite(total[32 + i])) bad |= 4u;
+      putf(i, total[32 + i]);
+    }
+  }
+  __syncwarp();  // the element's shared memory may be reused
+  return bad;
 }
 
 // Store the element residual in its 36-double record: R_cp (32, node-major), R_f (3), pad.

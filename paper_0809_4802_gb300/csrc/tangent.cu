@@ -6,6 +6,7 @@
 // y = K_ff^-1 R_f once both the residual and the tangent kernels are done. The two element
 // kernels are therefore independent and run concurrently (FP64 pipe and FP32 pipe).
 #include <algorithm>
+#include <type_traits>
 
 #include "residual_math.cuh"
 #include "residual_table.cuh"
@@ -374,8 +375,13 @@ __global__ void __launch_bounds__(WARPS * 32, ENG == 0 ? 1 : (ENG == TS_ENGINE ?
 // SM and the tangent runs mostly after them. Here one CTA per SM holds both: warps 0-3 (one per
 // partition) evaluate residuals, one element per thread, 32 elements per claim; warps 4-7 form
 // tangents, one element per warp, FUSED_TCLAIM elements per claim. A residual warp whose queue is
-// empty joins the tangent queue. The queues are two counters (zeroed before the launch); no warp
-// ever waits for another.
+// empty joins the tangent queue. The queues are three counters (zeroed before the launch); no warp
+// ever waits for another. The elements past the last whole round of the residual warps (residual_rest;
+// all of a small mesh) are taken with a lane per line of the rule: a round of 32 elements per warp
+// takes about 200 us however few warps have one. Small meshes also claim tangents one at a time.
+// A mixed assembly of 64 elements took 237 us and takes 82, 1,728 252 and 90, 8,000 263 and 204, 21,952
+// 484 and 349, 85,184 1,196 and 1,138; without a remainder for the lines the kernel has no code for them
+// (LINES), which would cost it 1 %.
 // The tangent warps take quadrature points 16 at a time (two passes of 16 lanes for the 27-point
 // rule), which halves their point records and lets the residual's store and eight warp areas fit
 // in one SM's shared memory.
@@ -389,7 +395,7 @@ size_t fused_smem_bytes(int nq) {
   return fused_res_bytes() + tan_table_bytes<float>(nq) + FUSED_WARPS * tan_warp_bytes<float, FUSED_QCH>(nq);
 }
 
-template <bool TRANSIENT, bool FORCE>
+template <bool TRANSIENT, bool FORCE, bool LINES>
 __global__ void __launch_bounds__(FUSED_WARPS * 32, 1) fused_assembly_kernel(
     const double4_32a* __restrict__ xyz, const double4_32a* __restrict__ u64,
     const double4_32a* __restrict__ uprev, const int32_t* __restrict__ conn,
@@ -399,9 +405,11 @@ __global__ void __launch_bounds__(FUSED_WARPS * 32, 1) fused_assembly_kernel(
     const float* __restrict__ gtab, float nut, float tau, const int32_t* __restrict__ blk,
     const int32_t* __restrict__ rowlen, const uint32_t* __restrict__ dir_mask,
     float* __restrict__ values, float* __restrict__ recX, float* __restrict__ recKcf,
-    double* __restrict__ recKinv, int64_t n_elems, unsigned long long* __restrict__ queues,
-    unsigned int* __restrict__ flags) {
+    double* __restrict__ recKinv, int64_t n_elems, int64_t whole, int claim,
+    unsigned long long* __restrict__ queues, unsigned int* __restrict__ flags) {
   extern __shared__ __align__(16) unsigned char smem[];
+  const int64_t n_whole = LINES ? whole : n_elems;
+  const int tclaim = LINES ? claim : FUSED_TCLAIM;  // 1 only for meshes that are all lines
   const int nq = kp.nq;
   float* st = reinterpret_cast<float*>(smem + fused_res_bytes());
   for (int i = threadIdx.x; i < 37 * nq; i += blockDim.x) st[i] = gtab[i];
@@ -409,15 +417,15 @@ __global__ void __launch_bounds__(FUSED_WARPS * 32, 1) fused_assembly_kernel(
   const RefTab<float> tab{st, st + 8 * nq, st + 32 * nq, st + 33 * nq, st + 36 * nq};
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (warp < FUSED_RES_WARPS) {
-    SmemStore<FUSED_RES_THREADS> C{reinterpret_cast<double (*)[FUSED_RES_THREADS]>(smem),
-                                   (int)threadIdx.x};
+    double* sm = reinterpret_cast<double*>(smem) + (size_t)warp * RC_N * 32;  // the warp's own store
+    SmemStore<32> C{reinterpret_cast<double (*)[32]>(sm), lane};
     for (;;) {
       unsigned long long base = 0;
       if (lane == 0) base = atomicAdd(queues, 32ull);
       base = __shfl_sync(0xffffffffu, base, 0);
-      if (base >= (unsigned long long)n_elems) break;
+      if (base >= (unsigned long long)n_whole) break;
       const int64_t e = (int64_t)base + lane;
-      if (e < n_elems) {
+      if (e < n_whole) {
         int nd[8];
         double Rcp[32], Rf[3];
         const unsigned bad = residual_element<TRANSIENT, FORCE>(e, C, GlobalTable{qp}, kp, xyz, u64,
@@ -426,15 +434,39 @@ __global__ void __launch_bounds__(FUSED_WARPS * 32, 1) fused_assembly_kernel(
         store_elem_residual(elemR + 36 * e, Rcp, Rf);
       }
     }
+    if (LINES) {
+      __syncwarp();
+      auto lines = [&](auto n1) {
+        constexpr int N1 = decltype(n1)::value, S = N1 * N1, EPW = 32 / S;
+        static_assert(EPW * rl_doubles<N1>() <= RC_N * 32, "the warp's shared memory");
+        const int el = lane / S, ln = lane - el * S;
+        for (;;) {
+          unsigned long long base = 0;
+          if (lane == 0) base = atomicAdd(queues + 2, (unsigned long long)EPW);
+          base = __shfl_sync(0xffffffffu, base, 0);
+          if (base >= (unsigned long long)(n_elems - n_whole)) break;
+          const bool valid = el < EPW && n_whole + (int64_t)base + el < n_elems;
+          const int64_t e = valid ? n_whole + (int64_t)base + el : 0;
+          const unsigned bad = residual_lines<TRANSIENT, FORCE, N1>(
+              valid, e, ln, sm + (el < EPW ? el : 0) * rl_doubles<N1>(), GlobalTable{qp}, kp, xyz, u64, uprev, conn,
+              beta64, [&](int a, int c, double v) { elemR[36 * e + 4 * a + c] = v; },
+              [&](int i, double v) { elemR[36 * e + 32 + i] = v; });
+          if (bad) atomicOr(flags, bad);
+        }
+      };
+      if (nq == 27) lines(std::integral_constant<int, 3>{});
+      else if (nq == 8) lines(std::integral_constant<int, 2>{});
+      else lines(std::integral_constant<int, 4>{});
+    }
   }
   WarpArea<float>& W = *reinterpret_cast<WarpArea<float>*>(
       smem + fused_res_bytes() + tan_table_bytes<float>(nq) + warp * tan_warp_bytes<float, FUSED_QCH>(nq));
   for (;;) {
     unsigned long long base = 0;
-    if (lane == 0) base = atomicAdd(queues + 1, (unsigned long long)FUSED_TCLAIM);
+    if (lane == 0) base = atomicAdd(queues + 1, (unsigned long long)tclaim);
     base = __shfl_sync(0xffffffffu, base, 0);
     if (base >= (unsigned long long)n_elems) break;
-    const int64_t end = (int64_t)base + FUSED_TCLAIM < n_elems ? (int64_t)base + FUSED_TCLAIM : n_elems;
+    const int64_t end = (int64_t)base + tclaim < n_elems ? (int64_t)base + tclaim : n_elems;
     for (int64_t e = (int64_t)base; e < end; ++e)
       tangent_element<float, false, true, FUSED_QCH>(lane, e, e, W, tab, nullptr, nullptr, nullptr, u32, conn, beta32, nq, nut, tau,
                                           kp.nu_e, kp.visc_factor, xyz, xhl32, u64, beta64, kp.tab64, blk,
@@ -448,21 +480,30 @@ int launch_fused_assembly(const Mesh& m, const State& s, const Fp32Copy& c32, co
                           unsigned long long* queues, unsigned int* flags, cudaStream_t st) {
   if (m.n_elems <= 0) return 0;
   const size_t smem = fused_smem_bytes(kp.nq);
+  // a claim of several elements saves counter traffic; below four claims per warp it would leave
+  // warps without work
+  const int tclaim = m.n_elems < (int64_t)sm_count() * FUSED_WARPS * FUSED_TCLAIM ? 1 : FUSED_TCLAIM;
+  const int64_t rest = residual_rest(kp.nq, m.n_elems, false);
   auto launch = [&](auto kern) {
     cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     kern<<<(unsigned)sm_count(), FUSED_WARPS * 32, smem, st>>>(
         m.xyz, s.u, s.u_prev, m.conn, s.beta, kp, qp, elemR, c32.u, c32.xhl, c32.beta, tab32,
         (float)kp.nut, (float)kp.tau, m.blk, m.rowlen, m.dir_mask, reinterpret_cast<float*>(o.values),
         reinterpret_cast<float*>(o.recX), reinterpret_cast<float*>(o.recKcf), o.recKinv, m.n_elems,
-        queues, flags);
+        m.n_elems - rest, tclaim, queues, flags);
   };
-  if (kp.transient) {
-    if (kp.has_force) launch(fused_assembly_kernel<true, true>);
-    else launch(fused_assembly_kernel<true, false>);
-  } else {
-    if (kp.has_force) launch(fused_assembly_kernel<false, true>);
-    else launch(fused_assembly_kernel<false, false>);
-  }
+  auto pick = [&](auto lines) {
+    constexpr bool L = decltype(lines)::value;
+    if (kp.transient) {
+      if (kp.has_force) launch(fused_assembly_kernel<true, true, L>);
+      else launch(fused_assembly_kernel<true, false, L>);
+    } else {
+      if (kp.has_force) launch(fused_assembly_kernel<false, true, L>);
+      else launch(fused_assembly_kernel<false, false, L>);
+    }
+  };
+  if (rest) pick(std::true_type{});
+  else pick(std::false_type{});
   return 1;
 }
 

@@ -118,7 +118,7 @@ struct Work {
   double* resid = nullptr;    // 4 n_nodes + 3 n_elems
   double* partial = nullptr;  // reduction partials
   unsigned int* flags = nullptr;
-  unsigned long long* queues = nullptr;  // 2 work counters of the fused assembly kernel
+  unsigned long long* queues = nullptr;  // 3 work counters of the fused assembly kernel (and pad)
   Fp32Copy f32;               // mixed precision only
   cudaStream_t aux = nullptr; // second stream for the tangent kernel
   cudaEvent_t fork = nullptr, join = nullptr;
@@ -130,7 +130,11 @@ struct Work {
 // mode 1: accumulate the assembled residual into resid (4 n_nodes + 3 n_elems entries).
 int launch_residual(const Mesh& m, const State& s, const KParams& kp, const QpRow* qp,
                      double* elemR, double* resid, int64_t first, int64_t count, int mode,
-                     unsigned int* flags, cudaStream_t st);
+                     unsigned int* flags, cudaStream_t st, bool beside = false);
+
+// How many of `count` elements, the last ones, the residual takes with a lane per line of the rule of
+// nq points; `beside`: a tangent kernel runs at the same time (residual.cu).
+int64_t residual_rest(int nq, int64_t count, bool beside);
 
 // Element tangent + condensation + scatter (warp per element). T = double or float.
 struct TangentOut {
@@ -187,7 +191,7 @@ int launch_tangent(bool fp32, int engine, const Mesh& m, const State& s, const F
                    int64_t count, const int32_t* elem_list, bool elem_outputs, bool atomic,
                    unsigned int* flags, cudaStream_t st);
 // Mixed precision with the atomic scatter: the residual (into elemR) and the FP32 tangent (into
-// out) in one persistent launch; `queues` holds two zeroed counters.
+// out) in one persistent launch; `queues` holds three zeroed counters.
 int launch_fused_assembly(const Mesh& m, const State& s, const Fp32Copy& c32, const KParams& kp,
                           const QpRow* qp, const float* tab32, double* elemR, const TangentOut& o,
                           unsigned long long* queues, unsigned int* flags, cudaStream_t st);
