@@ -594,7 +594,7 @@ static int mesh_upload_impl(vms_ctx* ctx, int npe, int64_t n_nodes, const double
   CK(cudaMalloc(&w.resid, sizeof(double) * (4 * n_nodes + 3 * n_elems)));
   CK(cudaMalloc(&w.partial, sizeof(double) * 1024));
   CK(cudaMalloc(&w.flags, sizeof(unsigned int)));
-  CK(cudaMalloc(&w.queues, 4 * sizeof(unsigned long long)));
+  CK(cudaMalloc(&w.queues, 3 * sizeof(unsigned long long)));
   return VMS_OK;
 }
 
@@ -660,9 +660,12 @@ static int enqueue_assembly(vms_ctx* ctx, cudaStream_t st) {
   const KParams kp = kparams(ctx);
   {
     KScope k(ctx, VMS_K_FILL, st);
-    k.add(launch_fill_zero(w.values, (size_t)m.nnz * (f32 ? sizeof(float) : sizeof(double)), st));
-    k.add(launch_fill_zero(w.rhs, sizeof(double) * 4 * m.n_nodes, st));
-    k.add(launch_fill_zero(w.flags, sizeof(unsigned int), st));
+    ZeroList z;
+    z.add(w.values, (size_t)m.nnz * (f32 ? sizeof(float) : sizeof(double)));
+    z.add(w.rhs, sizeof(double) * 4 * m.n_nodes);
+    z.add(w.flags, sizeof(unsigned int));
+    z.add(w.queues, 3 * sizeof(unsigned long long));
+    k.add(launch_prologue(m, ctx->state, f32 && m.npe == 8 ? &w.f32 : nullptr, z, st));
   }
   if (m.npe == 4) {  // tetrahedra: one kernel does residual, tangent, condensation and scatter
     TangentOut o;
@@ -686,10 +689,6 @@ static int enqueue_assembly(vms_ctx* ctx, cudaStream_t st) {
     CK(cudaGetLastError());
     return VMS_OK;
   }
-  if (f32) {
-    KScope k(ctx, VMS_K_FILL, st);
-    k.add(launch_to_fp32(m, ctx->state, w.f32, st));
-  }
   TangentOut o;
   o.values = w.values; o.rhs = w.rhs; o.recX = w.recX; o.recKcf = w.recKcf; o.recKinv = w.recKinv;
   o.recY = w.recY;
@@ -699,19 +698,14 @@ static int enqueue_assembly(vms_ctx* ctx, cudaStream_t st) {
   if (f32 && engine(ctx) == 0 && !colour && ctx->tune.schedule == VMS_SCHEDULE_FUSED) {
     // residual and tangent in one persistent launch, then r_e and the Dirichlet rows
     {
-      KScope k(ctx, VMS_K_FILL, st);
-      k.add(launch_fill_zero(w.queues, 4 * sizeof(unsigned long long), st));
-    }
-    {
       KScope k(ctx, VMS_K_FUSED, st);
       k.add(launch_fused_assembly(m, ctx->state, w.f32, kp, ctx->d_qp, ctx->d_tab32, w.elemR, o,
                                   w.queues, w.flags, st));
     }
     {
       KScope k(ctx, VMS_K_DIRICHLET, st);
-      k.add(launch_finish(f32, m, w.elemR, o, 0, m.n_elems, nullptr, true, st));
+      k.add(launch_finish(f32, m, w.elemR, o, 0, m.n_elems, nullptr, true, true, st));
     }
-    { KScope k(ctx, VMS_K_DIRICHLET, st); k.add(launch_dirichlet_diag(m, w.values, f32, w.rhs, st)); }
     CK(cudaGetLastError());
     return VMS_OK;
   }
@@ -743,13 +737,12 @@ static int enqueue_assembly(vms_ctx* ctx, cudaStream_t st) {
     if (colour) {
       for (int c = 0; c < m.n_colours; ++c) {
         const int64_t b = m.colour_start[c], n = m.colour_start[c + 1] - b;
-        k.add(launch_finish(f32, m, w.elemR, o, b, n, m.colour_order, false, st));
+        k.add(launch_finish(f32, m, w.elemR, o, b, n, m.colour_order, false, c == 0, st));
       }
     } else {
-      k.add(launch_finish(f32, m, w.elemR, o, 0, m.n_elems, nullptr, true, st));
+      k.add(launch_finish(f32, m, w.elemR, o, 0, m.n_elems, nullptr, true, true, st));
     }
   }
-  { KScope k(ctx, VMS_K_DIRICHLET, st); k.add(launch_dirichlet_diag(m, w.values, f32, w.rhs, st)); }
   CK(cudaGetLastError());
   return VMS_OK;
 }
@@ -895,8 +888,10 @@ int vms_residual(vms_ctx* ctx, double* norm, double* R) {
   const int64_t n = 4 * m.n_nodes + 3 * m.n_elems;
   {
     KScope k(ctx, VMS_K_FILL);
-    k.add(launch_fill_zero(w.resid, sizeof(double) * n, st));
-    k.add(launch_fill_zero(w.flags, sizeof(unsigned int), st));
+    ZeroList z;
+    z.add(w.resid, sizeof(double) * n);
+    z.add(w.flags, sizeof(unsigned int));
+    k.add(launch_prologue(m, ctx->state, nullptr, z, st));
   }
   {
     KScope k(ctx, VMS_K_RESIDUAL);
@@ -974,12 +969,13 @@ int vms_element_matrices(vms_ctx* ctx, int64_t first, int64_t count, double* S, 
   cudaStream_t st = ctx->stream;
   const KParams kp = kparams(ctx);
   const bool f32 = fp32_mode(ctx);
-  { KScope k(ctx, VMS_K_FILL); k.add(launch_fill_zero(w.flags, sizeof(unsigned int), st)); }
-  if (m.npe == 4) return element_matrices_tet(ctx, first, count, S, r, Kcc, Kcf, Kfc, Kff, Rcp, Rf);
-  if (f32) {
+  {
     KScope k(ctx, VMS_K_FILL);
-    k.add(launch_to_fp32(m, ctx->state, w.f32, st));
+    ZeroList z;
+    z.add(w.flags, sizeof(unsigned int));
+    k.add(launch_prologue(m, ctx->state, f32 && m.npe == 8 ? &w.f32 : nullptr, z, st));
   }
+  if (m.npe == 4) return element_matrices_tet(ctx, first, count, S, r, Kcc, Kcf, Kfc, Kff, Rcp, Rf);
   {
     KScope k(ctx, VMS_K_RESIDUAL);
     k.add(launch_residual(m, ctx->state, kp, ctx->d_qp, w.elemR, nullptr, first, count, 0, w.flags, st));
@@ -999,7 +995,7 @@ int vms_element_matrices(vms_ctx* ctx, int64_t first, int64_t count, double* S, 
   }
   {
     KScope k(ctx, VMS_K_DIRICHLET);
-    k.add(launch_finish(f32, m, w.elemR, o, first, count, nullptr, true, st));
+    k.add(launch_finish(f32, m, w.elemR, o, first, count, nullptr, true, false, st));
   }
   cudaError_t e = cudaGetLastError();
   struct Out { double* dst; double* src; size_t n; } outs[6] = {

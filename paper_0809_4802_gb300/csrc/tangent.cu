@@ -507,66 +507,125 @@ int launch_fused_assembly(const Mesh& m, const State& s, const Fp32Copy& c32, co
   return 1;
 }
 
+// A float as a double, exactly, without the FP64 pipe (its conversion instruction costs as much there
+// as a product): the exponent is rebiased by 1023 - 127 and the fraction's 23 bits are the double's
+// upper ones. Zeros keep their sign; subnormals, infinities and NaN take the conversion instruction.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t u = __float_as_uint(x), m = u << 1;
+  if (m == 0u || (m >= 0x01000000u && m < 0xff000000u))
+    return __hiloint2double((int)((u & 0x80000000u) | (m == 0u ? 0u : (m >> 4) + 0x38000000u)), (int)(u << 29));
+  return (double)x;
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+
 // y = K_ff^-1 R_f (FP64, kept for the recovery) and r_e = R_cp - K_cf y (FP64 arithmetic on the
-// stored K_cf, FP32 in mixed precision) scattered into the right-hand side. One thread per element.
+// stored K_cf, FP32 in mixed precision) scattered into the right-hand side. Eight threads per element, one
+// per node: y is formed by three of them and handed round, each thread reads its node's 4 x 3 block
+// of K_cf and 4 entries of R_cp as 16-byte words. It is bound by the FP64 pipe (3.75 warp
+// instructions per element; a thread per element with converted K_cf took 7.2) and then by reading the
+// records (0.8 KB per element). Blocks past `fin_blocks` set the constrained rows (atomic scatter: neither
+// the scatter of the tangent nor this one touches their entries): unit diagonal, zero right-hand side.
+constexpr int FIN_THREADS = 128, FIN_ELEMS = FIN_THREADS / 8;
 template <typename T, bool ATOMIC>
-__global__ void __launch_bounds__(128) finish_kernel(
+__global__ void __launch_bounds__(FIN_THREADS) finish_kernel(
     const int32_t* __restrict__ conn, const double* __restrict__ elemR, const T* __restrict__ recKcf,
     const double* __restrict__ recKinv, const uint32_t* __restrict__ dir_mask, int64_t first,
     int64_t count, const int32_t* __restrict__ elem_list, double* __restrict__ rhs,
-    double* __restrict__ recY, double* __restrict__ oR) {
-  const int64_t it = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (it >= count) return;
-  const int64_t e = elem_list ? (int64_t)elem_list[first + it] : first + it;
-  const double* R = elemR + 36 * e;
-  const double Rf[3] = {R[32], R[33], R[34]};
-  double y[3];
-#pragma unroll
-  for (int m = 0; m < 3; ++m) {
-    const double* K = recKinv + 9 * e + 3 * m;
-    y[m] = K[0] * Rf[0] + K[1] * Rf[1] + K[2] * Rf[2];
-    recY[3 * e + m] = y[m];
+    double* __restrict__ recY, double* __restrict__ oR, unsigned fin_blocks, const int64_t* __restrict__ diag_pos,
+    const int64_t* __restrict__ dir_dof, int64_t n_dir, T* __restrict__ values) {
+  if (blockIdx.x >= fin_blocks) {
+    const int64_t k = (int64_t)(blockIdx.x - fin_blocks) * FIN_THREADS + threadIdx.x;
+    if (k < n_dir) {
+      values[diag_pos[k]] = T(1);
+      rhs[dir_dof[k]] = 0.0;
+    }
+    return;
   }
-  const uint32_t msk = oR ? 0u : dir_mask[e];
-  const T* kc = recKcf + 96 * e;
-#pragma unroll 4
-  for (int t = 0; t < 32; ++t) {
-    const double r = R[t] - ((double)kc[3 * t] * y[0] + (double)kc[3 * t + 1] * y[1] +
-                             (double)kc[3 * t + 2] * y[2]);
-    if (oR) {
-      oR[32 * it + t] = r;
-    } else if (!(msk >> t & 1u)) {
-      double* dst = rhs + 4 * (int64_t)conn[8 * e + (t >> 2)] + (t & 3);
-      if (ATOMIC) atomicAdd(dst, r); else *dst += r;
+  const int a = threadIdx.x & 7;
+  int64_t it = (int64_t)blockIdx.x * FIN_ELEMS + (threadIdx.x >> 3);
+  const bool valid = it < count;
+  if (!valid) it = count - 1;  // takes part in the exchange only
+  const int64_t e = elem_list ? (int64_t)elem_list[first + it] : first + it;
+  const double2* R = reinterpret_cast<const double2*>(elemR + 36 * e);
+  const double2 rf01 = R[16], r01 = R[2 * a], r23 = R[2 * a + 1];
+  const double rf2 = elemR[36 * e + 34];
+  double kc[12];
+  if constexpr (sizeof(T) == 4) {
+    const float4* k4 = reinterpret_cast<const float4*>(recKcf + 96 * e + 12 * a);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+      const float4 v = k4[i];
+      kc[4 * i] = widen(v.x); kc[4 * i + 1] = widen(v.y); kc[4 * i + 2] = widen(v.z); kc[4 * i + 3] = widen(v.w);
+    }
+  } else {
+    const double2* k2 = reinterpret_cast<const double2*>(recKcf + 96 * e + 12 * a);
+#pragma unroll
+    for (int i = 0; i < 6; ++i) { const double2 v = k2[i]; kc[2 * i] = v.x; kc[2 * i + 1] = v.y; }
+  }
+  const int m = a < 3 ? a : 0;
+  const double* K = recKinv + 9 * e + 3 * m;
+  const double ym = K[0] * rf01.x + K[1] * rf01.y + K[2] * rf2;
+  if (valid && a < 3) recY[3 * e + a] = ym;
+  const double y0 = __shfl_sync(0xffffffffu, ym, 0, 8), y1 = __shfl_sync(0xffffffffu, ym, 1, 8),
+               y2 = __shfl_sync(0xffffffffu, ym, 2, 8);
+  if (!valid) return;
+  const double r[4] = {r01.x, r01.y, r23.x, r23.y};
+  const uint32_t msk = oR ? 0u : dir_mask[e] >> (4 * a);
+  double* dst = oR ? oR + 32 * it + 4 * a : rhs + 4 * (int64_t)conn[8 * e + a];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const double v = fma(-kc[3 * c], y0, fma(-kc[3 * c + 1], y1, fma(-kc[3 * c + 2], y2, r[c])));
+    if (oR) dst[c] = v;
+    else if (!(msk >> c & 1u)) {
+      if (ATOMIC) atomicAdd(dst + c, v); else dst[c] += v;
     }
   }
 }
 
-// FP32 copies of the nodal state and bubble coefficients for the mixed-precision tangent, and the
-// coordinates as FP32 high and low parts (x = hi + lo to about 2^-48 |x|) for its geometry.
-__global__ void to_fp32_kernel(const double4_32a* __restrict__ u, const double* __restrict__ beta,
-                               const double4_32a* __restrict__ xyz, float4* __restrict__ u32,
-                               float* __restrict__ beta32, float4* __restrict__ xhl,
-                               int64_t n_nodes, int64_t n_elems) {
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_nodes; i += stride) {
-    const double4_32a w = u[i];
-    u32[i] = make_float4((float)w.x, (float)w.y, (float)w.z, (float)w.w);
-    const double4_32a x = xyz[i];
-    const float hx = (float)x.x, hy = (float)x.y, hz = (float)x.z;
-    xhl[2 * i] = make_float4(hx, hy, hz, 0.f);
-    xhl[2 * i + 1] = make_float4((float)(x.x - hx), (float)(x.y - hy), (float)(x.z - hz), 0.f);
+// What precedes an assembly, in one launch: zeros in up to four arrays (a multiple of 4 bytes each) and,
+// in mixed precision, FP32 copies of the nodal state and bubble coefficients for the tangent, and the
+// coordinates as FP32 high and low parts (x = hi + lo to about 2^-48 |x|) for its geometry. Bound by the
+// bytes it writes; as five launches it cost a small mesh 10 us.
+struct PrologueArgs {
+  ZeroList z;
+  const double4_32a *u = nullptr, *xyz = nullptr;
+  const double* beta = nullptr;
+  float4 *u32 = nullptr, *xhl = nullptr;
+  float* beta32 = nullptr;
+  int64_t n_nodes = 0, n_beta = 0;
+};
+__global__ void __launch_bounds__(256) prologue_kernel(PrologueArgs a) {
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x, t0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int64_t n16 = (int64_t)(a.z.bytes[r] / 16), rest = (int64_t)(a.z.bytes[r] % 16) / 4;
+    uint4* p = reinterpret_cast<uint4*>(a.z.p[r]);
+    for (int64_t i = t0; i < n16; i += stride) p[i] = make_uint4(0u, 0u, 0u, 0u);
+    if (t0 < rest) reinterpret_cast<uint32_t*>(p + n16)[t0] = 0u;
   }
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < 3 * n_elems; i += stride)
-    beta32[i] = (float)beta[i];
+  for (int64_t i = t0; i < a.n_nodes; i += stride) {
+    const double4_32a w = a.u[i];
+    a.u32[i] = make_float4((float)w.x, (float)w.y, (float)w.z, (float)w.w);
+    const double4_32a x = a.xyz[i];
+    const float hx = (float)x.x, hy = (float)x.y, hz = (float)x.z;
+    a.xhl[2 * i] = make_float4(hx, hy, hz, 0.f);
+    a.xhl[2 * i + 1] = make_float4((float)(x.x - hx), (float)(x.y - hy), (float)(x.z - hz), 0.f);
+  }
+  for (int64_t i = t0; i < a.n_beta; i += stride) a.beta32[i] = (float)a.beta[i];
 }
 
-int launch_to_fp32(const Mesh& m, const State& s, const Fp32Copy& c, cudaStream_t st) {
-  const int64_t n = m.n_nodes > 3 * m.n_elems ? m.n_nodes : 3 * m.n_elems;
-  int64_t blocks = (n + 255) / 256;
-  if (blocks > (int64_t)sm_count() * 8) blocks = (int64_t)sm_count() * 8;
-  to_fp32_kernel<<<(unsigned)blocks, 256, 0, st>>>(s.u, s.beta, m.xyz, c.u, c.beta, c.xhl,
-                                                   m.n_nodes, m.n_elems);
+int launch_prologue(const Mesh& m, const State& s, const Fp32Copy* c, const ZeroList& z, cudaStream_t st) {
+  PrologueArgs a;
+  a.z = z;
+  int64_t n = 1;
+  for (int r = 0; r < 4; ++r) n = std::max(n, (int64_t)(z.bytes[r] / 16));
+  if (c) {
+    a.u = s.u; a.xyz = m.xyz; a.beta = s.beta; a.u32 = c->u; a.xhl = c->xhl; a.beta32 = c->beta;
+    a.n_nodes = m.n_nodes; a.n_beta = 3 * m.n_elems;
+    n = std::max(n, std::max(a.n_nodes, a.n_beta));
+  }
+  const int64_t blocks = std::min((n + 255) / 256, (int64_t)sm_count() * 16);
+  prologue_kernel<<<(unsigned)blocks, 256, 0, st>>>(a);
   return 1;
 }
 
@@ -648,20 +707,23 @@ int launch_tangent(bool fp32, int engine, const Mesh& m, const State& s, const F
 }
 
 int launch_finish(bool fp32, const Mesh& m, const double* elemR, const TangentOut& o,
-                  int64_t first, int64_t count, const int32_t* elem_list, bool atomic,
+                  int64_t first, int64_t count, const int32_t* elem_list, bool atomic, bool dirichlet,
                   cudaStream_t st) {
   if (count <= 0) return 0;
-  const unsigned blocks = (unsigned)((count + 127) / 128);
-  auto go = [&](auto kern, auto* kcf) {
-    kern<<<blocks, 128, 0, st>>>(m.conn, elemR, kcf, o.recKinv, m.dir_mask, first, count,
-                                 elem_list, o.rhs, o.recY, o.r);
+  const unsigned fin = (unsigned)((count + FIN_ELEMS - 1) / FIN_ELEMS);
+  const unsigned dir = dirichlet ? (unsigned)((m.n_dir + FIN_THREADS - 1) / FIN_THREADS) : 0u;
+  auto go = [&](auto kern, auto* kcf, auto* values) {
+    kern<<<fin + dir, FIN_THREADS, 0, st>>>(m.conn, elemR, kcf, o.recKinv, m.dir_mask, first, count, elem_list, o.rhs,
+                                            o.recY, o.r, fin, m.diag_pos, m.dir_dof, m.n_dir, values);
   };
   if (fp32) {
     const float* k = reinterpret_cast<const float*>(o.recKcf);
-    if (atomic) go(finish_kernel<float, true>, k); else go(finish_kernel<float, false>, k);
+    float* v = reinterpret_cast<float*>(o.values);
+    if (atomic) go(finish_kernel<float, true>, k, v); else go(finish_kernel<float, false>, k, v);
   } else {
     const double* k = reinterpret_cast<const double*>(o.recKcf);
-    if (atomic) go(finish_kernel<double, true>, k); else go(finish_kernel<double, false>, k);
+    double* v = reinterpret_cast<double*>(o.values);
+    if (atomic) go(finish_kernel<double, true>, k, v); else go(finish_kernel<double, false>, k, v);
   }
   return 1;
 }

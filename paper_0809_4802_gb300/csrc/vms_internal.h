@@ -118,7 +118,7 @@ struct Work {
   double* resid = nullptr;    // 4 n_nodes + 3 n_elems
   double* partial = nullptr;  // reduction partials
   unsigned int* flags = nullptr;
-  unsigned long long* queues = nullptr;  // 3 work counters of the fused assembly kernel (and pad)
+  unsigned long long* queues = nullptr;  // 3 work counters of the fused assembly kernel
   Fp32Copy f32;               // mixed precision only
   cudaStream_t aux = nullptr; // second stream for the tangent kernel
   cudaEvent_t fork = nullptr, join = nullptr;
@@ -195,12 +195,20 @@ int launch_tangent(bool fp32, int engine, const Mesh& m, const State& s, const F
 int launch_fused_assembly(const Mesh& m, const State& s, const Fp32Copy& c32, const KParams& kp,
                           const QpRow* qp, const float* tab32, double* elemR, const TangentOut& o,
                           unsigned long long* queues, unsigned int* flags, cudaStream_t st);
-// y = K_ff^-1 R_f into recY and r_e = R_cp - K_cf y (FP64) into rhs (or into out.r).
+// y = K_ff^-1 R_f into recY and r_e = R_cp - K_cf y (FP64) into rhs (or into out.r); with `dirichlet`
+// also the unit diagonal and zero right-hand side of the constrained dofs.
 int launch_finish(bool fp32, const Mesh& m, const double* elemR, const TangentOut& out,
-                  int64_t first, int64_t count, const int32_t* elem_list, bool atomic,
+                  int64_t first, int64_t count, const int32_t* elem_list, bool atomic, bool dirichlet,
                   cudaStream_t st);
-// FP32 copies of the nodal state and of beta.
-int launch_to_fp32(const Mesh& m, const State& s, const Fp32Copy& c, cudaStream_t st);
+// Arrays to be zeroed (sizes in bytes, multiples of 4).
+struct ZeroList {
+  void* p[4] = {};
+  size_t bytes[4] = {};
+  int n = 0;
+  void add(void* q, size_t b) { p[n] = q; bytes[n++] = b; }
+};
+// One launch before an assembly: the zeros and, with c, the FP32 copies of the state and coordinates.
+int launch_prologue(const Mesh& m, const State& s, const Fp32Copy* c, const ZeroList& z, cudaStream_t st);
 
 // Streaming multiprocessors of the current device (cudaDevAttrMultiProcessorCount, looked up once
 // per device). Grid sizes are multiples of it.
