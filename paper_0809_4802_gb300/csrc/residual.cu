@@ -117,7 +117,8 @@ static void launch_r(const Mesh& m, const State& s, const KParams& kp, const QpR
 // take less time than a part of a round of threads. Measured in us (27 points; 8; 64), U = 9,728
 // elements on 152 SMs: threads U 184, 2 U 195, 3 U 288, 4 U 371 (75, 82, 115, 146; 396, 420, 636, 815)
 // in steps of U and again from there; lines 29 up to 1,728 elements (25; 34), then 14 + 12.6 per
-// thousand (10 + 3.9; 10 + 24). The bounds below are where the two meet.
+// thousand (10 + 3.9; 10 + 24). The bounds below are where the two meet. (Both take 5 % less since the
+// lines' sums were shortened: 32,768 elements 371 -> 353, 10,648 142 -> 137.)
 // Beside an FP64 tangent (`beside`) the lines of up to 2 U elements fill the tangent's gaps better:
 // an assembly of 512 elements takes 130 us with lines, 228 with threads, 4,096 362 and 415, 12,167
 // 893 and 1,029, 17,576 1,279 and 1,346, 19,683 1,435 and 1,436; past that the lines' extra FP64 work

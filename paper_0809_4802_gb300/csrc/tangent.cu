@@ -419,11 +419,19 @@ __global__ void __launch_bounds__(FUSED_WARPS * 32, 1) fused_assembly_kernel(
   if (warp < FUSED_RES_WARPS) {
     double* sm = reinterpret_cast<double*>(smem) + (size_t)warp * RC_N * 32;  // the warp's own store
     SmemStore<32> C{reinterpret_cast<double (*)[32]>(sm), lane};
-    for (;;) {
+    // Whole rounds from a counter, then a group each of the last, partial round: spread over the SMs (as
+    // they come, some SMs would take four of them and others none), with at most three FP64 warps an SM
+    // a group takes 165 us, with four 196.
+    const int64_t round = (int64_t)gridDim.x * FUSED_RES_THREADS, n_round = n_whole / round * round;
+    for (bool last = false; !last;) {
       unsigned long long base = 0;
       if (lane == 0) base = atomicAdd(queues, 32ull);
       base = __shfl_sync(0xffffffffu, base, 0);
-      if (base >= (unsigned long long)n_whole) break;
+      if (base >= (unsigned long long)n_round) {
+        last = true;
+        base = n_round + 32 * ((int64_t)warp * gridDim.x + blockIdx.x);
+        if (base >= (unsigned long long)n_whole) break;
+      }
       const int64_t e = (int64_t)base + lane;
       if (e < n_whole) {
         int nd[8];
