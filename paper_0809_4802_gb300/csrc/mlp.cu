@@ -3,12 +3,12 @@
 // backward-Euler step. Weights are stored in BF16, biases, activations and accumulation in FP32.
 // Forward, backward (mean squared error) and Adam run in these kernels; Newton then converges to
 // the same tolerance from the predicted start, so the network only changes the starting point.
-// The three 128-wide contractions of a 64-node tile (H1 W2 in the forward pass; H1^T D and D W2^T
-// in the backward pass) run on the tensor cores (mma.sync m16n8k16, BF16 operands, FP32
-// accumulation), the FP32 activations split into sums of BF16 terms (mma_bf16.cuh): three terms
-// against the BF16 weights (exact products, FP32-level results), two times two terms (three
-// products) for H1^T D. The 12-wide input layer, the 4-wide output layer and the small gradient
-// blocks stay on the CUDA cores.
+// The forward pass runs both hidden layers on tcgen05 tensor cores (mlp_forward_kernel). In the gradient
+// kernel the three 128-wide contractions of a 64-node tile (H1 W2, H1^T D and D W2^T) run on mma.sync
+// m16n8k16, BF16 operands, FP32 accumulation. Either way the FP32 activations are split into sums of
+// BF16 terms: three terms against the BF16 weights (exact products, FP32-level results), two times
+// two terms (three products) for H1^T D. The 4-wide output layer and, in the gradient kernel, the
+// 12-wide input layer and the small gradient blocks stay on the CUDA cores.
 //
 // Layout of the parameter vector (row-major): W1 [12][128], b1 [128], W2 [128][128], b2 [128],
 // W3 [128][4], b3 [4].
@@ -182,25 +182,346 @@ __device__ float dense_out(const Smem& s, int r, int o) {
   return y;
 }
 
-__global__ void __launch_bounds__(THREADS) mlp_forward_kernel(const __nv_bfloat16* __restrict__ w,
-                                                              const float* __restrict__ bias,
-                                                              const float* __restrict__ X,
-                                                              int64_t n, float* __restrict__ Y) {
-  extern __shared__ __align__(16) unsigned char raw[];
-  Smem& s = *reinterpret_cast<Smem*>(raw);
-  load_weights(s, w, bias);
-  for (int64_t r0 = (int64_t)blockIdx.x * TILE; r0 < n; r0 += (int64_t)gridDim.x * TILE) {
-    __syncthreads();
-    load_tile(s, X, nullptr, r0, n);
-    __syncthreads();
-    dense_tanh<NI, NW>(s.X, &s.W1[0][0], s.b1, s.H1);
-    __syncthreads();
-    dense2_tanh(s);
-    __syncthreads();
-    const int r = threadIdx.x >> 2, o = threadIdx.x & 3;
-    const float y = dense_out(s, r, o);
-    if (r0 + r < n) Y[(r0 + r) * NO + o] = y;
+// ---------------------------------------------------------------------------------------------
+// Forward pass on the fifth-generation tensor cores (tcgen05.mma, accumulators in tensor memory)
+// ---------------------------------------------------------------------------------------------
+// A CTA takes tiles of 128 rows, one row per TMEM lane; two CTAs share an SM, so one's matrix products
+// run under the other's tanh. Both hidden layers are MMAs of 128 x 128 x 16 with BF16 operands from
+// shared memory: the FP32 activations as three BF16 terms whose sum is exact (truncated, 8 bits each),
+// the weights as they are stored; the low terms of a group of K are summed first. Biases ride along as
+// three rows of a K step whose activations are 1. Per tile: X -> D1 (K = 16, three MMAs) -> H1 = tanh ->
+// D2 (eight K steps, three MMAs each, in two halves of K so that the operand buffer holds half of H1
+// and two CTAs fit) -> tanh -> the 4-wide output layer in FP32 as the values leave tensor memory. H2 and D2
+// never touch shared memory, H1 only as an operand.
+// Bound by instruction issue and the FP32 pipe (tanh, the split); the products alone would take 60 us of
+// the 188 us for 975,583 rows. With mma.sync from FP32 tiles in shared memory, bound by the traffic there, it
+// took 661 us (1,024 rows 14.5, now 10.8; 100,000 79, now 29), with errors against 64 bits of 4.7e-7 rms, now
+// 3.9e-7 (the low terms are summed first).
+constexpr int FT = 128;                       // rows per tile
+constexpr uint32_t OP_K = FT * 16;            // bytes between core matrices along K (LBO)
+constexpr uint32_t OP_R = 128;                // bytes between groups of 8 rows (SBO)
+constexpr uint32_t OP_STEP = 2 * OP_K;        // a K step of 16: two core matrices
+struct SmemFwd {
+  // operands in the canonical K-major layout without swizzle: [k / 8][row][k % 8]
+  __nv_bfloat16 W1[2 * FT * 8];               // W1 (k < 12), the bias' three terms (k = 12..14), 0
+  __nv_bfloat16 B2[2 * FT * 8];               // 0, the second bias' three terms, 0
+  __nv_bfloat16 one[2 * FT * 8];              // its activations: 0 (not X's, which may be infinite), 1, 1, 1, 0
+  __nv_bfloat16 X[3][2 * FT * 8];             // the terms of X; 1 in k = 12..14 of the first
+  __nv_bfloat16 W2[16 * FT * 8];
+  __nv_bfloat16 H[3][8 * FT * 8];             // the terms of half of H1
+  float4 W3[NW];
+  float4 part[FT];                            // output sums of columns 64..127
+  float b3[NO];
+  uint32_t tmem;
+  unsigned long long bar[3];                  // D1; first half of D2 (operand buffers free); D2
+};
+
+__device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
+// Shared-memory matrix descriptor: start, LBO and SBO in 16-byte units, version 1, no swizzle.
+__device__ __forceinline__ uint64_t op_desc(uint32_t addr) {
+  return (uint64_t)((addr & 0x3ffffu) >> 4) | (uint64_t)(OP_K >> 4) << 16 | (uint64_t)(OP_R >> 4) << 32 | 1ull << 46;
+}
+// Instruction descriptor of kind::f16: FP32 accumulators, BF16 operands, both K-major, N = 128, M = 128.
+constexpr uint32_t OP_IDESC = 1u << 4 | 1u << 7 | 1u << 10 | (NW >> 3) << 17 | (FT >> 4) << 24;
+__device__ __forceinline__ void tc_mma(uint32_t d, uint32_t a, uint32_t b, bool add) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d),
+      "l"(op_desc(a)), "l"(op_desc(b)), "r"(OP_IDESC), "r"((uint32_t)add)
+      : "memory");
+}
+__device__ __forceinline__ void tc_commit(unsigned long long* bar) {
+  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar)) : "memory");
+}
+__device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
+__device__ __forceinline__ void fence_async_shared() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
+// Wait for the barrier's phase of this parity; false if it does not come within a second.
+__device__ __forceinline__ bool bar_wait(unsigned long long* bar, uint32_t parity) {
+  const uint32_t a = smem_u32(bar);
+  unsigned long long t0 = 0;
+  for (int it = 0; it < 4000000; ++it) {
+    uint32_t done;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done)
+        : "r"(a), "r"(parity)
+        : "memory");
+    if (done) return true;
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+    if (it == 0) t0 = t;
+    if (t - t0 > 1000000000ull) break;
   }
+  return false;
+}
+// 32 columns of the warp's 32 lanes of tensor memory; the values may be used when it returns.
+__device__ __forceinline__ void tc_load32(uint32_t addr, float v[32]) {
+  uint32_t* r = reinterpret_cast<uint32_t*>(v);
+  __syncwarp();
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
+      "{%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15,"
+      "%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%32];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]), "=r"(r[16]),
+        "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]), "=r"(r[24]),
+        "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+      : "r"(addr)
+      : "memory");
+}
+// x = h + m + l, each the leading 8 bits of what is left (bit patterns with the BF16 in the upper half):
+// exact for every finite x whose low term is a BF16 number; infinities and NaN stay in h.
+struct Terms {
+  uint32_t h, m, l;
+};
+__device__ __forceinline__ Terms split_exact(float x) {
+  Terms t;
+  t.h = __float_as_uint(x) & 0xffff0000u;
+  const float r = x - __uint_as_float(t.h);
+  t.m = __float_as_uint(r) & 0xffff0000u;
+  t.l = __float_as_uint(r - __uint_as_float(t.m));
+  return t;
+}
+// tanh of two values: x N(x^2) / D(x^2) with N of degree 4 and D of degree 5, the minimax quotient on [0, 9.02]
+// (relative error 1e-9; fitted with the Remez exchange algorithm in 40 digits), beyond which tanh rounds to +-1.
+// 3e-8 rms from tanh, against 4e-7 of the network's output from the sums of its products. Branch-free and two
+// at a time: the tile is bound by instruction issue, and tanhf took two thirds of it (975,583 rows 214 us).
+constexpr float NTH1 = 0.137853637f, NTH2 = 0.00400850875f, NTH3 = 3.15890575e-05f, NTH4 = 5.07622211e-08f;
+constexpr float DTH1 = 0.471186966f, DTH2 = 0.0277375113f, DTH3 = 0.000420740689f, DTH4 = 1.61748528e-06f,
+                DTH5 = 7.37443662e-10f;
+__device__ __forceinline__ float2 tanh2(float2 v) {
+  float2 x;
+  asm("{\n\t.reg .f32 t;\n\tmax.NaN.f32 t, %2, 0fC11051EC;\n\tmin.NaN.f32 %0, t, 0f411051EC;\n\t"
+      "max.NaN.f32 t, %3, 0fC11051EC;\n\tmin.NaN.f32 %1, t, 0f411051EC;\n\t}"
+      : "=f"(x.x), "=f"(x.y)
+      : "f"(v.x), "f"(v.y));
+  auto c = [](float a) { return make_float2(a, a); };
+  const float2 s = __fmul2_rn(x, x);
+  float2 n = __ffma2_rn(c(NTH4), s, c(NTH3)), d = __ffma2_rn(c(DTH5), s, c(DTH4));
+  n = __ffma2_rn(n, s, c(NTH2));
+  d = __ffma2_rn(d, s, c(DTH3));
+  n = __ffma2_rn(n, s, c(NTH1));
+  d = __ffma2_rn(d, s, c(DTH2));
+  n = __ffma2_rn(n, s, c(1.f));
+  d = __ffma2_rn(d, s, c(DTH1));
+  d = __ffma2_rn(d, s, c(1.f));
+  float2 r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.x) : "f"(d.x));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r.y) : "f"(d.y));
+  return __fmul2_rn(__fmul2_rn(n, x), r);
+}
+
+// Eight consecutive K of one row, as the three terms' 16-byte pieces.
+__device__ __forceinline__ void store_terms(__nv_bfloat16* h, __nv_bfloat16* m, __nv_bfloat16* l, const float v[8]) {
+  uint32_t H[4], M[4], L[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    const Terms a = split_exact(v[2 * i]), b = split_exact(v[2 * i + 1]);
+    H[i] = __byte_perm(a.h, b.h, 0x7632);
+    M[i] = __byte_perm(a.m, b.m, 0x7632);
+    L[i] = __byte_perm(a.l, b.l, 0x7632);
+  }
+  *reinterpret_cast<uint4*>(h) = make_uint4(H[0], H[1], H[2], H[3]);
+  *reinterpret_cast<uint4*>(m) = make_uint4(M[0], M[1], M[2], M[3]);
+  *reinterpret_cast<uint4*>(l) = make_uint4(L[0], L[1], L[2], L[3]);
+}
+__device__ __forceinline__ __nv_bfloat16 upper_bf16(uint32_t u) { return __ushort_as_bfloat16((unsigned short)(u >> 16)); }
+
+// Eight of the sixteen K of a row of X (half 0: columns 0..7; half 1: columns 8..11, 1, 1, 1, 0); `vec`: X is 16-byte aligned.
+__device__ __forceinline__ void load_x(const float* __restrict__ X, int64_t row, int64_t n, int half, bool vec, float v[8]) {
+#pragma unroll
+  for (int i = 0; i < 8; ++i) v[i] = half && i >= 4 && i < 7 ? 1.f : 0.f;
+  if (row >= n) return;
+  const float* p = X + row * NI + 8 * half;
+  if (vec) {
+    const float4 a = __ldg(reinterpret_cast<const float4*>(p));
+    v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w;
+    if (!half) {
+      const float4 b = __ldg(reinterpret_cast<const float4*>(p) + 1);
+      v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+    }
+  } else {
+#pragma unroll
+    for (int i = 0; i < 4; ++i) v[i] = __ldg(p + i);
+    if (!half)
+#pragma unroll
+      for (int i = 4; i < 8; ++i) v[i] = __ldg(p + i);
+  }
+}
+__device__ __forceinline__ void store_x(SmemFwd& s, int row, int half, const float v[8]) {
+  const int at = half * FT * 8 + row * 8;
+  store_terms(&s.X[0][at], &s.X[1][at], &s.X[2][at], v);
+#pragma unroll
+  for (int i = 0; i < 8; ++i)
+    if (fabsf(v[i]) == INFINITY) {  // infinity minus infinity would be NaN
+      s.X[1][at + i] = __ushort_as_bfloat16(0);
+      s.X[2][at + i] = __ushort_as_bfloat16(0);
+    }
+}
+
+__global__ void __launch_bounds__(THREADS, 2) mlp_forward_kernel(const __nv_bfloat16* __restrict__ w,
+                                                                 const float* __restrict__ bias,
+                                                                 const float* __restrict__ X, int64_t n,
+                                                                 float* __restrict__ Y) {
+  extern __shared__ __align__(128) unsigned char raw[];
+  SmemFwd& s = *reinterpret_cast<SmemFwd*>(raw);
+  const int tid = threadIdx.x, wp = tid >> 5, half = wp >> 2, row = (wp & 3) * 32 + (tid & 31);
+  const bool vec = (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+  const int64_t stride = (int64_t)gridDim.x * FT;
+  int64_t r0 = (int64_t)blockIdx.x * FT;
+  float x[8];
+  load_x(X, r0 + row, n, half, vec, x);
+  // operands of the weights, K (8 at a time) contiguous
+  for (int i = tid; i < 16 * NW; i += THREADS) {
+    const int c = i / NW, j = i % NW;
+    alignas(16) __nv_bfloat16 v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = w[WB_2 + (8 * c + k) * NW + j];
+    *reinterpret_cast<uint4*>(&s.W2[c * FT * 8 + j * 8]) = *reinterpret_cast<const uint4*>(v);
+  }
+  {
+    const int c = tid / NW, j = tid % NW;  // 2 x 128
+    const Terms b1 = split_exact(bias[BB_1 + j]), b2 = split_exact(bias[BB_2 + j]);
+    const __nv_bfloat16 z = __ushort_as_bfloat16(0);
+    alignas(16) __nv_bfloat16 v[8], u[8], o[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+      v[k] = 8 * c + k < NI ? w[WB_1 + (8 * c + k) * NW + j] : z;
+      u[k] = z;
+      o[k] = c && k >= 4 && k < 7 ? __ushort_as_bfloat16(0x3f80) : z;
+    }
+    *reinterpret_cast<uint4*>(&s.one[c * FT * 8 + j * 8]) = *reinterpret_cast<const uint4*>(o);
+    if (c) {
+      v[4] = upper_bf16(b1.h); v[5] = upper_bf16(b1.m); v[6] = upper_bf16(b1.l);
+      u[4] = upper_bf16(b2.h); u[5] = upper_bf16(b2.m); u[6] = upper_bf16(b2.l);
+    }
+    *reinterpret_cast<uint4*>(&s.W1[c * FT * 8 + j * 8]) = *reinterpret_cast<const uint4*>(v);
+    *reinterpret_cast<uint4*>(&s.B2[c * FT * 8 + j * 8]) = *reinterpret_cast<const uint4*>(u);
+  }
+  for (int i = tid; i < NW * NO; i += THREADS) reinterpret_cast<float*>(s.W3)[i] = __bfloat162float(w[WB_3 + i]);
+  if (tid < NO) s.b3[tid] = bias[BB_3 + tid];
+  store_x(s, row, half, x);
+  if (tid == 0) {
+    for (int i = 0; i < 3; ++i)
+      asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s.bar[i])) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (wp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 256;" ::"r"(smem_u32(&s.tmem)) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  fence_async_shared();
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t d1 = s.tmem, d2 = d1 + NW, lanes = (uint32_t)(wp & 3) << 21;  // the warp's lanes, in bits 16..31
+  const uint32_t aX = smem_u32(s.X), aH = smem_u32(s.H), aW1 = smem_u32(s.W1), aB2 = smem_u32(s.B2), aOne = smem_u32(s.one), aW2 = smem_u32(s.W2);
+  constexpr uint32_t XT = sizeof(s.X[0]), HT = sizeof(s.H[0]);
+  auto layer1 = [&]() {
+    for (int t = 2; t >= 0; --t) tc_mma(d1, aX + t * XT, aW1, t != 2);
+    tc_commit(&s.bar[0]);
+  };
+  if (tid == 0) layer1();
+  uint32_t par = 0;
+  bool ok = true;
+  for (; r0 < n; r0 += stride, par ^= 1u) {
+    const bool more = r0 + stride < n;
+    if (more) load_x(X, r0 + stride + row, n, half, vec, x);
+    // H1, columns 0..63 (the warp's 32), then their products
+    float v[32];
+    bool good = bar_wait(&s.bar[0], par);
+    tc_fence_after();
+    tc_load32(d1 + lanes + 32 * half, v);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      float h[8];
+#pragma unroll
+      for (int i = 0; i < 8; i += 2) {
+        const float2 t = tanh2(make_float2(v[8 * c + i], v[8 * c + i + 1]));
+        h[i] = t.x; h[i + 1] = t.y;
+      }
+      const int at = (4 * half + c) * FT * 8 + row * 8;
+      store_terms(&s.H[0][at], &s.H[1][at], &s.H[2][at], h);
+    }
+    fence_async_shared();
+    tc_fence_before();
+    if (__syncthreads_or(!good)) { ok = false; break; }
+    if (tid == 0) {
+      tc_fence_after();
+      tc_mma(d2, aOne, aB2, false);
+      for (int t = 2; t >= 0; --t)
+        for (int k = 0; k < 4; ++k) tc_mma(d2, aH + t * HT + k * OP_STEP, aW2 + k * OP_STEP, true);
+      tc_commit(&s.bar[1]);
+    }
+    // columns 64..127
+    tc_load32(d1 + lanes + 64 + 32 * half, v);
+#pragma unroll
+    for (int i = 0; i < 32; i += 2) {
+      const float2 t = tanh2(make_float2(v[i], v[i + 1]));
+      v[i] = t.x; v[i + 1] = t.y;
+    }
+    good = bar_wait(&s.bar[1], par);
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      const int at = (4 * half + c) * FT * 8 + row * 8;
+      store_terms(&s.H[0][at], &s.H[1][at], &s.H[2][at], v + 8 * c);
+    }
+    if (more) store_x(s, row, half, x);
+    fence_async_shared();
+    tc_fence_before();
+    if (__syncthreads_or(!good)) { ok = false; break; }
+    if (tid == 0) {
+      tc_fence_after();
+      for (int t = 2; t >= 0; --t)
+        for (int k = 0; k < 4; ++k) tc_mma(d2, aH + t * HT + k * OP_STEP, aW2 + (4 + k) * OP_STEP, true);
+      tc_commit(&s.bar[2]);
+      if (more) layer1();
+    }
+    // H2 and the output layer, columns 64 half ..
+    good = bar_wait(&s.bar[2], par);
+    tc_fence_after();
+    float2 ya = make_float2(0.f, 0.f), yb = ya;
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      tc_load32(d2 + lanes + 64 * half + 32 * q, v);
+#pragma unroll
+      for (int i = 0; i < 32; i += 2) {
+        const float2 h = tanh2(make_float2(v[i], v[i + 1]));
+        const float4 w0 = s.W3[64 * half + 32 * q + i], w1 = s.W3[64 * half + 32 * q + i + 1];
+        ya = __ffma2_rn(make_float2(h.x, h.x), make_float2(w0.x, w0.y), ya);
+        yb = __ffma2_rn(make_float2(h.x, h.x), make_float2(w0.z, w0.w), yb);
+        ya = __ffma2_rn(make_float2(h.y, h.y), make_float2(w1.x, w1.y), ya);
+        yb = __ffma2_rn(make_float2(h.y, h.y), make_float2(w1.z, w1.w), yb);
+      }
+    }
+    if (half) s.part[row] = make_float4(ya.x, ya.y, yb.x, yb.y);
+    tc_fence_before();
+    if (__syncthreads_or(!good)) { ok = false; break; }
+    if (!half && r0 + row < n) {
+      const float4 p = s.part[row];
+      const float y[4] = {s.b3[0] + ya.x + p.x, s.b3[1] + ya.y + p.y, s.b3[2] + yb.x + p.z, s.b3[3] + yb.y + p.w};
+      float* o = Y + (r0 + row) * NO;
+      if ((reinterpret_cast<uintptr_t>(Y) & 15) == 0) {
+        *reinterpret_cast<float4*>(o) = make_float4(y[0], y[1], y[2], y[3]);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) o[i] = y[i];
+      }
+    }
+  }
+  if (!ok) {
+    // a product did not finish in time: wait for what is in flight (with a limit) and say so in the result
+    for (int i = 0; i < 3; ++i) {
+      bar_wait(&s.bar[i], par);
+    }
+    for (; r0 < n; r0 += stride)
+      for (int i = tid; i < FT * NO; i += THREADS)
+        if (r0 + i / NO < n) Y[r0 * NO + i] = NAN;
+  }
+  __syncthreads();
+  if (wp == 0) asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 256;" ::"r"(d1) : "memory");
 }
 
 // Gradient of loss = sum over the n rows and 4 outputs of (y - t)^2 / (4 n), accumulated per CTA
@@ -541,7 +862,7 @@ int vms_mlp_create(vms_mlp** out, int device) {
     if (e == cudaSuccess) e = cudaMemset(p, 0, sizeof(float) * (p == (void*)mlp->bias ? BB_N : P_N));
   if (e == cudaSuccess) e = cudaMemset(mlp->w, 0, sizeof(__nv_bfloat16) * WB_N);
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(mlp_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Smem));
+    e = cudaFuncSetAttribute(mlp_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmemFwd));
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmemGrad));
   if (e != cudaSuccess) return cleanup(e == cudaErrorMemoryAllocation ? VMS_ERR_OUT_OF_MEMORY : VMS_ERR_CUDA);
@@ -599,7 +920,9 @@ int vms_mlp_forward(vms_mlp* mlp, int64_t n, const float* X, float* Y) {
   if (!mlp || n < 0 || (n > 0 && (!X || !Y))) return mfail(mlp, VMS_ERR_INVALID_ARG, "invalid arguments");
   if (n == 0) return VMS_OK;
   MCK(cudaSetDevice(mlp->device));
-  mlp_forward_kernel<<<grid_rows(n), THREADS, sizeof(Smem), mlp->stream>>>(mlp->w, mlp->bias, X, n, Y);
+  const int64_t tiles = (n + FT - 1) / FT, most = 2 * (int64_t)vms::sm_count();
+  mlp_forward_kernel<<<(unsigned)(tiles < most ? tiles : most), THREADS, sizeof(SmemFwd), mlp->stream>>>(
+      mlp->w, mlp->bias, X, n, Y);
   MCK(cudaGetLastError());
   return VMS_OK;
 }
