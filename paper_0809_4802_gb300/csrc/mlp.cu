@@ -16,6 +16,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <vector>
 
 #include "mma_bf16.cuh"
@@ -31,7 +32,8 @@ struct vms_mlp {
   float* grad = nullptr;    // gradient of the last vms_mlp_grad call
   __nv_bfloat16* w = nullptr;  // W1, W2, W3 in BF16 (offsets below)
   float* bias = nullptr;       // b1, b2, b3 in FP32
-  double* loss = nullptr;      // device loss accumulator
+  double* loss = nullptr;      // device loss accumulator, behind grad
+  float* host = nullptr;       // page-locked: gradient and loss on their way to the caller
   float* scratch = nullptr;    // P_N floats (parameter read-back)
   double* colsum = nullptr;    // 16 column sums of squares (vms_mlp_column_rms)
   int t = 0;                   // Adam steps taken
@@ -48,51 +50,67 @@ constexpr int NI = VMS_MLP_IN, NW = VMS_MLP_WIDTH, NO = VMS_MLP_OUT;
 constexpr int P_W1 = 0, P_B1 = P_W1 + NI * NW, P_W2 = P_B1 + NW, P_B2 = P_W2 + NW * NW,
               P_W3 = P_B2 + NW, P_B3 = P_W3 + NW * NO, P_N = P_B3 + NO;
 static_assert(P_N == VMS_MLP_PARAMS, "parameter count");
+constexpr size_t GRAD_BYTES = sizeof(float) * P_N + sizeof(double);  // the gradient, then the loss
+static_assert(P_N % 2 == 0, "the loss behind the gradient");
 // BF16 weight array: W1 | W2 | W3; FP32 bias array: b1 | b2 | b3
 constexpr int WB_1 = 0, WB_2 = NI * NW, WB_3 = WB_2 + NW * NW, WB_N = WB_3 + NW * NO;
 constexpr int BB_1 = 0, BB_2 = NW, BB_3 = 2 * NW, BB_N = 2 * NW + NO;
 
-constexpr int TILE = 64;       // rows (nodes) per tile
 constexpr int THREADS = 256;   // 8 warps
 constexpr int HLD = NW + 4;    // padded FP32 activation row (conflict-free MMA fragment loads)
 constexpr int WLD = NW + 8;    // padded BF16 weight row (68 words: conflict-free fragment loads)
 
-struct Smem {
+// ROWS (16, 32 or 64) rows (nodes) per tile.
+template <int ROWS>
+struct SmemGrad {
   float W1[NI][NW];
-  __nv_bfloat16 W2t[NW][WLD];  // W2^T [j][k]: B operand of H1 W2 (K index contiguous)
+  __nv_bfloat16 W2[NW][WLD];   // W2 [k][j]
   float W3[NW][NO];
   float b1[NW], b2[NW], b3[NO];
-  float X[TILE][NI];
-  float H1[TILE][HLD];
-  float H2[TILE][HLD];
-};
-struct SmemGrad : Smem {
-  __nv_bfloat16 W2[NW][WLD];   // W2 [k][j]: B operand of D W2^T
-  float D[TILE][HLD];
-  float dY[TILE][NO];
+  float X[ROWS][NI];
+  float H1[ROWS][HLD];
+  float H2[ROWS][HLD];
+  float D[ROWS][HLD];
+  float dY[ROWS][NO];
 };
 
-__device__ void load_weights(Smem& s, const __nv_bfloat16* __restrict__ w,
-                             const float* __restrict__ bias, __nv_bfloat16 (*W2)[WLD] = nullptr) {
-  for (int i = threadIdx.x; i < NI * NW; i += THREADS) s.W1[i / NW][i % NW] = __bfloat162float(w[WB_1 + i]);
-  for (int i = threadIdx.x; i < NW * NW; i += THREADS) {
-    const int k = i / NW, j = i % NW;
-    s.W2t[j][k] = w[WB_2 + i];
-    if (W2) W2[k][j] = w[WB_2 + i];
+// W2 arrives by asynchronous 16-byte copies while the first layer runs (wait_weights before its use).
+template <int ROWS>
+__device__ void load_weights(SmemGrad<ROWS>& s, const __nv_bfloat16* __restrict__ w, const float* __restrict__ bias) {
+  for (int i = threadIdx.x; i < NW * NW / 8; i += THREADS) {
+    const uint32_t dst = (uint32_t)__cvta_generic_to_shared(&s.W2[i / (NW / 8)][i % (NW / 8) * 8]);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(w + WB_2 + 8 * i) : "memory");
   }
-  for (int i = threadIdx.x; i < NW * NO; i += THREADS) s.W3[i / NO][i % NO] = __bfloat162float(w[WB_3 + i]);
-  for (int i = threadIdx.x; i < NW; i += THREADS) { s.b1[i] = bias[BB_1 + i]; s.b2[i] = bias[BB_2 + i]; }
+  asm volatile("cp.async.commit_group;" ::: "memory");
+#pragma unroll
+  for (int i = threadIdx.x; i < NI * NW / 2; i += THREADS) {
+    const float2 v = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(w + WB_1)[i]);
+    reinterpret_cast<float2*>(&s.W1[0][0])[i] = v;
+  }
+  {
+    const float2 v = __bfloat1622float2(reinterpret_cast<const __nv_bfloat162*>(w + WB_3)[threadIdx.x]);
+    reinterpret_cast<float2*>(&s.W3[0][0])[threadIdx.x] = v;
+    static_assert(NW * NO == 2 * THREADS && 2 * NW == THREADS, "one pair, one bias per thread");
+    (threadIdx.x < NW ? s.b1 : s.b2 - NW)[threadIdx.x] = bias[BB_1 + threadIdx.x];
+  }
   if (threadIdx.x < NO) s.b3[threadIdx.x] = bias[BB_3 + threadIdx.x];
 }
+__device__ __forceinline__ void wait_weights() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
-// C[64 x 128] = A[64 x 128] B on the tensor cores, B given as Bk[n][k] (BF16, K contiguous), A
-// FP32 split into three BF16 terms. Warp w owns rows 16 (w & 3) .. + 15 and columns
-// 64 (w >> 2) .. + 63 (eight 8-wide tiles); acc[nt][*] is the standard m16n8 C fragment (rows g,
-// g + 8 and columns 2t, 2t + 1 of tile nt, g = lane / 4, t = lane % 4), initialised by the caller.
-__device__ __forceinline__ void mma_rows64(const float (*A)[HLD], const __nv_bfloat16 (*Bk)[WLD],
-                                           float acc[8][4]) {
+// C[ROWS x 128] = A[ROWS x 128] B on the tensor cores, A FP32 split into three BF16 terms, B = W (BWD false)
+// or W^T (true), W [128][128] in BF16. A warp owns 16 rows (warp w rows 16 (w % RT) ..) and NT column
+// tiles of 8; acc[nt][*] is the standard m16n8 C fragment (rows g, g + 8 and columns 2t, 2t + 1 of
+// tile nt, g = lane / 4, t = lane % 4), initialised by the caller.
+template <int ROWS> struct WarpTile {
+  static constexpr int RT = ROWS / 16, NT = 2 * RT;  // row tiles; column tiles per warp
+  static __device__ __forceinline__ int row(int w) { return 16 * (w % RT); }
+  static __device__ __forceinline__ int col(int w) { return 8 * NT * (w / RT); }
+};
+template <int ROWS, bool BWD>
+__device__ __forceinline__ void mma_rows(const float (*A)[HLD], const __nv_bfloat16 (*W)[WLD], float (*acc)[4]) {
+  constexpr int NT = WarpTile<ROWS>::NT;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int r0 = 16 * (w & 3) + g, c0 = 64 * (w >> 2);
+  const int r0 = WarpTile<ROWS>::row(w) + g, c0 = WarpTile<ROWS>::col(w);
 #pragma unroll 2
   for (int k0 = 0; k0 < NW; k0 += 16) {
     uint32_t ah[4], am[4], al[4];
@@ -102,41 +120,56 @@ __device__ __forceinline__ void mma_rows64(const float (*A)[HLD], const __nv_bfl
       bf16x2_split3(x.x, x.y, ah[f], am[f], al[f]);
     }
 #pragma unroll
-    for (int nt = 0; nt < 8; ++nt) {
-      const __nv_bfloat16* br = &Bk[c0 + 8 * nt + g][k0 + 2 * t];
-      const uint32_t b0 = *reinterpret_cast<const uint32_t*>(br);
-      const uint32_t b1 = *reinterpret_cast<const uint32_t*>(br + 8);
-      mma_bf16(acc[nt], al, b0, b1);
-      mma_bf16(acc[nt], am, b0, b1);
-      mma_bf16(acc[nt], ah, b0, b1);
+    for (int nt = 0; nt < NT; nt += 2) {
+      // two column tiles: rows k0 .. + 15 of W transposed on the way in, or K contiguous as it lies
+      uint32_t b[4];
+      const int q = lane >> 3, i = lane & 7;
+      const __nv_bfloat16* at = BWD ? &W[c0 + 8 * (nt + (q >> 1)) + i][k0 + 8 * (q & 1)]
+                                    : &W[k0 + 8 * (q & 1) + i][c0 + 8 * (nt + (q >> 1))];
+      const uint32_t addr = (uint32_t)__cvta_generic_to_shared(at);
+      if (BWD)
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]) : "r"(addr) : "memory");
+      else
+        asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                     : "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3]) : "r"(addr) : "memory");
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        mma_bf16(acc[nt + h], al, b[2 * h], b[2 * h + 1]);
+        mma_bf16(acc[nt + h], am, b[2 * h], b[2 * h + 1]);
+        mma_bf16(acc[nt + h], ah, b[2 * h], b[2 * h + 1]);
+      }
     }
   }
 }
 
 // H2 = tanh(H1 W2 + b2) on the tensor cores
-__device__ __forceinline__ void dense2_tanh(Smem& s) {
+template <int ROWS>
+__device__ __forceinline__ void dense2_tanh(SmemGrad<ROWS>& s) {
+  constexpr int NT = WarpTile<ROWS>::NT;
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
-  const int r0 = 16 * (w & 3) + g, c0 = 64 * (w >> 2);
-  float acc[8][4];
+  const int r0 = WarpTile<ROWS>::row(w) + g, c0 = WarpTile<ROWS>::col(w);
+  float acc[NT][4];
 #pragma unroll
-  for (int nt = 0; nt < 8; ++nt) {
+  for (int nt = 0; nt < NT; ++nt) {
     const int c = c0 + 8 * nt + 2 * t;
     acc[nt][0] = acc[nt][2] = s.b2[c];
     acc[nt][1] = acc[nt][3] = s.b2[c + 1];
   }
-  mma_rows64(s.H1, s.W2t, acc);
+  mma_rows<ROWS, false>(s.H1, s.W2, acc);
 #pragma unroll
-  for (int nt = 0; nt < 8; ++nt) {
+  for (int nt = 0; nt < NT; ++nt) {
     const int c = c0 + 8 * nt + 2 * t;
     *reinterpret_cast<float2*>(&s.H2[r0][c]) = make_float2(tanhf(acc[nt][0]), tanhf(acc[nt][1]));
     *reinterpret_cast<float2*>(&s.H2[r0 + 8][c]) = make_float2(tanhf(acc[nt][2]), tanhf(acc[nt][3]));
   }
 }
 
-// rows [r0, r0 + TILE) of X (through `rows` if given) into shared memory, zero beyond n
-__device__ void load_tile(Smem& s, const float* __restrict__ X, const int32_t* __restrict__ rows,
+// rows [r0, r0 + ROWS) of X (through `rows` if given) into shared memory, zero beyond n
+template <int ROWS>
+__device__ void load_tile(SmemGrad<ROWS>& s, const float* __restrict__ X, const int32_t* __restrict__ rows,
                           int64_t r0, int64_t n) {
-  for (int i = threadIdx.x; i < TILE * NI; i += THREADS) {
+  for (int i = threadIdx.x; i < ROWS * NI; i += THREADS) {
     const int r = i / NI, c = i % NI;
     const int64_t g = r0 + r;
     float x = 0.f;
@@ -145,41 +178,32 @@ __device__ void load_tile(Smem& s, const float* __restrict__ X, const int32_t* _
   }
 }
 
-// H = tanh(A W + b) for the tile on the CUDA cores (the 12-wide input layer): A [TILE][K] in
-// shared memory, W [K][NW] (leading dimension LD); warp w owns rows 8w..8w+7, lane l columns
-// l + 32 j
-template <int K, int LD>
-__device__ void dense_tanh(const float (*A)[K], const float* W, const float* b, float (*H)[HLD]) {
+// H1 = tanh(X W1 + b1) for the tile on the CUDA cores; warp w owns ROWS / 8 rows, lane l columns l + 32 j
+template <int ROWS>
+__device__ void dense1_tanh(SmemGrad<ROWS>& s) {
+  constexpr int R = ROWS / 8;
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  float acc[8][4];
+  float acc[R][4];
 #pragma unroll
-  for (int r = 0; r < 8; ++r)
+  for (int r = 0; r < R; ++r)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) acc[r][j] = b[l + 32 * j];
+    for (int j = 0; j < 4; ++j) acc[r][j] = s.b1[l + 32 * j];
 #pragma unroll 4
-  for (int k = 0; k < K; ++k) {
+  for (int k = 0; k < NI; ++k) {
     float wv[4];
 #pragma unroll
-    for (int j = 0; j < 4; ++j) wv[j] = W[k * LD + l + 32 * j];
+    for (int j = 0; j < 4; ++j) wv[j] = s.W1[k][l + 32 * j];
 #pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      const float a = A[8 * w + r][k];
+    for (int r = 0; r < R; ++r) {
+      const float a = s.X[R * w + r][k];
 #pragma unroll
       for (int j = 0; j < 4; ++j) acc[r][j] = fmaf(a, wv[j], acc[r][j]);
     }
   }
 #pragma unroll
-  for (int r = 0; r < 8; ++r)
+  for (int r = 0; r < R; ++r)
 #pragma unroll
-    for (int j = 0; j < 4; ++j) H[8 * w + r][l + 32 * j] = tanhf(acc[r][j]);
-}
-
-// y[r][o] = b3[o] + sum_k H2[r][k] W3[k][o], thread = (r, o)
-__device__ float dense_out(const Smem& s, int r, int o) {
-  float y = s.b3[o];
-#pragma unroll 8
-  for (int k = 0; k < NW; ++k) y = fmaf(s.H2[r][k], s.W3[k][o], y);
-  return y;
+    for (int j = 0; j < 4; ++j) s.H1[R * w + r][l + 32 * j] = tanhf(acc[r][j]);
 }
 
 // ---------------------------------------------------------------------------------------------
@@ -525,14 +549,17 @@ __global__ void __launch_bounds__(THREADS, 2) mlp_forward_kernel(const __nv_bflo
 }
 
 // Gradient of loss = sum over the n rows and 4 outputs of (y - t)^2 / (4 n), accumulated per CTA
-// in registers and added to grad (FP32) once; the loss (FP64) likewise.
+// in registers and added to grad (FP32) once; the loss (FP64) likewise. ROWS rows per tile: a CTA's tile is a
+// chain of eight dependent stages whose length goes with ROWS, so as long as there are SMs for it a batch
+// is cut finer (grad_rows).
+template <int ROWS>
 __global__ void __launch_bounds__(THREADS) mlp_grad_kernel(
     const __nv_bfloat16* __restrict__ w, const float* __restrict__ bias, const float* __restrict__ X,
     const float* __restrict__ T, const int32_t* __restrict__ rows, int64_t n, float scale,
     float* __restrict__ grad, double* __restrict__ loss) {
   extern __shared__ __align__(16) unsigned char raw[];
-  SmemGrad& s = *reinterpret_cast<SmemGrad*>(raw);
-  load_weights(s, w, bias, s.W2);
+  SmemGrad<ROWS>& s = *reinterpret_cast<SmemGrad<ROWS>*>(raw);
+  load_weights(s, w, bias);
   const int tid = threadIdx.x, wp = tid >> 5, l = tid & 31, g = l >> 2, t = l & 3;
   // register partials: dW2 as MMA C fragments (warp wp: rows k = 16 wp + g (+ 8) of dW2, column
   // tiles 0..15), dW1 (6 entries), dW3 (2 entries), db1/db2 (threads < 128: column tid), db3
@@ -546,43 +573,52 @@ __global__ void __launch_bounds__(THREADS) mlp_grad_kernel(
   for (int i = 0; i < 6; ++i) gW1[i] = 0.f;
   gW3[0] = gW3[1] = 0.f;
   double lsum = 0.0;
-  for (int64_t r0 = (int64_t)blockIdx.x * TILE; r0 < n; r0 += (int64_t)gridDim.x * TILE) {
+  for (int64_t r0 = (int64_t)blockIdx.x * ROWS; r0 < n; r0 += (int64_t)gridDim.x * ROWS) {
     __syncthreads();
     load_tile(s, X, rows, r0, n);
     __syncthreads();
-    dense_tanh<NI, NW>(s.X, &s.W1[0][0], s.b1, s.H1);
+    dense1_tanh(s);
+    wait_weights();
     __syncthreads();
     dense2_tanh(s);
     __syncthreads();
     {
-      const int r = tid >> 2, o = tid & 3;
+      // y[r][o] = b3[o] + sum_k H2[r][k] W3[k][o]: KS threads per output
+      constexpr int KS = 64 / ROWS;
+      const int o = tid & 3, ks = (tid >> 2) % KS, r = tid / (4 * KS);
       const int64_t gr = r0 + r;
-      float d = 0.f;
+      float y = ks ? 0.f : s.b3[o], d = 0.f;
+#pragma unroll 8
+      for (int k = ks; k < NW; k += KS) y = fmaf(s.H2[r][k], s.W3[k][o], y);
+#pragma unroll
+      for (int m = 4; m < 4 * KS; m <<= 1) y += __shfl_xor_sync(0xffffffffu, y, m);
       if (gr < n) {
-        const float y = dense_out(s, r, o);
         const float e = y - T[(rows ? (int64_t)rows[gr] : gr) * NO + o];
-        lsum += (double)e * (double)e;
+        if (ks == 0) lsum += (double)e * (double)e;
         d = 2.f * scale * e;
       }
-      s.dY[r][o] = d;
+      if (ks == 0) s.dY[r][o] = d;
+      // db3: the warp's rows (lanes 0..3 of each warp keep the sums)
+      float c = ks == 0 ? d : 0.f;
+#pragma unroll
+      for (int m = 4; m < 32; m <<= 1) c += __shfl_xor_sync(0xffffffffu, c, m);
+      gb3 += c;
     }
     __syncthreads();
-    // dW3, db3
+    // dW3
 #pragma unroll
     for (int q = 0; q < 2; ++q) {
       const int e = tid + THREADS * q, k = e / NO, o = e % NO;
       float a = 0.f;
-      for (int r = 0; r < TILE; ++r) a = fmaf(s.H2[r][k], s.dY[r][o], a);
+      for (int r = 0; r < ROWS; ++r) a = fmaf(s.H2[r][k], s.dY[r][o], a);
       gW3[q] += a;
     }
-    if (tid < NO)
-      for (int r = 0; r < TILE; ++r) gb3 += s.dY[r][tid];
     // D = dH2 = (dY W3^T) * (1 - H2^2)
 #pragma unroll
-    for (int r = 0; r < 8; ++r)
+    for (int r = 0; r < ROWS / 8; ++r)
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        const int rr = 8 * wp + r, c = l + 32 * j;
+        const int rr = ROWS / 8 * wp + r, c = l + 32 * j;
         float a = 0.f;
 #pragma unroll
         for (int o = 0; o < NO; ++o) a = fmaf(s.dY[rr][o], s.W3[c][o], a);
@@ -593,7 +629,7 @@ __global__ void __launch_bounds__(THREADS) mlp_grad_kernel(
     // dW2[k][j] += sum_r H1[r][k] D[r][j] on the tensor cores: A = H1^T (rows k = 16 wp ..), B = D,
     // both split into two BF16 terms, products hi hi + hi lo + lo hi
 #pragma unroll 1
-    for (int k0 = 0; k0 < TILE; k0 += 16) {
+    for (int k0 = 0; k0 < ROWS; k0 += 16) {
       uint32_t ah[4], al[4];
 #pragma unroll
       for (int f = 0; f < 4; ++f) {
@@ -612,19 +648,21 @@ __global__ void __launch_bounds__(THREADS) mlp_grad_kernel(
       }
     }
     if (tid < NW)
-      for (int r = 0; r < TILE; ++r) gb2 += s.D[r][tid];
+#pragma unroll 16
+      for (int r = 0; r < ROWS; ++r) gb2 += s.D[r][tid];
     // dH1 = (D W2^T) * (1 - H1^2) on the tensor cores (B = W2 [k][j], K = j contiguous), written
     // over H2 (no longer needed)
     {
-      const int rr = 16 * (wp & 3) + g, c0 = 64 * (wp >> 2);
-      float acc[8][4];
+      constexpr int NT = WarpTile<ROWS>::NT;
+      const int rr = WarpTile<ROWS>::row(wp) + g, c0 = WarpTile<ROWS>::col(wp);
+      float acc[NT][4];
 #pragma unroll
-      for (int nt = 0; nt < 8; ++nt)
+      for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[nt][q] = 0.f;
-      mma_rows64(s.D, s.W2, acc);
+      mma_rows<ROWS, true>(s.D, s.W2, acc);
 #pragma unroll
-      for (int nt = 0; nt < 8; ++nt) {
+      for (int nt = 0; nt < NT; ++nt) {
         const int c = c0 + 8 * nt + 2 * t;
 #pragma unroll
         for (int hf = 0; hf < 2; ++hf) {
@@ -641,19 +679,20 @@ __global__ void __launch_bounds__(THREADS) mlp_grad_kernel(
     for (int q = 0; q < 6; ++q) {
       const int e = tid + THREADS * q, k = e / NW, j = e % NW;
       float a = 0.f;
-      for (int r = 0; r < TILE; ++r) a = fmaf(s.X[r][k], s.H2[r][j], a);
+      for (int r = 0; r < ROWS; ++r) a = fmaf(s.X[r][k], s.H2[r][j], a);
       gW1[q] += a;
     }
     if (tid < NW)
-      for (int r = 0; r < TILE; ++r) gb1 += s.H2[r][tid];
+#pragma unroll 16
+      for (int r = 0; r < ROWS; ++r) gb1 += s.H2[r][tid];
   }
   // flush the partials
 #pragma unroll
   for (int nt = 0; nt < 16; ++nt)
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      const int k = 16 * wp + g + 8 * (q >> 1), j = 8 * nt + 2 * t + (q & 1);
-      atomicAdd(grad + P_W2 + k * NW + j, gW2[nt][q]);
+    for (int q = 0; q < 2; ++q) {
+      const int k = 16 * wp + g + 8 * q, j = 8 * nt + 2 * t;
+      atomicAdd(reinterpret_cast<float2*>(grad + P_W2 + k * NW + j), make_float2(gW2[nt][2 * q], gW2[nt][2 * q + 1]));
     }
 #pragma unroll
   for (int q = 0; q < 6; ++q) atomicAdd(grad + P_W1 + tid + THREADS * q, gW1[q]);
@@ -663,7 +702,7 @@ __global__ void __launch_bounds__(THREADS) mlp_grad_kernel(
     atomicAdd(grad + P_B1 + tid, gb1);
     atomicAdd(grad + P_B2 + tid, gb2);
   }
-  if (tid < NO) atomicAdd(grad + P_B3 + tid, gb3);
+  if (l < NO) atomicAdd(grad + P_B3 + l, gb3);
   for (int o = 16; o > 0; o >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, o);
   if (l == 0) atomicAdd(loss, lsum * (double)scale);
 }
@@ -718,10 +757,17 @@ __global__ void mlp_stored_kernel(const __nv_bfloat16* __restrict__ w, const flo
   out[i] = x;
 }
 
-unsigned grid_rows(int64_t n) {
-  const int64_t tiles = (n + TILE - 1) / TILE;
+unsigned grid_rows(int64_t n, int rows) {
+  const int64_t tiles = (n + rows - 1) / rows;
   const int64_t sms = vms::sm_count();
   return (unsigned)(tiles < 1 ? 1 : (tiles > sms ? sms : tiles));
+}
+// Rows per tile of the gradient kernel: the fewest for which a batch is one round of CTAs. Measured in us with
+// 16, 32 and 64 rows: 1,024 rows 16.6, 20.7, 26.9; 2,432 20.7, 20.7, 26.8; 4,864 26.8, 22.7, 28.1; 9,728
+// 39.1, 32.9, 30.9 (64 rows with W2 read and transposed two bytes at a time: 31.5, and 36.4 for 9,728).
+int grad_rows(int64_t n) {
+  const int64_t sms = vms::sm_count();
+  return n <= 16 * sms ? 16 : (n <= 32 * sms ? 32 : 64);
 }
 
 int mfail(vms_mlp* p, int code, const char* msg) {
@@ -852,10 +898,11 @@ int vms_mlp_create(vms_mlp** out, int device) {
   cudaError_t e = cudaMalloc(&mlp->master, sizeof(float) * P_N);
   if (e == cudaSuccess) e = cudaMalloc(&mlp->m, sizeof(float) * P_N);
   if (e == cudaSuccess) e = cudaMalloc(&mlp->v, sizeof(float) * P_N);
-  if (e == cudaSuccess) e = cudaMalloc(&mlp->grad, sizeof(float) * P_N);
+  if (e == cudaSuccess) e = cudaMalloc(&mlp->grad, GRAD_BYTES);
+  if (e == cudaSuccess) e = cudaMallocHost(&mlp->host, GRAD_BYTES);
   if (e == cudaSuccess) e = cudaMalloc(&mlp->w, sizeof(__nv_bfloat16) * WB_N);
   if (e == cudaSuccess) e = cudaMalloc(&mlp->bias, sizeof(float) * BB_N);
-  if (e == cudaSuccess) e = cudaMalloc(&mlp->loss, sizeof(double));
+  mlp->loss = reinterpret_cast<double*>(mlp->grad + P_N);
   if (e == cudaSuccess) e = cudaMalloc(&mlp->scratch, sizeof(float) * P_N);
   if (e == cudaSuccess) e = cudaMalloc(&mlp->colsum, sizeof(double) * 16);
   for (void* p : {(void*)mlp->master, (void*)mlp->m, (void*)mlp->v, (void*)mlp->grad, (void*)mlp->bias})
@@ -864,7 +911,11 @@ int vms_mlp_create(vms_mlp** out, int device) {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(mlp_forward_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmemFwd));
   if (e == cudaSuccess)
-    e = cudaFuncSetAttribute(mlp_grad_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmemGrad));
+    e = cudaFuncSetAttribute(mlp_grad_kernel<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmemGrad<16>));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(mlp_grad_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmemGrad<32>));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(mlp_grad_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SmemGrad<64>));
   if (e != cudaSuccess) return cleanup(e == cudaErrorMemoryAllocation ? VMS_ERR_OUT_OF_MEMORY : VMS_ERR_CUDA);
   *out = mlp;
   return VMS_OK;
@@ -875,8 +926,9 @@ int vms_mlp_destroy(vms_mlp* mlp) {
   cudaSetDevice(mlp->device);
   if (mlp->stream) cudaStreamSynchronize(mlp->stream);
   for (void* p : {(void*)mlp->master, (void*)mlp->m, (void*)mlp->v, (void*)mlp->grad, (void*)mlp->w,
-                  (void*)mlp->bias, (void*)mlp->loss, (void*)mlp->scratch, (void*)mlp->colsum})
+                  (void*)mlp->bias, (void*)mlp->scratch, (void*)mlp->colsum})
     if (p) cudaFree(p);
+  if (mlp->host) cudaFreeHost(mlp->host);
   delete mlp;
   return VMS_OK;
 }
@@ -931,15 +983,32 @@ int vms_mlp_grad(vms_mlp* mlp, int64_t n, const int32_t* rows, const float* X, c
                  double* loss, float* grads) {
   if (!mlp || n <= 0 || !X || !T) return mfail(mlp, VMS_ERR_INVALID_ARG, "invalid arguments");
   MCK(cudaSetDevice(mlp->device));
-  MCK(cudaMemsetAsync(mlp->grad, 0, sizeof(float) * P_N, mlp->stream));
-  MCK(cudaMemsetAsync(mlp->loss, 0, sizeof(double), mlp->stream));
+  MCK(cudaMemsetAsync(mlp->grad, 0, GRAD_BYTES, mlp->stream));
   const float scale = (float)(1.0 / (4.0 * (double)n));
-  mlp_grad_kernel<<<grid_rows(n), THREADS, sizeof(SmemGrad), mlp->stream>>>(
-      mlp->w, mlp->bias, X, T, rows, n, scale, mlp->grad, mlp->loss);
+  auto launch = [&](auto kern, int r, size_t smem) {
+    kern<<<grid_rows(n, r), THREADS, smem, mlp->stream>>>(mlp->w, mlp->bias, X, T, rows, n, scale, mlp->grad, mlp->loss);
+  };
+  const int r = grad_rows(n);
+  if (r == 16) launch(mlp_grad_kernel<16>, r, sizeof(SmemGrad<16>));
+  else if (r == 32) launch(mlp_grad_kernel<32>, r, sizeof(SmemGrad<32>));
+  else launch(mlp_grad_kernel<64>, r, sizeof(SmemGrad<64>));
   MCK(cudaGetLastError());
-  if (loss) MCK(cudaMemcpyAsync(loss, mlp->loss, sizeof(double), cudaMemcpyDeviceToHost, mlp->stream));
-  if (grads) MCK(cudaMemcpyAsync(grads, mlp->grad, sizeof(float) * P_N, cudaMemcpyDefault, mlp->stream));
-  if (loss || grads) MCK(cudaStreamSynchronize(mlp->stream));
+  if (!loss && !grads) return VMS_OK;
+  // To ordinary host memory both go in one copy through the handle's page-locked buffer; a device (or
+  // managed) destination is copied to directly.
+  cudaPointerAttributes at{};
+  const bool host = grads && cudaPointerGetAttributes(&at, grads) == cudaSuccess &&
+                    (at.type == cudaMemoryTypeUnregistered || at.type == cudaMemoryTypeHost);
+  double* hl = reinterpret_cast<double*>(mlp->host + P_N);
+  if (host) {
+    MCK(cudaMemcpyAsync(mlp->host, mlp->grad, GRAD_BYTES, cudaMemcpyDeviceToHost, mlp->stream));
+  } else {
+    if (grads) MCK(cudaMemcpyAsync(grads, mlp->grad, sizeof(float) * P_N, cudaMemcpyDefault, mlp->stream));
+    if (loss) MCK(cudaMemcpyAsync(hl, mlp->loss, sizeof(double), cudaMemcpyDeviceToHost, mlp->stream));
+  }
+  MCK(cudaStreamSynchronize(mlp->stream));
+  if (host) std::memcpy(grads, mlp->host, sizeof(float) * P_N);
+  if (loss) *loss = *hl;
   return VMS_OK;
 }
 
