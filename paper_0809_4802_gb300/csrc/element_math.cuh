@@ -26,6 +26,16 @@ namespace vms {
 // non-positive (a degenerate element), so that recip_normal() applies.
 constexpr double DET_MIN = 2.2250738585072014e-308;
 
+// det J is a normal positive number (or infinite), as det >= DET_MIN tests; on the device on the high
+// word, since an FP64 compare takes an FP64 slot. NaN (quiet: from 0x7ff80000) is not.
+VMS_HD bool det_ok(double det) {
+#if defined(__CUDA_ARCH__)
+  return (unsigned)__double2hiint(det) - 0x00100000u <= 0x7fe00000u;
+#else
+  return det >= DET_MIN;
+#endif
+}
+
 // 1 / d for a normal d (|d| >= DET_MIN, finite). On the device: the approximate reciprocal of the
 // PTX instruction set, then two Newton steps r <- r + r (1 - d r), each of which squares the
 // relative error of the approximation, with fewer FP64 instructions than a division. Measured on a

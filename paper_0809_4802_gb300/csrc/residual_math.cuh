@@ -73,16 +73,6 @@ struct ResSums {
   double s0[3], s1[3], b0[3], c0[3], c1[3], d0[3], d1[3], t0, t1;
 };
 
-// det J is a normal positive number (or infinite), as det >= DET_MIN tests; on the device on the high
-// word, since an FP64 compare takes an FP64 slot. NaN (quiet: from 0x7ff80000) is not.
-VMS_HD bool det_ok(double det) {
-#if defined(__CUDA_ARCH__)
-  return (unsigned)__double2hiint(det) - 0x00100000u <= 0x7fe00000u;
-#else
-  return det >= DET_MIN;
-#endif
-}
-
 // The sums of the line whose first point is q0 (and R_f, added to); false if det J <= 0 at a point.
 template <bool TRANSIENT, bool FORCE, int N1, class Table>
 VMS_HD bool residual_line(const Table& tab, int q0, const ResLine& ln, const double bet[3], double nut, double tau,

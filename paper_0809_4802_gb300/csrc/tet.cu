@@ -165,27 +165,35 @@ namespace {
 constexpr int TET_WARPS = 2;     // warps per block
 constexpr int TET_PER_WARP = 8;  // tetrahedra per warp
 
-// What every lane of an element's group holds (a = the lane's node).
+// What every lane of an element's group holds (a = the lane's node). The kernel is bound by the FP64 pipe
+// (19 cycles of an SM per warp instruction), so integrals over the element are kept with the factor
+// det J that turns J^-1 into its cofactors: no entry of J^-1 and no product with det J is formed, only 1 /
+// det J where a product of two gradients needs it. With that, sums started from the value they are
+// subtracted from, y = K_ff^-1 R_f in place of K_cf K_ff^-1, K_ff's rows on the group's lanes and results
+// narrowed to FP32 by integer instructions a warp takes about 690 FP64 instructions for its eight elements
+// instead of 1,030.
 struct TetElem {
   int nd[4];
   int nda;           // node a
   bool ok;           // det J > 0
-  double det;
-  double Ji[3][3];   // J^-1: Ji[al][j] = d xi_al / d x_j
-  double g[4][3];    // P1 gradients g_c = grad lambda_c
-  double G[3][3];    // coarse velocity gradient G[i][j] = sum_c V_c[i] g_c[j]
+  double det, r;     // det J and 1 / det J
+  double C[3][3];    // det J J^-1: C[al][j] = det J d xi_al / d x_j
+  double g[4][3];    // det J grad lambda_c
+  double G[3][3];    // det J times the coarse velocity gradient: G[i][j] = sum_c V_c[i] g_c[j]
+  double Ga[3];      // its row a (a < 3)
+  double Ca[3];      // column a of C (lane 3: zero)
   double beta[3];
-  double Ua[3];      // int lambda_a v       (all integrals divided by det)
-  double Ub[3];      // int b v
+  double Ua[3];      // int lambda_a v / det
+  double Ub[3];      // int b v / det
   double Aa;         // int lambda_a v.d
   double Ab;         // int b v.d
   double Bd;         // int lambda_a beta.d
   double Dint[3];    // int d
   double DD;         // int d.d
-  double Pbar;       // int p
+  double Pbar;       // int p / det
   double PdJ[3];     // int p d
-  double dVa[3];     // int lambda_a (v - v_prev)
-  double dVb[3];     // int b (v - v_prev)
+  double dVa[3];     // int lambda_a (v - v_prev) / det
+  double dVb[3];     // int b (v - v_prev) / det
   double ga[3];      // g_a
   // the moment rows of node a (selected without dynamic indexing)
   double m1a, m1ba, m2a[4], m1da[3], m1bda[3], m2da[12];
@@ -227,28 +235,29 @@ __device__ __forceinline__ void tet_element(int a, int64_t e, const double4_32a*
 #pragma unroll
   for (int l = 0; l < 12; ++l)
     E.m2da[l] = sel4(a, M[TM_M2D + l], M[TM_M2D + 12 + l], M[TM_M2D + 24 + l], M[TM_M2D + 36 + l]);
-  // J[i][al] = x_{al+1,i} - x_{0,i}; Jinv[al][j] = cof[j][al] / det
+  // J[i][al] = x_{al+1,i} - x_{0,i}
   double J[3][3], cof[3][3];
 #pragma unroll
   for (int i = 0; i < 3; ++i)
 #pragma unroll
     for (int al = 0; al < 3; ++al) J[i][al] = X[al + 1][i] - X[0][i];
   double det = cofactor3(J, cof);
-  E.ok = det >= DET_MIN;
+  E.ok = det_ok(det);
   if (!E.ok) det = 1.0;
   E.det = det;
-  const double r = recip_normal(det);
+  E.r = recip_normal(det);
 #pragma unroll
   for (int al = 0; al < 3; ++al)
 #pragma unroll
-    for (int j = 0; j < 3; ++j) E.Ji[al][j] = cof[j][al] * r;
+    for (int j = 0; j < 3; ++j) E.C[al][j] = cof[j][al];
 #pragma unroll
   for (int j = 0; j < 3; ++j) {
-    E.g[1][j] = E.Ji[0][j];
-    E.g[2][j] = E.Ji[1][j];
-    E.g[3][j] = E.Ji[2][j];
-    E.g[0][j] = -(E.Ji[0][j] + E.Ji[1][j] + E.Ji[2][j]);
+    E.g[1][j] = E.C[0][j];
+    E.g[2][j] = E.C[1][j];
+    E.g[3][j] = E.C[2][j];
+    E.g[0][j] = -(E.C[0][j] + E.C[1][j] + E.C[2][j]);
     E.ga[j] = sel4(a, E.g[0][j], E.g[1][j], E.g[2][j], E.g[3][j]);
+    E.Ca[j] = sel4(a, E.C[j][0], E.C[j][1], E.C[j][2], 0.0);
   }
   // The element constants below are the same on the group's four lanes. Each lane forms one part
   // of each (its own node's, or row / column a), in the same instruction stream as the others,
@@ -267,14 +276,13 @@ __device__ __forceinline__ void tet_element(int a, int64_t e, const double4_32a*
   for (int c = 0; c < 4; ++c) w[c] = sel4(a, V[c][0], V[c][1], V[c][2], P[c]);
   // G[i][j] = sum_c V_c[i] g_c[j]: row a on lane a (lane 3 forms the pressure gradient, unused)
   {
-    double Ga[3];
 #pragma unroll
     for (int j = 0; j < 3; ++j)
-      Ga[j] = w[0] * E.g[0][j] + w[1] * E.g[1][j] + w[2] * E.g[2][j] + w[3] * E.g[3][j];
+      E.Ga[j] = w[0] * E.g[0][j] + w[1] * E.g[1][j] + w[2] * E.g[2][j] + w[3] * E.g[3][j];
 #pragma unroll
     for (int i = 0; i < 3; ++i)
 #pragma unroll
-      for (int j = 0; j < 3; ++j) E.G[i][j] = from(Ga[j], i);
+      for (int j = 0; j < 3; ++j) E.G[i][j] = from(E.Ga[j], i);
   }
   // Ub[j] = int b v_j: component a on lane a
   {
@@ -288,17 +296,20 @@ __device__ __forceinline__ void tet_element(int a, int64_t e, const double4_32a*
 #pragma unroll
   for (int j = 0; j < 3; ++j)
     E.Ua[j] = M2a[0] * V[0][j] + M2a[1] * V[1][j] + M2a[2] * V[2][j] + M2a[3] * V[3][j] + E.m1ba * E.beta[j];
-  // reference-frame components Vr_c = Jinv V_c (node c's on lane c) and br = Jinv beta
-  double Vra[3], Vr[4][3], br[3];
+  // reference-frame components Vr_c = C V_c (node c's on lane c) and br = C beta (component a on lane a)
+  double Vra[3], Vr[4][3], br[3], Cr[3];  // Cr: row a of C (lane 3: zero)
   {
     double Va[3];
 #pragma unroll
-    for (int j = 0; j < 3; ++j) Va[j] = sel4(a, V[0][j], V[1][j], V[2][j], V[3][j]);
-#pragma unroll
-    for (int al = 0; al < 3; ++al) {
-      Vra[al] = E.Ji[al][0] * Va[0] + E.Ji[al][1] * Va[1] + E.Ji[al][2] * Va[2];
-      br[al] = E.Ji[al][0] * E.beta[0] + E.Ji[al][1] * E.beta[1] + E.Ji[al][2] * E.beta[2];
+    for (int j = 0; j < 3; ++j) {
+      Va[j] = sel4(a, V[0][j], V[1][j], V[2][j], V[3][j]);
+      Cr[j] = sel4(a, E.C[0][j], E.C[1][j], E.C[2][j], 0.0);
     }
+#pragma unroll
+    for (int al = 0; al < 3; ++al) Vra[al] = E.C[al][0] * Va[0] + E.C[al][1] * Va[1] + E.C[al][2] * Va[2];
+    const double bra = Cr[0] * E.beta[0] + Cr[1] * E.beta[1] + Cr[2] * E.beta[2];
+#pragma unroll
+    for (int al = 0; al < 3; ++al) br[al] = from(bra, al);
 #pragma unroll
     for (int c = 0; c < 4; ++c)
 #pragma unroll
@@ -323,33 +334,26 @@ __device__ __forceinline__ void tet_element(int a, int64_t e, const double4_32a*
     E.Ab = gsum(ab) + M[TM_MBBD] * br[0] + M[TM_MBBD + 1] * br[1] + M[TM_MBBD + 2] * br[2];
   }
   E.Pbar = M[TM_M1] * P[0] + M[TM_M1 + 1] * P[1] + M[TM_M1 + 2] * P[2] + M[TM_M1 + 3] * P[3];
-  // column a of Jinv (lane 3: zero)
-  double Jc[3];
-#pragma unroll
-  for (int al = 0; al < 3; ++al) Jc[al] = sel4(a, E.Ji[al][0], E.Ji[al][1], E.Ji[al][2], 0.0);
-  // DD = int d.d = sum_{al,be} Mdd[al][be] (Jinv Jinv^T)[al][be]: row a of Jinv Jinv^T on lane a
+  // DD = int d.d = sum_{al,be} Mdd[al][be] (C C^T)[al][be] / det: row a of C C^T on lane a
   {
-    double Jr[3];  // row a of Jinv (lane 3: zero)
-#pragma unroll
-    for (int j = 0; j < 3; ++j) Jr[j] = sel4(a, E.Ji[0][j], E.Ji[1][j], E.Ji[2][j], 0.0);
     double dd = 0.0;
 #pragma unroll
     for (int be = 0; be < 3; ++be) {
-      const double jj = Jr[0] * E.Ji[be][0] + Jr[1] * E.Ji[be][1] + Jr[2] * E.Ji[be][2];
+      const double jj = Cr[0] * E.C[be][0] + Cr[1] * E.C[be][1] + Cr[2] * E.C[be][2];
       dd += sel4(a, M[TM_MDD + be], M[TM_MDD + 3 + be], M[TM_MDD + 6 + be], 0.0) * jj;
     }
-    E.DD = gsum(dd);
+    E.DD = E.r * gsum(dd);
   }
-  // Pd[al] = int p d_al (reference): component a on lane a; then PdJ = Jinv^T Pd and
-  // Dint = Jinv^T Md, component a on lane a
+  // Pd[al] = int p d_al (reference): component a on lane a; then PdJ = C^T Pd and
+  // Dint = C^T Md, component a on lane a
   {
     const double pda = sel4(a, M[TM_M1D], M[TM_M1D + 1], M[TM_M1D + 2], 0.0) * P[0] +
                        sel4(a, M[TM_M1D + 3], M[TM_M1D + 4], M[TM_M1D + 5], 0.0) * P[1] +
                        sel4(a, M[TM_M1D + 6], M[TM_M1D + 7], M[TM_M1D + 8], 0.0) * P[2] +
                        sel4(a, M[TM_M1D + 9], M[TM_M1D + 10], M[TM_M1D + 11], 0.0) * P[3];
     const double Pd[3] = {from(pda, 0), from(pda, 1), from(pda, 2)};
-    const double pdj = Pd[0] * Jc[0] + Pd[1] * Jc[1] + Pd[2] * Jc[2];
-    const double din = M[TM_MD] * Jc[0] + M[TM_MD + 1] * Jc[1] + M[TM_MD + 2] * Jc[2];
+    const double pdj = Pd[0] * E.Ca[0] + Pd[1] * E.Ca[1] + Pd[2] * E.Ca[2];
+    const double din = M[TM_MD] * E.Ca[0] + M[TM_MD + 1] * E.Ca[1] + M[TM_MD + 2] * E.Ca[2];
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
       E.PdJ[j] = from(pdj, j);
@@ -382,30 +386,70 @@ __device__ __forceinline__ double dot3(const double x[3], const double y[3]) {
   return x[0] * y[0] + x[1] * y[1] + x[2] * y[2];
 }
 
+// Combinations the residual and the tangent share: w = U_a + nut M0 g_a / det (so that G_i . w is the
+// convective and the viscous term of node a), the bubble's viscous term with lambda_a, and the diagonal
+// of K_ff.
+struct TetTerms {
+  double w[3], gD, kd;
+};
+__device__ __forceinline__ TetTerms tet_terms(const TetElem& E, const double* __restrict__ M, double nut) {
+  TetTerms t;
+  const double nr = nut * E.r, nm = nr * M[TM_M0];
+#pragma unroll
+  for (int j = 0; j < 3; ++j) t.w[j] = E.Ua[j] + nm * E.ga[j];
+  t.gD = nr * dot3(E.ga, E.Dint);
+  t.kd = E.Ab + nut * E.DD;
+  return t;
+}
+
 // R_cp rows of node a (Eqs. SC_Coarse_Resid_Vec, SC_Coarse_Resid_Vec_2) and R_f (Eq.
 // SC_Fine_Resid_Vec), every lane of the group holding the same R_f.
-__device__ __forceinline__ void tet_residual(int a, const TetElem& E, const double* __restrict__ M,
-                                             double nut, double tau, const double f[3],
-                                             double Rcp[4], double Rf[3]) {
-  const double gD = dot3(E.ga, E.Dint);
+__device__ __forceinline__ void tet_residual(int a, const TetElem& E, const TetTerms& t, const double* __restrict__ M,
+                                             const KParams& kp, double nut, double Rcp[4], double Rf[3]) {
+  const double nr = nut * E.r, ca = E.Aa + t.gD;
+  double wb[3];
+#pragma unroll
+  for (int j = 0; j < 3; ++j) wb[j] = E.Ub[j] + nr * E.Dint[j];
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
-    const double s = dot3(E.G[i], E.Ua) + E.beta[i] * E.Aa - f[i] * E.m1a + tau * E.dVa[i] -
-                     E.ga[i] * E.Pbar + nut * (M[TM_M0] * dot3(E.ga, E.G[i]) + E.beta[i] * gD);
-    Rcp[i] = E.det * s;
-    const double t = dot3(E.G[i], E.Ub) + E.beta[i] * E.Ab - f[i] * M[TM_MB] + tau * E.dVb[i] -
-                     E.PdJ[i] + nut * (dot3(E.G[i], E.Dint) + E.beta[i] * E.DD);
-    Rf[i] = E.det * t;
+    Rcp[i] = E.G[i][0] * t.w[0] + (E.G[i][1] * t.w[1] + (E.G[i][2] * t.w[2] + (E.beta[i] * ca - E.ga[i] * E.Pbar)));
+    Rf[i] = E.G[i][0] * wb[0] + (E.G[i][1] * wb[1] + (E.G[i][2] * wb[2] + (E.beta[i] * t.kd - E.PdJ[i])));
   }
-  Rcp[3] = -E.det * (E.m1a * (E.G[0][0] + E.G[1][1] + E.G[2][2]) + E.Bd);
+  if (kp.has_force) {
+    const double da = E.det * E.m1a, db = E.det * M[TM_MB];
+#pragma unroll
+    for (int i = 0; i < 3; ++i) { Rcp[i] -= kp.f[i] * da; Rf[i] -= kp.f[i] * db; }
+  }
+  if (kp.transient) {
+    const double dt = E.det * kp.tau;
+#pragma unroll
+    for (int i = 0; i < 3; ++i) { Rcp[i] += dt * E.dVa[i]; Rf[i] += dt * E.dVb[i]; }
+  }
+  Rcp[3] = -(E.m1a * (E.G[0][0] + E.G[1][1] + E.G[2][2]) + E.Bd);
+}
+
+// Tested on the bits: an FP64 compare takes a slot of the FP64 pipe.
+__device__ __forceinline__ bool finite(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
+
+// x in the type of the results. To FP32 (round to nearest, ties to even) by integer instructions where the
+// result is a normal number: the conversion instruction takes a slot of the FP64 pipe.
+template <typename T> __device__ __forceinline__ T narrow(double x);
+template <> __device__ __forceinline__ double narrow<double>(double x) { return x; }
+template <> __device__ __forceinline__ float narrow<float>(double x) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const uint32_t t = (hi & 0x7fffffffu) - 0x38000000u;  // exponent rebiased by 1023 - 127
+  if (t - 0x00100000u >= 0x0fe00000u) return (float)x;
+  uint32_t f = __funnelshift_l(lo, t, 3);
+  f += ((lo & 0x1fffffffu) + 0x0fffffffu + (f & 1u)) >> 29;
+  return __uint_as_float(f | (hi & 0x80000000u));
 }
 
 template <typename T>
-__device__ __forceinline__ void tet_scatter_row(T* p, const double v[4], bool atomic);
+__device__ __forceinline__ void tet_scatter_row(T* p, const T v[4], bool atomic);
 template <>
-__device__ __forceinline__ void tet_scatter_row<float>(float* p, const double v[4], bool atomic) {
+__device__ __forceinline__ void tet_scatter_row<float>(float* p, const float v[4], bool atomic) {
   // one row of a 4x4 node block: four contiguous values, 16-byte aligned (offsets are multiples of 4)
-  const float4 w = make_float4((float)v[0], (float)v[1], (float)v[2], (float)v[3]);
+  const float4 w = make_float4(v[0], v[1], v[2], v[3]);
   if (atomic) {
     atomicAdd(reinterpret_cast<float4*>(p), w);
   } else {
@@ -418,7 +462,7 @@ template <>
 __device__ __forceinline__ void tet_scatter_row<double>(double* p, const double v[4], bool atomic) {
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    if (v[k] == 0.0) continue;
+    if (__double_as_longlong(v[k]) << 1 == 0) continue;  // zero
     if (atomic) atomicAdd(p + k, v[k]); else p[k] += v[k];
   }
 }
@@ -447,92 +491,98 @@ __global__ void __launch_bounds__(TET_WARPS * 32) tet_assembly_kernel(
     const int64_t it = valid ? it0 : base;
     const int64_t e = elem_list ? (int64_t)elem_list[first + it] : first + it;
     const double nut = kp.nu_e ? kp.visc_factor * kp.nu_e[e] : kp.nut;
-    const double tau = kp.tau;
     TetElem E;
     tet_element(a, e, xyz, u, up, conn, beta, kp.transient != 0, M, E);
+    const TetTerms tt = tet_terms(E, M, nut);
     double Rcp[4], Rf[3];
-    tet_residual(a, E, M, nut, tau, kp.f, Rcp, Rf);
-    const double det = E.det;
+    tet_residual(a, E, tt, M, kp, nut, Rcp, Rf);
+    const double dtau = kp.transient ? E.det * kp.tau : 0.0;
 
-    // K_ff and its inverse (every lane)
-    double Q[3], Kff[9];
+    // K_ff (row a on lane a) and its inverse: row a's cofactors are the cross product of the next two
+    // rows, and give column a of the inverse
+    double Kff[3], Kinv[9];
+    bool bad;
+    {
+      const double q = M[TM_MBBD] * E.Ca[0] + M[TM_MBBD + 1] * E.Ca[1] + M[TM_MBBD + 2] * E.Ca[2];
+      const double ba = sel4(a, E.beta[0], E.beta[1], E.beta[2], 0.0);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) Q[k] = M[TM_MBBD] * E.Ji[0][k] + M[TM_MBBD + 1] * E.Ji[1][k] + M[TM_MBBD + 2] * E.Ji[2][k];
+      for (int k = 0; k < 3; ++k) {
+        const double qk = __shfl_sync(0xffffffffu, q, src0 | k);
+        Kff[k] = M[TM_MBB] * E.Ga[k] + (ba * qk + (a == k ? tt.kd : 0.0));
+      }
+      const int a1 = a == 2 ? 0 : a + 1, a2 = a == 0 ? 2 : a - 1;
+      double R1[3], R2[3], kc[3];
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+      for (int k = 0; k < 3; ++k) {
+        R1[k] = __shfl_sync(0xffffffffu, Kff[k], src0 | (a1 & 3));
+        R2[k] = __shfl_sync(0xffffffffu, Kff[k], src0 | a2);
+      }
 #pragma unroll
-      for (int k = 0; k < 3; ++k)
-        Kff[3 * i + k] = det * (M[TM_MBB] * E.G[i][k] + E.beta[i] * Q[k] + (i == k ? E.Ab + nut * E.DD : 0.0));
-    double Kc[9];
+      for (int k = 0; k < 3; ++k) kc[k] = R1[(k + 1) % 3] * R2[(k + 2) % 3] - R1[(k + 2) % 3] * R2[(k + 1) % 3];
+      const double kdet = __shfl_sync(0xffffffffu, Kff[0] * kc[0] + Kff[1] * kc[1] + Kff[2] * kc[2], src0);
+      // zero or not finite, tested on the bits (an FP64 compare takes a slot of the FP64 pipe)
+      const uint64_t kb = (uint64_t)__double_as_longlong(kdet);
+      bad = (kb << 1) == 0 || ((kb >> 52) & 0x7ffu) == 0x7ffu;
+      const double kr = bad ? 0.0 : recip(kdet);
 #pragma unroll
-    for (int l = 0; l < 9; ++l) {
-      const int i = l / 3, j = l % 3;
-      const int i1 = (i + 1) % 3, i2 = (i + 2) % 3, j1 = (j + 1) % 3, j2 = (j + 2) % 3;
-      Kc[l] = Kff[3 * i1 + j1] * Kff[3 * i2 + j2] - Kff[3 * i1 + j2] * Kff[3 * i2 + j1];
+      for (int k = 0; k < 3; ++k) {
+        const double v = kc[k] * kr;
+#pragma unroll
+        for (int j = 0; j < 3; ++j) Kinv[3 * k + j] = __shfl_sync(0xffffffffu, v, src0 | j);
+      }
     }
-    const double kdet = Kff[0] * Kc[0] + Kff[1] * Kc[1] + Kff[2] * Kc[2];
-    const bool bad = !(kdet != 0.0) || !isfinite(kdet);
-    const double kr = bad ? 0.0 : 1.0 / kdet;
-    double Kinv[9];
+    // row a of the inverse (a < 3), y = K_ff^-1 R_f
+    double kr3[3], y[3];
+    {
 #pragma unroll
-    for (int l = 0; l < 9; ++l) Kinv[l] = Kc[3 * (l % 3) + l / 3] * kr;
+      for (int k = 0; k < 3; ++k) kr3[k] = a == 0 ? Kinv[k] : a == 1 ? Kinv[3 + k] : Kinv[6 + k];
+      const double ya = kr3[0] * Rf[0] + kr3[1] * Rf[1] + kr3[2] * Rf[2];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) y[k] = __shfl_sync(0xffffffffu, ya, src0 | k);
+    }
 
-    // F_a = int lambda_a b d, H_a = int lambda_a d (divided by det)
+    // F_a = int lambda_a b d, H_a = int lambda_a d
     double F[3], H[3];
 #pragma unroll
     for (int m = 0; m < 3; ++m) {
-      F[m] = E.m1bda[0] * E.Ji[0][m] + E.m1bda[1] * E.Ji[1][m] + E.m1bda[2] * E.Ji[2][m];
-      H[m] = E.m1da[0] * E.Ji[0][m] + E.m1da[1] * E.Ji[1][m] + E.m1da[2] * E.Ji[2][m];
+      F[m] = E.m1bda[0] * E.C[0][m] + E.m1bda[1] * E.C[1][m] + E.m1bda[2] * E.C[2][m];
+      H[m] = E.m1da[0] * E.C[0][m] + E.m1da[1] * E.C[1][m] + E.m1da[2] * E.C[2][m];
     }
-    const double gD = dot3(E.ga, E.Dint);
-    const double m1b = E.m1ba;
-    // K_fc column block a (3 x 4) and X_a = K_ff^-1 K_fc[:, block a]
-    double Kfc[3][4], Xa[3][4];
+    // K_cf rows of node a (4 x 3) and K_fc column block a (3 x 4): they differ in their diagonals
+    double Kcf[4][3], Kfc[3][4], Xa[3][4], rr[4];
     {
-      const double gUb = dot3(E.ga, E.Ub);
+      const double dcf = E.Aa + tt.gD, dfc = dot3(E.ga, E.Ub) + tt.gD + dtau * E.m1ba;
 #pragma unroll
-      for (int m = 0; m < 3; ++m) {
+      for (int i = 0; i < 3; ++i) {
 #pragma unroll
-        for (int k = 0; k < 3; ++k)
-          Kfc[m][k] = det * (m1b * E.G[m][k] + E.beta[m] * F[k] + (m == k ? gUb + nut * gD + tau * m1b : 0.0));
-        Kfc[m][3] = -det * H[m];
+        for (int k = 0; k < 3; ++k) {
+          const double p = E.m1ba * E.G[i][k] + E.beta[i] * F[k];
+          Kcf[i][k] = i == k ? p + dcf : p;
+          Kfc[i][k] = i == k ? p + dfc : p;
+        }
+        Kcf[3][i] = -H[i];
+        Kfc[i][3] = -H[i];
       }
-#pragma unroll
-      for (int m = 0; m < 3; ++m)
-#pragma unroll
-        for (int k = 0; k < 4; ++k)
-          Xa[m][k] = Kinv[3 * m] * Kfc[0][k] + Kinv[3 * m + 1] * Kfc[1][k] + Kinv[3 * m + 2] * Kfc[2][k];
     }
-    // K_cf rows of node a (4 x 3), W_a = K_cf K_ff^-1, condensed residual r = R_cp - W_a R_f
-    double Kcf[4][3], rr[4];
+    // X_a = K_ff^-1 K_fc[:, block a], condensed residual r = R_cp - K_cf y
 #pragma unroll
-    for (int i = 0; i < 3; ++i)
+    for (int m = 0; m < 3; ++m)
 #pragma unroll
-      for (int m = 0; m < 3; ++m)
-        Kcf[i][m] = det * (m1b * E.G[i][m] + E.beta[i] * F[m] + (i == m ? E.Aa + nut * gD : 0.0));
+      for (int k = 0; k < 4; ++k)
+        Xa[m][k] = Kinv[3 * m] * Kfc[0][k] + Kinv[3 * m + 1] * Kfc[1][k] + Kinv[3 * m + 2] * Kfc[2][k];
 #pragma unroll
-    for (int m = 0; m < 3; ++m) Kcf[3][m] = -det * H[m];
-    double Wa[4][3];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-#pragma unroll
-      for (int m = 0; m < 3; ++m) Wa[i][m] = Kcf[i][0] * Kinv[m] + Kcf[i][1] * Kinv[3 + m] + Kcf[i][2] * Kinv[6 + m];
-      rr[i] = Rcp[i] - (Wa[i][0] * Rf[0] + Wa[i][1] * Rf[1] + Wa[i][2] * Rf[2]);
-    }
+    for (int i = 0; i < 4; ++i) rr[i] = Rcp[i] - Kcf[i][0] * y[0] - Kcf[i][1] * y[1] - Kcf[i][2] * y[2];
     const uint32_t msk = dir_mask[e];
     if (valid) {
-      if (!(isfinite(rr[0]) && isfinite(rr[1]) && isfinite(rr[2]) && isfinite(rr[3])))
+      if (!(finite(rr[0]) && finite(rr[1]) && finite(rr[2]) && finite(rr[3])))
         atomicOr(flags, FLAG_NAN);
       if (a == 0 && (!E.ok || bad)) atomicOr(flags, (E.ok ? 0u : FLAG_NEG_JACOBIAN) | (bad ? FLAG_SINGULAR_KFF : 0u));
 #pragma unroll
       for (int m = 0; m < 3; ++m)
 #pragma unroll
-        for (int k = 0; k < 4; ++k) recX[96 * e + 32 * m + 4 * a + k] = T(Xa[m][k]);
+        for (int k = 0; k < 4; ++k) recX[96 * e + 32 * m + 4 * a + k] = narrow<T>(Xa[m][k]);
       if (a < 3) {
-        double kr3[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) kr3[k] = a == 0 ? Kinv[k] : a == 1 ? Kinv[3 + k] : Kinv[6 + k];
-        recY[3 * e + a] = kr3[0] * Rf[0] + kr3[1] * Rf[1] + kr3[2] * Rf[2];
+        recY[3 * e + a] = a == 0 ? y[0] : a == 1 ? y[1] : y[2];
 #pragma unroll
         for (int k = 0; k < 3; ++k) recKinv[9 * e + 3 * a + k] = kr3[k];
       }
@@ -552,7 +602,7 @@ __global__ void __launch_bounds__(TET_WARPS * 32) tet_assembly_kernel(
             if (oKfc) oKfc[48 * it + 16 * m + 4 * a + k] = Kfc[m][k];
         if (oKff && a < 3)
 #pragma unroll
-          for (int k = 0; k < 3; ++k) oKff[9 * it + 3 * a + k] = a == 0 ? Kff[k] : a == 1 ? Kff[3 + k] : Kff[6 + k];
+          for (int k = 0; k < 3; ++k) oKff[9 * it + 3 * a + k] = Kff[k];
       } else {
 #pragma unroll
         for (int i = 0; i < 4; ++i)
@@ -575,24 +625,27 @@ __global__ void __launch_bounds__(TET_WARPS * 32) tet_assembly_kernel(
       double Eab[3];
 #pragma unroll
       for (int k = 0; k < 3; ++k)
-        Eab[k] = E.m2da[3 * b] * E.Ji[0][k] + E.m2da[3 * b + 1] * E.Ji[1][k] + E.m2da[3 * b + 2] * E.Ji[2][k];
-      const double sd = dot3(E.g[b], E.Ua) + tau * m2 + nut * M[TM_M0] * dot3(E.ga, E.g[b]);
+        Eab[k] = E.m2da[3 * b] * E.C[0][k] + E.m2da[3 * b + 1] * E.C[1][k] + E.m2da[3 * b + 2] * E.C[2][k];
+      const double sd = dot3(E.g[b], tt.w) + dtau * m2;
       double K[4][4];
 #pragma unroll
       for (int i = 0; i < 3; ++i) {
 #pragma unroll
-        for (int k = 0; k < 3; ++k) K[i][k] = det * (E.G[i][k] * m2 + E.beta[i] * Eab[k] + (i == k ? sd : 0.0));
-        K[i][3] = -det * E.ga[i] * M[TM_M1 + b];
+        for (int k = 0; k < 3; ++k) {
+          K[i][k] = E.G[i][k] * m2 + E.beta[i] * Eab[k];
+          if (i == k) K[i][k] += sd;
+        }
+        K[i][3] = -E.ga[i] * M[TM_M1 + b];
       }
 #pragma unroll
-      for (int k = 0; k < 3; ++k) K[3][k] = -det * E.g[b][k] * E.m1a;
+      for (int k = 0; k < 3; ++k) K[3][k] = -E.g[b][k] * E.m1a;
       K[3][3] = 0.0;
       if (!valid) continue;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         double v[4];
 #pragma unroll
-        for (int k = 0; k < 4; ++k) v[k] = K[i][k] - (Kcf[i][0] * Xb[0][k] + Kcf[i][1] * Xb[1][k] + Kcf[i][2] * Xb[2][k]);
+        for (int k = 0; k < 4; ++k) v[k] = K[i][k] - Kcf[i][0] * Xb[0][k] - Kcf[i][1] * Xb[1][k] - Kcf[i][2] * Xb[2][k];
         const int r = 4 * a + i;
         if (ELEM_OUT) {
 #pragma unroll
@@ -601,10 +654,10 @@ __global__ void __launch_bounds__(TET_WARPS * 32) tet_assembly_kernel(
             if (oKcc) oKcc[256 * it + 16 * r + 4 * b + k] = K[i][k];
           }
         } else if (!(msk >> r & 1u)) {
+          T o[4];
 #pragma unroll
-          for (int k = 0; k < 4; ++k)
-            if (msk >> (4 * b + k) & 1u) v[k] = 0.0;
-          tet_scatter_row<T>(values + blk[16 * e + 4 * a + b] + i * rl, v, ATOMIC);
+          for (int k = 0; k < 4; ++k) o[k] = msk >> (4 * b + k) & 1u ? T(0) : narrow<T>(v[k]);
+          tet_scatter_row<T>(values + blk[16 * e + 4 * a + b] + i * rl, o, ATOMIC);
         }
       }
     }
@@ -634,10 +687,10 @@ __global__ void __launch_bounds__(TET_WARPS * 32) tet_residual_kernel(
     TetElem E;
     tet_element(a, e, xyz, u, up, conn, beta, kp.transient != 0, M, E);
     double Rcp[4], Rf[3];
-    tet_residual(a, E, M, nut, kp.tau, kp.f, Rcp, Rf);
+    tet_residual(a, E, tet_terms(E, M, nut), M, kp, nut, Rcp, Rf);
     if (!valid) continue;
-    if (!(isfinite(Rcp[0]) && isfinite(Rcp[1]) && isfinite(Rcp[2]) && isfinite(Rcp[3]) &&
-          isfinite(Rf[0]) && isfinite(Rf[1]) && isfinite(Rf[2])))
+    if (!(finite(Rcp[0]) && finite(Rcp[1]) && finite(Rcp[2]) && finite(Rcp[3]) && finite(Rf[0]) &&
+          finite(Rf[1]) && finite(Rf[2])))
       atomicOr(flags, FLAG_NAN);
     if (a == 0 && !E.ok) atomicOr(flags, FLAG_NEG_JACOBIAN);
     if (mode == 0) {
