@@ -119,7 +119,7 @@ __device__ __forceinline__ void scatter_row(float* p, const float v[4], bool ato
 __device__ __forceinline__ void scatter_row(double* p, const double v[4], bool atomic) {
 #pragma unroll
   for (int k = 0; k < 4; ++k) {
-    if (v[k] == 0.0) continue;
+    if (__double_as_longlong(v[k]) << 1 == 0) continue;  // zero
     if (atomic) atomicAdd(p + k, v[k]); else p[k] += v[k];
   }
 }

@@ -105,7 +105,7 @@ struct WarpArea {
   T kffp[32][9];
   T Kcf[32][3];
   T Xs[3][32];     // X = K_ff^-1 K_fc rounded to T
-  T Xl[3][32];     // X - Xs (its low part in T; zero in FP64)
+  T Xl[3][32];     // X - Xs (its low part in T; not used in FP64)
   double Kff[9];
   double cof[9];
   double Kinv[9];
@@ -289,9 +289,22 @@ VMS_HD void tan_phase3a(int lane, WarpArea<T>& W, const LaneAcc<T>& A) {
   for (int j = 0; j < 9; ++j) W.kffp[lane][j] = A.kff[j];
 }
 
-// Phase 3b: lanes 0..8 sum one K_ff entry each over the 32 partials (in T), then widen to FP64.
+// Phase 3b: lanes 0..8 sum one K_ff entry each over the 32 partials (in T), then widen to FP64. In FP64
+// three lanes share an entry: 32 additions in a chain are 2,000 cycles of the warp.
 template <typename T>
 VMS_HD void tan_phase3b(int lane, WarpArea<T>& W) {
+#if defined(__CUDA_ARCH__)
+  if constexpr (sizeof(T) == 8) {
+    const int j = lane % 9, r = lane < 27 ? lane / 9 : 3;
+    T s = T(0);
+#pragma unroll
+    for (int i = 0; i < 11; ++i)
+      if (11 * r + i < 32) s += W.kffp[11 * r + i][j];
+    s += __shfl_sync(0xffffffffu, s, lane + 9 < 32 ? lane + 9 : lane) + __shfl_sync(0xffffffffu, s, lane + 18 < 32 ? lane + 18 : lane);
+    if (lane < 9) W.KffT[lane] = W.Kff[lane] = s;
+    return;
+  }
+#endif
   if (lane < 9) {
     T s = T(0);
     for (int l = 0; l < 32; ++l) s += W.kffp[l][lane];
@@ -355,7 +368,7 @@ VMS_HD void tan_phase3f(int lane, WarpArea<T>& W, const LaneAcc<T>& A, bool accu
       const double x = W.Kinv[3 * m] * f0 + W.Kinv[3 * m + 1] * f1 + W.Kinv[3 * m + 2] * f2;
       const T xh = T(x);
       W.Xs[m][lane] = xh;
-      W.Xl[m][lane] = T(x - (double)xh);
+      if (sizeof(T) == 4) W.Xl[m][lane] = T(x - (double)xh);
       W.Kcf[lane][m] = A.kcf[m];
     }
   } else {
@@ -393,7 +406,7 @@ __device__ __forceinline__ float comp_dot3(float s, const float c[3], const floa
 #endif
 
 // Phase 3e: S blocks of the lane's two node pairs, in place: K -= K_cf X (FP32 with `accurate`:
-// compensated, with X = Xs + Xl; otherwise plain FMA with X = Xs, and Xs + Xl in FP64).
+// compensated, with X = Xs + Xl; otherwise plain FMA with X = Xs).
 template <typename T>
 VMS_HD void tan_phase3e(int lane, const WarpArea<T>& W, LaneAcc<T>& A, bool accurate) {
   const int a0 = lane >> 3, a1 = a0 + 4, b = lane & 7;
@@ -427,9 +440,7 @@ VMS_HD void tan_phase3e(int lane, const WarpArea<T>& W, LaneAcc<T>& A, bool accu
     const auto c2 = pk(-W.Kcf[4 * a0 + i][2], -W.Kcf[4 * a1 + i][2]);
     VMS_UNROLL
     for (int k = 0; k < 4; ++k) {
-      const T x0 = sizeof(T) == 8 ? W.Xs[0][4 * b + k] + W.Xl[0][4 * b + k] : W.Xs[0][4 * b + k];
-      const T x1 = sizeof(T) == 8 ? W.Xs[1][4 * b + k] + W.Xl[1][4 * b + k] : W.Xs[1][4 * b + k];
-      const T x2 = sizeof(T) == 8 ? W.Xs[2][4 * b + k] + W.Xl[2][4 * b + k] : W.Xs[2][4 * b + k];
+      const T x0 = W.Xs[0][4 * b + k], x1 = W.Xs[1][4 * b + k], x2 = W.Xs[2][4 * b + k];
       auto acc = A.K[4 * i + k];
       acc = pfma(c0, pk(x0, x0), acc);
       acc = pfma(c1, pk(x1, x1), acc);
