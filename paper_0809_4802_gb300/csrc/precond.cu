@@ -7,9 +7,9 @@
 //   L_ik = A_ik U_kk^-1,   A_ij -= L_ik U_kj   for every block j > k present in both rows,
 // after which U_ii = A_ii and its inverse is kept for the backward sweep.
 //
-// GPU mapping of the factorisation: one warp owns one node row at a time and claims rows in order
-// from a counter, so a row only ever waits for rows claimed earlier, by warps that are already
-// running. A row publishes itself by writing its epoch into a flag with release semantics;
+// GPU mapping of the factorisation: one CTA owns one node row at a time and claims rows from a counter in
+// the order of their dependency levels, so a row only ever waits for rows claimed earlier, by CTAs that
+// are already running. A row publishes itself by writing its epoch into a flag with release semantics;
 // dependants poll the flag with acquire loads (bounded: after Ilu::spin_limit polls the kernel
 // records a timeout and returns), and read data published in the same launch through L2
 // (ld.global.cg), never through L1. The triangular sweeps read the finished factor from per-row
@@ -25,7 +25,7 @@ namespace vms {
 
 namespace {
 
-constexpr int ILU_FWARPS = 4;    // warps per CTA of the factorisation
+constexpr int ILU_FWARPS = 4;    // warps per row (and CTA) of the factorisation
 constexpr unsigned FULL = 0xffffffffu;
 
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
@@ -51,82 +51,109 @@ __device__ __forceinline__ bool wait_ready(const uint32_t* f, uint32_t epoch, in
   return false;
 }
 
-// Claim the next row of this launch: 0 <= t < n_rows, or n_rows when none is left. A claim below
-// the launch's base (the counter was disturbed by a launch that stopped early) records an error
-// and also returns n_rows, so that no row index outside [0, n_rows) is ever formed.
-__device__ __forceinline__ int64_t claim_row(unsigned long long* ticket, unsigned long long base,
-                                             int64_t n_rows, int* err, int lane) {
-  unsigned long long t = 0;
-  if (lane == 0) t = atomicAdd(ticket, 1ull);
-  t = __shfl_sync(FULL, t, 0);
-  if (t < base) {
-    if (lane == 0) atomicCAS(err, 0, ILU_ERR_TIMEOUT);
-    return n_rows;
-  }
-  t -= base;
-  return t < (unsigned long long)n_rows ? (int64_t)t : n_rows;
-}
-
 // ---------------------------------------------------------------------------------------------
-// factorisation: one warp per node row; the row is eliminated in shared memory
+// factorisation: one CTA per node row; the row is eliminated in shared memory
+//
+// What bounds it: the chain of rows (224 levels on a lattice of 33^3 nodes, about 160 rows wide), and in a
+// row the FP64 instructions of its block products, 64 cycles each on one warp: 34 for a lower block of 17
+// pairs, and up to three lower blocks were finished only one level before. So a row's pairs are shared
+// by four warps, one per FP64 unit, eight pairs a step; what is known beforehand (neighbours, row starts,
+// pairs) is read before the first wait; U_kk^-1 and the blocks of row k are read as soon as row k is
+// published, while the products of the block before are still under way; and a lower block costs one
+// barrier: every warp forms L_ik for itself, the row keeps A_ik. Rows are claimed by level: in natural order
+// the rows that can run lie planes apart, and 608 CTAs would hold half a plane (6.7 ms on 33^3 nodes). 33^3 nodes (jittered cavity) with one warp
+// per row 4.05 ms, now 1.7 (9^3 0.59, 0.30; 22^3 of a tetrahedral mesh 0.66, 0.43).
 // ---------------------------------------------------------------------------------------------
 template <typename T>
 __global__ void __launch_bounds__(ILU_FWARPS * 32)
     ilu_factor_kernel(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colidx,
                       const T* __restrict__ A, T* F, T* Dinv, const int32_t* __restrict__ dpos,
                       const int32_t* __restrict__ lptr, const int32_t* __restrict__ pptr,
-                      const uint16_t* __restrict__ pairs, int64_t n_nodes, uint32_t* flags,
+                      const uint16_t* __restrict__ pairs, const int32_t* __restrict__ order, int64_t n_nodes, uint32_t* flags,
                       uint32_t epoch, unsigned long long* ticket, unsigned long long base, int* err,
                       uint32_t lim) {
-  __shared__ T srow[ILU_FWARPS][ILU_MAX_DEG * 16];
-  const int lane = threadIdx.x & 31;
-  T* row = srow[threadIdx.x >> 5];
+  constexpr int PS = 2 * ILU_FWARPS, PMAX = (ILU_MAX_DEG + PS - 1) / PS;  // pairs a step; steps of a lower block
+  __shared__ T row[ILU_MAX_DEG * 16], lrow[ILU_MAX_DEG * 16];
+  __shared__ T lw[ILU_FWARPS][16];
+  __shared__ int32_t s_k[ILU_MAX_DEG], s_pp[ILU_MAX_DEG + 1], s_rk[ILU_MAX_DEG][4];
+  __shared__ uint16_t s_pairs[ILU_MAX_DEG * ILU_MAX_DEG];
+  __shared__ int64_t s_row;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int q = (lane >> 2) & 3, c = lane & 3, half = lane >> 4;
   for (;;) {
-    const int64_t t = claim_row(ticket, base, n_nodes, err, lane);
-    if (t >= n_nodes) return;
-    const int64_t i = t;
+    // the next row of this launch. A claim below the launch's base (the counter was disturbed by a launch that
+    // stopped early) records an error and ends the block, so that no row outside [0, n_nodes) is ever formed.
+    if (tid == 0) {
+      const unsigned long long t = atomicAdd(ticket, 1ull);
+      if (t < base) atomicCAS(err, 0, ILU_ERR_TIMEOUT);
+      s_row = t >= base && t - base < (unsigned long long)n_nodes ? (int64_t)(t - base) : -1;
+    }
+    __syncthreads();
+    if (s_row < 0) return;
+    const int64_t i = order[s_row];
     const int32_t r0 = rowptr[4 * i];
-    const int deg = (rowptr[4 * i + 1] - r0) >> 2;
+    const int deg = (rowptr[4 * i + 1] - r0) >> 2, dp = dpos[i];
+    const int32_t l0 = lptr[i], p0 = pptr[l0], np = pptr[l0 + dp] - p0;
     // row i into shared memory, block-major: row[16 kk + 4 q + c] = A(4i+q, 4 adj_kk + c)
-    for (int e = lane; e < deg * 16; e += 32)
+    for (int e = tid; e < deg * 16; e += ILU_FWARPS * 32)
       row[e] = A[rowptr[4 * i + ((e >> 2) & 3)] + 4 * (e >> 4) + (e & 3)];
-    __syncwarp();
-    const int dp = dpos[i];
-    const int32_t l0 = lptr[i];
-    const int q = (lane >> 2) & 3, c = lane & 3, half = lane >> 4;
+    for (int kk = tid; kk <= dp; kk += ILU_FWARPS * 32) {
+      s_pp[kk] = pptr[l0 + kk] - p0;
+      if (kk < dp) {
+        const int32_t k = colidx[r0 + 4 * kk] >> 2;
+        s_k[kk] = k;
+        for (int m = 0; m < 4; ++m) s_rk[kk][m] = rowptr[4 * (int64_t)k + m];
+      }
+    }
+    for (int p = tid; p < np; p += ILU_FWARPS * 32) s_pairs[p] = pairs[p0 + p];
+    __syncthreads();
     for (int kk = 0; kk < dp; ++kk) {
-      const int64_t k = colidx[r0 + 4 * kk] >> 2;
+      const int64_t k = s_k[kk];
       int ok = 1;
       if (lane == 0) ok = wait_ready(flags + k, epoch, err, lim);
-      if (!__shfl_sync(FULL, ok, 0)) return;
-      // L_ik = A_ik U_kk^-1 (lanes 0..15 hold entry (q, c))
+      ok = __shfl_sync(FULL, ok, 0);
+      // U_kk^-1 (lane: column c) and the blocks U_kj of this half-warp's pairs (lane: column c)
+      T d[4], u[PMAX][4];
+      int jj[PMAX];
+      if (ok) {
+        for (int m = 0; m < 4; ++m) d[m] = __ldcg(Dinv + 16 * k + 4 * m + c);
+#pragma unroll
+        for (int s = 0; s < PMAX; ++s) {
+          const int p = s_pp[kk] + PS * s + 2 * warp + half;
+          jj[s] = -1;
+          if (p < s_pp[kk + 1]) {
+            const uint32_t pr = s_pairs[p];
+            jj[s] = pr & 255;
+            for (int m = 0; m < 4; ++m) u[s][m] = __ldcg(F + s_rk[kk][m] + 4 * (int)(pr >> 8) + c);
+          }
+        }
+      }
+      // the products of the lower blocks before are done
+      if (__syncthreads_or(!ok)) return;
+      // L_ik = A_ik U_kk^-1 (lane: entry (q, c), both halves alike)
       T l = T(0);
-      if (lane < 16) {
-        const T* d = Dinv + 16 * k + c;
-        for (int m = 0; m < 4; ++m) l += row[16 * kk + 4 * q + m] * __ldcg(d + 4 * m);
+      for (int m = 0; m < 4; ++m) l += row[16 * kk + 4 * q + m] * d[m];
+      if (half == 0) {
+        lw[warp][lane] = l;
+        if (warp == 0) lrow[16 * kk + lane] = l;
       }
       __syncwarp();
-      if (lane < 16) row[16 * kk + lane] = l;
-      __syncwarp();
-      // A_ij -= L_ik U_kj over the pairs of this lower block, two pairs per step (the products
-      // are subtracted one by one, so that each is a fused multiply-add)
-      int32_t rk[4];
-      for (int m = 0; m < 4; ++m) rk[m] = rowptr[4 * k + m];
-      const int32_t pe = pptr[l0 + kk + 1];
-      for (int32_t p = pptr[l0 + kk] + half; p < pe; p += 2) {
-        const uint32_t pr = pairs[p];
-        const int jj = pr & 255, jk = pr >> 8;
-        T s = row[16 * jj + 4 * q + c];
-        for (int m = 0; m < 4; ++m) s -= row[16 * kk + 4 * q + m] * __ldcg(F + rk[m] + 4 * jk + c);
-        row[16 * jj + 4 * q + c] = s;
-      }
-      __syncwarp();
+      // A_ij -= L_ik U_kj (the products are subtracted one by one, so that each is a fused multiply-add)
+#pragma unroll
+      for (int s = 0; s < PMAX; ++s)
+        if (jj[s] >= 0) {
+          T v = row[16 * jj[s] + 4 * q + c];
+          for (int m = 0; m < 4; ++m) v -= lw[warp][4 * q + m] * u[s][m];
+          row[16 * jj[s] + 4 * q + c] = v;
+        }
+      __syncwarp();  // lw is read before the next block's is written
     }
-    // U_ii^-1 = adj(U_ii) / det on lanes 0..15 (lane 4r + c forms the cofactor of entry (r, c)):
-    // a handful of FP64 instructions per lane instead of a serial elimination on one lane
-    {
+    __syncthreads();
+    if (warp == 0) {
+      // U_ii^-1 = adj(U_ii) / det on lanes 0..15 (lane 4r + c forms the cofactor of entry (r, c)); lanes 16..31
+      // sum the squares of the rows in the same instructions
       const T* D = row + 16 * dp;
-      const int r = (lane >> 2) & 3, c = lane & 3;
+      const int r = q;
       double mnr[3][3];  // the minor: rows other than r, columns other than c
 #pragma unroll
       for (int a2 = 0; a2 < 3; ++a2)
@@ -137,27 +164,26 @@ __global__ void __launch_bounds__(ILU_FWARPS * 32)
                         mnr[0][1] * (mnr[1][0] * mnr[2][2] - mnr[1][2] * mnr[2][0]) +
                         mnr[0][2] * (mnr[1][0] * mnr[2][1] - mnr[1][1] * mnr[2][0]);
       const double cf = ((r + c) & 1) ? -m3 : m3;
-      const double dv = lane < 16 ? (double)D[lane] : 0.0;
-      double dt = lane < 4 ? dv * cf : 0.0;  // det by the first row
+      const double dv = (double)D[lane & 15];
+      double dt = dv * (half ? dv : cf);  // lanes 0..3: det by the first row; 16..31: squared row norms
       dt += __shfl_xor_sync(FULL, dt, 1);
       dt += __shfl_xor_sync(FULL, dt, 2);
       const double det = __shfl_sync(FULL, dt, 0);
       // singular unless |det| is a fair fraction of the product of the row norms (Hadamard's
       // bound; independent of the rows' scales), compared squared: det^2 > 1e-28 prod |row|^2
-      double rn = dv * dv;
-      rn += __shfl_xor_sync(FULL, rn, 1);
-      rn += __shfl_xor_sync(FULL, rn, 2);
-      const double hb2 = __shfl_sync(FULL, rn, 0) * __shfl_sync(FULL, rn, 4) *
-                         __shfl_sync(FULL, rn, 8) * __shfl_sync(FULL, rn, 12);
+      const double hb2 = __shfl_sync(FULL, dt, 16) * __shfl_sync(FULL, dt, 20) *
+                         __shfl_sync(FULL, dt, 24) * __shfl_sync(FULL, dt, 28);
       const bool good = isfinite(det) && hb2 > 0.0 && det * det > 1e-28 * hb2;
       if (!good && lane == 0) atomicCAS(err, 0, ILU_ERR_PIVOT);
       if (lane < 16) Dinv[16 * i + 4 * c + r] = good ? T(cf / det) : T(r == c ? 1.0 : 0.0);
+      __threadfence();
+    } else {
+      for (int e = tid - 32; e < deg * 16; e += (ILU_FWARPS - 1) * 32)
+        F[rowptr[4 * i + ((e >> 2) & 3)] + 4 * (e >> 4) + (e & 3)] = (e >> 4) < dp ? lrow[e] : row[e];
+      __threadfence();
     }
-    for (int e = lane; e < deg * 16; e += 32)
-      F[rowptr[4 * i + ((e >> 2) & 3)] + 4 * (e >> 4) + (e & 3)] = row[e];
-    __threadfence();
-    __syncwarp();
-    if (lane == 0) st_release(flags + i, epoch);
+    __syncthreads();
+    if (tid == 0) st_release(flags + i, epoch);
   }
 }
 
@@ -725,7 +751,7 @@ int build_pattern(vms_ctx* ctx, Ilu& p, const Mesh& m) {
   // on one side would exceed ILU_FAR_MAX (one segment alone never does: 64 rows of at most 31);
   // every neighbour's place in its row's chunk: the chunk's own rows first, then the far list of
   // its side
-  std::vector<int32_t> chunk(1, 0), at(adj.size(), 0), farptr[2], far[2], mark(N, -1);
+  std::vector<int32_t> chunk(1, 0), at(adj.size(), 0), farptr[2], far[2], mark(N, -1), order(N);
   p.slots = 0;
   {
     const int32_t n_segs = (int32_t)seg.size() - 1;
@@ -735,6 +761,11 @@ int build_pattern(vms_ctx* ctx, Ilu& p, const Mesh& m) {
       for (int32_t t = start[i]; t < start[i] + dpos[i]; ++t) level[0][i] = std::max(level[0][i], level[0][adj[t]] + 1);
     for (int64_t i = N - 1; i >= 0; --i)
       for (int32_t t = start[i] + dpos[i] + 1; t < start[i + 1]; ++t) level[1][i] = std::max(level[1][i], level[1][adj[t]] + 1);
+    // rows by level, for the factorisation
+    std::vector<int32_t> first(N + 1, 0);
+    for (int64_t i = 0; i < N; ++i) ++first[level[0][i] + 1];
+    for (int64_t l = 0; l < N; ++l) first[l + 1] += first[l];
+    for (int64_t i = 0; i < N; ++i) order[first[level[0][i]]++] = (int32_t)i;
     farptr[0].push_back(0);
     farptr[1].push_back(0);
     for (int32_t lo = 0; lo < n_segs;) {
@@ -791,6 +822,7 @@ int build_pattern(vms_ctx* ctx, Ilu& p, const Mesh& m) {
     if (e == cudaSuccess && !h.empty()) e = cudaMemcpy(d, h.data(), sizeof(int32_t) * h.size(), cudaMemcpyHostToDevice);
   };
   up(p.chunk, chunk);
+  up(p.order, order);
   up(p.at, at);
   for (int side = 0; side < 2; ++side) {
     up(p.farptr[side], farptr[side]);
@@ -900,7 +932,7 @@ int pack(const Ilu& p, const Mesh& m, unsigned char* const rec[2], cudaStream_t 
 
 void free_ilu(Ilu& p) {
   const uint32_t lim = p.spin_limit;  // a setting of the context, kept across meshes
-  void* bufs[] = {p.dpos, p.lptr, p.pptr, p.pairs, p.F, p.Dinv, p.y, p.yp64, p.xp64,
+  void* bufs[] = {p.dpos, p.order, p.lptr, p.pptr, p.pairs, p.F, p.Dinv, p.y, p.yp64, p.xp64,
                   p.vals64, p.flags, p.yp32, p.xp32, p.tickets, p.err, p.seg, p.inl, p.chunk, p.at,
                   p.farptr[0], p.farptr[1], p.far[0], p.far[1], p.rec[0], p.rec[1], p.rec32[0], p.rec32[1], p.y32};
   for (void* b : bufs)
@@ -925,12 +957,12 @@ int ilu_factor(vms_ctx* ctx, Ilu& p, const Mesh& m, bool fp32, const void* value
     *launches += convert<float, double>((const float*)values, p.vals64, m.nnz, st);
     A = p.vals64;
   }
-  const unsigned ctas = resident_ctas(m.n_nodes, ILU_FWARPS, 8 * sm_count());
+  const unsigned ctas = resident_ctas(m.n_nodes, 1, 4 * sm_count());
   const uint32_t ep = next_epoch(p, st);
   ilu_factor_kernel<double><<<ctas, ILU_FWARPS * 32, 0, st>>>(
-      m.rowptr, m.colidx, A, p.F, p.Dinv, p.dpos, p.lptr, p.pptr, p.pairs, m.n_nodes, p.flags, ep,
+      m.rowptr, m.colidx, A, p.F, p.Dinv, p.dpos, p.lptr, p.pptr, p.pairs, p.order, m.n_nodes, p.flags, ep,
       p.tickets, p.base, p.err, p.spin_limit);
-  p.base += (unsigned long long)m.n_nodes + (unsigned long long)ctas * ILU_FWARPS;
+  p.base += (unsigned long long)m.n_nodes + ctas;  // + each CTA's last claim
   *launches += 1;
   if (fp32) *launches += pack<float>(p, m, p.rec32, st);
   p.packed64 = false;  // the FP64 records are made on the first FP64 sweep
