@@ -63,6 +63,19 @@ VMS_HD double recip(double d) {
   return recip_normal(d);
 }
 
+#if defined(__CUDACC__)
+// A float as a double, exactly, without the FP64 pipe (its conversion instruction costs as much there
+// as a product): the exponent is rebiased by 1023 - 127 and the fraction's 23 bits are the double's
+// upper ones. Zeros keep their sign; subnormals, infinities and NaN take the conversion instruction.
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t u = __float_as_uint(x), m = u << 1;
+  if (m == 0u || (m >= 0x01000000u && m < 0xff000000u))
+    return __hiloint2double((int)((u & 0x80000000u) | (m == 0u ? 0u : (m >> 4) + 0x38000000u)), (int)(u << 29));
+  return (double)x;
+}
+__device__ __forceinline__ double widen(double x) { return x; }
+#endif
+
 // Local node a <-> lattice corner bits (i,j,k): a = 0..7 <-> 000 100 110 010 001 101 111 011.
 // Forward butterfly: nodal f[8] (local order) -> monomial coefficients, scaled by 8, of
 // {1, xi, eta, zeta, xi eta, xi zeta, eta zeta, xi eta zeta}.

@@ -14,6 +14,7 @@
 #include <type_traits>
 #include <vector>
 
+#include "element_math.cuh"
 #include "ortho.cuh"
 #include "solver.h"
 
@@ -36,7 +37,7 @@ void free_solver(SolverWork& s) {
 // ---------------------------------------------------------------------------------------------
 // kernels
 // ---------------------------------------------------------------------------------------------
-// y = S x on the rows of nodes [node0, node0 + n_nodes): one warp per node (its four scalar rows
+// y = S x on the rows of nodes [node0, node0 + n_nodes): a group of lanes per node (its four scalar rows
 // share one column pattern of 4x4 blocks), one lane per block, so a column index is read once per
 // block instead of once per value. x and y are compact (x[c - 4 node0], y[4 (node - node0) + q]).
 // FP32 accumulation when matrix and vectors are FP32 (the inner solve of the mixed mode), FP64
@@ -56,50 +57,67 @@ template <> struct Row4<double> {
   }
 };
 
-template <typename T, typename VT>
+// L lanes per node. 32: a block per lane, the shortest chain, for small meshes. 16: two nodes per warp, fewer
+// sums across lanes (a node of 27 blocks takes 18 FP64 warp instructions instead of 22, a tetrahedral one of 15
+// blocks 10 instead of 22) and two blocks' loads in flight per lane. Measured in us with 32 and 16 lanes, FP64
+// matrix and vectors; FP32 matrix, FP64 vectors; both FP32: 33^3 nodes 49 and 43; 84 and 78; 23.9 and 23.0; 22^3
+// nodes of a tetrahedral mesh 16.6 and 10.8; 28.9 and 16.7; 9.0 and 7.2; 15^3 nodes 8.5 and 8.5; 12.5 and 14.5;
+// 6.5 and 7.0. Eight lanes: slower on small meshes, no faster on large ones. FP32 values are widened by integer
+// instructions (a conversion takes a slot of the FP64 pipe).
+template <typename T, typename VT, int L>
 __global__ void __launch_bounds__(256) spmv_kernel(const int32_t* __restrict__ rowptr,
                                                    const int32_t* __restrict__ colidx,
                                                    const T* __restrict__ val,
                                                    const VT* __restrict__ x, VT* __restrict__ y,
-                                                   int64_t node0, int64_t n_nodes) {
+                                                   int64_t node0, int64_t n_nodes, bool vec) {
   using Acc = typename std::conditional<sizeof(T) == 4 && sizeof(VT) == 4, float, double>::type;
-  const int64_t nd = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int lane = threadIdx.x & 31;
-  if (nd >= n_nodes) return;  // uniform over the warp
-  const int64_t g = node0 + nd;
-  int32_t rp[4];
-  for (int m = 0; m < 4; ++m) rp[m] = rowptr[4 * g + m];
-  const int deg = (rp[1] - rp[0]) >> 2;
+  const int64_t nd = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) / L;
+  const int lane = threadIdx.x % L;
+  const bool valid = nd < n_nodes;
+  const int4 rp4 = __ldg(reinterpret_cast<const int4*>(rowptr) + node0 + (valid ? nd : 0));
+  const int32_t rp[4] = {rp4.x, rp4.y, rp4.z, rp4.w};
+  const int deg = valid ? (rp[1] - rp[0]) >> 2 : 0;
   Acc acc[4] = {Acc(0), Acc(0), Acc(0), Acc(0)};
-  for (int kk = lane; kk < deg; kk += 32) {
+#pragma unroll 4
+  for (int kk = lane; kk < deg; kk += L) {
     const int64_t c = (int64_t)colidx[rp[0] + 4 * kk] - 4 * node0;
-    Acc xv[4];
-    for (int m = 0; m < 4; ++m) xv[m] = (Acc)x[c + m];
+    VT xv[4];
+    if (vec) Row4<VT>::ld(x + c, xv);
+    else
+      for (int m = 0; m < 4; ++m) xv[m] = x[c + m];
+#pragma unroll
     for (int r = 0; r < 4; ++r) {
       T v[4];
       Row4<T>::ld(val + rp[r] + 4 * kk, v);
-      for (int m = 0; m < 4; ++m) acc[r] = fma((Acc)v[m], xv[m], acc[r]);
+#pragma unroll
+      for (int m = 0; m < 4; ++m) {
+        if constexpr (sizeof(Acc) == 4) acc[r] = fmaf(v[m], xv[m], acc[r]);
+        else acc[r] = fma(widen(v[m]), (double)xv[m], acc[r]);
+      }
     }
   }
-  // reduce-scatter of the four sums over the warp: lane L ends with component (L >> 3) & 3
-  const bool h16 = lane & 16, h8 = lane & 8;
-  const Acc s0 = h16 ? acc[0] : acc[2], s1 = h16 ? acc[1] : acc[3];
-  const Acc b0 = (h16 ? acc[2] : acc[0]) + __shfl_xor_sync(0xffffffffu, s0, 16);
-  const Acc b1 = (h16 ? acc[3] : acc[1]) + __shfl_xor_sync(0xffffffffu, s1, 16);
-  Acc t = (h8 ? b1 : b0) + __shfl_xor_sync(0xffffffffu, h8 ? b0 : b1, 8);
-  t += __shfl_xor_sync(0xffffffffu, t, 4);
-  t += __shfl_xor_sync(0xffffffffu, t, 2);
-  t += __shfl_xor_sync(0xffffffffu, t, 1);
-  if ((lane & 7) == 0) y[4 * nd + (lane >> 3)] = VT(t);
+  // reduce-scatter of the four sums over the node's lanes: lanes lane / (L / 4) = q end with component q
+  const bool hi = lane & (L / 2), lo = lane & (L / 4);
+  const Acc s0 = hi ? acc[0] : acc[2], s1 = hi ? acc[1] : acc[3];
+  const Acc b0 = (hi ? acc[2] : acc[0]) + __shfl_xor_sync(0xffffffffu, s0, L / 2);
+  const Acc b1 = (hi ? acc[3] : acc[1]) + __shfl_xor_sync(0xffffffffu, s1, L / 2);
+  Acc t = (lo ? b1 : b0) + __shfl_xor_sync(0xffffffffu, lo ? b0 : b1, L / 4);
+#pragma unroll
+  for (int o = L / 8; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if (valid && lane % (L / 4) == 0) y[4 * nd + lane / (L / 4)] = VT(t);
 }
 
 template <typename T, typename VT>
 static int spmv(const Mesh& m, const SysRange& R, const void* values, const VT* x, VT* y,
                 cudaStream_t st) {
   const int64_t nodes = R.nodes();
-  const unsigned blocks = (unsigned)((nodes * 32 + 255) / 256);
-  spmv_kernel<T, VT><<<blocks, 256, 0, st>>>(m.rowptr, m.colidx, (const T*)values, x, y, R.n0,
-                                             nodes);
+  const bool vec = (reinterpret_cast<uintptr_t>(x) & 15) == 0;  // a caller's vector (vms_apply) may not be
+  auto go = [&](auto kern, int lanes) {
+    kern<<<(unsigned)((nodes * lanes + 255) / 256), 256, 0, st>>>(m.rowptr, m.colidx, (const T*)values, x, y, R.n0,
+                                                                  nodes, vec);
+  };
+  if (nodes < 32 * (int64_t)sm_count()) go(spmv_kernel<T, VT, 32>, 32);
+  else go(spmv_kernel<T, VT, 16>, 16);
   return 1;
 }
 

@@ -515,17 +515,6 @@ int launch_fused_assembly(const Mesh& m, const State& s, const Fp32Copy& c32, co
   return 1;
 }
 
-// A float as a double, exactly, without the FP64 pipe (its conversion instruction costs as much there
-// as a product): the exponent is rebiased by 1023 - 127 and the fraction's 23 bits are the double's
-// upper ones. Zeros keep their sign; subnormals, infinities and NaN take the conversion instruction.
-__device__ __forceinline__ double widen(float x) {
-  const uint32_t u = __float_as_uint(x), m = u << 1;
-  if (m == 0u || (m >= 0x01000000u && m < 0xff000000u))
-    return __hiloint2double((int)((u & 0x80000000u) | (m == 0u ? 0u : (m >> 4) + 0x38000000u)), (int)(u << 29));
-  return (double)x;
-}
-__device__ __forceinline__ double widen(double x) { return x; }
-
 // y = K_ff^-1 R_f (FP64, kept for the recovery) and r_e = R_cp - K_cf y (FP64 arithmetic on the
 // stored K_cf, FP32 in mixed precision) scattered into the right-hand side. Eight threads per element, one
 // per node: y is formed by three of them and handed round, each thread reads its node's 4 x 3 block
