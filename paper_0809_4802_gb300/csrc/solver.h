@@ -33,6 +33,7 @@ struct SolverWork {
   double* Dinv = nullptr;    // n_nodes * 16: inverted 4x4 diagonal node blocks
   double* h = nullptr;       // device scalars for dots
   double* hcol = nullptr;    // page-locked: the Hessenberg column of the current step (ortho_kernel)
+  cudaEvent_t col_done = nullptr;  // ... has been written
   double* og = nullptr;      // 2 OG_SET: exchange words of ortho_kernel, two launches' taking turns
   bool og_turn = false;
   int og_k = 0, og_blocks = 0;  // vectors and blocks of the last launch
