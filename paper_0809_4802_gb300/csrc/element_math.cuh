@@ -65,13 +65,14 @@ VMS_HD double recip(double d) {
 
 #if defined(__CUDACC__)
 // A float as a double, exactly, without the FP64 pipe (its conversion instruction costs as much there
-// as a product): the exponent is rebiased by 1023 - 127 and the fraction's 23 bits are the double's
-// upper ones. Zeros keep their sign; subnormals, infinities and NaN take the conversion instruction.
+// as a product): the exponent is rebiased by 1023 - 127 (infinities and NaN by 2047 - 255) and the
+// fraction's 23 bits are the double's upper ones; a subnormal number is first scaled by 2^64, exactly.
+// Straight-line: behind a test the compiler runs the conversion for every value and selects.
 __device__ __forceinline__ double widen(float x) {
-  const uint32_t u = __float_as_uint(x), m = u << 1;
-  if (m == 0u || (m >= 0x01000000u && m < 0xff000000u))
-    return __hiloint2double((int)((u & 0x80000000u) | (m == 0u ? 0u : (m >> 4) + 0x38000000u)), (int)(u << 29));
-  return (double)x;
+  const bool sub = __float_as_uint(x) << 1 < 0x01000000u;  // or zero
+  const uint32_t u = __float_as_uint(x * (sub ? 0x1p64f : 1.f)), m = u << 1;
+  const uint32_t bias = sub ? 0x38000000u - (64u << 20) : (m >= 0xff000000u ? 0x70000000u : 0x38000000u);
+  return __hiloint2double((int)((u & 0x80000000u) | (m == 0u ? 0u : (m >> 4) + bias)), (int)(u << 29));
 }
 __device__ __forceinline__ double widen(double x) { return x; }
 #endif

@@ -60,11 +60,11 @@ template <> struct Row4<double> {
 
 // L lanes per node. 32: a block per lane, the shortest chain, for small meshes. 16: two nodes per warp, fewer
 // sums across lanes (a node of 27 blocks takes 18 FP64 warp instructions instead of 22, a tetrahedral one of 15
-// blocks 10 instead of 22) and two blocks' loads in flight per lane. Measured in us with 32 and 16 lanes, FP64
-// matrix and vectors; FP32 matrix, FP64 vectors; both FP32: 33^3 nodes 49 and 43; 84 and 78; 23.9 and 23.0; 22^3
-// nodes of a tetrahedral mesh 16.6 and 10.8; 28.9 and 16.7; 9.0 and 7.2; 15^3 nodes 8.5 and 8.5; 12.5 and 14.5;
-// 6.5 and 7.0. Eight lanes: slower on small meshes, no faster on large ones. FP32 values are widened by integer
-// instructions (a conversion takes a slot of the FP64 pipe).
+// blocks 10 instead of 22) and two blocks' loads in flight per lane. FP32 values are widened by integer
+// instructions (a conversion takes a slot of the FP64 pipe). Measured in us, before (32 lanes, conversions) and now,
+// FP64 matrix and vectors; FP32 matrix, FP64 vectors; both FP32: 33^3 nodes 49 and 43; 84 and 40; 23.9 and 21.4;
+// 22^3 nodes of a tetrahedral mesh 16.6 and 10.5; 28.9 and 10.5; 9.0 and 6.7. On 15^3 nodes 16 lanes took 8.5, 14.5
+// and 7.0 where 32 took 8.5, 12.5 and 6.5. Eight lanes: slower on small meshes, no faster on large ones.
 template <typename T, typename VT, int L>
 __global__ void __launch_bounds__(256) spmv_kernel(const int32_t* __restrict__ rowptr,
                                                    const int32_t* __restrict__ colidx,

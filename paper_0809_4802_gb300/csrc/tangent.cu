@@ -379,9 +379,9 @@ __global__ void __launch_bounds__(WARPS * 32, ENG == 0 ? 1 : (ENG == TS_ENGINE ?
 // ever waits for another. The elements past the last whole round of the residual warps (residual_rest;
 // all of a small mesh) are taken with a lane per line of the rule: a round of 32 elements per warp
 // takes about 200 us however few warps have one. Small meshes also claim tangents one at a time.
-// A mixed assembly of 64 elements took 237 us and takes 82, 1,728 252 and 90, 8,000 263 and 204, 21,952
-// 484 and 349, 85,184 1,196 and 1,138; without a remainder for the lines the kernel has no code for them
-// (LINES), which would cost it 1 %.
+// A mixed assembly of 64 elements took 237 us and took 82 with the lines, 1,728 252 and 90, 8,000 263 and 204, 21,952
+// 484 and 349, 85,184 1,196 and 1,138 (55, 56, 166, 302 and 1,067 with fewer launches and instructions since);
+// without a remainder for the lines the kernel has no code for them (LINES), which would cost it 1 %.
 // The tangent warps take quadrature points 16 at a time (two passes of 16 lanes for the 27-point
 // rule), which halves their point records and lets the residual's store and eight warp areas fit
 // in one SM's shared memory.

@@ -170,8 +170,8 @@ constexpr int TET_PER_WARP = 8;  // tetrahedra per warp
 // det J that turns J^-1 into its cofactors: no entry of J^-1 and no product with det J is formed, only 1 /
 // det J where a product of two gradients needs it. With that, sums started from the value they are
 // subtracted from, y = K_ff^-1 R_f in place of K_cf K_ff^-1, K_ff's rows on the group's lanes and results
-// narrowed to FP32 by integer instructions a warp takes about 690 FP64 instructions for its eight elements
-// instead of 1,030.
+// narrowed to FP32 by integer instructions a warp takes 670 FP64 instructions for its eight elements instead
+// of 1,030: 355,914 elements 2,805 -> 1,745 us in mixed precision, 1,955 in FP64 (the wider scatter).
 struct TetElem {
   int nd[4];
   int nda;           // node a
@@ -431,17 +431,33 @@ __device__ __forceinline__ void tet_residual(int a, const TetElem& E, const TetT
 // Tested on the bits: an FP64 compare takes a slot of the FP64 pipe.
 __device__ __forceinline__ bool finite(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
 
-// x in the type of the results. To FP32 (round to nearest, ties to even) by integer instructions where the
-// result is a normal number: the conversion instruction takes a slot of the FP64 pipe.
-template <typename T> __device__ __forceinline__ T narrow(double x);
-template <> __device__ __forceinline__ double narrow<double>(double x) { return x; }
-template <> __device__ __forceinline__ float narrow<float>(double x) {
-  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
-  const uint32_t t = (hi & 0x7fffffffu) - 0x38000000u;  // exponent rebiased by 1023 - 127
-  if (t - 0x00100000u >= 0x0fe00000u) return (float)x;
-  uint32_t f = __funnelshift_l(lo, t, 3);
-  f += ((lo & 0x1fffffffu) + 0x0fffffffu + (f & 1u)) >> 29;
-  return __uint_as_float(f | (hi & 0x80000000u));
+// Four values in the type of the results. To FP32 (round to nearest, ties to even) by integer instructions
+// where the results are normal numbers or zero: the conversion instruction takes a slot of the FP64 pipe.
+// Otherwise (subnormal results, infinities, NaN) all four are converted, in a call: conversions behind a test are
+// issued for every value, predicated.
+__device__ __noinline__ float4 convert4(double a, double b, double c, double d) {
+  return make_float4((float)a, (float)b, (float)c, (float)d);
+}
+__device__ __forceinline__ void narrow4(const double v[4], double o[4]) {
+#pragma unroll
+  for (int k = 0; k < 4; ++k) o[k] = v[k];
+}
+__device__ __forceinline__ void narrow4(const double v[4], float o[4]) {
+  bool special = false;
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const uint32_t hi = (uint32_t)__double2hiint(v[k]), lo = (uint32_t)__double2loint(v[k]);
+    const uint32_t t = (hi & 0x7fffffffu) - 0x38000000u;  // exponent rebiased by 1023 - 127
+    const bool zero = ((hi << 1) | lo) == 0u;
+    uint32_t f = __funnelshift_l(lo, t, 3);
+    f += ((lo & 0x1fffffffu) + 0x0fffffffu + (f & 1u)) >> 29;
+    o[k] = __uint_as_float((zero ? 0u : f) | (hi & 0x80000000u));
+    special = special || (!zero && t - 0x00100000u >= 0x0fe00000u);
+  }
+  if (__builtin_expect(special, 0)) {
+    const float4 c = convert4(v[0], v[1], v[2], v[3]);
+    o[0] = c.x; o[1] = c.y; o[2] = c.z; o[3] = c.w;
+  }
 }
 
 template <typename T>
@@ -579,8 +595,12 @@ __global__ void __launch_bounds__(TET_WARPS * 32) tet_assembly_kernel(
       if (a == 0 && (!E.ok || bad)) atomicOr(flags, (E.ok ? 0u : FLAG_NEG_JACOBIAN) | (bad ? FLAG_SINGULAR_KFF : 0u));
 #pragma unroll
       for (int m = 0; m < 3; ++m)
+      {
+        T x[4];
+        narrow4(Xa[m], x);
 #pragma unroll
-        for (int k = 0; k < 4; ++k) recX[96 * e + 32 * m + 4 * a + k] = narrow<T>(Xa[m][k]);
+        for (int k = 0; k < 4; ++k) recX[96 * e + 32 * m + 4 * a + k] = x[k];
+      }
       if (a < 3) {
         recY[3 * e + a] = a == 0 ? y[0] : a == 1 ? y[1] : y[2];
 #pragma unroll
@@ -655,8 +675,10 @@ __global__ void __launch_bounds__(TET_WARPS * 32) tet_assembly_kernel(
           }
         } else if (!(msk >> r & 1u)) {
           T o[4];
+          narrow4(v, o);
 #pragma unroll
-          for (int k = 0; k < 4; ++k) o[k] = msk >> (4 * b + k) & 1u ? T(0) : narrow<T>(v[k]);
+          for (int k = 0; k < 4; ++k)
+            if (msk >> (4 * b + k) & 1u) o[k] = T(0);
           tet_scatter_row<T>(values + blk[16 * e + 4 * a + b] + i * rl, o, ATOMIC);
         }
       }
