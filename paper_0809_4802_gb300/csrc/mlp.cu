@@ -228,6 +228,7 @@ constexpr uint32_t OP_STEP = 2 * OP_K;        // a K step of 16: two core matric
 struct SmemFwd {
   // operands in the canonical K-major layout without swizzle: [k / 8][row][k % 8]
   __nv_bfloat16 W1[2 * FT * 8];               // W1 (k < 12), the bias' three terms (k = 12..14), 0
+  __nv_bfloat16 W1f[2 * FT * 8];              // W1 with 0 for its infinities, 0: the partner of X's lower terms
   __nv_bfloat16 B2[2 * FT * 8];               // 0, the second bias' three terms, 0
   __nv_bfloat16 one[2 * FT * 8];              // its activations: 0 (not X's, which may be infinite), 1, 1, 1, 0
   __nv_bfloat16 X[3][2 * FT * 8];             // the terms of X; 1 in k = 12..14 of the first
@@ -239,6 +240,7 @@ struct SmemFwd {
   uint32_t tmem;
   unsigned long long bar[3];                  // D1; first half of D2 (operand buffers free); D2
 };
+static_assert(sizeof(SmemFwd) + 1024 <= (228 << 10) / 2, "two CTAs per SM");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 // Shared-memory matrix descriptor: start, LBO and SBO in 16-byte units, version 1, no swizzle.
@@ -296,7 +298,8 @@ __device__ __forceinline__ void tc_load32(uint32_t addr, float v[32]) {
       : "memory");
 }
 // x = h + m + l, each the leading 8 bits of what is left (bit patterns with the BF16 in the upper half):
-// exact for every finite x whose low term is a BF16 number; infinities and NaN stay in h.
+// exact for every finite x whose low term is a BF16 number. NaN makes all of them NaN, an infinity m and l: where x
+// may be one, finite_terms() keeps it in h alone.
 struct Terms {
   uint32_t h, m, l;
 };
@@ -306,6 +309,11 @@ __device__ __forceinline__ Terms split_exact(float x) {
   const float r = x - __uint_as_float(t.h);
   t.m = __float_as_uint(r) & 0xffff0000u;
   t.l = __float_as_uint(r - __uint_as_float(t.m));
+  return t;
+}
+__device__ __forceinline__ Terms finite_terms(float x) {
+  Terms t = split_exact(x);
+  if (fabsf(x) == INFINITY) t.m = t.l = 0u;
   return t;
 }
 // tanh of two values: x N(x^2) / D(x^2) with N of degree 4 and D of degree 5, the minimax quotient on [0, 9.02]
@@ -407,12 +415,13 @@ __global__ void __launch_bounds__(THREADS, 2) mlp_forward_kernel(const __nv_bflo
   }
   {
     const int c = tid / NW, j = tid % NW;  // 2 x 128
-    const Terms b1 = split_exact(bias[BB_1 + j]), b2 = split_exact(bias[BB_2 + j]);
+    const Terms b1 = finite_terms(bias[BB_1 + j]), b2 = finite_terms(bias[BB_2 + j]);
     const __nv_bfloat16 z = __ushort_as_bfloat16(0);
-    alignas(16) __nv_bfloat16 v[8], u[8], o[8];
+    alignas(16) __nv_bfloat16 v[8], f[8], u[8], o[8];
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
       v[k] = 8 * c + k < NI ? w[WB_1 + (8 * c + k) * NW + j] : z;
+      f[k] = (__bfloat16_as_ushort(v[k]) & 0x7fffu) == 0x7f80u ? z : v[k];
       u[k] = z;
       o[k] = c && k >= 4 && k < 7 ? __ushort_as_bfloat16(0x3f80) : z;
     }
@@ -422,6 +431,7 @@ __global__ void __launch_bounds__(THREADS, 2) mlp_forward_kernel(const __nv_bflo
       u[4] = upper_bf16(b2.h); u[5] = upper_bf16(b2.m); u[6] = upper_bf16(b2.l);
     }
     *reinterpret_cast<uint4*>(&s.W1[c * FT * 8 + j * 8]) = *reinterpret_cast<const uint4*>(v);
+    *reinterpret_cast<uint4*>(&s.W1f[c * FT * 8 + j * 8]) = *reinterpret_cast<const uint4*>(f);
     *reinterpret_cast<uint4*>(&s.B2[c * FT * 8 + j * 8]) = *reinterpret_cast<const uint4*>(u);
   }
   for (int i = tid; i < NW * NO; i += THREADS) reinterpret_cast<float*>(s.W3)[i] = __bfloat162float(w[WB_3 + i]);
@@ -441,10 +451,10 @@ __global__ void __launch_bounds__(THREADS, 2) mlp_forward_kernel(const __nv_bflo
   __syncthreads();
   tc_fence_after();
   const uint32_t d1 = s.tmem, d2 = d1 + NW, lanes = (uint32_t)(wp & 3) << 21;  // the warp's lanes, in bits 16..31
-  const uint32_t aX = smem_u32(s.X), aH = smem_u32(s.H), aW1 = smem_u32(s.W1), aB2 = smem_u32(s.B2), aOne = smem_u32(s.one), aW2 = smem_u32(s.W2);
+  const uint32_t aX = smem_u32(s.X), aH = smem_u32(s.H), aW1 = smem_u32(s.W1), aW1f = smem_u32(s.W1f), aB2 = smem_u32(s.B2), aOne = smem_u32(s.one), aW2 = smem_u32(s.W2);
   constexpr uint32_t XT = sizeof(s.X[0]), HT = sizeof(s.H[0]);
   auto layer1 = [&]() {
-    for (int t = 2; t >= 0; --t) tc_mma(d1, aX + t * XT, aW1, t != 2);
+    for (int t = 2; t >= 0; --t) tc_mma(d1, aX + t * XT, t ? aW1f : aW1, t != 2);  // (a zero term times an infinity is NaN)
     tc_commit(&s.bar[0]);
   };
   if (tid == 0) layer1();

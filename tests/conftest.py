@@ -11,3 +11,12 @@ if ROOT not in sys.path:
 def pytest_configure(config):
     config.addinivalue_line("markers", "gpu: needs a CUDA GPU (GB300, sm_103a)")
     config.addinivalue_line("markers", "slow: takes more than a few seconds on CPU")
+
+
+@pytest.fixture(scope="session")
+def vms():
+    """The binding, with the library built and loaded."""
+    from paper_0809_4802_gb300 import build, vms as v
+    build.build()
+    v.load_library()
+    return v
