@@ -409,9 +409,10 @@ __global__ void sweep_pack_kernel(const int32_t* __restrict__ rowptr, const int3
 // chunk's far list) from the L2 publication as they appear, so that the L2 round trips run beside
 // the rows instead of inside them. The last warp streams the row records and right-hand sides into
 // a ring per compute warp with bulk copies. Chunks are claimed in order by running CTAs, so every
-// wait is for work that is already in progress.
+// wait is for work that is already in progress. The blocks per SM of the launch bounds are what leaves every variant
+// its registers without spills (56 to 168 a thread); left to itself the compiler spilled up to 68 bytes in the row loop.
 template <typename T, bool LOWER, int NP, int W, int FW>
-__global__ void __launch_bounds__((W + FW + 1) * 32)
+__global__ void __launch_bounds__((W + FW + 1) * 32, sizeof(T) == 4 ? (NP <= 3 ? 4 : 3) : 2)
     ilu_sweep_kernel(const unsigned char* __restrict__ rec, const int32_t* __restrict__ seg,
                      const int32_t* __restrict__ chunk, const int32_t* __restrict__ farptr,
                      const int32_t* __restrict__ far, int64_t c0, int64_t n_chunks, const T* __restrict__ v,
@@ -450,7 +451,12 @@ __global__ void __launch_bounds__((W + FW + 1) * 32)
     }
     __syncthreads();
     const int64_t c = s_chunk;
-    if (c < 0) return;
+    if (c < 0) {
+      // no copy may land after the block has ended: a warp that gave up has left some unread
+      if (warp == W + FW && lane < W)
+        for (unsigned n = copies < ST ? 0 : copies - ST; n < copies; ++n) mbar_wait(full(lane, n), (n / ST) & 1);
+      return;
+    }
     const int slo = chunk[c], shi = chunk[c + 1];  // its segments
     const int a = seg[slo];                        // its first node (slot 1)
     // rows r = 0 .. len - 1 of a segment in sweep order are the nodes first + r * dir
@@ -490,12 +496,7 @@ __global__ void __launch_bounds__((W + FW + 1) * 32)
           break;
         }
       }
-      if (stop) {
-        if (lane == 0) atomicCAS(err, 0, ILU_ERR_TIMEOUT);
-        // no copy may land after the block has ended
-        if (lane < W)
-          for (unsigned n = copies < ST ? 0 : copies - ST; n < copies; ++n) mbar_wait(full(lane, n), (n / ST) & 1);
-      }
+      if (stop && lane == 0) atomicCAS(err, 0, ILU_ERR_TIMEOUT);
     } else if (warp >= W) {
       // far neighbours: lane takes entries of the list in order, each until it is published
       const int b = seg[shi], fb = farptr[c], nf = farptr[c + 1] - fb;
@@ -642,9 +643,15 @@ __global__ void __launch_bounds__((W + FW + 1) * 32)
         }
         return true;
       };
+      // Whether the copy has landed: its producer may have stopped before starting it, which an error tells.
+      auto landed = [&](unsigned bar, unsigned parity) {
+        for (uint32_t it = 0; !mbar_try(bar, parity); ++it)
+          if (it >= lim || ((it & 15u) == 15u && *(volatile int*)err != 0)) return false;
+        return true;
+      };
       for (int r0 = 0; r0 < len && ok; r0 += RB) {
         const int n = len - r0 < RB ? len - r0 : RB;
-        if (!__all_sync(FULL, mbar_wait(full(warp, copies), (copies / ST) & 1))) {
+        if (!__all_sync(FULL, landed(full(warp, copies), (copies / ST) & 1))) {
           ok = false;
           break;
         }
