@@ -374,8 +374,15 @@ int vms_mlp_set_params(vms_mlp* mlp, const float* params);
 /* Read the parameters: stored != 0 gives the values the kernels use (BF16 weights as FP32),
  * stored == 0 the FP32 master copy the optimiser updates. */
 int vms_mlp_get_params(vms_mlp* mlp, float* params, int stored);
-/* Y (n x 4, device FP32) = network(X) for X (n x 12, device FP32), queued on the stream. */
+/* Y (n x 4, device FP32) = network(X) for X (n x 12, device FP32), queued on the stream. Its waits for the
+ * tensor cores are bounded (vms_mlp_set_wait_limit): a pass that gives up makes the rows it did not
+ * finish NaN, and the next call on the network after that which computes, synchronises or is given
+ * work (vms_mlp_forward, _grad, _adam, _get_params, _column_rms) returns VMS_ERR_TIMEOUT, once. */
 int vms_mlp_forward(vms_mlp* mlp, int64_t n, const float* X, float* Y);
+/* Limit of every device-side wait of vms_mlp_forward, in polls (the first a test, later ones up to
+ * about a microsecond each); 0 restores the default (2^20, about a second). Failure detection, as
+ * vms_set_wait_limit. Errors: VMS_ERR_INVALID_ARG (polls < 0 or > 2^30). */
+int vms_mlp_set_wait_limit(vms_mlp* mlp, int64_t polls);
 /* Gradient of the loss sum_r sum_c (y_rc - T_rc)^2 / (4 n) over n rows (rows: device int32
  * indices into X and T, or NULL for the first n rows); kept for vms_mlp_adam. *loss (host, may be
  * NULL) and grads (VMS_MLP_PARAMS, host or device, may be NULL) receive the loss and gradient

@@ -33,7 +33,9 @@ struct vms_mlp {
   __nv_bfloat16* w = nullptr;  // W1, W2, W3 in BF16 (offsets below)
   float* bias = nullptr;       // b1, b2, b3 in FP32
   double* loss = nullptr;      // device loss accumulator, behind grad
-  float* host = nullptr;       // page-locked: gradient and loss on their way to the caller
+  float* host = nullptr;       // page-locked: gradient and loss on their way to the caller, the status word
+  int* status = nullptr;       // behind them: 1 once a forward pass has given up (until it is reported)
+  uint32_t wait_limit = 0;     // polls of one wait of the forward pass; 0: the default
   float* scratch = nullptr;    // P_N floats (parameter read-back)
   double* colsum = nullptr;    // 16 column sums of squares (vms_mlp_column_rms)
   int t = 0;                   // Adam steps taken
@@ -52,6 +54,7 @@ constexpr int P_W1 = 0, P_B1 = P_W1 + NI * NW, P_W2 = P_B1 + NW, P_B2 = P_W2 + N
 static_assert(P_N == VMS_MLP_PARAMS, "parameter count");
 constexpr size_t GRAD_BYTES = sizeof(float) * P_N + sizeof(double);  // the gradient, then the loss
 static_assert(P_N % 2 == 0, "the loss behind the gradient");
+constexpr size_t HOST_BYTES = GRAD_BYTES + sizeof(int);
 // BF16 weight array: W1 | W2 | W3; FP32 bias array: b1 | b2 | b3
 constexpr int WB_1 = 0, WB_2 = NI * NW, WB_3 = WB_2 + NW * NW, WB_N = WB_3 + NW * NO;
 constexpr int BB_1 = 0, BB_2 = NW, BB_3 = 2 * NW, BB_N = 2 * NW + NO;
@@ -238,7 +241,7 @@ struct SmemFwd {
   float4 part[FT];                            // output sums of columns 64..127
   float b3[NO];
   uint32_t tmem;
-  unsigned long long bar[3];                  // D1; first half of D2 (operand buffers free); D2
+  unsigned long long bar[4];                  // D1; first half of D2 (operand buffers free); D2; all, after giving up
 };
 static_assert(sizeof(SmemFwd) + 1024 <= (228 << 10) / 2, "two CTAs per SM");
 
@@ -262,24 +265,20 @@ __device__ __forceinline__ void tc_commit(unsigned long long* bar) {
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_shared() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
-// Wait for the barrier's phase of this parity; false if it does not come within a second.
-__device__ __forceinline__ bool bar_wait(unsigned long long* bar, uint32_t parity) {
+// Wait of a whole warp for the barrier's phase of this parity; false for all its lanes if it has not come after `lim`
+// polls: a test, then waits of up to a microsecond each (counted, not timed: a process that is switched out has not
+// waited).
+constexpr uint32_t WAIT_DEFAULT = 1u << 20;
+__device__ __forceinline__ bool bar_wait(unsigned long long* bar, uint32_t parity, uint32_t lim) {
   const uint32_t a = smem_u32(bar);
-  unsigned long long t0 = 0;
-  for (int it = 0; it < 4000000; ++it) {
-    uint32_t done;
+  uint32_t done;
+  asm volatile("{\n\t.reg .pred p;\n\tmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+               : "=r"(done) : "r"(a), "r"(parity) : "memory");
+  for (uint32_t it = 1; !done && it < lim; ++it)
     asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\tselp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(done)
-        : "r"(a), "r"(parity)
-        : "memory");
-    if (done) return true;
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-    if (it == 0) t0 = t;
-    if (t - t0 > 1000000000ull) break;
-  }
-  return false;
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n\tselp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(done) : "r"(a), "r"(parity), "r"(1000u) : "memory");
+  return __all_sync(0xffffffffu, done);
 }
 // 32 columns of the warp's 32 lanes of tensor memory; the values may be used when it returns.
 __device__ __forceinline__ void tc_load32(uint32_t addr, float v[32]) {
@@ -396,7 +395,7 @@ __device__ __forceinline__ void store_x(SmemFwd& s, int row, int half, const flo
 __global__ void __launch_bounds__(THREADS, 2) mlp_forward_kernel(const __nv_bfloat16* __restrict__ w,
                                                                  const float* __restrict__ bias,
                                                                  const float* __restrict__ X, int64_t n,
-                                                                 float* __restrict__ Y) {
+                                                                 float* __restrict__ Y, uint32_t lim, int* status) {
   extern __shared__ __align__(128) unsigned char raw[];
   SmemFwd& s = *reinterpret_cast<SmemFwd*>(raw);
   const int tid = threadIdx.x, wp = tid >> 5, half = wp >> 2, row = (wp & 3) * 32 + (tid & 31);
@@ -438,7 +437,7 @@ __global__ void __launch_bounds__(THREADS, 2) mlp_forward_kernel(const __nv_bflo
   if (tid < NO) s.b3[tid] = bias[BB_3 + tid];
   store_x(s, row, half, x);
   if (tid == 0) {
-    for (int i = 0; i < 3; ++i)
+    for (int i = 0; i < 4; ++i)
       asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(smem_u32(&s.bar[i])) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -464,10 +463,10 @@ __global__ void __launch_bounds__(THREADS, 2) mlp_forward_kernel(const __nv_bflo
     const bool more = r0 + stride < n;
     if (more) load_x(X, r0 + stride + row, n, half, vec, x);
     // H1, columns 0..63 (the warp's 32), then their products
-    float v[32];
-    bool good = bar_wait(&s.bar[0], par);
+    float v[32] = {};
+    bool good = bar_wait(&s.bar[0], par, lim);
     tc_fence_after();
-    tc_load32(d1 + lanes + 32 * half, v);
+    if (good) tc_load32(d1 + lanes + 32 * half, v);
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
       float h[8];
@@ -496,12 +495,13 @@ __global__ void __launch_bounds__(THREADS, 2) mlp_forward_kernel(const __nv_bflo
       const float2 t = tanh2(make_float2(v[i], v[i + 1]));
       v[i] = t.x; v[i + 1] = t.y;
     }
-    good = bar_wait(&s.bar[1], par);
+    good = bar_wait(&s.bar[1], par, lim);
+    if (good)
 #pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      const int at = (4 * half + c) * FT * 8 + row * 8;
-      store_terms(&s.H[0][at], &s.H[1][at], &s.H[2][at], v + 8 * c);
-    }
+      for (int c = 0; c < 4; ++c) {
+        const int at = (4 * half + c) * FT * 8 + row * 8;
+        store_terms(&s.H[0][at], &s.H[1][at], &s.H[2][at], v + 8 * c);
+      }
     if (more) store_x(s, row, half, x);
     fence_async_shared();
     tc_fence_before();
@@ -514,11 +514,11 @@ __global__ void __launch_bounds__(THREADS, 2) mlp_forward_kernel(const __nv_bflo
       if (more) layer1();
     }
     // H2 and the output layer, columns 64 half ..
-    good = bar_wait(&s.bar[2], par);
+    good = bar_wait(&s.bar[2], par, lim);
     tc_fence_after();
     float2 ya = make_float2(0.f, 0.f), yb = ya;
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
+    for (int q = 0; q < 2 && good; ++q) {
       tc_load32(d2 + lanes + 64 * half + 32 * q, v);
 #pragma unroll
       for (int i = 0; i < 32; i += 2) {
@@ -546,10 +546,15 @@ __global__ void __launch_bounds__(THREADS, 2) mlp_forward_kernel(const __nv_bflo
     }
   }
   if (!ok) {
-    // a product did not finish in time: wait for what is in flight (with a limit) and say so in the result
-    for (int i = 0; i < 3; ++i) {
-      bar_wait(&s.bar[i], par);
+    // a product did not finish in time. Wait for all that are in flight (the next tile's first layer may be), which
+    // write tensor memory and read shared memory; then say so in the rows and in the handle's status.
+    if (tid == 0) {
+      tc_commit(&s.bar[3]);
+      *reinterpret_cast<volatile int*>(status) = 1;
+      __threadfence_system();
     }
+    __syncwarp();
+    bar_wait(&s.bar[3], 0, WAIT_DEFAULT);
     for (; r0 < n; r0 += stride)
       for (int i = tid; i < FT * NO; i += THREADS)
         if (r0 + i / NO < n) Y[r0 * NO + i] = NAN;
@@ -794,6 +799,18 @@ int mfail(vms_mlp* p, int code, const char* msg) {
                    cudaGetErrorString(e_));                                   \
   } while (0)
 
+// Reports, once, a forward pass that has given up by now.
+int mlp_status(vms_mlp* mlp) {
+  volatile int* s = mlp->status;
+  if (*s == 0) return VMS_OK;
+  *s = 0;
+  return mfail(mlp, VMS_ERR_TIMEOUT, "a forward pass waited longer than its limit: rows of its result are NaN");
+}
+#define MSTATUS()                            \
+  do {                                       \
+    if (int s_ = mlp_status(mlp)) return s_; \
+  } while (0)
+
 // ---------------------------------------------------------------------------------------------
 // node features and increments on a context's state
 // ---------------------------------------------------------------------------------------------
@@ -909,7 +926,11 @@ int vms_mlp_create(vms_mlp** out, int device) {
   if (e == cudaSuccess) e = cudaMalloc(&mlp->m, sizeof(float) * P_N);
   if (e == cudaSuccess) e = cudaMalloc(&mlp->v, sizeof(float) * P_N);
   if (e == cudaSuccess) e = cudaMalloc(&mlp->grad, GRAD_BYTES);
-  if (e == cudaSuccess) e = cudaMallocHost(&mlp->host, GRAD_BYTES);
+  if (e == cudaSuccess) e = cudaMallocHost(&mlp->host, HOST_BYTES);
+  if (e == cudaSuccess) {
+    mlp->status = reinterpret_cast<int*>(reinterpret_cast<char*>(mlp->host) + GRAD_BYTES);
+    *mlp->status = 0;
+  }
   if (e == cudaSuccess) e = cudaMalloc(&mlp->w, sizeof(__nv_bfloat16) * WB_N);
   if (e == cudaSuccess) e = cudaMalloc(&mlp->bias, sizeof(float) * BB_N);
   mlp->loss = reinterpret_cast<double*>(mlp->grad + P_N);
@@ -975,16 +996,24 @@ int vms_mlp_get_params(vms_mlp* mlp, float* params, int stored) {
     MCK(cudaMemcpyAsync(params, mlp->master, sizeof(float) * P_N, cudaMemcpyDefault, mlp->stream));
   }
   MCK(cudaStreamSynchronize(mlp->stream));
+  MSTATUS();
+  return VMS_OK;
+}
+
+int vms_mlp_set_wait_limit(vms_mlp* mlp, int64_t polls) {
+  if (!mlp || polls < 0 || polls > ((int64_t)1 << 30)) return mfail(mlp, VMS_ERR_INVALID_ARG, "wait limit out of range");
+  mlp->wait_limit = (uint32_t)polls;
   return VMS_OK;
 }
 
 int vms_mlp_forward(vms_mlp* mlp, int64_t n, const float* X, float* Y) {
   if (!mlp || n < 0 || (n > 0 && (!X || !Y))) return mfail(mlp, VMS_ERR_INVALID_ARG, "invalid arguments");
+  MSTATUS();
   if (n == 0) return VMS_OK;
   MCK(cudaSetDevice(mlp->device));
   const int64_t tiles = (n + FT - 1) / FT, most = 2 * (int64_t)vms::sm_count();
   mlp_forward_kernel<<<(unsigned)(tiles < most ? tiles : most), THREADS, sizeof(SmemFwd), mlp->stream>>>(
-      mlp->w, mlp->bias, X, n, Y);
+      mlp->w, mlp->bias, X, n, Y, mlp->wait_limit ? mlp->wait_limit : WAIT_DEFAULT, mlp->status);
   MCK(cudaGetLastError());
   return VMS_OK;
 }
@@ -992,6 +1021,7 @@ int vms_mlp_forward(vms_mlp* mlp, int64_t n, const float* X, float* Y) {
 int vms_mlp_grad(vms_mlp* mlp, int64_t n, const int32_t* rows, const float* X, const float* T,
                  double* loss, float* grads) {
   if (!mlp || n <= 0 || !X || !T) return mfail(mlp, VMS_ERR_INVALID_ARG, "invalid arguments");
+  MSTATUS();
   MCK(cudaSetDevice(mlp->device));
   MCK(cudaMemsetAsync(mlp->grad, 0, GRAD_BYTES, mlp->stream));
   const float scale = (float)(1.0 / (4.0 * (double)n));
@@ -1019,11 +1049,13 @@ int vms_mlp_grad(vms_mlp* mlp, int64_t n, const int32_t* rows, const float* X, c
   MCK(cudaStreamSynchronize(mlp->stream));
   if (host) std::memcpy(grads, mlp->host, sizeof(float) * P_N);
   if (loss) *loss = *hl;
+  MSTATUS();
   return VMS_OK;
 }
 
 int vms_mlp_adam(vms_mlp* mlp, float lr) {
   if (!mlp || !(lr > 0.f)) return mfail(mlp, VMS_ERR_INVALID_ARG, "invalid arguments");
+  MSTATUS();
   MCK(cudaSetDevice(mlp->device));
   mlp->t += 1;
   const double b1 = 0.9, b2 = 0.999;
@@ -1048,6 +1080,7 @@ int vms_mlp_column_rms(vms_mlp* mlp, int64_t n, int cols, const float* X, double
   MCK(cudaMemcpyAsync(h, mlp->colsum, sizeof(double) * cols, cudaMemcpyDeviceToHost, mlp->stream));
   MCK(cudaStreamSynchronize(mlp->stream));
   for (int c = 0; c < cols; ++c) rms[c] = std::sqrt(h[c] / (double)n);
+  MSTATUS();
   return VMS_OK;
 }
 

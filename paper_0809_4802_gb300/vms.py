@@ -52,7 +52,7 @@ EXPORTS = [
     "vms_set_tuning", "vms_get_tuning", "vms_autotune",
     "vms_mlp_create", "vms_mlp_destroy", "vms_mlp_last_error", "vms_mlp_set_stream",
     "vms_mlp_set_params", "vms_mlp_get_params", "vms_mlp_forward", "vms_mlp_grad", "vms_mlp_adam",
-    "vms_mlp_column_rms", "vms_mlp_scale_columns",
+    "vms_mlp_column_rms", "vms_mlp_scale_columns", "vms_mlp_set_wait_limit",
     "vms_node_features", "vms_node_increment", "vms_apply_increment", "vms_shift_time",
     "vms_newton_solve_to", "vms_state_download_prev", "vms_mesh_upload_tet", "vms_tet_rule",
     "vms_set_wait_limit", "vms_csr_download", "vms_fma_throughput", "vms_csr_download_async",
@@ -136,6 +136,7 @@ def load_library(path: str = LIB_PATH):
         "vms_mlp_destroy": (c_int, [p]),
         "vms_mlp_last_error": (c_char_p, [p]),
         "vms_mlp_set_stream": (c_int, [p, p]),
+        "vms_mlp_set_wait_limit": (c_int, [p, c_int64]),
         "vms_mlp_set_params": (c_int, [p, p]),
         "vms_mlp_get_params": (c_int, [p, p, c_int]),
         "vms_mlp_forward": (c_int, [p, c_int64, p, p]),
@@ -469,6 +470,11 @@ class Mlp:
 
     def set_stream(self, stream_handle: int):
         self._check(self.lib.vms_mlp_set_stream(self.h, c_void_p(stream_handle)))
+
+    def set_wait_limit(self, polls: int):
+        """Polls of one device-side wait of forward() before it gives up (NaN rows, VMS_ERR_TIMEOUT
+        from a later call); 0 restores the default."""
+        self._check(self.lib.vms_mlp_set_wait_limit(self.h, int(polls)))
 
     def set_params(self, params):
         a = np.ascontiguousarray(params, dtype=np.float32)
