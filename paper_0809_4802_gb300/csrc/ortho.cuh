@@ -19,7 +19,6 @@ namespace vms {
 constexpr int OG_THREADS = 512, OG_WARPS = OG_THREADS / 32;
 constexpr int OG_K = 8;                  // vectors a warp takes at a time
 constexpr int OG_MAX = 480;              // most basis vectors (MAX_RESTART)
-constexpr uint32_t OG_WAIT = 1u << 22;   // polls of one wait before the kernel gives up
 constexpr int OG_BLOCKS = 256;           // most blocks
 constexpr unsigned long long OG_UNSET = ~0ull;
 // Exchange words of one launch (doubles): the blocks' shares of the dot products of the two passes
@@ -28,9 +27,10 @@ constexpr int64_t OG_P = 0, OG_N = 2 * (int64_t)OG_MAX * OG_BLOCKS, OG_H = OG_N 
                   OG_SET = OG_H + 2 * OG_MAX;
 
 // Words are exchanged between blocks by their values: a buffer holds an all-ones pattern (a NaN that
-// arithmetic never produces) until a word is written, once, and its readers poll the word itself.
-// Two buffers take turns; each launch sets the other one's used words back for the next.
+// arithmetic never produces but from an operand that is one) until a word is written, once, and its readers
+// poll the word itself. Two buffers take turns; each launch sets the other one's used words back for the next.
 __device__ __forceinline__ void og_put(double* p, double v) {
+  if (__double_as_longlong(v) == (long long)OG_UNSET) v = __longlong_as_double(0x7ff8000000000000ll);  // another NaN
   asm volatile("st.relaxed.gpu.global.f64 [%0], %1;" ::"l"(p), "d"(v) : "memory");
 }
 __device__ __forceinline__ unsigned long long og_peek(const double* p) {
@@ -38,11 +38,12 @@ __device__ __forceinline__ unsigned long long og_peek(const double* p) {
   asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
 }
-// The word at p once it is written; clears `ok` when it does not come within OG_WAIT polls.
-__device__ __forceinline__ double og_get(const double* p, bool& ok) {
+// The word at p once it is written; clears `ok` when it does not come within `lim` polls, or at once where
+// an earlier wait of the thread has.
+__device__ __forceinline__ double og_get(const double* p, uint32_t lim, bool& ok) {
   unsigned long long v = og_peek(p);
   for (uint32_t it = 0; v == OG_UNSET; ++it) {
-    if (it >= OG_WAIT) {
+    if (it >= lim || !ok) {
       ok = false;
       return 0.0;
     }
@@ -114,10 +115,10 @@ __device__ __forceinline__ double og_rsqrt(double d) {
 // launch's exchange words, Y: those of the launch before, which had kprev vectors and gprev blocks.
 // out (host or device, kk + 2 doubles) receives the coefficients V_k . w of both passes added, the
 // squared norm of what is left of w before it is scaled to unit length (to zero if that norm is zero
-// or not a number), and the status: left alone, or 1 when a wait gave up.
+// or not a number), and the status: left alone, or 1 when a wait gave up after `lim` polls.
 template <typename VT>
 __global__ void __launch_bounds__(OG_THREADS, 1)
-    ortho_kernel(VT* V, int64_t n, int kk, double* X, double* Y, int kprev, int gprev, double* out) {
+    ortho_kernel(VT* V, int64_t n, int kk, double* X, double* Y, int kprev, int gprev, uint32_t lim, double* out) {
   using Q = OgQuad<VT>;
   using V4 = typename Q::V4;
   __shared__ double sh[512];       // warps' sums (parts x vectors)
@@ -201,12 +202,12 @@ __global__ void __launch_bounds__(OG_THREADS, 1)
     // vector k is summed over the blocks by block k mod G, its sum taken by all
     for (int k = c + G * warp; k < kk; k += G * OG_WARPS) {
       double s = 0.0;
-      for (int b = lane; b < G; b += 32) s += og_get(P + (int64_t)k * G + b, ok);
+      for (int b = lane; b < G; b += 32) s += og_get(P + (int64_t)k * G + b, lim, ok);
       for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
       if (lane == 0) og_put(H + k, s);
     }
     for (int k = tid; k < kk; k += OG_THREADS) {
-      const double x = og_get(H + k, ok);
+      const double x = og_get(H + k, lim, ok);
       hs[pass][k] = x;
       cs[k] = (VT)-x;
     }
@@ -262,7 +263,7 @@ __global__ void __launch_bounds__(OG_THREADS, 1)
   }
   if (warp == 0) {  // every block forms the same norm
     double s = 0.0;
-    for (int b = lane; b < G; b += 32) s += og_get(X + OG_N + b, ok);
+    for (int b = lane; b < G; b += 32) s += og_get(X + OG_N + b, lim, ok);
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     if (lane == 0) {
       s_norm = s;

@@ -520,8 +520,9 @@ struct Gmres {
     int64_t nn = n;
     int blocks = (int)std::min<int64_t>({(n / 4 + 127) / 128, (int64_t)sm_count(), (int64_t)OG_BLOCKS});
     double *X = w.og + (w.og_turn ? OG_SET : 0), *Y = w.og + (w.og_turn ? 0 : OG_SET), *out = w.hcol;
+    uint32_t lim = w.use_ilu ? w.ilu.spin_limit : ILU_SPIN_DEFAULT;
     out[kk + 1] = 0.0;
-    void* args[] = {&V, &nn, &kk, &X, &Y, &w.og_k, &w.og_blocks, &out};
+    void* args[] = {&V, &nn, &kk, &X, &Y, &w.og_k, &w.og_blocks, &lim, &out};
     const cudaError_t e = cudaLaunchCooperativeKernel((const void*)ortho_kernel<VT>, dim3((unsigned)blocks),
                                                       dim3(OG_THREADS), args, 0, st);
     if (e != cudaSuccess) return ctx_fail(ctx, VMS_ERR_CUDA, cudaGetErrorString(e));
@@ -843,12 +844,17 @@ static int linear_solve(vms_ctx* ctx, const SysRange& R, double rtol, int maxit,
     *rel_out = 0.0;
     return VMS_OK;
   }
+  // Where the preconditioner's kernels have recorded an error, that is the solve's, whatever else came of it; asking
+  // also sets their claims, flags and publications back, so that no later solve meets them.
+  auto report = [&](int rc) {
+    if (w.use_ilu)
+      if (int rc2 = ilu_status(ctx, w.ilu, st)) return rc2;
+    return rc;
+  };
   if (!f32) {
     int it = 0;
     double rel = 0.0;
-    if (int rc = G.solve<double, double>(wk.values, w.r, w.x, bnorm, rtol, maxit, restart, &it, &rel)) return rc;
-    if (w.use_ilu)
-      if (int rc = ilu_status(ctx, w.ilu, st)) return rc;
+    if (int rc = report(G.solve<double, double>(wk.values, w.r, w.x, bnorm, rtol, maxit, restart, &it, &rel))) return rc;
     *iters_out = it;
     *rel_out = rel;
     return rel <= rtol ? VMS_OK : ctx_fail(ctx, VMS_ERR_KRYLOV_MAXIT, "GMRES reached maxit");
@@ -933,8 +939,8 @@ static int linear_solve(vms_ctx* ctx, const SysRange& R, double rtol, int maxit,
       w.Zf = nullptr;
       const cudaError_t e = cudaMalloc(&w.Zf, sizeof(double) * (size_t)w.n * restart);
       if (e != cudaSuccess)
-        return ctx_fail(ctx, e == cudaErrorMemoryAllocation ? VMS_ERR_OUT_OF_MEMORY : VMS_ERR_CUDA,
-                        cudaGetErrorString(e));
+        return report(ctx_fail(ctx, e == cudaErrorMemoryAllocation ? VMS_ERR_OUT_OF_MEMORY : VMS_ERR_CUDA,
+                               cudaGetErrorString(e)));
       w.zf_restart = restart;
     }
     G.Zflex = w.Zf;
@@ -963,9 +969,7 @@ static int linear_solve(vms_ctx* ctx, const SysRange& R, double rtol, int maxit,
       rel = std::sqrt(r2) / bnorm;
     }
   }
-  if (rc) return rc;
-  if (w.use_ilu)
-    if (int rc2 = ilu_status(ctx, w.ilu, st)) return rc2;
+  if ((rc = report(rc))) return rc;
   *iters_out = total;
   *rel_out = rel;
   return rel <= rtol ? VMS_OK : ctx_fail(ctx, VMS_ERR_KRYLOV_MAXIT, "refined GMRES reached maxit");
