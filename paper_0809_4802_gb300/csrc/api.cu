@@ -102,6 +102,7 @@ namespace {
 
 int fail(vms_ctx* c, int code, const std::string& msg) {
   if (c) c->err = msg;
+  if (code == VMS_ERR_OUT_OF_MEMORY) cudaGetLastError();  // not sticky: clear it for the next launch's check
   return code;
 }
 

@@ -952,9 +952,13 @@ int ilu_factor(vms_ctx* ctx, Ilu& p, const Mesh& m, bool fp32, const void* value
                int* launches) {
   *launches = 0;
   if (p.dpos && p.n_nodes != m.n_nodes) free_ilu(p);
-  if (!p.dpos)
-    if (int rc = build_pattern(ctx, p, m)) return rc;
-  if (int rc = ensure_work(ctx, p, m, fp32)) return rc;
+  // a part that was allocated would be taken for the whole by the next call: none is kept
+  int rc = p.dpos ? VMS_OK : build_pattern(ctx, p, m);
+  if (rc == VMS_OK) rc = ensure_work(ctx, p, m, fp32);
+  if (rc != VMS_OK) {
+    free_ilu(p);
+    return rc;
+  }
   // The elimination always runs in FP64 (from the FP32 values in mixed precision): FP32
   // elimination of the condensed systems of distorted meshes, whose condition numbers reach
   // 1e9-1e10, gives factors too poor for GMRES to converge. Mixed precision then rounds the
