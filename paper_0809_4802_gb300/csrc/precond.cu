@@ -869,12 +869,6 @@ int ensure_work(vms_ctx* ctx, Ilu& p, const Mesh& m, bool fp32) {
   if (!p.F) {
     e = cudaMalloc(&p.F, sizeof(double) * m.nnz);
     if (e == cudaSuccess) e = cudaMalloc(&p.Dinv, sizeof(double) * 16 * m.n_nodes);
-    for (double** b : {&p.y, &p.yp64, &p.xp64})
-      if (e == cudaSuccess) e = cudaMalloc(b, sizeof(double) * 4 * m.n_nodes);
-    for (int side = 0; side < 2; ++side)
-      if (e == cudaSuccess) e = cudaMalloc(&p.rec[side], rec_bytes<double>(p, side));
-    for (double* b : {p.yp64, p.xp64})
-      if (e == cudaSuccess) e = cudaMemset(b, 0xff, sizeof(double) * 4 * m.n_nodes);
   }
   if (e == cudaSuccess && fp32 && !p.vals64) {
     e = cudaMalloc(&p.vals64, sizeof(double) * m.nnz);
@@ -946,6 +940,27 @@ void free_ilu(Ilu& p) {
     if (b) cudaFree(b);
   p = Ilu();
   p.spin_limit = lim;
+}
+
+int ilu_sweeps64(vms_ctx* ctx, Ilu& p, const Mesh& m) {
+  if (p.rec[1]) return VMS_OK;
+  cudaError_t e = cudaSuccess;
+  for (double** b : {&p.y, &p.yp64, &p.xp64})
+    if (e == cudaSuccess) e = cudaMalloc(b, sizeof(double) * 4 * m.n_nodes);
+  for (double* b : {p.yp64, p.xp64})
+    if (e == cudaSuccess) e = cudaMemset(b, 0xff, sizeof(double) * 4 * m.n_nodes);
+  for (int side = 0; side < 2; ++side)
+    if (e == cudaSuccess) e = cudaMalloc(&p.rec[side], rec_bytes<double>(p, side));
+  if (e == cudaSuccess) return VMS_OK;
+  for (double** b : {&p.y, &p.yp64, &p.xp64}) {
+    cudaFree(*b);
+    *b = nullptr;
+  }
+  for (unsigned char*& r : p.rec) {
+    cudaFree(r);
+    r = nullptr;
+  }
+  return ctx_fail(ctx, e == cudaErrorMemoryAllocation ? VMS_ERR_OUT_OF_MEMORY : VMS_ERR_CUDA, cudaGetErrorString(e));
 }
 
 int ilu_factor(vms_ctx* ctx, Ilu& p, const Mesh& m, bool fp32, const void* values, cudaStream_t st,
@@ -1053,8 +1068,8 @@ int ilu_status(vms_ctx* ctx, Ilu& p, cudaStream_t st) {
   cudaMemsetAsync(p.flags, 0, sizeof(uint32_t) * p.n_nodes, st);
   if (p.yp32) cudaMemsetAsync(p.yp32, 0xff, sizeof(float) * 4 * p.n_nodes, st);
   if (p.xp32) cudaMemsetAsync(p.xp32, 0xff, sizeof(float) * 4 * p.n_nodes, st);
-  cudaMemsetAsync(p.yp64, 0xff, sizeof(double) * 4 * p.n_nodes, st);
-  cudaMemsetAsync(p.xp64, 0xff, sizeof(double) * 4 * p.n_nodes, st);
+  if (p.yp64) cudaMemsetAsync(p.yp64, 0xff, sizeof(double) * 4 * p.n_nodes, st);
+  if (p.xp64) cudaMemsetAsync(p.xp64, 0xff, sizeof(double) * 4 * p.n_nodes, st);
   cudaStreamSynchronize(st);
   p.base = 0;
   p.epoch = 0;

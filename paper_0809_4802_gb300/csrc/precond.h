@@ -46,11 +46,11 @@ struct Ilu {
   double* F = nullptr;         // nnz: L (unit lower, strictly lower blocks) and U, CSR layout
   double* Dinv = nullptr;      // n_nodes * 16: inverses of the diagonal blocks of U
   // the factor as the sweeps read it, one record per row (forward, backward)
-  unsigned char* rec[2] = {nullptr, nullptr};    // FP64 (made on the first FP64 sweep)
+  unsigned char* rec[2] = {nullptr, nullptr};    // FP64 (ilu_sweeps64; filled on the first FP64 sweep)
   unsigned char* rec32[2] = {nullptr, nullptr};  // rounded to FP32 (mixed precision)
   bool packed64 = false;       // rec holds the current factor
   double* vals64 = nullptr;    // mixed precision: FP64 copy of the FP32 matrix values
-  double* y = nullptr;         // 4 n_nodes: L^-1 v (FP64 sweeps; compact over the rows solved)
+  double* y = nullptr;         // 4 n_nodes: L^-1 v (FP64 sweeps, as yp64 and xp64; compact over the rows solved)
   float* y32 = nullptr;        // 4 n_nodes: L^-1 v (FP32 sweeps)
   double* yp64 = nullptr;      // 4 n_nodes: FP64 forward-sweep publication, all ones between sweeps
   double* xp64 = nullptr;      // 4 n_nodes: FP64 backward-sweep publication, all ones between sweeps
@@ -74,7 +74,11 @@ void free_ilu(Ilu& p);
 int ilu_factor(vms_ctx* ctx, Ilu& p, const Mesh& m, bool fp32, const void* values, cudaStream_t st,
                int* launches);
 
-// z = (LU)^-1 v. T is the element type of the factor, VT the vector type. Returns the launches.
+// Allocate what the FP64 sweeps need beside the factor, on first use: their records take 2 (8 NP (16 x 8 + 4)) bytes
+// a node (4.2 KB on hexahedra), which a mixed solve whose FP32 refinement gets there never reads.
+int ilu_sweeps64(vms_ctx* ctx, Ilu& p, const Mesh& m);
+
+// z = (LU)^-1 v (FP64: after ilu_sweeps64). T is the element type of the factor, VT the vector type. Returns the launches.
 // Rows of nodes [n0, n1) only (a block of the matrix with no couplings outside it); v and z are
 // compact: entry 4 (i - n0) + c belongs to node i.
 template <typename T, typename VT>

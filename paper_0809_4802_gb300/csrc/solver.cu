@@ -854,6 +854,8 @@ static int linear_solve(vms_ctx* ctx, const SysRange& R, double rtol, int maxit,
   if (!f32) {
     int it = 0;
     double rel = 0.0;
+    if (w.use_ilu)
+      if (int rc = ilu_sweeps64(ctx, w.ilu, m)) return report(rc);
     if (int rc = report(G.solve<double, double>(wk.values, w.r, w.x, bnorm, rtol, maxit, restart, &it, &rel))) return rc;
     *iters_out = it;
     *rel_out = rel;
@@ -943,6 +945,8 @@ static int linear_solve(vms_ctx* ctx, const SysRange& R, double rtol, int maxit,
                                cudaGetErrorString(e)));
       w.zf_restart = restart;
     }
+    if (w.use_ilu)
+      if (int rc2 = ilu_sweeps64(ctx, w.ilu, m)) return report(rc2);
     G.Zflex = w.Zf;
     rc = G.solve<float, double>(wk.values, rfull, w.cx, std::sqrt(r2), rtol / rel, maxit - total,
                                 restart, &it, &irel);
