@@ -332,17 +332,22 @@ __device__ __forceinline__ bool mbar_wait(unsigned bar, unsigned parity) {
 // block products in either sweep (the forward one adds its right-hand side). Places without a
 // block hold zeros and point to slot 0, which holds zeros.
 template <typename T, int NP> constexpr int sweep_rec_bytes() { return 8 * NP * (16 * (int)sizeof(T) + 4); }
-// rows of a bulk copy (8: 190 us instead of 213 on 49^3 nodes, but 331 instead of 237 on lines of 151
-// nodes, and fewer blocks fit an SM), and copies in flight per warp
-template <typename T, int NP> constexpr int sweep_rb() { return NP <= 2 ? 4 : 2; }
-constexpr int SWEEP_ST = 3;
+// Rows of a bulk copy and copies in flight per warp; one each where segments are SHORT (sweep_short). (8 rows: 190 us
+// instead of 213 on 49^3 nodes, but 331 instead of 237 on lines of 151 nodes, and fewer blocks fit an SM.)
+template <int NP, bool SHORT> constexpr int sweep_rb() { return SHORT ? 1 : (NP <= 2 ? 4 : 2); }
+template <bool SHORT> constexpr int sweep_st() { return SHORT ? 1 : 3; }
 // shared memory of a sweep: value slots (zeros, the chunk's rows, their far neighbours), the rings
 // of row records and right-hand sides, the barriers
-template <typename T, int NP>
-size_t sweep_smem_bytes(int warps, int slots) {
+template <typename T, int NP, bool SHORT>
+constexpr size_t sweep_smem_bytes(int warps, int slots) {
   return (size_t)slots * 4 * sizeof(T) +
-         (size_t)warps * SWEEP_ST * (sweep_rb<T, NP>() * (sweep_rec_bytes<T, NP>() + 4 * sizeof(T)) + 16);
+         (size_t)warps * sweep_st<SHORT>() * (sweep_rb<NP, SHORT>() * (sweep_rec_bytes<T, NP>() + 4 * sizeof(T)) + 16);
 }
+
+// a chunk of one segment may have any number of far neighbours: 64 rows of at most 31
+static_assert(sweep_smem_bytes<double, 5, false>(ILU_CHUNK, 1 + ILU_SEG_MAX * ILU_MAX_DEG) + 1024 <= (227 << 10) &&
+                  ILU_CHUNK * ILU_SEG_MAX + ILU_FAR_MAX < ILU_SEG_MAX * ILU_MAX_DEG,
+              "the largest chunk's shared memory");
 
 // The records of one sweep from the factor (CSR layout, FP64): one thread per 16-byte piece.
 template <typename T, bool LOWER, int NP>
@@ -411,14 +416,14 @@ __global__ void sweep_pack_kernel(const int32_t* __restrict__ rowptr, const int3
 // a ring per compute warp with bulk copies. Chunks are claimed in order by running CTAs, so every
 // wait is for work that is already in progress. The blocks per SM of the launch bounds are what leaves every variant
 // its registers without spills (56 to 168 a thread); left to itself the compiler spilled up to 68 bytes in the row loop.
-template <typename T, bool LOWER, int NP, int W, int FW>
-__global__ void __launch_bounds__((W + FW + 1) * 32, sizeof(T) == 4 ? (NP <= 3 ? 4 : 3) : 2)
+template <typename T, bool LOWER, int NP, int W, int FW, bool SHORT>
+__global__ void __launch_bounds__((W + FW + 1) * 32, sizeof(T) == 4 ? (SHORT ? 5 : NP <= 3 ? 4 : 3) : (SHORT ? 3 : 2))
     ilu_sweep_kernel(const unsigned char* __restrict__ rec, const int32_t* __restrict__ seg,
                      const int32_t* __restrict__ chunk, const int32_t* __restrict__ farptr,
                      const int32_t* __restrict__ far, int64_t c0, int64_t n_chunks, const T* __restrict__ v,
                      T* pub, uint4* __restrict__ clr, T* __restrict__ out, int n0, int n_rows, int slots,
                      unsigned long long* ticket, unsigned long long base, int* err, uint32_t lim) {
-  constexpr int ST = SWEEP_ST, RB = sweep_rb<T, NP>(), VB = 4 * (int)sizeof(T);  // VB: bytes of a node's values
+  constexpr int ST = sweep_st<SHORT>(), RB = sweep_rb<NP, SHORT>(), VB = 4 * (int)sizeof(T);  // VB: bytes of a node's values
   constexpr int RS = sweep_rec_bytes<T, NP>(), STAGE = RB * (RS + VB);
   constexpr int dir = LOWER ? 1 : -1;
   __shared__ int64_t s_chunk;
@@ -755,7 +760,7 @@ int build_pattern(vms_ctx* ctx, Ilu& p, const Mesh& m) {
       p.side_up = std::max(p.side_up, deg - 1 - dpos[i] - (i + 1 < seg[s + 1] ? 1 : 0));
     }
   // chunks of at most ILU_CHUNK segments, fewer where a chunk's distinct neighbours in other chunks
-  // on one side would exceed ILU_FAR_MAX (one segment alone never does: 64 rows of at most 31);
+  // on one side would exceed ILU_FAR_MAX (one segment alone is a chunk whatever their number);
   // every neighbour's place in its row's chunk: the chunk's own rows first, then the far list of
   // its side
   std::vector<int32_t> chunk(1, 0), at(adj.size(), 0), farptr[2], far[2], mark(N, -1), order(N);
@@ -855,13 +860,22 @@ int build_pattern(vms_ctx* ctx, Ilu& p, const Mesh& m) {
 // (backward sweep) the diagonal block
 int sweep_np(const Ilu& p, int side) {
   const int places = side ? p.side_up + 2 : p.side_lo + 1;
-  return places <= 8 ? 1 : (places <= 16 ? 2 : (places <= 24 ? 3 : 5));
+  return places <= 8 ? 1 : (places <= 16 ? 2 : (places <= 24 ? 3 : (places <= 32 ? 4 : 5)));
+}
+// f(std::integral_constant<int, NP>) for the sweep's number of passes
+template <class F>
+auto with_np(const Ilu& p, int side, const F& f) {
+  switch (sweep_np(p, side)) {
+    case 1: return f(std::integral_constant<int, 1>{});
+    case 2: return f(std::integral_constant<int, 2>{});
+    case 3: return f(std::integral_constant<int, 3>{});
+    case 4: return f(std::integral_constant<int, 4>{});
+    default: return f(std::integral_constant<int, 5>{});
+  }
 }
 template <typename T>
 size_t rec_bytes(const Ilu& p, int side) {
-  const int np = sweep_np(p, side);
-  return (size_t)p.n_nodes * (np == 1 ? sweep_rec_bytes<T, 1>() : np == 2 ? sweep_rec_bytes<T, 2>()
-                                    : np == 3 ? sweep_rec_bytes<T, 3>() : sweep_rec_bytes<T, 5>());
+  return with_np(p, side, [&](auto np) { return (size_t)p.n_nodes * sweep_rec_bytes<T, decltype(np)::value>(); });
 }
 
 int ensure_work(vms_ctx* ctx, Ilu& p, const Mesh& m, bool fp32) {
@@ -913,14 +927,10 @@ int convert(const A* x, B* y, int64_t n, cudaStream_t st) {
 // The row records of both sweeps from the factor.
 template <typename T, bool LOWER>
 void pack_side(const Ilu& p, const Mesh& m, unsigned char* rec, cudaStream_t st) {
-  auto go = [&](auto kern) {
-    kern<<<16 * (unsigned)sm_count(), 256, 0, st>>>(m.rowptr, p.dpos, p.inl, p.at, p.F, p.Dinv, m.n_nodes, rec);
-  };
-  const int np = sweep_np(p, LOWER ? 0 : 1);
-  if (np == 1) go(sweep_pack_kernel<T, LOWER, 1>);
-  else if (np == 2) go(sweep_pack_kernel<T, LOWER, 2>);
-  else if (np == 3) go(sweep_pack_kernel<T, LOWER, 3>);
-  else go(sweep_pack_kernel<T, LOWER, 5>);
+  with_np(p, LOWER ? 0 : 1, [&](auto np) {
+    sweep_pack_kernel<T, LOWER, decltype(np)::value>
+        <<<16 * (unsigned)sm_count(), 256, 0, st>>>(m.rowptr, p.dpos, p.inl, p.at, p.F, p.Dinv, m.n_nodes, rec);
+  });
 }
 template <typename T>
 int pack(const Ilu& p, const Mesh& m, unsigned char* const rec[2], cudaStream_t st) {
@@ -997,6 +1007,13 @@ int ilu_factor(vms_ctx* ctx, Ilu& p, const Mesh& m, bool fp32, const void* value
   return e == cudaSuccess ? VMS_OK : ctx_fail(ctx, VMS_ERR_CUDA, cudaGetErrorString(e));
 }
 
+// Rows without lines: one row a copy and one copy a warp, so that an SM holds more CTAs (FP32 5, FP64 3 instead of 3 and 1
+// on hexahedra); rings for the rows to come stay empty there. A GMRES step's two sweeps in us, with the rings and
+// without, random node order (one row a segment): 33^3 nodes FP32 180, 139, FP64 343, 272; 91^3 2,925, 1,958 and 6,357, 4,863;
+// 40^3 nodes of a tetrahedral mesh 191, 144 and 421, 265. With segments of 5 rows on average (13^3 nodes in reverse
+// Cuthill-McKee order) and more the rings win: a solve's sweeps 8.6 and 12.0 ms in FP32.
+static bool sweep_short(const Ilu& p) { return p.n_nodes < 2 * p.n_segs; }
+
 // One sweep over rows [n0, n1): the chunks that cover it (rows outside are clamped away in the kernel;
 // a block solve has no couplings outside its rows, so n0 and n1 are segment starts).
 template <typename T>
@@ -1007,17 +1024,17 @@ struct SweepArgs {
   T *pub, *clr;
   T* out;
 };
-template <typename T, bool LOWER, int NP>
+template <typename T, bool LOWER, int NP, bool SHORT>
 static void launch_sweep(Ilu& p, const SweepArgs<T>& s, cudaStream_t st) {
   const std::vector<int32_t>& cn = p.chunk_node;
   const int64_t c0 = std::max<int64_t>(0, (int64_t)(std::upper_bound(cn.begin(), cn.end() - 1, (int32_t)s.n0) - cn.begin()) - 1);
   const int64_t nc = (int64_t)(std::lower_bound(cn.begin(), cn.end() - 1, (int32_t)s.n1) - cn.begin()) - c0;
   constexpr int W = ILU_CHUNK, FW = 1;
   const int side = LOWER ? 0 : 1;
-  const size_t smem = sweep_smem_bytes<T, NP>(W, p.slots);
+  const size_t smem = sweep_smem_bytes<T, NP, SHORT>(W, p.slots);
   const int per_sm = (int)std::min<size_t>(48 / (W + FW + 1), (size_t)(227 << 10) / (smem + 2048));
   const unsigned ctas = resident_ctas(nc, 1, (unsigned)std::max(1, per_sm) * sm_count());
-  auto kern = ilu_sweep_kernel<T, LOWER, NP, W, FW>;
+  auto kern = ilu_sweep_kernel<T, LOWER, NP, W, FW, SHORT>;
   // more than the default 48 KB of dynamic shared memory (set for the current device)
   cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   kern<<<ctas, (W + FW + 1) * 32, smem, st>>>(s.rec, p.seg, p.chunk, p.farptr[side], p.far[side], c0, nc, s.v,
@@ -1027,11 +1044,11 @@ static void launch_sweep(Ilu& p, const SweepArgs<T>& s, cudaStream_t st) {
 }
 template <typename T, bool LOWER>
 static void sweep(Ilu& p, const SweepArgs<T>& s, cudaStream_t st) {
-  const int np = sweep_np(p, LOWER ? 0 : 1);
-  if (np == 1) launch_sweep<T, LOWER, 1>(p, s, st);
-  else if (np == 2) launch_sweep<T, LOWER, 2>(p, s, st);
-  else if (np == 3) launch_sweep<T, LOWER, 3>(p, s, st);
-  else launch_sweep<T, LOWER, 5>(p, s, st);
+  const bool short_segs = sweep_short(p);
+  with_np(p, LOWER ? 0 : 1, [&](auto np) {
+    if (short_segs) launch_sweep<T, LOWER, decltype(np)::value, true>(p, s, st);
+    else launch_sweep<T, LOWER, decltype(np)::value, false>(p, s, st);
+  });
 }
 
 template <>
