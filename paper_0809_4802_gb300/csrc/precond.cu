@@ -25,7 +25,7 @@ namespace vms {
 
 namespace {
 
-constexpr int ILU_FWARPS = 4;    // warps per row (and CTA) of the factorisation
+constexpr int FACTOR_CTAS = 6, FACTOR_WIDE_CTAS = 24;  // of the factorisation, per SM: four warps a row; one
 constexpr unsigned FULL = 0xffffffffu;
 
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t* p) {
@@ -54,27 +54,33 @@ __device__ __forceinline__ bool wait_ready(const uint32_t* f, uint32_t epoch, in
 // ---------------------------------------------------------------------------------------------
 // factorisation: one CTA per node row; the row is eliminated in shared memory
 //
-// What bounds it: the chain of rows (224 levels on a lattice of 33^3 nodes, about 160 rows wide), and in a
+// What bounds it where levels are narrow: the chain of rows (224 levels on a lattice of 33^3 nodes, about 160 rows wide), and in a
 // row the FP64 instructions of its block products, 64 cycles each on one warp: 34 for a lower block of 17
 // pairs, and up to three lower blocks were finished only one level before. So a row's pairs are shared
 // by four warps, one per FP64 unit, eight pairs a step; what is known beforehand (neighbours, row starts,
 // pairs) is read before the first wait; U_kk^-1 and the blocks of row k are read as soon as row k is
 // published, while the products of the block before are still under way; and a lower block costs one
 // barrier: every warp forms L_ik for itself, the row keeps A_ik. Rows are claimed by level: in natural order
-// the rows that can run lie planes apart, and 608 CTAs would hold half a plane (6.7 ms on 33^3 nodes). 33^3 nodes (jittered cavity) with one warp
-// per row 4.05 ms, now 1.7 (9^3 0.59, 0.30; 22^3 of a tetrahedral mesh 0.66, 0.43).
+// the rows that can run lie planes apart, and the resident CTAs would hold half a plane (6.7 ms on 33^3 nodes).
+// Where a level has more rows than the GPU has SMs (factor_wide), the rows in flight bound it instead: one warp
+// per row, so that an SM holds 24 rows, not 6. Measured in ms, one warp per row in natural order; four warps; one warp
+// now: lattices of 13^3 nodes (26 rows a level) 0.91, 0.46, 0.55; 25^3 (93) 1.96, 1.02, 1.19; 33^3 (160) 4.05, 1.66, 1.68;
+// 45^3 (296) 11.6, 3.3, 2.8; 91^3 (1,183) 120, 24.2, 14.7; 40^3 nodes of a tetrahedral mesh 3.99, 1.34, 0.99; in random
+// node order, whose levels are few, 25^3 0.45, 0.53, 0.40; 45^3 1.71, 3.06, 1.78; 91^3 15.9, 26.2, 14.8.
 // ---------------------------------------------------------------------------------------------
-template <typename T>
-__global__ void __launch_bounds__(ILU_FWARPS * 32)
+template <typename T, int FW>
+__global__ void __launch_bounds__(FW * 32, FW == 1 ? FACTOR_WIDE_CTAS : FACTOR_CTAS)
     ilu_factor_kernel(const int32_t* __restrict__ rowptr, const int32_t* __restrict__ colidx,
                       const T* __restrict__ A, T* F, T* Dinv, const int32_t* __restrict__ dpos,
                       const int32_t* __restrict__ lptr, const int32_t* __restrict__ pptr,
                       const uint16_t* __restrict__ pairs, const int32_t* __restrict__ order, int64_t n_nodes, uint32_t* flags,
                       uint32_t epoch, unsigned long long* ticket, unsigned long long base, int* err,
                       uint32_t lim) {
-  constexpr int PS = 2 * ILU_FWARPS, PMAX = (ILU_MAX_DEG + PS - 1) / PS;  // pairs a step; steps of a lower block
-  __shared__ T row[ILU_MAX_DEG * 16], lrow[ILU_MAX_DEG * 16];
-  __shared__ T lw[ILU_FWARPS][16];
+  constexpr int PS = 2 * FW, PMAX = FW == 1 ? 4 : (ILU_MAX_DEG + PS - 1) / PS;  // pairs a step; steps read ahead
+  __shared__ T row[ILU_MAX_DEG * 16];
+  // FW > 1: L_ik as each warp reads it and as the row is stored (other warps may still need A_ik); 1: in A_ik's place
+  __shared__ T lrows[FW == 1 ? 1 : ILU_MAX_DEG * 16], lw[FW][FW == 1 ? 1 : 16];
+  T* const lrow = FW == 1 ? row : lrows;
   __shared__ int32_t s_k[ILU_MAX_DEG], s_pp[ILU_MAX_DEG + 1], s_rk[ILU_MAX_DEG][4];
   __shared__ uint16_t s_pairs[ILU_MAX_DEG * ILU_MAX_DEG];
   __shared__ int64_t s_row;
@@ -95,9 +101,9 @@ __global__ void __launch_bounds__(ILU_FWARPS * 32)
     const int deg = (rowptr[4 * i + 1] - r0) >> 2, dp = dpos[i];
     const int32_t l0 = lptr[i], p0 = pptr[l0], np = pptr[l0 + dp] - p0;
     // row i into shared memory, block-major: row[16 kk + 4 q + c] = A(4i+q, 4 adj_kk + c)
-    for (int e = tid; e < deg * 16; e += ILU_FWARPS * 32)
+    for (int e = tid; e < deg * 16; e += FW * 32)
       row[e] = A[rowptr[4 * i + ((e >> 2) & 3)] + 4 * (e >> 4) + (e & 3)];
-    for (int kk = tid; kk <= dp; kk += ILU_FWARPS * 32) {
+    for (int kk = tid; kk <= dp; kk += FW * 32) {
       s_pp[kk] = pptr[l0 + kk] - p0;
       if (kk < dp) {
         const int32_t k = colidx[r0 + 4 * kk] >> 2;
@@ -105,7 +111,7 @@ __global__ void __launch_bounds__(ILU_FWARPS * 32)
         for (int m = 0; m < 4; ++m) s_rk[kk][m] = rowptr[4 * (int64_t)k + m];
       }
     }
-    for (int p = tid; p < np; p += ILU_FWARPS * 32) s_pairs[p] = pairs[p0 + p];
+    for (int p = tid; p < np; p += FW * 32) s_pairs[p] = pairs[p0 + p];
     __syncthreads();
     for (int kk = 0; kk < dp; ++kk) {
       const int64_t k = s_k[kk];
@@ -133,20 +139,30 @@ __global__ void __launch_bounds__(ILU_FWARPS * 32)
       // L_ik = A_ik U_kk^-1 (lane: entry (q, c), both halves alike)
       T l = T(0);
       for (int m = 0; m < 4; ++m) l += row[16 * kk + 4 * q + m] * d[m];
+      if (FW == 1) __syncwarp();
       if (half == 0) {
-        lw[warp][lane] = l;
+        if (FW > 1) lw[warp][lane] = l;
         if (warp == 0) lrow[16 * kk + lane] = l;
       }
       __syncwarp();
+      const T* L = FW == 1 ? row + 16 * kk : lw[warp];
       // A_ij -= L_ik U_kj (the products are subtracted one by one, so that each is a fused multiply-add)
 #pragma unroll
       for (int s = 0; s < PMAX; ++s)
         if (jj[s] >= 0) {
           T v = row[16 * jj[s] + 4 * q + c];
-          for (int m = 0; m < 4; ++m) v -= lw[warp][4 * q + m] * u[s][m];
+          for (int m = 0; m < 4; ++m) v -= L[4 * q + m] * u[s][m];
           row[16 * jj[s] + 4 * q + c] = v;
         }
-      __syncwarp();  // lw is read before the next block's is written
+      if constexpr (PS * PMAX < ILU_MAX_DEG)
+        for (int p = s_pp[kk] + PS * PMAX + 2 * warp + half; p < s_pp[kk + 1]; p += PS) {
+          const uint32_t pr = s_pairs[p];
+          const int j = pr & 255;
+          T v = row[16 * j + 4 * q + c];
+          for (int m = 0; m < 4; ++m) v -= L[4 * q + m] * __ldcg(F + s_rk[kk][m] + 4 * (int)(pr >> 8) + c);
+          row[16 * j + 4 * q + c] = v;
+        }
+      __syncwarp();  // L is read before the next block's is written
     }
     __syncthreads();
     if (warp == 0) {
@@ -176,12 +192,13 @@ __global__ void __launch_bounds__(ILU_FWARPS * 32)
       const bool good = isfinite(det) && hb2 > 0.0 && det * det > 1e-28 * hb2;
       if (!good && lane == 0) atomicCAS(err, 0, ILU_ERR_PIVOT);
       if (lane < 16) Dinv[16 * i + 4 * c + r] = good ? T(cf / det) : T(r == c ? 1.0 : 0.0);
-      __threadfence();
-    } else {
-      for (int e = tid - 32; e < deg * 16; e += (ILU_FWARPS - 1) * 32)
-        F[rowptr[4 * i + ((e >> 2) & 3)] + 4 * (e >> 4) + (e & 3)] = (e >> 4) < dp ? lrow[e] : row[e];
-      __threadfence();
     }
+    if (FW == 1 || warp > 0) {
+      constexpr int SW = FW == 1 ? 1 : FW - 1;  // warps that store
+      for (int e = tid - (FW - SW) * 32; e < deg * 16; e += SW * 32)
+        F[rowptr[4 * i + ((e >> 2) & 3)] + 4 * (e >> 4) + (e & 3)] = (e >> 4) < dp ? lrow[e] : row[e];
+    }
+    __threadfence();
     __syncthreads();
     if (tid == 0) st_release(flags + i, epoch);
   }
@@ -776,6 +793,7 @@ int build_pattern(vms_ctx* ctx, Ilu& p, const Mesh& m) {
     // rows by level, for the factorisation
     std::vector<int32_t> first(N + 1, 0);
     for (int64_t i = 0; i < N; ++i) ++first[level[0][i] + 1];
+    p.n_levels = 1 + *std::max_element(level[0].begin(), level[0].end());
     for (int64_t l = 0; l < N; ++l) first[l + 1] += first[l];
     for (int64_t i = 0; i < N; ++i) order[first[level[0][i]]++] = (int32_t)i;
     farptr[0].push_back(0);
@@ -952,6 +970,9 @@ void free_ilu(Ilu& p) {
   p.spin_limit = lim;
 }
 
+// One warp per row where the levels hold more rows than there are SMs on average (see ilu_factor_kernel).
+static bool factor_wide(const Ilu& p) { return p.n_nodes > (int64_t)sm_count() * p.n_levels; }
+
 int ilu_sweeps64(vms_ctx* ctx, Ilu& p, const Mesh& m) {
   if (p.rec[1]) return VMS_OK;
   cudaError_t e = cudaSuccess;
@@ -993,11 +1014,15 @@ int ilu_factor(vms_ctx* ctx, Ilu& p, const Mesh& m, bool fp32, const void* value
     *launches += convert<float, double>((const float*)values, p.vals64, m.nnz, st);
     A = p.vals64;
   }
-  const unsigned ctas = resident_ctas(m.n_nodes, 1, 4 * sm_count());
+  const bool wide = factor_wide(p);
+  const unsigned ctas = resident_ctas(m.n_nodes, 1, (wide ? FACTOR_WIDE_CTAS : FACTOR_CTAS) * sm_count());
   const uint32_t ep = next_epoch(p, st);
-  ilu_factor_kernel<double><<<ctas, ILU_FWARPS * 32, 0, st>>>(
-      m.rowptr, m.colidx, A, p.F, p.Dinv, p.dpos, p.lptr, p.pptr, p.pairs, p.order, m.n_nodes, p.flags, ep,
-      p.tickets, p.base, p.err, p.spin_limit);
+  auto go = [&](auto kern, int warps) {
+    kern<<<ctas, warps * 32, 0, st>>>(m.rowptr, m.colidx, A, p.F, p.Dinv, p.dpos, p.lptr, p.pptr, p.pairs, p.order,
+                                      m.n_nodes, p.flags, ep, p.tickets, p.base, p.err, p.spin_limit);
+  };
+  if (wide) go(ilu_factor_kernel<double, 1>, 1);
+  else go(ilu_factor_kernel<double, 4>, 4);
   p.base += (unsigned long long)m.n_nodes + ctas;  // + each CTA's last claim
   *launches += 1;
   if (fp32) *launches += pack<float>(p, m, p.rec32, st);

@@ -20,6 +20,7 @@ constexpr int ILU_FAR_MAX = 1024;    // distinct far neighbours on one side of a
 struct Ilu {
   // pattern (built once per mesh, on first use)
   int32_t* order = nullptr;    // rows by their level in the forward dependencies: the order of the factorisation
+  int64_t n_levels = 0;        // of those dependencies
   int32_t* dpos = nullptr;     // n_nodes: position of the diagonal block in the node row
   int32_t* lptr = nullptr;     // n_nodes + 1: first lower-block entry of each node row
   int32_t* pptr = nullptr;     // n_lower + 1: first update pair of each lower block
