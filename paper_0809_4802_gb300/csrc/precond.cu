@@ -732,21 +732,26 @@ int build_pattern(vms_ctx* ctx, Ilu& p, const Mesh& m) {
     dpos[i] = d;
   }
   start[N] = (int32_t)adj.size();
+  std::vector<uint8_t> place(N, 0);  // of row i's neighbours in it, from 1; 0: no neighbour
   for (int64_t i = 0; i < N; ++i) {
     const int32_t* ai = adj.data() + start[i];
     const int degi = start[i + 1] - start[i];
+    for (int jj = 0; jj < degi; ++jj) place[ai[jj]] = (uint8_t)(jj + 1);
     for (int kk = 0; kk < dpos[i]; ++kk) {
       const int32_t k = ai[kk];
       const int32_t* ak = adj.data() + start[k];
       const int degk = start[k + 1] - start[k];
-      int jj = kk + 1;
-      for (int jk = dpos[k] + 1; jk < degk; ++jk) {
-        const int32_t j = ak[jk];
-        while (jj < degi && ai[jj] < j) ++jj;
-        if (jj < degi && ai[jj] == j) pairs.push_back((uint16_t)(jj | (jk << 8)));
+      uint16_t found[ILU_MAX_DEG];
+      int n = 0;
+      for (int jk = dpos[k] + 1; jk < degk; ++jk) {  // without a branch: in random order none could be predicted
+        const int jj = place[ak[jk]];
+        found[n] = (uint16_t)((jj - 1) | (jk << 8));
+        n += jj != 0;
       }
+      pairs.insert(pairs.end(), found, found + n);
       pptr.push_back((int32_t)pairs.size());
     }
+    for (int jj = 0; jj < degi; ++jj) place[ai[jj]] = 0;
     lptr[i + 1] = lptr[i] + dpos[i];
   }
   if (pairs.size() >= (size_t)INT32_MAX)
@@ -798,40 +803,41 @@ int build_pattern(vms_ctx* ctx, Ilu& p, const Mesh& m) {
     for (int64_t i = 0; i < N; ++i) order[first[level[0][i]]++] = (int32_t)i;
     farptr[0].push_back(0);
     farptr[1].push_back(0);
+    std::vector<uint64_t> lists[2];  // far neighbours of a chunk, level and node
     for (int32_t lo = 0; lo < n_segs;) {
       int32_t hi = std::min(lo + ILU_CHUNK, n_segs);
       for (;; --hi) {
         const int32_t a = seg[lo], b = seg[hi];
-        size_t most = 0;
-        std::vector<int32_t> lists[2];
-        for (int side = 0; side < 2; ++side) {
-          for (int32_t t = start[a]; t < start[b]; ++t) {
-            const int32_t j = adj[t];
-            if ((side ? j >= b : j < a) && mark[j] == -1) {
-              mark[j] = 0;
-              lists[side].push_back(j);
-            }
+        for (int32_t t = start[a]; t < start[b]; ++t) {
+          const int32_t j = adj[t];
+          if (j >= a && j < b) {
+            at[t] = 1 + j - a;
+          } else if (mark[j] == -1) {
+            const int side = j >= b;
+            mark[j] = 0;
+            lists[side].push_back((uint64_t)level[side][j] << 32 | (uint32_t)j);
           }
-          std::sort(lists[side].begin(), lists[side].end(), [&](int32_t x, int32_t y) {
-            return level[side][x] != level[side][y] ? level[side][x] < level[side][y] : x < y;
-          });
-          for (size_t k = 0; k < lists[side].size(); ++k) mark[lists[side][k]] = (int32_t)k;
-          for (int32_t i = a; i < b; ++i)
-            for (int32_t t = start[i]; t < start[i + 1]; ++t) {
-              const int32_t j = adj[t];
-              if (j >= a && j < b) at[t] = 1 + j - a;
-              else if (side ? j >= b : j < a) at[t] = 1 + b - a + mark[j];
-            }
-          for (int32_t j : lists[side]) mark[j] = -1;
-          most = std::max(most, lists[side].size());
         }
-        if (most > (size_t)ILU_FAR_MAX && hi > lo + 1) continue;
+        for (auto& list : lists) {
+          std::sort(list.begin(), list.end());
+          for (size_t k = 0; k < list.size(); ++k) mark[(uint32_t)list[k]] = (int32_t)k;
+        }
+        const size_t most = std::max(lists[0].size(), lists[1].size());
+        const bool fits = most <= (size_t)ILU_FAR_MAX || hi == lo + 1;
+        if (fits) {
+          for (int32_t t = start[a]; t < start[b]; ++t)
+            if (adj[t] < a || adj[t] >= b) at[t] = 1 + b - a + mark[adj[t]];
+          p.slots = std::max(p.slots, 1 + (int)(b - a + (int32_t)most));
+        }
         for (int side = 0; side < 2; ++side) {
-          far[side].insert(far[side].end(), lists[side].begin(), lists[side].end());
-          farptr[side].push_back((int32_t)far[side].size());
+          for (uint64_t e : lists[side]) {
+            mark[(uint32_t)e] = -1;
+            if (fits) far[side].push_back((int32_t)(uint32_t)e);
+          }
+          if (fits) farptr[side].push_back((int32_t)far[side].size());
+          lists[side].clear();
         }
-        p.slots = std::max(p.slots, 1 + (int)(b - a + (int32_t)most));
-        break;
+        if (fits) break;
       }
       chunk.push_back(hi);
       lo = hi;
