@@ -96,11 +96,16 @@ __device__ __forceinline__ void ts_phase1(int lane, int nq, WarpArea<double>& W,
   double det = cofactor3(J, cof);
   if (!det_ok(det)) { W.flag = 1u; det = 1.0; }
   const double nr = nut * recip_normal(det), tom = tau * (wq * det);
-  double P[3][3], omd[3];  // omega (J^-1)[al][j] = w cof[j][al]; omega d
+  // omega (J^-1)[al][j] = w cof[j][al]; nut (J^-1)[al][j] (the product of two cofactors, divided by det J after it,
+  // would be subnormal for edges below 1e-77); omega d
+  double P[3][3], Q[3][3], omd[3];
 #pragma unroll
   for (int al = 0; al < 3; ++al)
 #pragma unroll
-    for (int j = 0; j < 3; ++j) P[al][j] = wq * cof[j][al];
+    for (int j = 0; j < 3; ++j) {
+      P[al][j] = wq * cof[j][al];
+      Q[al][j] = nr * cof[j][al];
+    }
 #pragma unroll
   for (int j = 0; j < 3; ++j) omd[j] = db[0] * P[0][j] + db[1] * P[1][j] + db[2] * P[2][j];
   const double omcd = v[0] * omd[0] + v[1] * omd[1] + v[2] * omd[2];
@@ -116,7 +121,7 @@ __device__ __forceinline__ void ts_phase1(int lane, int nq, WarpArea<double>& W,
   const int pa[6] = {0, 1, 2, 0, 0, 1}, pb[6] = {0, 1, 2, 1, 2, 2};
 #pragma unroll
   for (int m = 0; m < 6; ++m) {
-    const double g = nr * (P[pa[m]][0] * cof[0][pb[m]] + P[pa[m]][1] * cof[1][pb[m]] + P[pa[m]][2] * cof[2][pb[m]]);
+    const double g = P[pa[m]][0] * Q[pb[m]][0] + P[pa[m]][1] * Q[pb[m]][1] + P[pa[m]][2] * Q[pb[m]][2];
     Gm[pa[m]][pb[m]] = Gm[pb[m]][pa[m]] = g;
     F[(TF_G + m) * ld + q] = g;
   }

@@ -334,15 +334,17 @@ __device__ __forceinline__ void tet_element(int a, int64_t e, const double4_32a*
     E.Ab = gsum(ab) + M[TM_MBBD] * br[0] + M[TM_MBBD + 1] * br[1] + M[TM_MBBD + 2] * br[2];
   }
   E.Pbar = M[TM_M1] * P[0] + M[TM_M1 + 1] * P[1] + M[TM_M1 + 2] * P[2] + M[TM_M1 + 3] * P[3];
-  // DD = int d.d = sum_{al,be} Mdd[al][be] (C C^T)[al][be] / det: row a of C C^T on lane a
+  // DD = int d.d = sum_{al,be} Mdd[al][be] (C C^T)[al][be] / det: row a of C C^T / det on lane a (a product of two
+  // cofactors by itself would be subnormal for edges below 1e-77)
   {
+    const double rC[3] = {E.r * Cr[0], E.r * Cr[1], E.r * Cr[2]};
     double dd = 0.0;
 #pragma unroll
     for (int be = 0; be < 3; ++be) {
-      const double jj = Cr[0] * E.C[be][0] + Cr[1] * E.C[be][1] + Cr[2] * E.C[be][2];
+      const double jj = rC[0] * E.C[be][0] + rC[1] * E.C[be][1] + rC[2] * E.C[be][2];
       dd += sel4(a, M[TM_MDD + be], M[TM_MDD + 3 + be], M[TM_MDD + 6 + be], 0.0) * jj;
     }
-    E.DD = E.r * gsum(dd);
+    E.DD = gsum(dd);
   }
   // Pd[al] = int p d_al (reference): component a on lane a; then PdJ = C^T Pd and
   // Dint = C^T Md, component a on lane a
@@ -390,14 +392,17 @@ __device__ __forceinline__ double dot3(const double x[3], const double y[3]) {
 // convective and the viscous term of node a), the bubble's viscous term with lambda_a, and the diagonal
 // of K_ff.
 struct TetTerms {
-  double w[3], gD, kd;
+  double w[3], nD[3], gD, kd;  // nD = nut D / det
 };
 __device__ __forceinline__ TetTerms tet_terms(const TetElem& E, const double* __restrict__ M, double nut) {
   TetTerms t;
   const double nr = nut * E.r, nm = nr * M[TM_M0];
 #pragma unroll
-  for (int j = 0; j < 3; ++j) t.w[j] = E.Ua[j] + nm * E.ga[j];
-  t.gD = nr * dot3(E.ga, E.Dint);
+  for (int j = 0; j < 3; ++j) {
+    t.w[j] = E.Ua[j] + nm * E.ga[j];
+    t.nD[j] = nr * E.Dint[j];
+  }
+  t.gD = dot3(E.ga, t.nD);
   t.kd = E.Ab + nut * E.DD;
   return t;
 }
@@ -405,11 +410,11 @@ __device__ __forceinline__ TetTerms tet_terms(const TetElem& E, const double* __
 // R_cp rows of node a (Eqs. SC_Coarse_Resid_Vec, SC_Coarse_Resid_Vec_2) and R_f (Eq.
 // SC_Fine_Resid_Vec), every lane of the group holding the same R_f.
 __device__ __forceinline__ void tet_residual(int a, const TetElem& E, const TetTerms& t, const double* __restrict__ M,
-                                             const KParams& kp, double nut, double Rcp[4], double Rf[3]) {
-  const double nr = nut * E.r, ca = E.Aa + t.gD;
+                                             const KParams& kp, double Rcp[4], double Rf[3]) {
+  const double ca = E.Aa + t.gD;
   double wb[3];
 #pragma unroll
-  for (int j = 0; j < 3; ++j) wb[j] = E.Ub[j] + nr * E.Dint[j];
+  for (int j = 0; j < 3; ++j) wb[j] = E.Ub[j] + t.nD[j];
 #pragma unroll
   for (int i = 0; i < 3; ++i) {
     Rcp[i] = E.G[i][0] * t.w[0] + (E.G[i][1] * t.w[1] + (E.G[i][2] * t.w[2] + (E.beta[i] * ca - E.ga[i] * E.Pbar)));
@@ -511,7 +516,7 @@ __global__ void __launch_bounds__(TET_WARPS * 32) tet_assembly_kernel(
     tet_element(a, e, xyz, u, up, conn, beta, kp.transient != 0, M, E);
     const TetTerms tt = tet_terms(E, M, nut);
     double Rcp[4], Rf[3];
-    tet_residual(a, E, tt, M, kp, nut, Rcp, Rf);
+    tet_residual(a, E, tt, M, kp, Rcp, Rf);
     const double dtau = kp.transient ? E.det * kp.tau : 0.0;
 
     // K_ff (row a on lane a) and its inverse: row a's cofactors are the cross product of the next two
@@ -709,7 +714,7 @@ __global__ void __launch_bounds__(TET_WARPS * 32) tet_residual_kernel(
     TetElem E;
     tet_element(a, e, xyz, u, up, conn, beta, kp.transient != 0, M, E);
     double Rcp[4], Rf[3];
-    tet_residual(a, E, tet_terms(E, M, nut), M, kp, nut, Rcp, Rf);
+    tet_residual(a, E, tet_terms(E, M, nut), M, kp, Rcp, Rf);
     if (!valid) continue;
     if (!(finite(Rcp[0]) && finite(Rcp[1]) && finite(Rcp[2]) && finite(Rcp[3]) && finite(Rf[0]) &&
           finite(Rf[1]) && finite(Rf[2])))
