@@ -15,8 +15,9 @@ constexpr int ILU_SEG_MAX = 64;
 constexpr int ILU_CHUNK = 4;         // segments of a sweep chunk
 constexpr int ILU_FAR_MAX = 1024;    // distinct far neighbours on one side of a chunk of several segments
 
-// Block ILU(0) of the node-block matrix (4x4 blocks, natural node order), factored and applied on
-// the device by warps that each own one node row and wait for the rows their row depends on.
+// Block ILU(0) of the node-block matrix (4x4 blocks, natural node order), factored and applied on the device:
+// the factorisation by blocks that each eliminate one node row, the sweeps by blocks that each solve the rows of a
+// chunk of segments; both wait for the rows that theirs depend on.
 struct Ilu {
   // pattern (built once per mesh, on first use)
   int32_t* order = nullptr;    // rows by their level in the forward dependencies: the order of the factorisation
@@ -29,7 +30,6 @@ struct Ilu {
   // sweep segments: maximal runs of consecutive nodes each coupled to the one before (at most
   // ILU_SEG_MAX long); segment s is nodes seg[s] .. seg[s+1] - 1
   int32_t* seg = nullptr;           // device, n_segs + 1
-  std::vector<int32_t> seg_host;    // host copy (segment ranges of node blocks)
   int64_t n_segs = 0;
   // chunks of segments: chunk c is segments chunk[c] .. chunk[c+1] - 1, chunk_node its first nodes
   // (host); far[0]/far[1]: its distinct neighbours in earlier / later chunks, from farptr[.][c] on

@@ -49,12 +49,19 @@ template <> struct Row4<float> {
     const float4 t = __ldg(reinterpret_cast<const float4*>(p));
     o[0] = t.x; o[1] = t.y; o[2] = t.z; o[3] = t.w;
   }
+  __device__ __forceinline__ static void st(float* p, const float v[4]) {
+    *reinterpret_cast<float4*>(p) = make_float4(v[0], v[1], v[2], v[3]);
+  }
 };
 template <> struct Row4<double> {
   __device__ __forceinline__ static void ld(const double* p, double o[4]) {
     const double2 a = __ldg(reinterpret_cast<const double2*>(p));
     const double2 b = __ldg(reinterpret_cast<const double2*>(p) + 1);
     o[0] = a.x; o[1] = a.y; o[2] = b.x; o[3] = b.y;
+  }
+  __device__ __forceinline__ static void st(double* p, const double v[4]) {
+    reinterpret_cast<double2*>(p)[0] = make_double2(v[0], v[1]);
+    reinterpret_cast<double2*>(p)[1] = make_double2(v[2], v[3]);
   }
 };
 
@@ -207,190 +214,71 @@ __device__ __forceinline__ double block_reduce(double v, double* sh) {
   return v;
 }
 
-// Four consecutive entries of a vector as doubles (16-byte loads for FP32, two for FP64).
-template <typename VT> struct Quad;
-template <> struct Quad<float> {
-  __device__ __forceinline__ static void ld(const float* p, double o[4]) {
-    const float4 t = *reinterpret_cast<const float4*>(p);
-    o[0] = t.x; o[1] = t.y; o[2] = t.z; o[3] = t.w;
-  }
-  __device__ __forceinline__ static void st(float* p, const double v[4]) {
-    *reinterpret_cast<float4*>(p) = make_float4((float)v[0], (float)v[1], (float)v[2], (float)v[3]);
-  }
-};
-template <> struct Quad<double> {
-  __device__ __forceinline__ static void ld(const double* p, double o[4]) {
-    const double2 a = reinterpret_cast<const double2*>(p)[0], b = reinterpret_cast<const double2*>(p)[1];
-    o[0] = a.x; o[1] = a.y; o[2] = b.x; o[3] = b.y;
-  }
-  __device__ __forceinline__ static void st(double* p, const double v[4]) {
-    reinterpret_cast<double2*>(p)[0] = make_double2(v[0], v[1]);
-    reinterpret_cast<double2*>(p)[1] = make_double2(v[2], v[3]);
-  }
-};
-
-constexpr int MD_K = 8;          // vectors per block of the multi-dot and per step of the combine
+constexpr int MD_K = 8;          // vector loads in flight per thread of the combine
 constexpr int MD_THREADS = 256;
 constexpr int MD_MAX_BLOCKS = 256;
-constexpr int H_SIZE = H_PART + (MAX_RESTART + 1) * MD_MAX_BLOCKS;
+constexpr int H_SIZE = H_PART + MD_MAX_BLOCKS;
 
-// partial[k * nb + bx] = this block's share of V_k . w for k in [MD_K by, MD_K by + MD_K) and
-// k < m (FP64 accumulation). Rows are taken four at a time (quad) when every vector allows it.
+// partial[bx] = this block's share of v . v (n4 quads of entries). FP64 accumulation; of an FP32 vector each thread's
+// squares and the warp's sum (at most 128 squares in the usual one quad per thread) are formed in FP32: the FP64
+// pipe, 1/64 of FP32, would otherwise bound the kernel.
 template <typename VT>
-__global__ void __launch_bounds__(MD_THREADS) mdot_kernel(const VT* __restrict__ V, int64_t ld, int m,
-                                                          const VT* __restrict__ w, int64_t n,
-                                                          bool quad, double* __restrict__ partial) {
-  __shared__ double sh[MD_K][MD_THREADS / 32];
-  const int k0 = blockIdx.y * MD_K;
-  const int nb = gridDim.x;
-  double acc[MD_K];
+__global__ void __launch_bounds__(MD_THREADS) norm2_kernel(const VT* __restrict__ v, int64_t n4, double* __restrict__ partial) {
+  __shared__ double sh[MD_THREADS / 32];
+  VT acc = VT(0);
+  for (int64_t i = (int64_t)blockIdx.x * MD_THREADS + threadIdx.x; i < n4; i += (int64_t)gridDim.x * MD_THREADS) {
+    VT x[4];
+    Row4<VT>::ld(v + 4 * i, x);
 #pragma unroll
-  for (int t = 0; t < MD_K; ++t) acc[t] = 0.0;
-  const int lane = threadIdx.x & 31, wp = threadIdx.x >> 5;
-  if (quad && sizeof(VT) == 4) {
-    // FP32 vectors: each thread's products and the warp's sum (at most 128 products per warp in
-    // the usual one quad per thread) are formed in FP32, the warps' and blocks' sums in FP64: the
-    // FP64 pipe, 1/64 of FP32, would otherwise bound the kernel
-    float accf[MD_K];
-#pragma unroll
-    for (int t = 0; t < MD_K; ++t) accf[t] = 0.f;
-    const int64_t n4 = n >> 2;
-    const float4* w4 = reinterpret_cast<const float4*>(w);
-    for (int64_t i = (int64_t)blockIdx.x * MD_THREADS + threadIdx.x; i < n4; i += (int64_t)nb * MD_THREADS) {
-      const float4 wv = w4[i];
-      float4 vv[MD_K];
-#pragma unroll
-      for (int t = 0; t < MD_K; ++t)
-        if (k0 + t < m) vv[t] = reinterpret_cast<const float4*>(V + (int64_t)(k0 + t) * ld)[i];
-#pragma unroll
-      for (int t = 0; t < MD_K; ++t)
-        if (k0 + t < m)
-          accf[t] = fmaf(vv[t].w, wv.w, fmaf(vv[t].z, wv.z, fmaf(vv[t].y, wv.y, fmaf(vv[t].x, wv.x, accf[t]))));
-    }
-#pragma unroll
-    for (int t = 0; t < MD_K; ++t) {
-      float v = accf[t];
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) sh[t][wp] = (double)v;
-    }
-  } else {
-    if (quad) {
-      const int64_t n4 = n >> 2;
-      for (int64_t i = (int64_t)blockIdx.x * MD_THREADS + threadIdx.x; i < n4; i += (int64_t)nb * MD_THREADS) {
-        double wv[4], vv[MD_K][4];
-        Quad<VT>::ld(w + 4 * i, wv);
-#pragma unroll
-        for (int t = 0; t < MD_K; ++t)
-          if (k0 + t < m) Quad<VT>::ld(V + (int64_t)(k0 + t) * ld + 4 * i, vv[t]);
-#pragma unroll
-        for (int t = 0; t < MD_K; ++t)
-          if (k0 + t < m)
-            acc[t] = fma(vv[t][3], wv[3], fma(vv[t][2], wv[2], fma(vv[t][1], wv[1], fma(vv[t][0], wv[0], acc[t]))));
-      }
-    } else {
-      for (int64_t i = (int64_t)blockIdx.x * MD_THREADS + threadIdx.x; i < n; i += (int64_t)nb * MD_THREADS) {
-        const double wi = (double)w[i];
-#pragma unroll
-        for (int t = 0; t < MD_K; ++t)
-          if (k0 + t < m) acc[t] = fma((double)V[(int64_t)(k0 + t) * ld + i], wi, acc[t]);
-      }
-    }
-#pragma unroll
-    for (int t = 0; t < MD_K; ++t) {
-      double v = acc[t];
-      for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-      if (lane == 0) sh[t][wp] = v;
-    }
+    for (int t = 0; t < 4; ++t) acc = fma(x[t], x[t], acc);
   }
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = (double)acc;
   __syncthreads();
-  if (threadIdx.x < MD_K && k0 + (int)threadIdx.x < m) {
-    double v = 0.0;
-    for (int q = 0; q < MD_THREADS / 32; ++q) v += sh[threadIdx.x][q];
-    partial[(int64_t)(k0 + threadIdx.x) * nb + blockIdx.x] = v;
+  if (threadIdx.x == 0) {
+    double s = 0.0;
+    for (int q = 0; q < MD_THREADS / 32; ++q) s += sh[q];
+    partial[blockIdx.x] = s;
   }
 }
 
-// out[k] = sum_b partial[k * nb + b], one block per k
+// *out = sum_b partial[b], one block
 __global__ void __launch_bounds__(DOT_THREADS) reduce_partials_kernel(const double* __restrict__ partial,
                                                                       int nb, double* __restrict__ out) {
   __shared__ double sh[DOT_THREADS / 32];
-  const int k = blockIdx.x;
   double s = 0.0;
-  for (int b = threadIdx.x; b < nb; b += DOT_THREADS) s += partial[(int64_t)k * nb + b];
+  for (int b = threadIdx.x; b < nb; b += DOT_THREADS) s += partial[b];
   s = block_reduce(s, sh);
-  if (threadIdx.x == 0) out[k] = s;
+  if (threadIdx.x == 0) *out = s;
 }
 
-// out = (base ? base : 0) + sign * sum_{k < m} c[k] V_k, rows four at a time when aligned, with
-// MD_K vector loads in flight per thread
+// out = sum_{k < m} c[k] V_k in the vectors' type (FP32: the inner solve's working precision), V_k = V + k ld, four
+// rows at a time with MD_K loads in flight per thread
 template <typename VT>
-__global__ void __launch_bounds__(256) vcomb_kernel(const VT* __restrict__ V, int64_t ld,
-                                                    const double* __restrict__ c, int m, double sign,
-                                                    const VT* base, VT* out, int64_t n, bool quad) {
-  __shared__ double cs[MAX_RESTART + 1];
-  __shared__ float cs32[MAX_RESTART + 1];
-  for (int k = threadIdx.x; k < m; k += blockDim.x) {
-    cs[k] = sign * c[k];
-    cs32[k] = (float)(sign * c[k]);
-  }
+__global__ void __launch_bounds__(256) vcomb_kernel(const VT* __restrict__ V, int64_t ld, const double* __restrict__ c, int m,
+                                                    VT* out, int64_t n4) {
+  __shared__ VT cs[MAX_RESTART + 1];
+  for (int k = threadIdx.x; k < m; k += blockDim.x) cs[k] = (VT)c[k];
   __syncthreads();
-  if (quad && sizeof(VT) == 4) {
-    // FP32 vectors are combined in FP32 (the inner solve's working precision)
-    const int64_t n4 = n >> 2;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4;
-         i += (int64_t)gridDim.x * blockDim.x) {
-      float4 s = base ? reinterpret_cast<const float4*>(base)[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-      int k = 0;
-      for (; k + MD_K <= m; k += MD_K) {
-        float4 vv[MD_K];
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (int64_t)gridDim.x * blockDim.x) {
+    VT s[4] = {VT(0), VT(0), VT(0), VT(0)};
+    int k = 0;
+    for (; k + MD_K <= m; k += MD_K) {
+      VT vv[MD_K][4];
 #pragma unroll
-        for (int t = 0; t < MD_K; ++t) vv[t] = reinterpret_cast<const float4*>(V + (int64_t)(k + t) * ld)[i];
+      for (int t = 0; t < MD_K; ++t) Row4<VT>::ld(V + (int64_t)(k + t) * ld + 4 * i, vv[t]);
 #pragma unroll
-        for (int t = 0; t < MD_K; ++t) {
-          const float ct = cs32[k + t];
-          s.x = fmaf(ct, vv[t].x, s.x); s.y = fmaf(ct, vv[t].y, s.y);
-          s.z = fmaf(ct, vv[t].z, s.z); s.w = fmaf(ct, vv[t].w, s.w);
-        }
-      }
-      for (; k < m; ++k) {
-        const float4 vv = reinterpret_cast<const float4*>(V + (int64_t)k * ld)[i];
-        const float ct = cs32[k];
-        s.x = fmaf(ct, vv.x, s.x); s.y = fmaf(ct, vv.y, s.y);
-        s.z = fmaf(ct, vv.z, s.z); s.w = fmaf(ct, vv.w, s.w);
-      }
-      reinterpret_cast<float4*>(out)[i] = s;
+      for (int t = 0; t < MD_K; ++t)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) s[e] = fma(cs[k + t], vv[t][e], s[e]);
     }
-  } else if (quad) {
-    const int64_t n4 = n >> 2;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4;
-         i += (int64_t)gridDim.x * blockDim.x) {
-      double s[4] = {0.0, 0.0, 0.0, 0.0};
-      if (base) Quad<VT>::ld(base + 4 * i, s);
-      int k = 0;
-      for (; k + MD_K <= m; k += MD_K) {
-        double vv[MD_K][4];
+    for (; k < m; ++k) {
+      VT vv[4];
+      Row4<VT>::ld(V + (int64_t)k * ld + 4 * i, vv);
 #pragma unroll
-        for (int t = 0; t < MD_K; ++t) Quad<VT>::ld(V + (int64_t)(k + t) * ld + 4 * i, vv[t]);
-#pragma unroll
-        for (int t = 0; t < MD_K; ++t)
-#pragma unroll
-          for (int e = 0; e < 4; ++e) s[e] = fma(cs[k + t], vv[t][e], s[e]);
-      }
-      for (; k < m; ++k) {
-        double vv[4];
-        Quad<VT>::ld(V + (int64_t)k * ld + 4 * i, vv);
-#pragma unroll
-        for (int e = 0; e < 4; ++e) s[e] = fma(cs[k], vv[e], s[e]);
-      }
-      Quad<VT>::st(out + 4 * i, s);
+      for (int e = 0; e < 4; ++e) s[e] = fma(cs[k], vv[e], s[e]);
     }
-  } else {
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n;
-         i += (int64_t)gridDim.x * blockDim.x) {
-      double s = base ? (double)base[i] : 0.0;
-      for (int k = 0; k < m; ++k) s = fma(cs[k], (double)V[(int64_t)k * ld + i], s);
-      out[i] = VT(s);
-    }
+    Row4<VT>::st(out + 4 * i, s);
   }
 }
 
@@ -438,37 +326,21 @@ static unsigned grid_for(int64_t n) {
   return (unsigned)(b > cap ? cap : (b < 1 ? 1 : b));
 }
 
-// Rows can be taken four at a time when the length, the stride and every pointer allow 16-byte
-// (FP32) or 32-byte (FP64) accesses.
-static bool quad_ok(int64_t n, int64_t ld, size_t elem, std::initializer_list<const void*> ptrs) {
-  if ((n & 3) || (ld & 3)) return false;
-  for (const void* q : ptrs)
-    if (q && ((uintptr_t)q % (4 * elem))) return false;
-  return true;
-}
-
-// out[k] = V_k . w for k < m (m <= MAX_RESTART + 1), FP64 accumulation; `partial` holds
-// m * MD_MAX_BLOCKS doubles. Returns the launches.
+// *out = v . v for a solver's vector (n a multiple of 4, v 16-byte aligned); `partial` holds MD_MAX_BLOCKS doubles.
+// Returns the launches.
 template <typename VT>
-static int dots(const VT* V, int64_t ld, int m, const VT* w, int64_t n, double* partial,
-                double* out, cudaStream_t st) {
-  const bool quad = quad_ok(n, ld, sizeof(VT), {V, w});
-  const int groups = (m + MD_K - 1) / MD_K;
-  const int64_t units = quad ? n / 4 : n;
-  int64_t nb = (4 * (int64_t)sm_count() + groups - 1) / groups;  // about four blocks per SM in all
-  nb = std::min<int64_t>(nb, (units + MD_THREADS - 1) / MD_THREADS);
-  nb = std::max<int64_t>(1, std::min<int64_t>(nb, MD_MAX_BLOCKS));
-  mdot_kernel<VT><<<dim3((unsigned)nb, (unsigned)groups), MD_THREADS, 0, st>>>(V, ld, m, w, n, quad, partial);
-  reduce_partials_kernel<<<m, DOT_THREADS, 0, st>>>(partial, (int)nb, out);
+static int norm2(const VT* v, int64_t n, double* partial, double* out, cudaStream_t st) {
+  const int64_t n4 = n / 4;
+  const int64_t nb = std::max<int64_t>(1, std::min<int64_t>({4 * (int64_t)sm_count(), (n4 + MD_THREADS - 1) / MD_THREADS, MD_MAX_BLOCKS}));
+  norm2_kernel<VT><<<(unsigned)nb, MD_THREADS, 0, st>>>(v, n4, partial);
+  reduce_partials_kernel<<<1, DOT_THREADS, 0, st>>>(partial, (int)nb, out);
   return 2;
 }
 
-// out = (base ? base : 0) + sign * sum_{k < m} c[k] V_k (c on the device). Returns the launches.
+// out = sum_{k < m} c[k] V_k (c on the device). Returns the launches.
 template <typename VT>
-static int vcomb(const VT* V, int64_t ld, const double* c, int m, double sign, const VT* base,
-                 VT* out, int64_t n, cudaStream_t st) {
-  const bool quad = quad_ok(n, ld, sizeof(VT), {V, base, out});
-  vcomb_kernel<VT><<<grid_for(quad ? n / 4 : n), 256, 0, st>>>(V, ld, c, m, sign, base, out, n, quad);
+static int vcomb(const VT* V, int64_t ld, const double* c, int m, VT* out, int64_t n, cudaStream_t st) {
+  vcomb_kernel<VT><<<grid_for(n / 4), 256, 0, st>>>(V, ld, c, m, out, n / 4);
   return 1;
 }
 
@@ -587,7 +459,7 @@ struct Gmres {
       // V_0 = r / |r|
       {
         KScope k(ctx, VMS_K_REDUCE);
-        k.add(dots<VT>(V, n, 1, V, n, hd + H_PART, hd + H_NORM, st));
+        k.add(norm2<VT>(V, n, hd + H_PART, hd + H_NORM, st));
       }
       int rc = sync_host(&res, hd + H_NORM, sizeof(double));
       if (rc) return rc;
@@ -672,11 +544,11 @@ struct Gmres {
       cudaMemcpyAsync(hd + H_Y, y.data(), sizeof(double) * j, cudaMemcpyHostToDevice, st);
       if (Zflex) {  // x += Z y with the kept preconditioned vectors
         KScope k(ctx, VMS_K_KRYLOV);
-        k.add(vcomb<VT>(reinterpret_cast<const VT*>(Zflex), n, hd + H_Y, j, 1.0, nullptr, V + n, n, st));
+        k.add(vcomb<VT>(reinterpret_cast<const VT*>(Zflex), n, hd + H_Y, j, V + n, n, st));
       } else {      // x += M^-1 V y
         {
           KScope k(ctx, VMS_K_KRYLOV);
-          k.add(vcomb<VT>(V, n, hd + H_Y, j, 1.0, nullptr, z, n, st));
+          k.add(vcomb<VT>(V, n, hd + H_Y, j, z, n, st));
         }
         precond<T, VT>(z, V + n);
       }
@@ -717,7 +589,7 @@ struct Gmres {
       // true residual norm for the next cycle's test is computed at the top of the loop
       if (!(res > rtol * bnorm)) {
         KScope k(ctx, VMS_K_REDUCE);
-        k.add(dots<VT>(V, n, 1, V, n, hd + H_PART, hd + H_NORM, st));
+        k.add(norm2<VT>(V, n, hd + H_PART, hd + H_NORM, st));
         double r2 = 0.0;
         if (int rc2 = sync_host(&r2, hd + H_NORM, sizeof(double))) return rc2;
         res = std::sqrt(r2);
@@ -813,7 +685,7 @@ static int linear_solve(vms_ctx* ctx, const SysRange& R, double rtol, int maxit,
   double bnorm2 = 0.0;
   {
     KScope k(ctx, VMS_K_REDUCE);
-    dots<double>(w.r, n, 1, w.r, n, hd + H_PART, hd + H_NORM, st);
+    norm2<double>(w.r, n, hd + H_PART, hd + H_NORM, st);
     k.add(2);
   }
   Gmres G{ctx, m, w, st, n, R};
@@ -891,7 +763,7 @@ static int linear_solve(vms_ctx* ctx, const SysRange& R, double rtol, int maxit,
     }
     {
       KScope k(ctx, VMS_K_REDUCE);
-      dots<double>(rfull, n, 1, rfull, n, hd + H_PART, hd + H_NORM, st);
+      norm2<double>(rfull, n, hd + H_PART, hd + H_NORM, st);
       k.add(2);
     }
     if ((rc = G.sync_host(&r2, hd + H_NORM, sizeof(double)))) break;
@@ -966,7 +838,7 @@ static int linear_solve(vms_ctx* ctx, const SysRange& R, double rtol, int maxit,
       }
       {
         KScope k(ctx, VMS_K_REDUCE);
-        dots<double>(rfull, n, 1, rfull, n, hd + H_PART, hd + H_NORM, st);
+        norm2<double>(rfull, n, hd + H_PART, hd + H_NORM, st);
         k.add(2);
       }
       rc = G.sync_host(&r2, hd + H_NORM, sizeof(double));
@@ -1350,10 +1222,10 @@ static int band_direct(vms_ctx* ctx, const SysRange& R, double* rel_out) {
   ks.add(1);
   double* hd = w.h;
   double nb2 = 0.0, nr2 = 0.0;
-  dots<double>(w.rb, n, 1, w.rb, n, hd + H_PART, hd + H_NORM, st);
+  norm2<double>(w.rb, n, hd + H_PART, hd + H_NORM, st);
   cudaMemcpyAsync(&nb2, hd + H_NORM, sizeof(double), cudaMemcpyDeviceToHost, st);
   e = cudaStreamSynchronize(st);
-  dots<double>(y, n, 1, y, n, hd + H_PART, hd + H_NORM, st);
+  norm2<double>(y, n, hd + H_PART, hd + H_NORM, st);
   ks.add(4);
   cudaMemcpyAsync(&nr2, hd + H_NORM, sizeof(double), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
