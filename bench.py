@@ -33,19 +33,19 @@ UNIT = "elements/s"
 # ~300, tangent blocks K_vv ~1.7k + K_vp ~0.4k + fine-coupled blocks ~0.5k) plus the condensation
 # (~7k flops per element). The kernels execute fewer flops than these counts where their
 # formulation needs fewer; `executed` gives ncu opcode counts (FMA = 2 flops) on the 32^3 cavity:
-# the FP64 residual's line-factored monomial form 8,038, the FP64 tangent's factorised sums 37,739,
+# the FP64 residual's line-factored monomial form 8,038, the FP64 tangent's factorised sums 37,820,
 # the fused kernel's FP64 part (residual + the tangent's FP64 K_ff work) 8,490, the tetrahedral
-# kernel 4,382 (21^3 tetrahedral cavity).
+# kernel 4,407 (21^3 tetrahedral cavity).
 ALG_FLOPS = {"residual": (600 + 300) * 27, "tangent": (600 + 1700 + 400 + 500) * 27 + 7000}
-EXECUTED_FLOPS = {"residual": 8_038, "tangent_fp64": 37_739, "fused_fp64": 8_490, "tet": 4_382}
+EXECUTED_FLOPS = {"residual": 8_038, "tangent_fp64": 37_820, "fused_fp64": 8_490, "tet": 4_407}
 
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from ncu captures of the
 # current kernels on the named workloads (profiles/); no entry where none was taken.
-NCU_TRAFFIC_BYTES = {("fused", "cavity32_re400_mixed"): 68_558_848 + 34_623_744,
-                     ("fused", "channel_re1000_mixed"): 2_074_687_744 + 3_088_019_200,
-                     ("residual", "cavity32_re400_fp64"): 4_220_928 + 256,
-                     ("tangent", "cavity32_re400_fp64"): 119_526_656 + 101_442_816,
-                     ("tangent", "tetcavity21_re400_mixed"): 15_452_928 + 25_088}
+NCU_TRAFFIC_BYTES = {("fused", "cavity32_re400_mixed"): 68_583_424 + 34_924_544,
+                     ("fused", "channel_re1000_mixed"): 2_090_000_000 + 3_080_000_000,
+                     ("residual", "cavity32_re400_fp64"): 4_220_672 + 256,
+                     ("tangent", "cavity32_re400_fp64"): 119_561_216 + 101_812_224,
+                     ("tangent", "tetcavity21_re400_mixed"): 15_458_304 + 29_696}
 
 WORKLOADS = {
     # the 32^3 jittered lid-driven cavity at Re 400, random state (mixed precision by default)

@@ -221,7 +221,7 @@ __device__ void dense1_tanh(SmemGrad<ROWS>& s) {
 // and two CTAs fit) -> tanh -> the 4-wide output layer in FP32 as the values leave tensor memory. H2 and D2
 // never touch shared memory, H1 only as an operand.
 // Bound by instruction issue and the FP32 pipe (tanh, the split); the products alone would take 60 us of
-// the 188 us for 975,583 rows. With mma.sync from FP32 tiles in shared memory, bound by the traffic there, it
+// the 191 us for 975,583 rows. With mma.sync from FP32 tiles in shared memory, bound by the traffic there, it
 // took 661 us (1,024 rows 14.5, now 10.8; 100,000 79, now 29), with errors against 64 bits of 4.7e-7 rms, now
 // 3.9e-7 (the low terms are summed first).
 constexpr int FT = 128;                       // rows per tile
@@ -316,9 +316,13 @@ __device__ __forceinline__ Terms finite_terms(float x) {
   return t;
 }
 // tanh of two values: x N(x^2) / D(x^2) with N of degree 4 and D of degree 5, the minimax quotient on [0, 9.02]
-// (relative error 1e-9; fitted with the Remez exchange algorithm in 40 digits), beyond which tanh rounds to +-1.
-// 3e-8 rms from tanh, against 4e-7 of the network's output from the sums of its products. Branch-free and two
-// at a time: the tile is bound by instruction issue, and tanhf took two thirds of it (975,583 rows 214 us).
+// (fitted with the Remez exchange algorithm in 40 digits), beyond which tanh rounds to +-1. Its relative error is 1.1e-8
+// with the coefficients rounded to FP32 and, evaluated in FP32, 6.4e-8 rms and at most 2.8e-7 over 28,000 arguments
+// (tanhf: 2.6e-8 and 1.7e-7), largest near +-8.8, where a value may also be 1 + 2^-22. The sums of products leave
+// more: the output's error is 0.80 to 0.88 of the earlier kernel's rms (mma.sync, tanhf) on inputs of unit variance and
+// initial weights, and over 45 settings of weights (1 to 10 times) and inputs (0.01 to 100) 0.36 to 1.10 of it (above 1
+// in one) and 0.16 to 0.99 of its largest. Branch-free and two at a time: the tile is bound by instruction issue, and
+// tanhf took two thirds of it (975,583 rows 214 us, now 191).
 constexpr float NTH1 = 0.137853637f, NTH2 = 0.00400850875f, NTH3 = 3.15890575e-05f, NTH4 = 5.07622211e-08f;
 constexpr float DTH1 = 0.471186966f, DTH2 = 0.0277375113f, DTH3 = 0.000420740689f, DTH4 = 1.61748528e-06f,
                 DTH5 = 7.37443662e-10f;

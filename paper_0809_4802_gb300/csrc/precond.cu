@@ -212,8 +212,8 @@ __global__ void __launch_bounds__(FW * 32, FW == 1 ? FACTOR_WIDE_CTAS : FACTOR_C
 // data, 39 MB of FP32 records, would take 6 us of HBM. So everything off the chain is moved off the
 // warp that solves a row: values of earlier chunks are fetched by one warp, records by another, and
 // a row is one sum of block products without a test in its way. Measured on 33^3 nodes (jittered
-// cavity): FP32 sweep 239 -> 129 us, FP64 524 -> 260 us; 22^3 nodes of a tetrahedral mesh 57 -> 47
-// and 160 -> 67 us. What is left: a row takes about 0.2 us (FP32; FP64 11 instructions of 64 cycles
+// cavity): FP32 sweep 239 -> 127 us, FP64 524 -> 260 us; 22^3 nodes of a tetrahedral mesh 57 -> 46
+// and 160 -> 65 us; in random node order, where rows in flight bound them, 33^3 nodes 61 -> 70 and 184 -> 136 us. What is left: a row takes about 0.2 us (FP32; FP64 11 instructions of 64 cycles
 // each on its partition's FP64 unit, about 0.5 us), and a value from another chunk about 0.9 us from
 // its publication to the slot. Four segments a chunk: eight are alike in FP32 and slower in FP64
 // (315 us: the SM's FP64 unit is shared), and a second fetching warp changes nothing.
@@ -1038,7 +1038,7 @@ int ilu_factor(vms_ctx* ctx, Ilu& p, const Mesh& m, bool fp32, const void* value
   return e == cudaSuccess ? VMS_OK : ctx_fail(ctx, VMS_ERR_CUDA, cudaGetErrorString(e));
 }
 
-// Rows without lines: one row a copy and one copy a warp, so that an SM holds more CTAs (FP32 5, FP64 3 instead of 3 and 1
+// Rows without lines: one row a copy and one copy a warp, so that an SM holds more CTAs (FP32 5, FP64 3 instead of 3 and 2
 // on hexahedra); rings for the rows to come stay empty there. A GMRES step's two sweeps in us, with the rings and
 // without, random node order (one row a segment): 33^3 nodes FP32 180, 139, FP64 343, 272; 91^3 2,925, 1,958 and 6,357, 4,863;
 // 40^3 nodes of a tetrahedral mesh 191, 144 and 421, 265. With segments of 5 rows on average (13^3 nodes in reverse

@@ -119,10 +119,12 @@ static void launch_r(const Mesh& m, const State& s, const KParams& kp, const QpR
 // in steps of U and again from there; lines 29 up to 1,728 elements (25; 34), then 14 + 12.6 per
 // thousand (10 + 3.9; 10 + 24). The bounds below are where the two meet. (Both take 5 % less since the
 // lines' sums were shortened: 32,768 elements 371 -> 353, 10,648 142 -> 137.)
-// Beside an FP64 tangent (`beside`) the lines of up to 2 U elements fill the tangent's gaps better:
-// an assembly of 512 elements takes 130 us with lines, 228 with threads, 4,096 362 and 415, 12,167
-// 893 and 1,029, 17,576 1,279 and 1,346, 19,683 1,435 and 1,436; past that the lines' extra FP64 work
-// (a third) costs more than it hides (32,768: 2,318 and 2,253; a part of them in lines: up to 4 % more).
+// Beside a tangent kernel (`beside`) the lines of up to 2 U elements fill the tangent's gaps better. An assembly in us
+// with lines and with threads, FP64; FP32 tangent on a second stream; split-TF32 tangent: 512 elements 109 and 196, 53
+// and 195, 57 and 198; 4,096 303 and 341, 115 and 232, 137 and 222; 6,069 415 and 566, 158 and 316, 177 and 237; 9,702
+// 639 and 858, 232 and 380, 259 and 426; 12,696 822 and 982, 280 and 426, 319 and 463; 17,576 1,129 and 1,229, 386 and
+// 514, 436 and 565. Past 2 U the lines' extra FP64 work (a third) costs more than it hides (32,768 in FP64, before the
+// tangent took a fifth less: 2,318 and 2,253; a part of them in lines: up to 4 % more).
 int64_t residual_rest(int nq, int64_t count, bool beside) {
   const int64_t U = 64 * (int64_t)sm_count(), r = count % (2 * U);
   if (beside) return count <= 2 * U ? count : 0;

@@ -42,7 +42,7 @@ __host__ __device__ inline size_t ts_area_bytes(int nq) {
 // The kernel is bound by the FP64 pipe (19 cycles of an SM per warp instruction, one warp alone 64 each), so
 // every field is taken from ones already formed: with P = omega J^-1 = w cof^T, omega L = G P + beta (omega
 // d)^T, the K_fc coefficients are the K_cf ones transposed, (J^-1 d) comes from J^-1 J^-T, and K_ff from
-// the K_cf coefficients. 250 FP64 instructions for the point instead of 380, of about 700 for an element
+// the K_cf coefficients. About 250 FP64 instructions for the point instead of 380, of 779 for an element
 // (950). Assembly of 13,824 elements in FP64 1,010 -> 900 us.
 // B is the one-dimensional basis table (its row TS_ROW_X holds the Gauss points).
 __device__ __forceinline__ void ts_phase1(int lane, int nq, WarpArea<double>& W, TsArea& C,

@@ -170,8 +170,8 @@ constexpr int TET_PER_WARP = 8;  // tetrahedra per warp
 // det J that turns J^-1 into its cofactors: no entry of J^-1 and no product with det J is formed, only 1 /
 // det J where a product of two gradients needs it. With that, sums started from the value they are
 // subtracted from, y = K_ff^-1 R_f in place of K_cf K_ff^-1, K_ff's rows on the group's lanes and results
-// narrowed to FP32 by integer instructions a warp takes 670 FP64 instructions for its eight elements instead
-// of 1,030: 355,914 elements 2,805 -> 1,745 us in mixed precision, 1,955 in FP64 (the wider scatter).
+// narrowed to FP32 by integer instructions a warp takes 677 FP64 instructions for its eight elements instead
+// of 1,030: 355,914 elements 2,805 -> 1,758 us in mixed precision, 1,970 in FP64 (the wider scatter).
 struct TetElem {
   int nd[4];
   int nda;           // node a
