@@ -300,7 +300,8 @@ int vms_set_graph(vms_ctx* ctx, int enable);
 int vms_set_preconditioner(vms_ctx* ctx, int kind);
 
 /* Limit of every device-side wait of a solve with ILU(0): of its factorisation and sweeps (a row waiting
- * for a row it depends on) and of the Arnoldi step (a block waiting for the others' sums): after `polls` polls (about 32 ns apart) the kernel records a timeout and stops
+ * for a row it depends on) and of the Arnoldi step (a block waiting for the others' sums; 64 times as many, at
+ * most 2^22 or `polls`): after `polls` polls (about 32 ns apart) the kernel records a timeout and stops
  * its remaining work, and the solve returns VMS_ERR_TIMEOUT with the state unchanged; the context
  * stays usable. polls = 0 restores the default (2^22, about 0.13 s). A limit too small for the
  * rows' normal hand-over times makes every ILU(0) solve time out. Not part of the paper's method:

@@ -392,7 +392,9 @@ struct Gmres {
     int64_t nn = n;
     int blocks = (int)std::min<int64_t>({(n / 4 + 127) / 128, (int64_t)sm_count(), (int64_t)OG_BLOCKS});
     double *X = w.og + (w.og_turn ? OG_SET : 0), *Y = w.og + (w.og_turn ? 0 : OG_SET), *out = w.hcol;
-    uint32_t lim = w.use_ilu ? w.ilu.spin_limit : ILU_SPIN_DEFAULT;
+    // the polls of a block for the others' sums are shorter than a row's (no sleep) and wait for whole passes
+    uint32_t lim = w.use_ilu ? (uint32_t)std::min<uint64_t>(64ull * w.ilu.spin_limit, std::max(w.ilu.spin_limit, ILU_SPIN_DEFAULT))
+                             : ILU_SPIN_DEFAULT;
     out[kk + 1] = 0.0;
     void* args[] = {&V, &nn, &kk, &X, &Y, &w.og_k, &w.og_blocks, &lim, &out};
     const cudaError_t e = cudaLaunchCooperativeKernel((const void*)ortho_kernel<VT>, dim3((unsigned)blocks),
