@@ -54,8 +54,8 @@ __device__ __forceinline__ bool wait_ready(const uint32_t* f, uint32_t epoch, in
 // ---------------------------------------------------------------------------------------------
 // factorisation: one CTA per node row; the row is eliminated in shared memory
 //
-// What bounds it where levels are narrow: the chain of rows (224 levels on a lattice of 33^3 nodes, about 160 rows wide), and in a
-// row the FP64 instructions of its block products, 64 cycles each on one warp: 34 for a lower block of 17
+// What bounds it where levels are narrow: the chain of rows (224 levels on a lattice of 33^3 nodes, about 160
+// rows wide), and in a row the FP64 instructions of its block products, 64 cycles each on one warp: 34 for a lower block of 17
 // pairs, and up to three lower blocks were finished only one level before. So a row's pairs are shared
 // by four warps, one per FP64 unit, eight pairs a step; what is known beforehand (neighbours, row starts,
 // pairs) is read before the first wait; U_kk^-1 and the blocks of row k are read as soon as row k is
@@ -213,8 +213,8 @@ __global__ void __launch_bounds__(FW * 32, FW == 1 ? FACTOR_WIDE_CTAS : FACTOR_C
 // warp that solves a row: values of earlier chunks are fetched by one warp, records by another, and
 // a row is one sum of block products without a test in its way. Measured on 33^3 nodes (jittered
 // cavity): FP32 sweep 239 -> 127 us, FP64 524 -> 260 us; 22^3 nodes of a tetrahedral mesh 57 -> 46
-// and 160 -> 65 us; in random node order, where rows in flight bound them, 33^3 nodes 61 -> 70 and 184 -> 136 us. What is left: a row takes about 0.2 us (FP32; FP64 11 instructions of 64 cycles
-// each on its partition's FP64 unit, about 0.5 us), and a value from another chunk about 0.9 us from
+// and 160 -> 65 us; in random node order, where rows in flight bound them, 33^3 nodes 61 -> 70 and 184 -> 136 us.
+// What is left: a row takes about 0.2 us (FP32; FP64 11 instructions of 64 cycles each on its partition's FP64 unit, about 0.5 us), and a value from another chunk about 0.9 us from
 // its publication to the slot. Four segments a chunk: eight are alike in FP32 and slower in FP64
 // (315 us: the SM's FP64 unit is shared), and a second fetching warp changes nothing.
 // ---------------------------------------------------------------------------------------------
@@ -431,8 +431,9 @@ __global__ void sweep_pack_kernel(const int32_t* __restrict__ rowptr, const int3
 // chunk's far list) from the L2 publication as they appear, so that the L2 round trips run beside
 // the rows instead of inside them. The last warp streams the row records and right-hand sides into
 // a ring per compute warp with bulk copies. Chunks are claimed in order by running CTAs, so every
-// wait is for work that is already in progress. The blocks per SM of the launch bounds are what leaves every variant
-// its registers without spills (56 to 168 a thread); left to itself the compiler spilled up to 68 bytes in the row loop.
+// wait is for work that is already in progress. The blocks per SM of the launch bounds leave the variants their
+// registers without spills (44 to 168 a thread; FP64 with 40 places and SHORT spills 84 bytes); left to itself the
+// compiler spilled up to 68 bytes in the row loop.
 template <typename T, bool LOWER, int NP, int W, int FW, bool SHORT>
 __global__ void __launch_bounds__((W + FW + 1) * 32, sizeof(T) == 4 ? (SHORT ? 5 : NP <= 3 ? 4 : 3) : (SHORT ? 3 : 2))
     ilu_sweep_kernel(const unsigned char* __restrict__ rec, const int32_t* __restrict__ seg,
