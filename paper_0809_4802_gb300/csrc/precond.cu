@@ -214,8 +214,8 @@ __global__ void __launch_bounds__(FW * 32, FW == 1 ? FACTOR_WIDE_CTAS : FACTOR_C
 // a row is one sum of block products without a test in its way. Measured on 33^3 nodes (jittered
 // cavity): FP32 sweep 239 -> 127 us, FP64 524 -> 260 us; 22^3 nodes of a tetrahedral mesh 57 -> 46
 // and 160 -> 65 us; in random node order, where rows in flight bound them, 33^3 nodes 61 -> 70 and 184 -> 136 us.
-// What is left: a row takes about 0.2 us (FP32; FP64 11 instructions of 64 cycles each on its partition's FP64 unit, about 0.5 us), and a value from another chunk about 0.9 us from
-// its publication to the slot. Four segments a chunk: eight are alike in FP32 and slower in FP64
+// What is left: a row takes about 0.2 us (FP32; FP64 11 instructions of 64 cycles each on its partition's FP64
+// unit, about 0.5 us), and a value from another chunk about 0.9 us from its publication to the slot. Four segments a chunk: eight are alike in FP32 and slower in FP64
 // (315 us: the SM's FP64 unit is shared), and a second fetching warp changes nothing.
 // ---------------------------------------------------------------------------------------------
 
